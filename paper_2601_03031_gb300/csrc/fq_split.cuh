@@ -26,18 +26,30 @@ struct FqSplitScratch {
 };
 
 namespace fqs {
-// acc[O .. O + 12] += a v (v: 12 limbs), the carry into acc[O + 13]
-template <int O>
-FPG_DEV void row_mac(uint32_t* acc, uint32_t a, const uint32_t* v) {
-    acc[O] = ptx::mad_lo_cc(a, v[0], acc[O]);
+// E + 2^32 D += a v 2^(32 O) for 12 limbs v: the products that start at an even column go to E, the others
+// to D (mp::mont_mul keeps its sum the same way, so that both halves of a product are one instruction);
+// each chain's carry goes up to limb CAP of its accumulator
+template <int O, int CAP>
+FPG_DEV void row_mac(uint32_t* E, uint32_t* D, uint32_t a, const uint32_t* v) {
+    uint32_t* e = E + O + (O & 1);                    // limbs of v of O's parity
+    uint32_t* d = D + O - (O & 1);                    // the others, one column up
+    mp::mac_chain<12, false>(e, v + (O & 1), a);
 #pragma unroll
-    for (int j = 1; j < 12; j++) acc[O + j] = ptx::madc_lo_cc(a, v[j], acc[O + j]);
-    acc[O + 12] = ptx::addc_cc(acc[O + 12], 0);
-    acc[O + 13] = ptx::addc(acc[O + 13], 0);
-    acc[O + 1] = ptx::mad_hi_cc(a, v[0], acc[O + 1]);
+    for (int j = O + (O & 1) + 12; j < CAP; j++) E[j] = ptx::addc_cc(E[j], 0);
+    E[CAP] = ptx::addc(E[CAP], 0);
+    mp::mac_chain<12, false>(d, v + 1 - (O & 1), a);
 #pragma unroll
-    for (int j = 1; j < 12; j++) acc[O + j + 1] = ptx::madc_hi_cc(a, v[j], acc[O + j + 1]);
-    acc[O + 13] = ptx::addc(acc[O + 13], 0);
+    for (int j = O - (O & 1) + 12; j < CAP; j++) D[j] = ptx::addc_cc(D[j], 0);
+    D[CAP] = ptx::addc(D[CAP], 0);
+}
+// r[0 .. N) = limbs 0 .. N - 1 of E + 2^32 D
+template <int N>
+FPG_DEV void row_sum(uint32_t* r, const uint32_t* E, const uint32_t* D) {
+    r[0] = E[0];
+    r[1] = ptx::add_cc(E[1], D[0]);
+#pragma unroll
+    for (int j = 2; j < N - 1; j++) r[j] = ptx::addc_cc(E[j], D[j - 1]);
+    r[N - 1] = ptx::addc(E[N - 1], D[N - 2]);
 }
 
 // the three limbs x_{3w}, x_{3w+1}, x_{3w+2} of warp w, chosen by selects so that every warp runs one
@@ -47,12 +59,13 @@ FPG_DEV uint32_t limb_of_warp(const uint32_t* v, int w, int i) {
 }
 
 FPG_DEV void phase1(FqSplitScratch& sc, int w, int t, const fq& x, const fq& y) {
-    uint32_t P[16];
+    uint32_t E[15], D[15], P[15];
 #pragma unroll
-    for (int j = 0; j < 16; j++) P[j] = 0;
-    row_mac<0>(P, limb_of_warp(x.v, w, 0), y.v);
-    row_mac<1>(P, limb_of_warp(x.v, w, 1), y.v);
-    row_mac<2>(P, limb_of_warp(x.v, w, 2), y.v);
+    for (int j = 0; j < 15; j++) E[j] = D[j] = 0;
+    row_mac<0, 14>(E, D, limb_of_warp(x.v, w, 0), y.v);
+    row_mac<1, 14>(E, D, limb_of_warp(x.v, w, 1), y.v);
+    row_mac<2, 14>(E, D, limb_of_warp(x.v, w, 2), y.v);
+    row_sum<15>(P, E, D);
 #pragma unroll
     for (int k = 0; k < 15; k++) sc.a[w][k][t] = P[k];
 }
@@ -73,28 +86,33 @@ FPG_DEV void phase2(FqSplitScratch& sc, int w, int t) {
         for (int k = 3 * v + 15; k < 24; k++) T[k] = ptx::addc_cc(T[k], 0);
     }
     const uint32_t hi = w == 3 ? 0xffffffffu : 0u;
-    uint32_t A[15];
+    uint32_t A[14], D[14];
 #pragma unroll
-    for (int j = 0; j < 14; j++) A[j] = T[10 + j] & hi;
-    A[14] = 0;
+    for (int j = 0; j < 14; j++) {
+        A[j] = T[10 + j] & hi;
+        D[j] = 0;
+    }
 #pragma unroll
     for (int i = 0; i < 3; i++) {
         const int k = 3 * w + i;
         uint32_t c[12];
 #pragma unroll
         for (int j = 0; j < 12; j++) c[j] = FQ_FOLD[k][j];
-        row_mac<0>(A, limb_of_warp(T, w, i), c);
+        row_mac<0, 13>(A, D, limb_of_warp(T, w, i), c);
     }
+    uint32_t S[14];
+    row_sum<14>(S, A, D);
 #pragma unroll
-    for (int k = 0; k < 14; k++) sc.b[w][k][t] = A[k];
+    for (int k = 0; k < 14; k++) sc.b[w][k][t] = S[k];
 }
 
 FPG_DEV fq phase3(const FqSplitScratch& sc, int t) {
-    uint32_t U[16];
+    uint32_t U[15], D[15], V[15];
 #pragma unroll
     for (int k = 0; k < 14; k++) U[k] = sc.b[0][k][t];
     U[14] = 0;
-    U[15] = 0;
+#pragma unroll
+    for (int k = 0; k < 15; k++) D[k] = 0;
 #pragma unroll
     for (int w = 1; w < 4; w++) {
         U[0] = ptx::add_cc(U[0], sc.b[w][0][t]);
@@ -107,16 +125,17 @@ FPG_DEV fq phase3(const FqSplitScratch& sc, int t) {
     uint32_t pl[12];
 #pragma unroll
     for (int j = 0; j < 12; j++) pl[j] = FQ_P[j];
-    row_mac<0>(U, m0, pl);
-    row_mac<1>(U, m1, pl);
-    fq X, D;
+    row_mac<0, 14>(U, D, m0, pl);
+    row_mac<1, 14>(U, D, m1, pl);
+    row_sum<15>(V, U, D);
+    fq X, Y;
 #pragma unroll
-    for (int j = 0; j < 12; j++) X.v[j] = U[2 + j];
-    D.v[0] = ptx::sub_cc(X.v[0], pl[0]);
+    for (int j = 0; j < 12; j++) X.v[j] = V[2 + j];
+    Y.v[0] = ptx::sub_cc(X.v[0], pl[0]);
 #pragma unroll
-    for (int j = 1; j < 12; j++) D.v[j] = ptx::subc_cc(X.v[j], pl[j]);
-    const uint32_t borrow = ptx::subc(U[14], 0);      // all-ones when X < p
-    return fq_select(borrow != 0, X, D);
+    for (int j = 1; j < 12; j++) Y.v[j] = ptx::subc_cc(X.v[j], pl[j]);
+    const uint32_t borrow = ptx::subc(V[14], 0);      // all-ones when X < p
+    return fq_select(borrow != 0, X, Y);
 }
 }  // namespace fqs
 
