@@ -237,6 +237,90 @@ out.append("__constant__ uint32_t FQ_FOLD[12][12] = {" + ", ".join(
     for k in range(12)) + "};\n")
 out.append(f"#define FQ_PINV64_LO 0x{(-pow(P, -1, 2**64)) % 2**32:08x}u\n")
 out.append(f"#define FQ_PINV64_HI 0x{((-pow(P, -1, 2**64)) % 2**64) >> 32:08x}u\n")
+
+
+# the limb-lane engine (limb.cuh): 15 limbs of 26 bits, one per lane, Montgomery factor 2^390.  Lane l
+# of a slot's 16 holds: the fold constants c_k = 2^(26 k - 338) mod p, k < 13, of output column l + 2
+# (lanes 13 and 14: of columns 0 and 1), and the limbs l + 2 and l + 1 of p for the closing two-limb
+# Montgomery step
+def limbs26(v):
+    return [(v >> (26 * i)) & ((1 << 26) - 1) for i in range(15)] + [0]
+
+
+def rows(name, vals):
+    return (f"static __device__ const int32_t {name}[{len(vals)}][{len(vals[0])}] = {{" +
+            ", ".join("{" + ", ".join(str(v) for v in r) + "}" for r in vals) + "};\n")
+
+
+def mont26(v):
+    return limbs26(v * 2**390 % P)
+
+
+FOLD26 = [limbs26(pow(2, 26 * k - 338, P)) for k in range(13)]
+COL26 = [(lane + 2 if lane < 13 else lane - 13) for lane in range(15)]
+P26 = limbs26(P) + [0, 0]
+out.append(rows("LIMB_FOLD", [[FOLD26[k][c] if c < 15 else 0 for k in range(13)] for c in COL26] + [[0] * 13]))
+out.append(rows("LIMB_P", [[P26[lane + 2] if lane < 13 else 0, P26[lane + 1] if lane < 14 else 0, P26[lane]]
+                           for lane in range(16)]))
+out.append(f"#define LIMB_P0 {P26[0]}\n#define LIMB_P1 {P26[1]}\n")
+out.append(f"#define LIMB_PINV52 0x{(-pow(P, -1, 2**52)) % 2**52:x}ull\n")
+out.append(f"#define LIMB_PTOP_INV {((1 << 32) << 364) // P}\n")
+# factors 2^396 (a residue times 2^384 into the engine's form) and 2^384 (back)
+out.append(rows("LIMB_CONV", [limbs26(2**396 % P), limbs26(2**384 % P)]))
+out.append(rows("LIMB_FROB1", [mont26(FROB1[k][e]) for k in range(6) for e in range(2)]))
+out.append(rows("LIMB_FROB2", [mont26(FROB2[k][0]) for k in range(6)]))
+
+# the final exponentiation as a list of Fq12 operations on value buffers (limb12.cuh runs it): the
+# operation, its destination and one or two sources; destinations differ from sources.  f starts in
+# buffer 0; the first part ends with n u in Fq2 in buffer 3, whose inverse is put into buffer 4 before
+# the second part.  Easy part through norms (n = f conj(f) in Fq6, u = n^(p^2 + p^4), n u in Fq2),
+# g^h1 on the width-4 NAF of h1, then a = g^h1, b = a^(x + p), b^(x^2 + p^2 - 1) g.
+SQR, MUL, MULC, CONJ, FROB, FROB2 = range(6)          # MULC: the second source conjugated
+prog = [(CONJ, 1, 0, 0), (MUL, 2, 0, 1), (FROB2, 3, 2, 0), (FROB2, 4, 3, 0), (MUL, 5, 3, 4), (MUL, 3, 2, 5)]
+split = len(prog)
+prog += [(MUL, 2, 1, 1), (MUL, 3, 2, 5), (MUL, 2, 3, 4), (FROB2, 3, 2, 0), (MUL, 6, 3, 2)]      # g in 6
+prog += [(SQR, 0, 6, 0), (MUL, 3, 0, 6), (MUL, 5, 3, 0), (MUL, 1, 5, 0)]                       # g^3, g^5, g^7
+POW = {1: 6, 3: 3, 5: 5, 7: 1}
+
+
+def chain(cur, digits, power, b0, b1):
+    """cur, then per digit a squaring and, if it is not zero, a product, alternating b0 and b1"""
+    nxt, oth = b0, b1
+    for d in digits:
+        prog.append((SQR, nxt, cur, 0))
+        cur, nxt, oth = nxt, oth, nxt
+        if d:
+            prog.append((MULC if d < 0 else MUL, nxt, cur, power[abs(d)]))
+            cur, nxt, oth = nxt, oth, nxt
+    return cur
+
+
+XBITS = [int(c) for c in bin(XABS)[3:]]
+a = chain(POW[H1_WNAF[-1]], H1_WNAF[-2::-1], POW, 7, 8)
+ax = chain(a, XBITS, {1: a}, 0, 1)
+prog += [(FROB, 2, a, 0), (MULC, 3, 2, ax)]                                                    # b in 3
+bx = chain(3, XBITS, {1: 3}, 0, 1)
+bx2 = chain(bx, XBITS, {1: bx}, 4, 5)
+prog += [(FROB2, 7, 3, 0), (MUL, 8, bx2, 7), (MULC, 7, 8, 3), (MUL, 2, 7, 6)]                  # result in 2
+assert all(d != s and d != t for _, d, s, t in prog if _ in (MUL, MULC)) and all(d != s for _, d, s, _t in prog)
+
+
+def run_exponents():
+    """the list on exponents of f, modulo p^12 - 1: the result is (p^12 - 1)/r"""
+    q = P**12 - 1
+    v = {0: 1}
+    for i, (o, d, s, t) in enumerate(prog):
+        if i == split:
+            v[4] = -v[3]
+        v[d] = (2 * v[s] if o == SQR else v[s] + v[t] if o == MUL else v[s] + P**6 * v[t] if o == MULC else
+                v[s] * P**6 if o == CONJ else v[s] * P if o == FROB else v[s] * P**2) % q
+    return v[2]
+
+
+assert run_exponents() == (P**12 - 1) // R
+out.append(f"#define L12_FE_SPLIT {split}\n#define L12_FE_LEN {len(prog)}\n#define L12_FE_RESULT 2\n")
+out.append(f"__constant__ unsigned char L12_FE[{len(prog)}][4] = {{" +
+           ", ".join("{" + ", ".join(map(str, q)) + "}" for q in prog) + "};\n")
 out.append("__constant__ uint32_t SHA256_K[64] = {" + ", ".join(f"0x{k:08x}u" for k in SHA_K) + "};\n")
 out.append("__constant__ uint32_t SHA256_H0[8] = {" + ", ".join(f"0x{k:08x}u" for k in SHA_H) + "};\n")
 open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "constants.cuh"), "w").write("".join(out))

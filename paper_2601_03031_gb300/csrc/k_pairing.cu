@@ -1,5 +1,6 @@
 // Batched Miller loops and final exponentiations.
 #include "k_common.cuh"
+#include "limb12.cuh"
 #include "warp12.cuh"
 
 namespace fpk {
@@ -64,20 +65,23 @@ __global__ void __launch_bounds__(128) k_final_exp_w(const fq12* in, uint32_t n,
     }
 }
 
-// one 128-thread block per final exponentiation (few of them: the 108 products of an Fq12
-// product take one round instead of four)
-__global__ void __launch_bounds__(128) k_final_exp_c(const fq12* in, uint32_t n, fq12* out, uint8_t* ser,
-                                                     uint32_t per, size_t stride_a, size_t stride_b) {
-    __shared__ W12 W;
-    const int L = threadIdx.x;
+// one block of twelve 16-lane slots per final exponentiation, one limb per lane (limb12.cuh): few of
+// them, so the latency of one counts
+__global__ void __launch_bounds__(L12_THREADS) k_final_exp_c(const fq12* in, uint32_t n, fq12* out, uint8_t* ser,
+                                                             uint32_t per, size_t stride_a, size_t stride_b) {
+    __shared__ L12 W;
     const uint64_t t = blockIdx.x;
-    w_from_tower<4>(W.s[0], in[t]);
-    w_final_exp<4>(W);
-    if (L < 12) {
-        const int tp = w_tower_pos(L >> 1), e = L & 1;
-        const fq v = W.s[2][L];
-        if (out) reinterpret_cast<fq*>(&out[t])[2 * tp + e] = v;
-        if (ser) fq_to_be(ser + (t / per) * stride_a + (t % per) * stride_b + 96 * tp + 48 * e, v);
+    {
+        const L12Lane c = l12_lane();
+        l12_load(W, c, W.v[0], W.v[1], reinterpret_cast<const fq*>(&in[t])[2 * w_tower_pos(c.kc) + c.e]);
+    }
+    l12_final_exp(W);
+    const L12Lane c = l12_lane();
+    const int tp = w_tower_pos(c.kc);
+    const fq v = l12_store(W, c, W.v[L12_FE_RESULT], W.v[0]);
+    if (c.k.l == 0) {
+        if (out) reinterpret_cast<fq*>(&out[t])[2 * tp + c.e] = v;
+        if (ser) fq_to_be(ser + (t / per) * stride_a + (t % per) * stride_b + 96 * tp + 48 * c.e, v);
     }
 }
 
@@ -105,7 +109,7 @@ void final_exp_group(const void* in, uint32_t n, void* out, void* ser, uint32_t 
         return;
     }
     if (n <= lim.fe_block_max) {
-        FP_KERNEL("k_final_exp_c", s, k_final_exp_c<<<n, 128, 0, s>>>((const fq12*)in, n, (fq12*)out, (uint8_t*)ser, per,
+        FP_KERNEL("k_final_exp_c", s, k_final_exp_c<<<n, L12_THREADS, 0, s>>>((const fq12*)in, n, (fq12*)out, (uint8_t*)ser, per,
                                                                      stride_a, stride_b));
         return;
     }

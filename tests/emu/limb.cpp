@@ -1,0 +1,63 @@
+// Host build of the limb-lane engine (limb.cuh, limb12.cuh): every lane of a block as a host thread.
+// Field elements cross as canonical big-endian bytes (Fq12 576 in the tower order of the serialisation).
+#include "limb_shim.h"
+#include "pairing.cuh"
+#include "limb12.cuh"
+
+#include <vector>
+
+namespace {
+fq be_fq(const uint8_t* b) {
+    fq a;
+    for (int j = 0; j < 12; j++) {
+        const uint8_t* p = b + 44 - 4 * j;
+        a.v[j] = ((uint32_t)p[0] << 24) | ((uint32_t)p[1] << 16) | ((uint32_t)p[2] << 8) | p[3];
+    }
+    return fq_to_mont(a);
+}
+template <typename Fn>
+void lanes(int n, Fn fn) {
+    std::barrier<> bar(n);
+    g_lanes = &bar;
+    emu_setup_quads(n);
+    std::vector<std::thread> th;
+    for (int lane = 0; lane < n; lane++) th.emplace_back([&, lane] { threadIdx.x = lane; fn(); });
+    for (auto& t : th) t.join();
+}
+int tower_pos(int k) { return (k & 1) ? 3 + (k >> 1) : (k >> 1); }
+L12 g_w;
+}  // namespace
+
+extern "C" {
+// sum of nt products (12 little-endian words per operand, not Montgomery form) times 2^-390 mod p
+void emu_limb_dot3(const uint32_t* x, const uint32_t* y, uint32_t* out) {
+    lanes(16, [&] {
+        const LimbLane k = limb_lane();
+        alignas(16) static int32_t win[3][LIMB_WIN], u[16], r[16], row[3][LIMB_ROW];
+        const int32_t *w[3] = {win[0], win[1], win[2]}, *y3[3] = {row[0], row[1], row[2]};
+        for (int t = 0; t < 3; t++) {
+            limb_put_window(win[t], k.l, limb_of_words(x + 12 * t, k.l));
+            limb_put(row[t], k.l, limb_of_words(y + 12 * t, k.l));
+        }
+        __syncwarp();
+        int64_t lo, hi;
+        limb_dot<3>(k, lo, hi, y3, w);
+        limb_put(r, k.l, limb_carry(limb_reduce(k, lo, hi, u), k.l));
+        __syncwarp();
+        if (k.l == 0) {
+            const fq v = limb_canon(r);
+            for (int j = 0; j < 12; j++) out[j] = v.v[j];
+        }
+    });
+}
+void emu_limb_final_exp(const uint8_t* f_be, uint8_t* out) {
+    lanes(L12_THREADS, [&] {
+        const L12Lane c = l12_lane();
+        const int pos = 2 * tower_pos(c.kc) + c.e;
+        l12_load(g_w, c, g_w.v[0], g_w.v[1], be_fq(f_be + 48 * pos));
+        l12_final_exp(g_w);
+        const fq v = l12_store(g_w, c, g_w.v[L12_FE_RESULT], g_w.v[0]);
+        if (c.k.l == 0) fq_to_be(out + 48 * pos, v);
+    });
+}
+}

@@ -1,0 +1,57 @@
+"""The limb-lane engine (limb.cuh: Fq sums of products with one limb per lane; limb12.cuh: Fq12
+operations on it), compiled for the host with every lane as a thread, against Python integers and the
+oracle (no GPU)."""
+import ctypes
+import os
+import random
+import shutil
+import subprocess
+
+import pytest
+
+import oracle as O
+from tests import _pyref as ref
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2601_03031_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def emu(tmp_path_factory):
+    gxx = shutil.which("g++")
+    if not gxx:
+        pytest.skip("g++ not available")
+    so = str(tmp_path_factory.mktemp("emu_limb") / "liblimb.so")
+    subprocess.check_call([gxx, "-std=c++20", "-O1", "-shared", "-fPIC", f"-I{CSRC}", "-o", so,
+                           os.path.join(HERE, "emu", "limb.cpp")])
+    L = ctypes.CDLL(so)
+    L.emu_limb_dot3.restype = L.emu_limb_final_exp.restype = None
+    return L
+
+
+def test_sum_of_products_against_python(emu):
+    """x0 y0 + x1 y1 + x2 y2 times 2^-390 mod p, at values with all limbs at their largest, zero and
+    random ones."""
+    P = ref.P
+    rnd = random.Random(3)
+    vals = [0, 1, P - 1, (1 << 380) - 1, (1 << 338) - 1, 1 << 338, P >> 1]
+    cases = [[(a, b)] * 3 for a in vals for b in vals[1:4]]
+    cases += [[(rnd.randrange(P), rnd.randrange(P)) for _ in range(3)] for _ in range(20)]
+    out = (ctypes.c_uint32 * 12)()
+    for c in cases:
+        x, y = [(ctypes.c_uint32 * 36)(*[(t[i] >> (32 * j)) & 0xFFFFFFFF for t in c for j in range(12)])
+                for i in (0, 1)]
+        emu.emu_limb_dot3(x, y, out)
+        want = sum(a * b for a, b in c) * pow(2, -390, P) % P
+        assert sum(out[j] << (32 * j) for j in range(12)) == want, c
+
+
+def test_final_exponentiation_against_oracle(emu):
+    rnd = random.Random(8)
+    for n in range(2):
+        f = b"".join(rnd.randrange(ref.P).to_bytes(48, "big") for _ in range(12))
+        if n:
+            f = (1).to_bytes(48, "big") + bytes(528)
+        out = ctypes.create_string_buffer(576)
+        emu.emu_limb_final_exp(f, out)
+        assert out.raw == O.final_exp(f)
