@@ -109,7 +109,6 @@ SPLIT_ROUNDS = {"k_final_exp_c": (H1.bit_length() + 1) + 3 * (X_ABS.bit_length()
 CHAIN_KERNELS = ("k_final_exp_c", "k_round_miller_c", "k_fold_c", "k_challenge2")
 
 
-FOLD_COMB_MAX = 256           # rounds with at most this many fold points use the comb folds
 LAM_COMB_MAX_M = 1024         # setups with M <= this commit by the fixed-base combs of their bases
 G2_COMB_MAX_R = 1024          # setups with R <= this keep the W proofs' comb tables
 
@@ -154,7 +153,6 @@ def step_units(log_n: int, b: int, msm_window: int, msm_window_g2: int = 16, lim
     fe[engine(2 * K, lim["fe_block_max"], lim["fe_warp_max"])] += 2 * K * lr     # two per block and round
     cm = {"c": 0, "w": 0, "t": 0}
     cm[engine(R, lim["commit_block_max"], lim["commit_warp_max"])] += R
-    comb = sum(K * h for h in hs if K * h <= FOLD_COMB_MAX)
     fw = lim["fold_warp_max"]
     w_terms = K * (2 * R - 2) if not w_msm and R > G2_COMB_MAX_R else 0
     return {
@@ -169,11 +167,12 @@ def step_units(log_n: int, b: int, msm_window: int, msm_window_g2: int = 16, lim
         "k_commit_miller_w": ("miller_loop", cm["w"]),
         "k_commit_miller": ("miller_loop", cm["t"]),
         "k_sparse_g": ("g1_mul", sum(K * min(b, 2 * h) for h in hs)),
-        "k_fold_c": ("comb_fold", comb),
-        "k_comb_chain": ("comb_chain", comb),
-        "k_comb_tab": ("comb_tab", comb),
-        "k_fold_w": (("g1_mul", "g2_mul"), sum(K * h for h in hs if FOLD_COMB_MAX < K * h <= fw)),
-        "k_fold": (("g1_mul", "g2_mul"), sum(K * h for h in hs if K * h > max(fw, FOLD_COMB_MAX))),
+        # folds by comb tables of the round's bases: none (every fold is a scalar multiplication)
+        "k_fold_c": ("comb_fold", 0),
+        "k_comb_chain": ("comb_chain", 0),
+        "k_comb_tab": ("comb_tab", 0),
+        "k_fold_w": (("g1_mul", "g2_mul"), sum(K * h for h in hs if K * h <= fw)),
+        "k_fold": (("g1_mul", "g2_mul"), sum(K * h for h in hs if K * h > fw)),
         "k_lamc_sum": ("lamc_term", R * M if M <= LAM_COMB_MAX_M else 0),
         "k_msm_chunk": ("msm_madd", 2 * R * M * W if M > LAM_COMB_MAX_M else 0),
         "k_msm_chunk_g2": ("g2_msm_madd", 4 * 2 * R * K * W2 if w_msm else 0),

@@ -326,9 +326,8 @@ typedef enum { FP_SCHEDULE_DIRECT = 0, FP_SCHEDULE_LOOKAHEAD = 1 } fp_schedule;
  *   commit_block_max / commit_warp_max   Commit's R Miller loops, the same way (default 1024 / 16384)
  *   fe_block_max / fe_warp_max           final exponentiations: block / warp / thread (256 / 2^32-1)
  *   pair_block_max                       pairwise Fq12 products: <= a block each, above a thread (2048)
- *   fold_warp_max                        fold points of rounds beyond the split folds (more than 256
- *                                        points): <= a warp (G2) and 8 lanes (G1) each, above a thread
- *                                        (4096)
+ *   fold_warp_max                        fold points of a round: <= a block (G2) and half a block (G1)
+ *                                        each, above a thread (4096)
  *   wterm_warp_max                       terms of the v_l proof W when not by MSM: <= a warp each,
  *                                        above a thread (4096)
  *   msm_chunks                           MSM bucket pass: about this many chunks of the sorted entry

@@ -267,6 +267,8 @@ out.append(f"#define LIMB_PINV52 0x{(-pow(P, -1, 2**52)) % 2**52:x}ull\n")
 out.append(f"#define LIMB_PTOP_INV {((1 << 32) << 364) // P}\n")
 # factors 2^396 (a residue times 2^384 into the engine's form) and 2^384 (back)
 out.append(rows("LIMB_CONV", [limbs26(2**396 % P), limbs26(2**384 % P)]))
+out.append(f"static __device__ const int32_t LIMB_OMEGA[16] = {{{', '.join(map(str, mont26(OMEGA)))}}};\n")
+out.append(rows("LIMB_PSI", [mont26(PSI_CX[0]), mont26(PSI_CX[1]), mont26(PSI_CY[0]), mont26(PSI_CY[1])]))
 out.append(rows("LIMB_FROB1", [mont26(FROB1[k][e]) for k in range(6) for e in range(2)]))
 out.append(rows("LIMB_FROB2", [mont26(FROB2[k][0]) for k in range(6)]))
 

@@ -4,6 +4,7 @@
 #include <algorithm>
 
 #include "group_ec.cuh"
+#include "limb_ec.cuh"
 #include "k_common.cuh"
 
 namespace fpk {
@@ -121,243 +122,68 @@ __global__ void __launch_bounds__(64) k_round_g1_out(const g1j* sp, uint32_t K, 
     }
 }
 
-// Both folds of round j for few points: blocks [0, nb2) fold 4 points of v each (one warp per point,
-// group_ec.cuh GEcW), the remaining blocks 16 points of A (8-lane groups) and the entries of b.
+// Both folds of round j with one limb per lane (limb_ec.cuh): blocks [0, n) fold a point of v each, the
+// remaining blocks two points of A (96 threads each) and their entries of b, n = K h points t = (k, i).
+// Latency-bound up to about one block per SM: 0.25 ms for 1 to 64 points, 0.31 ms for 128, 0.79 for 512,
+// 2.8 for 2048, 5.5 for 4096 (one GB300).  A warp per G2 point and 8 lanes per G1 point took 1.21 ms for
+// 512 points and 6.1 for 4096; one thread per point (k_fold) takes 4.5 ms for 8192, which is where the
+// default limit leaves off.  It replaces comb tables of the round's bases formed beside the pairings
+// (0.16 ms for 64 points after the challenge, but 0.96 ms of chains and tables per round before it).
 union FoldSmemW {
-    GEcW g2[4];
-    GEc<fq> g1[16];
+    LimbEc2 g2;
+    LimbEc g1[2];
 };
-__global__ void __launch_bounds__(128) k_fold_w(g1a* A, g2a* v, fr* bvec, const fr* x_mont, const fr* xinv_mont,
-                                                uint32_t K, uint32_t R, uint32_t h, uint32_t nb2) {
+__global__ void __launch_bounds__(LEC2_THREADS) k_fold_w(g1a* A, g2a* v, fr* bvec, const fr* x_mont,
+                                                         const fr* xinv_mont, uint32_t K, uint32_t R, uint32_t h) {
     __shared__ FoldSmemW sm;
-    uint32_t kw[8];
-    if (blockIdx.x < nb2) {
-        const int w = threadIdx.x >> 5, L = threadIdx.x & 31;
-        const uint64_t t = (uint64_t)blockIdx.x * 4 + w;
-        if (t >= (uint64_t)K * h) return;                     // warp-uniform
-        const uint64_t k = t / h;
-        const uint32_t i = (uint32_t)(t % h);
-        const uint64_t lo = k * R + i, hi = k * R + h + i;
-        fr_canon_words(kw, xinv_mont[k]);
-        const GPt<fq2> r = gecw_add(sm.g2[w], L, gecw_g2_mul_proj(sm.g2[w], L, v[hi], kw),
-                                    gec_from_affine_or_inf(v[lo].x, v[lo].y));
-        g2a o;
-        gec_to_affine(o.x, o.y, r);
-        __syncwarp();
-        if (L == 0) v[lo] = o;
-        return;
-    }
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
-    const uint64_t t0 = (uint64_t)(blockIdx.x - nb2) * 16 + grp;
-    const bool valid = t0 < (uint64_t)K * h;
-    const uint64_t t = valid ? t0 : 0;
-    const uint64_t k = t / h;
-    const uint32_t i = (uint32_t)(t % h);
-    const uint64_t lo = k * R + i, hi = k * R + h + i;
-    fr_canon_words(kw, x_mont[k]);
-    const GPt<fq> r = gec_add(sm.g1[grp], lane, gec_g1_mul_proj_w2(sm.g1[grp], lane, A[hi], kw),
-                              gec_from_affine_or_inf(A[lo].x, A[lo].y));
-    g1a o;
-    gec_to_affine(o.x, o.y, r);
-    __syncwarp();
-    if (valid && lane == 0) {
-        A[lo] = o;
-        bvec[lo] = fr_add(bvec[lo], fr_mul(bvec[hi], xinv_mont[k]));
-    }
-}
-
-// Comb folds for few points.  The scalar multiplications x_j A[h + i] and x_j^-1 v[h + i] are the
-// longest chain of a round after the challenge, but their bases are known one round earlier.  So
-// k_comb_chain, run beside the round's Miller loops and final exponentiations, forms every
-// 2^i A[h + i'] (i < 128) and 2^i v[h + i'] (i < 64), k_comb_tab the 16-entry table of each G1 window
-// (B = 4^w A: entries a B + b (-phi(B)), a, b < 4) and of each G2 position (B = 2^i v: entries
-// sum_{j in s} (-1)^j psi^j(B)) (group_ec.cuh, fixed-base combs), and k_fold_c, after the challenge,
-// only adds one table entry per window or position: 64 independent additions per point, summed
-// as 16 (G1) or 8 (G2) chains and a tree instead of a chain of 64 doublings and additions.
-// Point t = (k, i < h) as in k_fold_w; the tables of point t start at t 64 16.
-struct CombPtrs {
-    GPt<fq>* chain1;     // [n][128]
-    GPt<fq2>* chain2;    // [n][64]
-    GPt<fq>* tab1;       // [n 64][16]
-    GPt<fq2>* tab2;      // [n 64][16]
-};
-static CombPtrs comb_ptrs(void* base, uint32_t n) {
-    CombPtrs c;
-    uint8_t* p = (uint8_t*)base;
-    c.chain1 = (GPt<fq>*)p;
-    p += (size_t)n * 128 * sizeof(GPt<fq>);
-    c.chain2 = (GPt<fq2>*)p;
-    p += (size_t)n * 64 * sizeof(GPt<fq2>);
-    c.tab1 = (GPt<fq>*)p;
-    p += (size_t)n * 64 * 16 * sizeof(GPt<fq>);
-    c.tab2 = (GPt<fq2>*)p;
-    return c;
-}
-size_t fold_comb_bytes(uint32_t n) {
-    return (size_t)n * 128 * sizeof(GPt<fq>) + (size_t)n * 64 * sizeof(GPt<fq2>) +
-           (size_t)n * 64 * 16 * sizeof(GPt<fq>) + (size_t)n * 64 * 16 * sizeof(GPt<fq2>);
-}
-
-union CombSmem {
-    GEcWs g2[4];
-    GEcs<fq> g1[16];
-};
-// blocks [0, nb2): one warp per G2 point; the others: one 8-lane group per G1 point
-__global__ void __launch_bounds__(128) k_comb_chain(const g1a* A, const g2a* v, uint32_t K, uint32_t R, uint32_t h,
-                                                    uint32_t nb2, GPt<fq>* chain1, GPt<fq2>* chain2) {
-    __shared__ CombSmem sm;
-    const uint64_t n = (uint64_t)K * h;
-    if (blockIdx.x < nb2) {
-        const int w = threadIdx.x >> 5, L = threadIdx.x & 31;
-        const uint64_t t = (uint64_t)blockIdx.x * 4 + w;
-        if (t >= n) return;                                   // warp-uniform
-        const uint64_t hi = (t / h) * R + h + (uint32_t)(t % h);
-        GPt<fq2> acc = gec_from_affine_or_inf(v[hi].x, v[hi].y);
-        GPt<fq2>* out = chain2 + t * 64;
-        for (int i = 0; i < 64; i++) {
-            if (i) acc = gecw_dbl(sm.g2[w], L, acc);
-            if (L == 0) out[i] = acc;
-        }
-        return;
-    }
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
-    const uint64_t t0 = (uint64_t)(blockIdx.x - nb2) * 16 + grp;
-    const bool valid = t0 < n;
-    const uint64_t t = valid ? t0 : 0;                        // idle groups repeat point 0, store nothing
-    const uint64_t hi = (t / h) * R + h + (uint32_t)(t % h);
-    GPt<fq> acc = gec_from_affine_or_inf(A[hi].x, A[hi].y);
-    GPt<fq>* out = chain1 + t * 128;
-    for (int i = 0; i < 128; i++) {
-        if (i) acc = gec_dbl(sm.g1[grp], lane, acc);
-        if (valid && lane == 0) out[i] = acc;
-    }
-}
-
-// one thread per table: u < n 64 the G1 window table u = t 64 + w, then the G2 position tables
-// (independent tables keep every lane busy, so one lane per table issues far fewer instructions per
-// entry than the lane-parallel engines, which leaves more of the GPU to the round's pairings)
-__global__ void __launch_bounds__(64) k_comb_tab(uint32_t n, const GPt<fq>* chain1, const GPt<fq2>* chain2,
-                                                 GPt<fq>* tab1, GPt<fq2>* tab2) {
-    const uint64_t m = (uint64_t)n * 64, u = gtid();
-    if (u < m) {
-        const uint64_t t = u / 64, w = u % 64;
-        gpt_g1_comb_table(chain1[t * 128 + 2 * w], chain1[t * 128 + 2 * w + 1], tab1 + u * 16);
-    } else if (u < 2 * m) {
-        gpt_g2_comb_table(chain2[u - m], tab2 + (u - m) * 16);
-    }
-}
-
-// blocks [0, n): one G2 point each, 8 warps (warp g adds the entries of positions g, g + 8, ...,
-// g + 56, then a tree over the warps, then v[lo]); the others two G1 points each, 16 groups per
-// point (group g adds windows g, g + 16, g + 32, g + 48, then a tree over the groups, then A[lo]).
-// Every group of a warp runs every addition (the groups of a warp share one instruction stream);
-// additions whose result is not needed are discarded.
-struct FoldSmemC {
-    union {
-        GEcWs g2[8];
-        GEcs<fq> g1[32];
-    } e;
-    union {
-        GPt<fq2> g2[8];
-        GPt<fq> g1[2][16];
-    } part;
-};
-__global__ void __launch_bounds__(256) k_fold_c(g1a* A, g2a* v, fr* bvec, const fr* x_mont, const fr* xinv_mont,
-                                                uint32_t K, uint32_t R, uint32_t h, const GPt<fq>* tab1,
-                                                const GPt<fq2>* tab2) {
-    __shared__ FoldSmemC sm;
     const uint64_t n = (uint64_t)K * h;
     uint32_t kw[8];
     if (blockIdx.x < n) {
-        const int w = threadIdx.x >> 5, L = threadIdx.x & 31;
         const uint64_t t = blockIdx.x, k = t / h;
-        const uint64_t lo = k * R + (uint32_t)(t % h);
+        const uint64_t lo = k * R + (uint32_t)(t % h), hi = lo + h;
         fr_canon_words(kw, xinv_mont[k]);
-        uint32_t d[4][2];
-        gls_digits(d, kw);
-        const GPt<fq2>* tb = tab2 + t * 64 * 16;
-        GPt<fq2> acc = tb[w * 16 + gls_position(d, w)];
-        for (int j = 1; j < 8; j++) {
-            const int i = w + 8 * j;
-            acc = gecw_add(sm.e.g2[w], L, acc, tb[i * 16 + gls_position(d, i)]);
-        }
-        for (int sh = 4; sh >= 1; sh >>= 1) {
-            __syncthreads();
-            if (L == 0) sm.part.g2[w] = acc;
-            __syncthreads();
-            if (w < sh) acc = gecw_add(sm.e.g2[w], L, acc, sm.part.g2[w + sh]);
-        }
-        if (w == 0) {
-            acc = gecw_add(sm.e.g2[0], L, acc, gec_from_affine_or_inf(v[lo].x, v[lo].y));
-            g2a o;
-            gec_to_affine_quad(o.x, o.y, acc);                 // every quad of warp 0 (converged)
-            __syncwarp();
-            if (L == 0) v[lo] = o;
-        }
+        const Lec2Lane c = lec2_lane();
+        lec2_g2_mul(sm.g2, c, v[hi], kw);
+        lec2_add_affine(sm.g2, c, v[lo]);
+        const fq r = lec2_affine(sm.g2, c);
+        if (c.k.l == 0 && c.slot < 4) reinterpret_cast<fq*>(&v[lo])[c.slot] = r;
         return;
     }
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7, half = grp >> 4, g = grp & 15;
-    const uint64_t t0 = (blockIdx.x - n) * 2 + half;
-    const bool valid = t0 < n;
-    const uint64_t t = valid ? t0 : 0;                        // an idle half repeats point 0, stores nothing
+    const int half = (int)(threadIdx.x / LEC_THREADS);
+    const uint64_t t = (blockIdx.x - n) * 2 + half;
+    if (t >= n) return;                                       // three whole warps, with a barrier of their own
     const uint64_t k = t / h;
-    const uint32_t i = (uint32_t)(t % h);
-    const uint64_t lo = k * R + i, hi = k * R + h + i;
+    const uint64_t lo = k * R + (uint32_t)(t % h), hi = lo + h;
     fr_canon_words(kw, x_mont[k]);
-    uint32_t k1[5], k0[4];
-    div_by_const<4, 5>(k1, k0, kw, GLV_D, GLV_BARRETT);
-    const GPt<fq>* tb = tab1 + t * 64 * 16;
-    GPt<fq> acc = tb[g * 16 + glv_window(k0, k1, g)];
-    for (int j = 1; j < 4; j++) {
-        const int w = g + 16 * j;
-        acc = gec_add(sm.e.g1[grp], lane, acc, tb[w * 16 + glv_window(k0, k1, w)]);
-    }
-    for (int sh = 8; sh >= 1; sh >>= 1) {
-        __syncthreads();
-        if (lane == 0) sm.part.g1[half][g] = acc;
-        __syncthreads();
-        const GPt<fq> r = gec_add(sm.e.g1[grp], lane, acc, sm.part.g1[half][g < sh ? g + sh : g]);
-        if (g < sh) acc = r;
-    }
-    acc = gec_add(sm.e.g1[grp], lane, acc, gec_from_affine_or_inf(A[lo].x, A[lo].y));
-    g1a o;
-    gec_to_affine_quad(o.x, o.y, acc);                        // the two quads of each group
-    __syncthreads();                                          // every read of A[lo] before the store
-    if (valid && g == 0 && lane == 0) {
-        A[lo] = o;
-        bvec[lo] = fr_add(bvec[lo], fr_mul(bvec[hi], xinv_mont[k]));
-    }
+    const LecLane c = lec_lane();
+    lec_g1_mul(sm.g1[half], c, A[hi], kw);
+    lec_add_affine(sm.g1[half], c, A[lo]);
+    const fq r = lec_affine(sm.g1[half], c);
+    if (c.k.l == 0 && c.slot < 2) reinterpret_cast<fq*>(&A[lo])[c.slot] = r;
+    if (c.k.l == 0 && c.slot == 2) bvec[lo] = fr_add(bvec[lo], fr_mul(bvec[hi], xinv_mont[k]));
 }
 
-// L_j.1 and R_j.1 terms at the support of b only, one 8-lane group per term, for the blocks
+// L_j.1 and R_j.1 terms at the support of b only, one block per term (limb_ec.cuh), for the blocks
 // k0 .. k0 + K - 1 (local index k - k0).  Block k's vector b is
 // non-zero only at its statement indices S_k = [k b, k b + |S_k|) folded mod the current length 2h:
 // term t < min(|S_k|, 2h) sits at p = (k b + t) mod 2h (all p < 2h when |S_k| > 2h); p < h is an
 // L_j.1 term b[p] A[h + p], p >= h an R_j.1 term b[p] A[p - h].  Results go to the dense per-block
 // layout out[k 2h + p] (Jacobian), whose other entries the caller has zeroed (Z = 0: identity).
-__global__ void __launch_bounds__(128) k_sparse_g(const g1a* A, const fr* bvec, uint32_t k0, uint32_t K, uint32_t R,
-                                                  uint32_t h, uint32_t b, uint32_t cmax, g1j* out) {
-    __shared__ GEc<fq> sm[16];
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
-    const uint64_t u0 = (uint64_t)blockIdx.x * 16 + grp;
-    uint64_t k = u0 / cmax;
-    uint32_t t = (uint32_t)(u0 % cmax);
-    bool valid = k < K;
-    uint32_t sk = valid ? min(b, R - (k0 + (uint32_t)k) * b) : 1;
-    valid = valid && t < min(sk, 2 * h);
-    if (!valid) { k = 0; t = 0; sk = min(b, R - k0 * b); }    // dummy work keeps the warp uniform
+__global__ void __launch_bounds__(LEC_THREADS) k_sparse_g(const g1a* A, const fr* bvec, uint32_t k0, uint32_t K,
+                                                          uint32_t R, uint32_t h, uint32_t b, uint32_t cmax,
+                                                          g1j* out) {
+    __shared__ LimbEc S;
+    const uint64_t k = blockIdx.x / cmax;
+    const uint32_t t = (uint32_t)(blockIdx.x % cmax);
+    const uint32_t sk = min(b, R - (k0 + (uint32_t)k) * b);
+    if (t >= min(sk, 2 * h)) return;                          // block-uniform
     const uint32_t p = sk <= 2 * h ? (uint32_t)(((uint64_t)(k0 + k) * b + t) % (2 * h)) : t;
     uint32_t kw[8];
     fr_canon_words(kw, bvec[k * R + p]);
-    const GPt<fq> r = gec_g1_mul_proj_w2(sm[grp], lane, A[k * R + (p < h ? h + p : p - h)], kw);
-    __syncwarp();
-    if (valid && lane == 0) {
-        g1j o;                                                // (X : Y : Z) -> Jacobian (X Z, Y Z^2, Z)
-        o.X = fq_mul(r.X, r.Z);
-        o.Y = fq_mul(r.Y, fq_sqr(r.Z));
-        o.Z = r.Z;
-        out[k * 2 * h + p] = o;
-    }
+    const LecLane c = lec_lane();
+    lec_g1_mul(S, c, A[k * R + (p < h ? h + p : p - h)], kw);
+    const fq v = lec_jacobian(S, c);
+    if (c.k.l == 0 && c.slot < 3) reinterpret_cast<fq*>(&out[k * 2 * h + p])[c.slot] = v;
 }
 
 // the same with the two SHA-256 halves of HFr on two lanes of a warp per block (they are
@@ -529,7 +355,7 @@ void step1_sparse_terms(const void* A, const void* bvec, uint32_t k0, uint32_t K
                         void* out, cudaStream_t s) {
     const uint32_t cmax = std::min(b, 2 * h);
     cudaMemsetAsync(out, 0, (size_t)K * 2 * h * G1J_BYTES, s);
-    FP_KERNEL("k_sparse_g", s, k_sparse_g<<<(unsigned)(((uint64_t)K * cmax + 15) / 16), 128, 0, s>>>(
+    FP_KERNEL("k_sparse_g", s, k_sparse_g<<<(unsigned)((uint64_t)K * cmax), LEC_THREADS, 0, s>>>(
                                    (const g1a*)A, (const fr*)bvec, k0, K, R, h, b, cmax, (g1j*)out));
 }
 void step1_gt_out(const void* ml, uint32_t K, int j, void* blocks, size_t bopen_len, cudaStream_t s) {
@@ -644,31 +470,12 @@ uint64_t step1_miller_g(const void* A, const void* v, uint32_t K, uint32_t R, ui
     round_miller_w(A, v, K, R, h, ml_out, s);      // few pairs: one warp or block each, for latency
     return n;
 }
-void step1_fold_pre(const void* A, const void* v, void* comb, uint32_t n_max, uint32_t K, uint32_t R, uint32_t h,
-                    cudaStream_t s) {
-    const uint32_t n = K * h;
-    if (n > n_max) return;
-    const CombPtrs c = comb_ptrs(comb, n_max);
-    const uint32_t nb2 = (n + 3) / 4, nb1 = (n + 15) / 16;
-    FP_KERNEL("k_comb_chain", s, k_comb_chain<<<nb2 + nb1, 128, 0, s>>>((const g1a*)A, (const g2a*)v, K, R, h, nb2,
-                                                                       c.chain1, c.chain2));
-    FP_KERNEL("k_comb_tab", s, k_comb_tab<<<grid_for((uint64_t)n * 128, 64), 64, 0, s>>>(n, c.chain1, c.chain2,
-                                                                                       c.tab1, c.tab2));
-}
 void step1_fold(void* A, void* v, void* bvec, const void* x_mont, const void* xinv_mont, uint32_t K, uint32_t R,
-                uint32_t h, const void* comb, uint32_t n_max, cudaStream_t s) {
-    if (comb && (uint64_t)K * h <= n_max) {            // comb tables ready: table entries only
-        const uint32_t n = K * h;
-        const CombPtrs c = comb_ptrs(const_cast<void*>(comb), n_max);
-        FP_KERNEL("k_fold_c", s, k_fold_c<<<n + (n + 1) / 2, 256, 0, s>>>((g1a*)A, (g2a*)v, (fr*)bvec,
-                                                                         (const fr*)x_mont, (const fr*)xinv_mont, K,
-                                                                         R, h, c.tab1, c.tab2));
-        return;
-    }
-    if ((uint64_t)K * h <= engine_limits().fold_warp_max) {   // few points: a warp per G2 point, 8 lanes per G1
-        const uint32_t nb2 = (uint32_t)(((uint64_t)K * h + 3) / 4), nb1 = (uint32_t)(((uint64_t)K * h + 15) / 16);
-        FP_KERNEL("k_fold_w", s, k_fold_w<<<nb2 + nb1, 128, 0, s>>>((g1a*)A, (g2a*)v, (fr*)bvec, (const fr*)x_mont,
-                                                                  (const fr*)xinv_mont, K, R, h, nb2));
+                uint32_t h, cudaStream_t s) {
+    const uint64_t n = (uint64_t)K * h;
+    if (n <= engine_limits().fold_warp_max) {          // few points: a block per G2 point, half a block per G1
+        FP_KERNEL("k_fold_w", s, k_fold_w<<<(unsigned)(n + (n + 1) / 2), LEC2_THREADS, 0, s>>>(
+                                     (g1a*)A, (g2a*)v, (fr*)bvec, (const fr*)x_mont, (const fr*)xinv_mont, K, R, h));
         return;
     }
     uint32_t nb = grid_for((uint64_t)K * h, 64);

@@ -33,7 +33,7 @@ struct EngineLimits {
     uint32_t fe_block_max = 256;            // final exponentiations per launch: <= this, a block each
     uint32_t fe_warp_max = 0xffffffffu;     //   <= this, a warp each; above, a thread each
     uint32_t pair_block_max = 2048;         // pairwise Fq12 products: <= this, a block each; above, a thread
-    uint32_t fold_warp_max = 4096;          // fold points (beyond the split folds): <= this, a warp / 8 lanes
+    uint32_t fold_warp_max = 4096;          // fold points: <= this, a block per G2 point and half a block per G1
                                             //   per point; above, a thread per point
     uint32_t wterm_warp_max = 4096;         // W terms: <= this, a warp per term; above, a thread per term
     uint32_t msm_chunks = 1u << 17;         // MSM bucket pass: about this many chunks of the entry list
@@ -104,16 +104,10 @@ uint64_t step1_miller_g(const void* A, const void* v, uint32_t K, uint32_t R, ui
                         cudaStream_t s);
 void step1_g1_out(const void* sp_g1j, uint32_t K, int j, void* blocks, size_t bopen_len, cudaStream_t s);
 void step1_gt_out(const void* ml_fq12, uint32_t K, int j, void* blocks, size_t bopen_len, cudaStream_t s);
-// Round j's folds.  For rounds of at most FOLD_COMB_MAX points, step1_fold_pre forms the comb tables
-// of the round's bases in `comb` (fold_comb_bytes(n_max) bytes for up to n_max points) beside the
-// round's pairings, and step1_fold then adds one table entry per window; other rounds run the
-// whole scalar multiplications after the challenge.
-constexpr uint32_t FOLD_COMB_MAX = 256;
-size_t fold_comb_bytes(uint32_t n_max);
-void step1_fold_pre(const void* A, const void* v, void* comb, uint32_t n_max, uint32_t K, uint32_t R, uint32_t h,
-                    cudaStream_t s);
+// Round j's folds: at most fold_warp_max points on the limb lanes (a block per G2 point, half a block per
+// G1 point), more on one thread per point.
 void step1_fold(void* A, void* v, void* bvec, const void* x_mont, const void* xinv_mont, uint32_t K, uint32_t R,
-                uint32_t h, const void* comb, uint32_t n_max, cudaStream_t s);
+                uint32_t h, cudaStream_t s);
 // Look-ahead rounds (lookahead.cuh): round j's record from round j-1's state (half-length h = 2 h2)
 // and challenge.  Before the challenge: la_miller (the 8 K h2 Miller values by class; then pairwise
 // products to 8 K and their final exponentiations, fe), la_sparse (the 6 K (4 h2) G1 terms; then

@@ -148,14 +148,14 @@ constexpr uint64_t TREE_REDUCE_MAX = 8192;
 
 size_t bopen_len(uint32_t log_r) { return (size_t)log_r * ROUND_BYTES + G1_SER + 2 * G2_SER; }
 
-// Internal non-blocking streams: OpenAll's latency-bound Step 1 runs on three high-priority
-// streams (the round chain, and beside it the sparse G1 terms and the shifted fold bases), the
+// Internal non-blocking streams: OpenAll's latency-bound Step 1 runs on two high-priority
+// streams (the round chain, and beside it the sparse G1 terms), the
 // throughput-bound Step 2 on a low-priority stream; all are forked from and joined back to the caller's stream with events
 // created per call.  Each caller stream (per device) gets its own set, so calls on different caller
 // streams run concurrently; past 256 caller streams the sets are shared (still correct, less
 // concurrent).
 struct Streams {
-    cudaStream_t hi = nullptr, sp = nullptr, pre = nullptr, la[2] = {nullptr, nullptr}, fold = nullptr, lo = nullptr;
+    cudaStream_t hi = nullptr, sp = nullptr, la[2] = {nullptr, nullptr}, fold = nullptr, lo = nullptr;
     cudaStream_t tail = nullptr;   // Commit's pairings of the row commitments (high priority)
 };
 struct StreamKey { int dev; cudaStream_t user; Streams set; };
@@ -167,7 +167,6 @@ Streams make_set() {
     check(cudaDeviceGetStreamPriorityRange(&lo, &hi), "priority range");
     check(cudaStreamCreateWithPriority(&a.hi, cudaStreamNonBlocking, hi), "cudaStreamCreate");
     check(cudaStreamCreateWithPriority(&a.sp, cudaStreamNonBlocking, hi), "cudaStreamCreate");
-    check(cudaStreamCreateWithPriority(&a.pre, cudaStreamNonBlocking, hi), "cudaStreamCreate");
     check(cudaStreamCreateWithPriority(&a.la[0], cudaStreamNonBlocking, hi), "cudaStreamCreate");
     check(cudaStreamCreateWithPriority(&a.la[1], cudaStreamNonBlocking, hi), "cudaStreamCreate");
     check(cudaStreamCreateWithPriority(&a.fold, cudaStreamNonBlocking, hi), "cudaStreamCreate");
@@ -503,8 +502,6 @@ namespace {
 // outputs, the challenges and the fast-verification proof of v_l
 struct Step1Bufs {
     void *A, *v, *bvec, *xprev, *x_mont, *xinv_mont, *xinv_all, *ml, *ml2, *sp, *sp2, *pcoef, *q;
-    void* comb = nullptr;                // comb tables of rounds with few points (step1_fold_pre)
-    uint32_t comb_n = 0;                 // points they hold
     void *wt = nullptr, *wt2 = nullptr, *wscr = nullptr;
     MsmShape wsh{};
     bool w_msm = false;
@@ -527,8 +524,6 @@ Step1Bufs step1_bufs(const fp_pp* pp, uint32_t Kc, Alloc&& T) {
     B.sp2 = T((KR / 2 + 1) * G1J_BYTES);
     B.pcoef = T((size_t)Kc * (2 * R - 1) * FR_BYTES);
     B.q = T((size_t)Kc * 2 * R * FR_BYTES);
-    B.comb_n = (uint32_t)std::min<uint64_t>(FOLD_COMB_MAX, KR / 2);
-    if (B.comb_n) B.comb = T(fold_comb_bytes(B.comb_n));
     // W proofs: one batched G2 MSM over the shared bases g2^{beta^i} when many blocks share them,
     // else one scalar multiplication per term and pairwise sums (with few batches the MSM's bucket
     // reduction runs nearly serially per window)
@@ -574,23 +569,16 @@ LaBufs la_bufs(const fp_pp* pp, uint32_t Kc, Alloc&& T) {
 
 // FC.BOpen rounds (Sec. 3, Eq. folding) and the fast-verification proof of v_l for the Kc blocks
 // k0 .. k0 + Kc - 1 of size b, whose combined vectors are in B.bvec (their support is the block):
-// the round chain on s1, each round's G1 parts on s3 (joined before the challenge) and, in rounds
-// with few points, the shifted fold bases on s4 (joined before the fold); the records go to
+// the round chain on s1, each round's G1 parts on s3 (joined before the challenge); the records go to
 // blocks1 (stride blen).  s3 must already be ordered after whatever filled B.bvec.
 void step1_rounds(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, const Step1Bufs& B, uint8_t* blocks1,
-                  size_t blen, cudaStream_t s1, cudaStream_t s3, cudaStream_t s4) {
+                  size_t blen, cudaStream_t s1, cudaStream_t s3) {
     const uint32_t R = pp->R;
     const int lr = (int)pp->log_r;
-    cudaEvent_t ev_folded = new_event(), ev_sparse = new_event(), ev_pre = new_event();
+    cudaEvent_t ev_folded = new_event(), ev_sparse = new_event();
     for (int j = 1; j <= lr; j++) {
         const uint32_t h = R >> j;
         check(cudaEventRecord(ev_folded, s1), "event");
-        const bool split = (uint64_t)Kc * h <= B.comb_n;
-        if (split) {
-            check(cudaStreamWaitEvent(s4, ev_folded, 0), "wait");
-            step1_fold_pre(B.A, B.v, B.comb, B.comb_n, Kc, R, h, s4);
-            check(cudaEventRecord(ev_pre, s4), "event");
-        }
         check(cudaStreamWaitEvent(s3, ev_folded, 0), "wait");
         step1_sparse_terms(B.A, B.bvec, k0, Kc, R, h, b, B.sp, s3);
         void* spr = (uint64_t)Kc * 2 * h <= TREE_REDUCE_MAX
@@ -603,8 +591,7 @@ void step1_rounds(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, const S
         step1_gt_out(mlr, Kc, j, blocks1, blen, s1);
         check(cudaStreamWaitEvent(s1, ev_sparse, 0), "wait");
         step1_challenge(blocks1, blen, Kc, j, B.xprev, B.x_mont, B.xinv_mont, B.xinv_all, lr, s1);
-        if (split) check(cudaStreamWaitEvent(s1, ev_pre, 0), "wait");
-        step1_fold(B.A, B.v, B.bvec, B.x_mont, B.xinv_mont, Kc, R, h, split ? B.comb : nullptr, B.comb_n, s1);
+        step1_fold(B.A, B.v, B.bvec, B.x_mont, B.xinv_mont, Kc, R, h, s1);
     }
     step1_kzg(B.A, B.v, B.xprev, B.xinv_all, Kc, R, lr, blocks1, blen, B.pcoef, B.q, s1);
     uint8_t* w_out = blocks1 + (size_t)lr * ROUND_BYTES + G1_SER + G2_SER;
@@ -620,7 +607,6 @@ void step1_rounds(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, const S
     }
     cudaEventDestroy(ev_folded);
     cudaEventDestroy(ev_sparse);
-    cudaEventDestroy(ev_pre);
 }
 
 // The rounds with look-ahead (lookahead.cuh): round 1 as in step1_rounds; for j >= 2 round j's record
@@ -632,11 +618,11 @@ void step1_rounds(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, const S
 // j-1's fold runs on sF after x_{j-1} and round j's snapshot.  Challenges alternate between two
 // buffers (B.x_mont, B.xinv_mont hold 2 Kc entries); a fold still reading x_{j-1} never meets x_{j+1},
 // because x_{j+1} waits for round j+1's look-ahead, which waits for that fold.  Streams: s1 challenges,
-// s3 round 1's sparse G1 terms, s4 the shifted fold bases, sL[0..1] the look-aheads, sF the folds;
+// s3 round 1's sparse G1 terms, sL[0..1] the look-aheads, sF the folds;
 // s3 must already be ordered after whatever filled B.bvec, s1 after B.A and B.v.
 void step1_rounds_la(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, const Step1Bufs& B,
                      const LaBufs& L, uint8_t* blocks1, size_t blen, cudaStream_t s1, cudaStream_t s3,
-                     cudaStream_t s4, const cudaStream_t* sL, cudaStream_t sF) {
+                     const cudaStream_t* sL, cudaStream_t sF) {
     const uint32_t R = pp->R;
     const int lr = (int)pp->log_r;
     const uint64_t KR = (uint64_t)Kc * R;
@@ -647,7 +633,7 @@ void step1_rounds_la(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, cons
     auto wait = [&](cudaStream_t st, cudaEvent_t e) { check(cudaStreamWaitEvent(st, e, 0), "wait"); };
     auto rec = [&](cudaStream_t st) { cudaEvent_t e = ev(); check(cudaEventRecord(e, st), "event"); return e; };
     std::vector<cudaEvent_t> ev_S(lr + 2, nullptr), ev_snap(lr + 2, nullptr), ev_la(lr + 2, nullptr),
-        ev_pre(lr + 2, nullptr), ev_x(lr + 2, nullptr);
+        ev_x(lr + 2, nullptr);
 
     // round j's look-ahead from the state S_{j-1} (the caller has ordered sL[j & 1] after it)
     auto lookahead = [&](int j) {
@@ -668,31 +654,20 @@ void step1_rounds_la(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, cons
         la_pre(L.fe[q], L.acc[q], Kc, L.gpre[q], L.acc2[q], st);
         ev_la[j] = rec(st);
     };
-    // round j's fold on sF (after x_j, the shifted bases and the snapshot of S_j for round j + 1)
+    // round j's fold on sF (after x_j and the snapshot of S_j for round j + 1)
     auto fold = [&](int j) {
         const uint32_t h = R >> j;
-        const bool split = (uint64_t)Kc * h <= B.comb_n;
         wait(sF, ev_x[j]);
-        if (split) wait(sF, ev_pre[j]);
         if (j + 1 <= lr) wait(sF, ev_snap[j + 1]);
-        step1_fold(B.A, B.v, B.bvec, xm(j), xim(j), Kc, R, h, split ? B.comb : nullptr, B.comb_n, sF);
+        step1_fold(B.A, B.v, B.bvec, xm(j), xim(j), Kc, R, h, sF);
         ev_S[j + 1] = rec(sF);
     };
-    auto fold_pre = [&](int j, cudaEvent_t ready) {
-        const uint32_t h = R >> j;
-        if ((uint64_t)Kc * h > B.comb_n) return;
-        wait(s4, ready);
-        step1_fold_pre(B.A, B.v, B.comb, B.comb_n, Kc, R, h, s4);
-        ev_pre[j] = rec(s4);
-    };
-
     cudaEvent_t ev_a = rec(s1), ev_b = rec(s3);     // S_1: A, v (s1) and b (s3)
     if (lr >= 2) {
         wait(sL[0], ev_a);
         wait(sL[0], ev_b);
         lookahead(2);
     }
-    fold_pre(1, ev_a);
     {   // round 1, direct
         const uint32_t h = R >> 1;
         step1_sparse_terms(B.A, B.bvec, k0, Kc, R, h, b, B.sp, s3);
@@ -714,7 +689,6 @@ void step1_rounds_la(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, cons
             wait(sL[(j + 1) & 1], ev_S[j]);
             lookahead(j + 1);
         }
-        fold_pre(j, ev_S[j]);
         wait(s1, ev_la[j]);
         la_gt(L.fe[j & 1], L.gpre[j & 1], xm(j - 1), xim(j - 1), Kc, L.pwp, s1);
         la_out(L.fe[j & 1], L.pwp, L.acc[j & 1], L.acc2[j & 1], xm(j - 1), xim(j - 1), Kc, j, blocks1, blen, s1);
@@ -833,8 +807,8 @@ fp_proofs* prove_impl(const fp_pp* pp, const fp_commit* cm, uint32_t b, uint32_t
             if (track_use && cm->done) check(cudaStreamWaitEvent(s3, cm->done, 0), "wait");
             step1_stmt_hash(cm->C_ser, cm->rows_ser, k0, Kc, R, b, hscr, hstmt, s3);
             step1_block_r(hstmt, k0, Kc, R, b, B.bvec, s3);
-            if (la) step1_rounds_la(pp, k0, Kc, b, B, L, blocks1, blen, s1, s3, st.pre, st.la, st.fold);
-            else step1_rounds(pp, k0, Kc, b, B, blocks1, blen, s1, s3, st.pre);
+            if (la) step1_rounds_la(pp, k0, Kc, b, B, L, blocks1, blen, s1, s3, st.la, st.fold);
+            else step1_rounds(pp, k0, Kc, b, B, blocks1, blen, s1, s3);
             check(cudaEventRecord(ev_join1, s1), "event");
             check(cudaStreamWaitEvent(s, ev_join1, 0), "join");
             cudaEventDestroy(ev_init);
@@ -1166,8 +1140,8 @@ fp_status vc_eval_prove(const fp_pp* pp, const fp_commit* cm, const uint8_t* r, 
             eval_bvec(cm->C_ser, r_be, ln, proof + 32, Tm, R, r0, B.bvec, s1);
             check(cudaEventRecord(ev_bvec, s1), "event");
             check(cudaStreamWaitEvent(s3, ev_bvec, 0), "wait");
-            if (la) step1_rounds_la(pp, 0, 1, R, B, L, proof + 128, blen, s1, s3, st.pre, st.la, st.fold);
-            else step1_rounds(pp, 0, 1, R, B, proof + 128, blen, s1, s3, st.pre);
+            if (la) step1_rounds_la(pp, 0, 1, R, B, L, proof + 128, blen, s1, s3, st.la, st.fold);
+            else step1_rounds(pp, 0, 1, R, B, proof + 128, blen, s1, s3);
             // step 3: PST.Eval of F = sum_j T_j f_j at r_R
             eval_ftable(cm->m_mont, Tm, R, M, F, s1);
             eval_pst_fold(F, r_mont, lc, q, proof, s1);

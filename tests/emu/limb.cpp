@@ -3,6 +3,7 @@
 #include "limb_shim.h"
 #include "pairing.cuh"
 #include "limb12.cuh"
+#include "limb_ec.cuh"
 
 #include <vector>
 
@@ -20,12 +21,15 @@ void lanes(int n, Fn fn) {
     std::barrier<> bar(n);
     g_lanes = &bar;
     emu_setup_quads(n);
+    emu_setup_warps(n);
     std::vector<std::thread> th;
     for (int lane = 0; lane < n; lane++) th.emplace_back([&, lane] { threadIdx.x = lane; fn(); });
     for (auto& t : th) t.join();
 }
 int tower_pos(int k) { return (k & 1) ? 3 + (k >> 1) : (k >> 1); }
 L12 g_w;
+LimbEc g_ec;
+LimbEc2 g_ec2;
 }  // namespace
 
 extern "C" {
@@ -58,6 +62,51 @@ void emu_limb_final_exp(const uint8_t* f_be, uint8_t* out) {
         l12_final_exp(g_w);
         const fq v = l12_store(g_w, c, g_w.v[L12_FE_RESULT], g_w.v[0]);
         if (c.k.l == 0) fq_to_be(out + 48 * pos, v);
+    });
+}
+// k P (96 bytes in and out, k as 8 little-endian words)
+void emu_limb_g1_mul(const uint8_t* p, const uint32_t* k, uint8_t* out) {
+    g1a P;
+    P.x = be_fq(p);
+    P.y = be_fq(p + 48);
+    g1j r;
+    lanes(LEC_THREADS, [&] {
+        const LecLane c = lec_lane();
+        lec_g1_mul(g_ec, c, P, k);
+        const fq v = lec_jacobian(g_ec, c);
+        if (c.k.l == 0 && c.slot < 3) (c.slot == 0 ? r.X : c.slot == 1 ? r.Y : r.Z) = v;
+    });
+    g1a a;
+    jac_to_affine(a.x, a.y, r);
+    fq_to_be(out, a.x);
+    fq_to_be(out + 48, a.y);
+}
+// k P + Q on G2 (192 bytes each)
+void emu_limb_g2_mul_add(const uint8_t* p, const uint32_t* k, const uint8_t* q, uint8_t* out) {
+    auto pt = [](const uint8_t* b) {
+        g2a P;
+        P.x.c0 = be_fq(b); P.x.c1 = be_fq(b + 48); P.y.c0 = be_fq(b + 96); P.y.c1 = be_fq(b + 144);
+        return P;
+    };
+    const g2a P = pt(p), Q = pt(q);
+    lanes(LEC2_THREADS, [&] {
+        const Lec2Lane c = lec2_lane();
+        lec2_g2_mul(g_ec2, c, P, k);
+        lec2_add_affine(g_ec2, c, Q);
+        const fq v = lec2_affine(g_ec2, c);
+        if (c.k.l == 0 && c.slot < 4) fq_to_be(out + 48 * c.slot, v);
+    });
+}
+// k P + Q on G1, affine
+void emu_limb_g1_mul_add(const uint8_t* p, const uint32_t* k, const uint8_t* q, uint8_t* out) {
+    g1a P, Q;
+    P.x = be_fq(p); P.y = be_fq(p + 48); Q.x = be_fq(q); Q.y = be_fq(q + 48);
+    lanes(LEC_THREADS, [&] {
+        const LecLane c = lec_lane();
+        lec_g1_mul(g_ec, c, P, k);
+        lec_add_affine(g_ec, c, Q);
+        const fq v = lec_affine(g_ec, c);
+        if (c.k.l == 0 && c.slot < 2) fq_to_be(out + 48 * c.slot, v);
     });
 }
 }

@@ -25,7 +25,8 @@ def emu(tmp_path_factory):
     subprocess.check_call([gxx, "-std=c++20", "-O1", "-shared", "-fPIC", f"-I{CSRC}", "-o", so,
                            os.path.join(HERE, "emu", "limb.cpp")])
     L = ctypes.CDLL(so)
-    L.emu_limb_dot3.restype = L.emu_limb_final_exp.restype = None
+    for f in (L.emu_limb_dot3, L.emu_limb_final_exp, L.emu_limb_g1_mul, L.emu_limb_g2_mul_add, L.emu_limb_g1_mul_add):
+        f.restype = None
     return L
 
 
@@ -55,3 +56,43 @@ def test_final_exponentiation_against_oracle(emu):
         out = ctypes.create_string_buffer(576)
         emu.emu_limb_final_exp(f, out)
         assert out.raw == O.final_exp(f)
+
+
+def test_g1_scalar_mul_against_oracle(emu):
+    """k P for edge and random k (digits that carry past bit 127 of a GLV half among them), and the
+    identity."""
+    rnd = random.Random(5)
+    r, x2 = ref.R, 0xD201000000010000 ** 2
+    ks = [0, 1, 2, 7, 8, 15, r - 1, x2, x2 - 1, x2 + 1, (x2 - 1) * (x2 + 1), r // 2] + [rnd.randrange(r) for _ in range(3)]
+    P = O.g1_mul(O.g1_gen(), 12345)
+    out = ctypes.create_string_buffer(96)
+    for k in ks:
+        for pt in (P, bytes(96)) if k == 7 else (P,):
+            emu.emu_limb_g1_mul(pt, (ctypes.c_uint32 * 8)(*[((k % r) >> (32 * i)) & 0xFFFFFFFF for i in range(8)]), out)
+            assert out.raw == O.g1_mul(pt, k % r), hex(k)
+
+
+def test_g2_scalar_mul_and_add_against_oracle(emu):
+    """k P + Q for edge and random k, with P = Q, P = -Q sums and identities among them."""
+    rnd = random.Random(6)
+    r, x = ref.R, 0xD201000000010000
+    P = O.g2_mul(O.g2_gen(), 777)
+    Q = O.g2_mul(O.g2_gen(), 4242)
+    inf = bytes(192)
+    cases = [(P, 0, Q), (P, 1, P), (P, r - 1, P), (P, 8, inf), (inf, 5, Q), (inf, 3, inf), (P, x, Q), (P, x - 1, Q),
+             (P, x**3 + x**2 - 1, Q)] + [(P, rnd.randrange(r), Q) for _ in range(2)]
+    out = ctypes.create_string_buffer(192)
+    for p, k, q in cases:
+        emu.emu_limb_g2_mul_add(p, (ctypes.c_uint32 * 8)(*[(k >> (32 * i)) & 0xFFFFFFFF for i in range(8)]), q, out)
+        assert out.raw == O.g2_add(O.g2_mul(p, k), q), hex(k)
+
+
+def test_g1_scalar_mul_and_add_against_oracle(emu):
+    rnd = random.Random(7)
+    r = ref.R
+    P, Q, inf = O.g1_mul(O.g1_gen(), 777), O.g1_mul(O.g1_gen(), 4242), bytes(96)
+    cases = [(P, 0, Q), (P, 1, P), (P, r - 1, P), (P, 8, inf), (inf, 5, Q), (inf, 3, inf), (P, rnd.randrange(r), Q)]
+    out = ctypes.create_string_buffer(96)
+    for p, k, q in cases:
+        emu.emu_limb_g1_mul_add(p, (ctypes.c_uint32 * 8)(*[(k >> (32 * i)) & 0xFFFFFFFF for i in range(8)]), q, out)
+        assert out.raw == O.g1_add(O.g1_mul(p, k), q), hex(k)
