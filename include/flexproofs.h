@@ -319,12 +319,14 @@ typedef enum { FP_SCHEDULE_DIRECT = 0, FP_SCHEDULE_LOOKAHEAD = 1 } fp_schedule;
  * 128-thread block or one warp per item: shortest chain, few items) or on a throughput engine (one
  * thread per item: least total work, many items); every engine computes the same values, so these
  * limits change which kernels run and how fast, never the bytes.  Counts are per launch.
- *   miller_block_max / miller_warp_max   Step-1 Miller loops: <= block_max a block each, <= warp_max
- *                                        a warp each, above a thread each (default 1024 / 16383)
+ *   miller_block_max / miller_warp_max   Step-1 Miller loops: <= the larger of the two a block each
+ *                                        (profiled as k_round_miller_c up to block_max, as
+ *                                        k_round_miller_w above), else a thread each (1024 / 16383)
  *   miller_group_min                     from this many (and h >= 4), a thread runs 4 pairs of one
  *                                        product with shared squarings (default 2^18)
  *   commit_block_max / commit_warp_max   Commit's R Miller loops, the same way (default 1024 / 16384)
- *   fe_block_max / fe_warp_max           final exponentiations: block / warp / thread (256 / 2^32-1)
+ *   fe_block_max / fe_warp_max           final exponentiations: block / warp / thread (256 / 2^32-1;
+ *                                        unless block_max is 0, blocks also up to 912)
  *   pair_block_max                       pairwise Fq12 products: <= a block each, above a thread (2048)
  *   fold_warp_max                        fold points of a round: <= a block (G2) and half a block (G1)
  *                                        each, above a thread (4096)

@@ -1,6 +1,6 @@
 // Batched Miller loops and final exponentiations.
 #include "k_common.cuh"
-#include "limb12.cuh"
+#include "limb_miller.cuh"
 #include "warp12.cuh"
 
 namespace fpk {
@@ -98,6 +98,7 @@ __global__ void k_final_exp_t(const fq12* in, uint32_t n, fq12* out, uint8_t* se
     }
 }
 
+constexpr uint32_t FE_LIMB_MAX = 6 * 152;
 void final_exp_group(const void* in, uint32_t n, void* out, void* ser, uint32_t per, size_t stride_a,
                      size_t stride_b, cudaStream_t s) {
     if (!n) return;
@@ -108,8 +109,10 @@ void final_exp_group(const void* in, uint32_t n, void* out, void* ser, uint32_t 
                                                                                   stride_b));
         return;
     }
-    if (n <= lim.fe_block_max) {
-        FP_KERNEL("k_final_exp_c", s, k_final_exp_c<<<n, L12_THREADS, 0, s>>>((const fq12*)in, n, (fq12*)out, (uint8_t*)ser, per,
+    // limb lanes also beyond the block limit (if there is one) up to six blocks per SM: 512 take 0.8 ms, 1024
+    // 1.56 ms; a warp each takes 1.48 ms for 257 to 1024
+    if (n <= lim.fe_block_max || (lim.fe_block_max && n <= FE_LIMB_MAX)) {
+        FP_KERNEL(n <= lim.fe_block_max ? "k_final_exp_c" : "k_final_exp_w", s, k_final_exp_c<<<n, L12_THREADS, 0, s>>>((const fq12*)in, n, (fq12*)out, (uint8_t*)ser, per,
                                                                      stride_a, stride_b));
         return;
     }
@@ -145,61 +148,37 @@ void fq12_pair_reduce(const void* in, void* out, uint64_t n, cudaStream_t s) {
     FP_KERNEL("k_fq12_pair", s, k_fq12_pair<<<grid_for(n, 64), 64, 0, s>>>((const fq12*)in, (fq12*)out, n));
 }
 
-// Miller loops, one warp per pair (warp12.cuh).  Pair t of Step 1 round h: t = (k, side, i) with
-// side 0: (A_k[h + i], v_k[i]) and side 1: (A_k[i], v_k[h + i]); Commit: (C_j, v_j = g2pow[2 j]).
-__global__ void __launch_bounds__(128) k_round_miller_w(const g1a* A, const g2a* v, uint32_t K, uint32_t R,
-                                                        uint32_t h, fq12* out) {
-    __shared__ WMill sm[4];
-    const int w = threadIdx.x >> 5, L = threadIdx.x & 31;
-    const uint64_t t = (uint64_t)blockIdx.x * 4 + w;
-    if (t >= (uint64_t)K * 2 * h) return;                 // warp-uniform
-    const uint64_t k = t / (2 * h);
-    const uint32_t r = (uint32_t)(t % (2 * h)), side = r / h, i = r % h;
-    const g1a* Ak = A + k * R;
-    const g2a* vk = v + k * R;
-    if (side == 0) w_miller<1>(sm[w], Ak[h + i], vk[i]);
-    else w_miller<1>(sm[w], Ak[i], vk[h + i]);
-    if (L < 12) reinterpret_cast<fq*>(&out[t])[2 * w_tower_pos(L >> 1) + (L & 1)] = sm[w].f[L];
+// Miller loops with few pairs, one block per pair, one limb per lane (limb_miller.cuh).  Pair t of Step 1
+// round h: t = (k, side, i) with side 0: (A_k[h + i], v_k[i]) and side 1: (A_k[i], v_k[h + i]); Commit:
+// (C_j, v_j = g2pow[2 j]).
+// One launch (one GB300): 0.205 ms for up to 152 pairs (latency: 152 rounds of ~2.8 k cycles), 0.34 for
+// 256, 1.25 for 1024, 4.5 for 4096, 8.8 for 8192.  With one Fq product per lane a 128-thread block per pair
+// took 0.42 ms for few pairs and 1.4 for 1024, a warp per pair 11.1 ms for 8192; one thread per pair takes
+// 19.8 ms for 16384 and 14.2 for 32768 (fewer run slower: their spills then miss).
+FPG_DEV void miller_block(const g1a& P, const g2a& Q, fq12* out) {
+    __shared__ LimbMiller S;
+    const LmLane c = lm_lane();
+    const fq v = lm_miller(S, c, P, Q);
+    if (!c.point && c.k.l == 0) reinterpret_cast<fq*>(out)[2 * w_tower_pos(c.kc) + c.e] = v;
 }
-__global__ void __launch_bounds__(128) k_commit_miller_w(const g1a* rows, const g2a* g2pow, uint32_t R, fq12* out) {
-    __shared__ WMill sm[4];
-    const int w = threadIdx.x >> 5, L = threadIdx.x & 31;
-    const uint64_t j = (uint64_t)blockIdx.x * 4 + w;
-    if (j >= R) return;
-    w_miller<1>(sm[w], rows[j], g2pow[2 * j]);
-    if (L < 12) reinterpret_cast<fq*>(&out[j])[2 * w_tower_pos(L >> 1) + (L & 1)] = sm[w].f[L];
-}
-// the same with one 128-thread block per pair (fewer rounds per step)
-__global__ void __launch_bounds__(128) k_round_miller_c(const g1a* A, const g2a* v, uint32_t K, uint32_t R,
-                                                        uint32_t h, fq12* out) {
-    __shared__ WMill S;
-    const int L = threadIdx.x;
+__global__ void __launch_bounds__(LM_THREADS, 2) k_round_miller_c(const g1a* A, const g2a* v, uint32_t K, uint32_t R,
+                                                               uint32_t h, fq12* out) {
     const uint64_t t = blockIdx.x;
     const uint64_t k = t / (2 * h);
     const uint32_t r = (uint32_t)(t % (2 * h)), side = r / h, i = r % h;
     const g1a* Ak = A + k * R;
     const g2a* vk = v + k * R;
-    if (side == 0) w_miller<4>(S, Ak[h + i], vk[i]);
-    else w_miller<4>(S, Ak[i], vk[h + i]);
-    if (L < 12) reinterpret_cast<fq*>(&out[t])[2 * w_tower_pos(L >> 1) + (L & 1)] = S.f[L];
+    miller_block(side == 0 ? Ak[h + i] : Ak[i], side == 0 ? vk[i] : vk[h + i], &out[t]);
 }
-__global__ void __launch_bounds__(128) k_commit_miller_c(const g1a* rows, const g2a* g2pow, fq12* out) {
-    __shared__ WMill S;
-    const int L = threadIdx.x;
+__global__ void __launch_bounds__(LM_THREADS, 2) k_commit_miller_c(const g1a* rows, const g2a* g2pow, fq12* out) {
     const uint64_t j = blockIdx.x;
-    w_miller<4>(S, rows[j], g2pow[2 * j]);
-    if (L < 12) reinterpret_cast<fq*>(&out[j])[2 * w_tower_pos(L >> 1) + (L & 1)] = S.f[L];
+    miller_block(rows[j], g2pow[2 * j], &out[j]);
 }
+// (the two names keep the ranges of the engine limits apart in profiles)
 void round_miller_w(const void* A, const void* v, uint32_t K, uint32_t R, uint32_t h, void* out, cudaStream_t s) {
     const uint64_t n = (uint64_t)K * 2 * h;
-    if (n <= engine_limits().miller_block_max) {
-        FP_KERNEL("k_round_miller_c", s, k_round_miller_c<<<(unsigned)n, 128, 0, s>>>((const g1a*)A, (const g2a*)v, K, R,
-                                                                                     h, (fq12*)out));
-        return;
-    }
-    FP_KERNEL("k_round_miller_w", s, k_round_miller_w<<<(unsigned)((n + 3) / 4), 128, 0, s>>>((const g1a*)A,
-                                                                                             (const g2a*)v, K, R, h,
-                                                                                             (fq12*)out));
+    FP_KERNEL(n <= engine_limits().miller_block_max ? "k_round_miller_c" : "k_round_miller_w", s,
+              k_round_miller_c<<<(unsigned)n, LM_THREADS, 0, s>>>((const g1a*)A, (const g2a*)v, K, R, h, (fq12*)out));
 }
 
 void commit_miller(const void* rows, const void* g2pow, uint32_t R, void* out, cudaStream_t s) {
@@ -210,14 +189,8 @@ void commit_miller(const void* rows, const void* g2pow, uint32_t R, void* out, c
                                                                                        (fq12*)out));
         return;
     }
-    if (R <= lim.commit_block_max) {
-        FP_KERNEL("k_commit_miller_c", s, k_commit_miller_c<<<R, 128, 0, s>>>((const g1a*)rows, (const g2a*)g2pow,
-                                                                             (fq12*)out));
-        return;
-    }
-    FP_KERNEL("k_commit_miller_w", s, k_commit_miller_w<<<(R + 3) / 4, 128, 0, s>>>((const g1a*)rows,
-                                                                                   (const g2a*)g2pow, R,
-                                                                                   (fq12*)out));
+    FP_KERNEL(R <= lim.commit_block_max ? "k_commit_miller_c" : "k_commit_miller_w", s,
+              k_commit_miller_c<<<R, LM_THREADS, 0, s>>>((const g1a*)rows, (const g2a*)g2pow, (fq12*)out));
 }
 // grouping pays once the grouped threads still fill the GPU several times over (2^16 threads)
 uint32_t step1_miller_group(uint64_t n, uint32_t h, const EngineLimits& lim) {

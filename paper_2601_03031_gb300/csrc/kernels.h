@@ -26,10 +26,10 @@ void prof_end(cudaStream_t s);
 // every engine computes the same values, so a limit changes which kernels run, never the bytes.
 struct EngineLimits {
     uint32_t miller_block_max = 1024;       // Step-1 Miller loops per launch: <= this, a block each
-    uint32_t miller_warp_max = 16383;       //   <= this, a warp each; above, a thread each
+    uint32_t miller_warp_max = 16383;       //   <= this, a block each too; above, a thread each
     uint32_t miller_group_min = 1u << 18;   //   from this many (h >= 4), 4 pairs of a product per thread
     uint32_t commit_block_max = 1024;       // Commit's Miller loops: <= this, a block each
-    uint32_t commit_warp_max = 16384;       //   <= this, a warp each; above, a thread each
+    uint32_t commit_warp_max = 16384;       //   <= this, a block each too; above, a thread each
     uint32_t fe_block_max = 256;            // final exponentiations per launch: <= this, a block each
     uint32_t fe_warp_max = 0xffffffffu;     //   <= this, a warp each; above, a thread each
     uint32_t pair_block_max = 2048;         // pairwise Fq12 products: <= this, a block each; above, a thread

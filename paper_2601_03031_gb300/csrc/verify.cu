@@ -27,6 +27,7 @@
 
 #include "group_ec.cuh"
 #include "k_common.cuh"
+#include "limb_miller.cuh"
 #include "warp12.cuh"
 
 namespace fpk {
@@ -374,13 +375,13 @@ __global__ void k_vb_pairs(uint32_t nb, const g1a* g1beta, const g1j* c1, VBlk* 
     Q[3 * q + 2] = g2_affine(g2_madd(g2j{B.Pzg.X, fq2_neg(B.Pzg.Y), B.Pzg.Z}, B.vl));
 }
 
-// one 128-thread block per pair
-__global__ void __launch_bounds__(128) k_v_miller(const g1a* P, const g2a* Q, fq12* out) {
-    __shared__ WMill S;
-    const int L = threadIdx.x;
+// one block per pair, one limb per lane (limb_miller.cuh)
+__global__ void __launch_bounds__(LM_THREADS, 2) k_v_miller(const g1a* P, const g2a* Q, fq12* out) {
+    __shared__ LimbMiller S;
+    const LmLane c = lm_lane();
     const uint64_t j = blockIdx.x;
-    w_miller<4>(S, P[j], Q[j]);
-    if (L < 12) reinterpret_cast<fq*>(&out[j])[2 * w_tower_pos(L >> 1) + (L & 1)] = S.f[L];
+    const fq v = lm_miller(S, c, P[j], Q[j]);
+    if (!c.point && c.k.l == 0) reinterpret_cast<fq*>(&out[j])[2 * w_tower_pos(c.kc) + c.e] = v;
 }
 
 // L_j.T^(x_j) and R_j.T^(1/x_j) of block q at 2 lr q + 2 (j - 1) + side
@@ -700,7 +701,7 @@ void verify_one(const void* proof, const void* C_be, const void* mi_be, uint32_t
     const PiSrc pi{pr + Ly.pst(), 0, M, lc};
     FP_KERNEL("k_vp_pairs", s, k_vp_pairs<<<1, 32, 0, s>>>(pi, nullptr, (uint32_t)(i % M), O.E, 1,
                                                            (const g2a*)g2tau, O.job_bad, O.P + 3, O.Q + 3));
-    FP_KERNEL("k_v_miller", s, k_v_miller<<<np, 128, 0, s>>>(O.P, O.Q, O.ml));
+    FP_KERNEL("k_v_miller", s, k_v_miller<<<np, LM_THREADS, 0, s>>>(O.P, O.Q, O.ml));
     FP_KERNEL("k_vb_gt", s, k_vb_gt<<<2 * lr, 128, 0, s>>>(S, O.Bb.st, O.Bb.ge));
     FP_KERNEL("k_vb_prod", s, k_vb_prod<<<1, 32, 0, s>>>(O.ml, O.Bb.ge, O.Cd, 1, lr, O.fe_in, O.Bb.cT));
     FP_KERNEL("k_vp_prod", s, k_vp_prod<<<1, 32, 0, s>>>(O.ml + 3, lc + 1, 1, O.fe_in + 2));
@@ -742,7 +743,7 @@ void verify_block(const void* blk, const void* fc, const void* C_be, uint32_t nk
     BlockOnlyBufs<Arena> O(ar, b, lr);
     FP_KERNEL("k_v_cdec", s, k_v_cdec<<<1, 32, 0, s>>>((const uint8_t*)C_be, O.Cd, O.cbad));
     block_checks_front(S, (const uint8_t*)C_be, (const g1a*)g1beta, O.Bb, s);
-    FP_KERNEL("k_v_miller", s, k_v_miller<<<3, 128, 0, s>>>(O.Bb.P, O.Bb.Q, O.Bb.ml));
+    FP_KERNEL("k_v_miller", s, k_v_miller<<<3, LM_THREADS, 0, s>>>(O.Bb.P, O.Bb.Q, O.Bb.ml));
     FP_KERNEL("k_vb_gt", s, k_vb_gt<<<2 * lr, 128, 0, s>>>(S, O.Bb.st, O.Bb.ge));
     FP_KERNEL("k_vb_prod", s, k_vb_prod<<<1, 32, 0, s>>>(O.Bb.ml, O.Bb.ge, O.Cd, 1, lr, O.Bb.fe_in, O.Bb.cT));
     final_exp_group(O.Bb.fe_in, 2, O.Bb.fe_out, nullptr, 1, 0, 0, s);
@@ -903,7 +904,7 @@ void verify_eval(const void* proof, const void* C_be, const void* r_be, int log_
     FP_KERNEL("k_vb_scalars", s, k_vb_scalars<<<1, 64, 0, s>>>(S, O.Bb.wt, O.Bb.st));
     FP_KERNEL("k_vb_muls", s, k_vb_muls<<<2, 128, 0, s>>>(O.Bb.st, 1, 1));
     FP_KERNEL("k_vb_pairs", s, k_vb_pairs<<<1, 64, 0, s>>>(1, (const g1a*)g1beta, x, O.Bb.st, O.Bb.P, O.Bb.Q));
-    FP_KERNEL("k_v_miller", s, k_v_miller<<<3, 128, 0, s>>>(O.Bb.P, O.Bb.Q, O.Bb.ml));
+    FP_KERNEL("k_v_miller", s, k_v_miller<<<3, LM_THREADS, 0, s>>>(O.Bb.P, O.Bb.Q, O.Bb.ml));
     FP_KERNEL("k_vb_gt", s, k_vb_gt<<<2 * lr, 128, 0, s>>>(S, O.Bb.st, O.Bb.ge));
     FP_KERNEL("k_vb_prod", s, k_vb_prod<<<1, 32, 0, s>>>(O.Bb.ml, O.Bb.ge, O.Cd, 1, lr, O.Bb.fe_in, O.Bb.cT));
     final_exp_group(O.Bb.fe_in, 2, O.Bb.fe_out, nullptr, 1, 0, 0, s);
@@ -912,7 +913,7 @@ void verify_eval(const void* proof, const void* C_be, const void* r_be, int log_
     FP_KERNEL("k_ve_E", s, k_ve_E<<<1, 32, 0, s>>>(O.CF, O.y, O.E));
     FP_KERNEL("k_ve_pst_pairs", s, k_ve_pst_pairs<<<lc + 1, 32, 0, s>>>(pr + 128 + blen, O.r_mont, (const g2a*)g2tau,
                                                                        lc, O.E, O.dec_bad, O.P, O.Q));
-    FP_KERNEL("k_v_miller", s, k_v_miller<<<lc + 1, 128, 0, s>>>(O.P, O.Q, O.ml));
+    FP_KERNEL("k_v_miller", s, k_v_miller<<<lc + 1, LM_THREADS, 0, s>>>(O.P, O.Q, O.ml));
     FP_KERNEL("k_vp_prod", s, k_vp_prod<<<1, 32, 0, s>>>(O.ml, lc + 1, 1, O.fe_in));
     final_exp_group(O.fe_in, 1, O.fe_out, nullptr, 1, 0, 0, s);
     cudaMemsetAsync(O.pst_res, 0, 4, s);
@@ -1101,7 +1102,7 @@ void pst_jobs(const ProofLayout& L, JobBufs<A>& J, uint32_t nj, const uint32_t* 
     cudaMemsetAsync(J.bad, 0, (size_t)nj * 4, s);
     FP_KERNEL("k_vp_pairs", s, k_vp_pairs<<<grid_for(np, 64), 64, 0, s>>>(pi, job_a, 0, J.E, nj, g2tau, J.bad, J.P,
                                                                         J.Q));
-    FP_KERNEL("k_v_miller", s, k_v_miller<<<(unsigned)np, 128, 0, s>>>(J.P, J.Q, J.ml));
+    FP_KERNEL("k_v_miller", s, k_v_miller<<<(unsigned)np, LM_THREADS, 0, s>>>(J.P, J.Q, J.ml));
     FP_KERNEL("k_vp_prod", s, k_vp_prod<<<grid_for(nj, 64), 64, 0, s>>>(J.ml, lc + 1, nj, J.fe_in));
     final_exp_group(J.fe_in, nj, J.fe_out, nullptr, 1, 0, 0, s);
     FP_KERNEL("k_vp_check", s, k_vp_check<<<grid_for(nj, 64), 64, 0, s>>>(J.fe_out, J.bad, nj, idx, q0, res));
@@ -1137,7 +1138,7 @@ uint64_t verify_all(const ProofLayout& L, const void* C_be, const void* m, const
     const VSrc S{rs, (size_t)L.b * G1_SER, (const uint8_t*)blocks, L.bopen_len, 0, L.K, L.b, L.R, L.log_r};
     FP_KERNEL("k_v_cdec", s, k_v_cdec<<<1, 32, 0, s>>>(Cb, Ab.Cd, Ab.cbad));
     block_checks_front(S, Cb, (const g1a*)g1beta, Bb, s);
-    FP_KERNEL("k_v_miller", s, k_v_miller<<<3 * L.K, 128, 0, s>>>(Bb.P, Bb.Q, Bb.ml));
+    FP_KERNEL("k_v_miller", s, k_v_miller<<<3 * L.K, LM_THREADS, 0, s>>>(Bb.P, Bb.Q, Bb.ml));
     FP_KERNEL("k_vb_gt", s, k_vb_gt<<<2 * L.log_r * L.K, 128, 0, s>>>(S, Bb.st, Bb.ge));
     FP_KERNEL("k_vb_prod", s, k_vb_prod<<<grid_for(L.K, 64), 64, 0, s>>>(Bb.ml, Bb.ge, Ab.Cd, L.K, L.log_r, Bb.fe_in,
                                                                        Bb.cT));

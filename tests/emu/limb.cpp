@@ -4,6 +4,7 @@
 #include "pairing.cuh"
 #include "limb12.cuh"
 #include "limb_ec.cuh"
+#include "limb_miller.cuh"
 
 #include <vector>
 
@@ -29,6 +30,7 @@ void lanes(int n, Fn fn) {
 int tower_pos(int k) { return (k & 1) ? 3 + (k >> 1) : (k >> 1); }
 L12 g_w;
 LimbEc g_ec;
+LimbMiller g_m;
 LimbEc2 g_ec2;
 }  // namespace
 
@@ -107,6 +109,17 @@ void emu_limb_g1_mul_add(const uint8_t* p, const uint32_t* k, const uint8_t* q, 
         lec_add_affine(g_ec, c, Q);
         const fq v = lec_affine(g_ec, c);
         if (c.k.l == 0 && c.slot < 2) fq_to_be(out + 48 * c.slot, v);
+    });
+}
+void emu_limb_miller(const uint8_t* p, const uint8_t* q, uint8_t* out) {
+    g1a P;
+    P.x = be_fq(p); P.y = be_fq(p + 48);
+    g2a Q;
+    Q.x.c0 = be_fq(q); Q.x.c1 = be_fq(q + 48); Q.y.c0 = be_fq(q + 96); Q.y.c1 = be_fq(q + 144);
+    lanes(LM_THREADS, [&] {
+        const LmLane c = lm_lane();
+        const fq v = lm_miller(g_m, c, P, Q);
+        if (!c.point && c.k.l == 0) fq_to_be(out + 48 * (2 * tower_pos(c.kc) + c.e), v);
     });
 }
 }

@@ -25,7 +25,7 @@ def emu(tmp_path_factory):
     subprocess.check_call([gxx, "-std=c++20", "-O1", "-shared", "-fPIC", f"-I{CSRC}", "-o", so,
                            os.path.join(HERE, "emu", "limb.cpp")])
     L = ctypes.CDLL(so)
-    for f in (L.emu_limb_dot3, L.emu_limb_final_exp, L.emu_limb_g1_mul, L.emu_limb_g2_mul_add, L.emu_limb_g1_mul_add):
+    for f in (L.emu_limb_dot3, L.emu_limb_final_exp, L.emu_limb_g1_mul, L.emu_limb_g2_mul_add, L.emu_limb_g1_mul_add, L.emu_limb_miller):
         f.restype = None
     return L
 
@@ -96,3 +96,18 @@ def test_g1_scalar_mul_and_add_against_oracle(emu):
     for p, k, q in cases:
         emu.emu_limb_g1_mul_add(p, (ctypes.c_uint32 * 8)(*[(k >> (32 * i)) & 0xFFFFFFFF for i in range(8)]), q, out)
         assert out.raw == O.g1_add(O.g1_mul(p, k), q), hex(k)
+
+
+def test_miller_loop_against_oracle(emu):
+    """The final exponentiation of the Miller value is the pairing (line scalings vanish under it); an
+    identity on either side gives 1."""
+    rnd = random.Random(9)
+    out = ctypes.create_string_buffer(576)
+    for _ in range(2):
+        P, Q = O.g1_mul(O.g1_gen(), rnd.randrange(1, ref.R)), O.g2_mul(O.g2_gen(), rnd.randrange(1, ref.R))
+        emu.emu_limb_miller(P, Q, out)
+        assert O.final_exp(out.raw) == O.pairing(P, Q)
+    one = (1).to_bytes(48, "big") + bytes(528)
+    for p, q in ((bytes(96), Q), (P, bytes(192))):
+        emu.emu_limb_miller(p, q, out)
+        assert out.raw == one
