@@ -120,6 +120,37 @@ void final_exp_group(const void* in, uint32_t n, void* out, void* ser, uint32_t 
                                                                            (uint8_t*)ser, per, stride_a, stride_b));
 }
 
+// out[q out_stride] = (base ? *base : 1) prod_{u < per} in[q stride + u], one block per q, one limb per lane:
+// a factor costs its conversion and a product, 1.8 us, where a launch of pairwise products takes 8
+__global__ void __launch_bounds__(L12_THREADS) k_fq12_prod(const fq12* base, const fq12* in, uint32_t stride,
+                                                           uint32_t per, fq12* out, uint32_t out_stride) {
+    __shared__ L12 W;
+    const L12Lane c = l12_lane();
+    const uint64_t q = blockIdx.x;
+    const int pos = 2 * w_tower_pos(c.kc) + c.e;
+    const fq12* src = in + q * stride;
+    const uint32_t n = per + (base ? 1 : 0);
+    int32_t *acc = W.v[0], *nxt = W.v[1];
+    for (uint32_t u = 0; u < n; u++) {
+        const fq12* f = base ? (u ? src + (u - 1) : base) : src + u;
+        l12_load(W, c, u ? W.v[2] : acc, W.v[3], reinterpret_cast<const fq*>(f)[pos]);
+        if (u) {
+            l12_mul(W, c, nxt, acc, W.v[2], false);
+            int32_t* t = acc;
+            acc = nxt;
+            nxt = t;
+        }
+    }
+    const fq v = l12_store(W, c, acc, W.v[3]);
+    if (c.k.l == 0) reinterpret_cast<fq*>(&out[q * out_stride])[pos] = v;
+}
+void fq12_products(const void* base, const void* in, uint32_t stride, uint32_t per, void* out, uint32_t out_stride,
+                   uint64_t n, cudaStream_t s) {
+    if (!n) return;
+    FP_KERNEL("k_fq12_prod", s, k_fq12_prod<<<(unsigned)n, L12_THREADS, 0, s>>>((const fq12*)base, (const fq12*)in, stride,
+                                                                               per, (fq12*)out, out_stride));
+}
+
 // pairwise Fq12 products out[i] = in[2i] in[2i+1]: one 128-thread block per product when there are
 // few (latency), one thread per product otherwise
 __global__ void k_fq12_pair(const fq12* in, fq12* out, uint64_t n) {

@@ -65,6 +65,9 @@ void g2_pair_reduce(const void* in_g2j, void* out_g2j, uint64_t n_out, cudaStrea
 void g1_tree_reduce(const void* in_g1j, void* out_g1j, uint64_t n_in, uint32_t gs, cudaStream_t s);
 void g2_tree_reduce(const void* in_g2j, void* out_g2j, uint64_t n_in, uint32_t gs, cudaStream_t s);
 void fq12_pair_reduce(const void* in, void* out, uint64_t n_out, cudaStream_t s);
+// out[q out_stride] = (base ? *base : 1) prod_{u < per} in[q stride + u] for q < n, one block each
+void fq12_products(const void* base, const void* in, uint32_t stride, uint32_t per, void* out, uint32_t out_stride,
+                   uint64_t n, cudaStream_t s);
 void g1j_to_affine(const void* in_g1j, void* out_g1a, void* ser_out, size_t ser_stride, uint64_t n, cudaStream_t s);
 void g2j_to_affine(const void* in_g2j, void* out_g2a, void* ser_out, size_t ser_stride, uint64_t n, cudaStream_t s);
 void g1a_serialize(const void* in_g1a, void* ser_out, size_t ser_stride, uint64_t n, cudaStream_t s);
@@ -199,26 +202,29 @@ void eval_bvec(const void* C_ser, const void* r_be, int log_n, const void* CF_se
 void eval_pst_fold(void* F, const void* r_mont, int log_c, void* q, void* y_out, cudaStream_t s);
 void eval_pst_terms(const void* q, const void* lam, uint32_t M, void* out, cudaStream_t s);
 
-// ---- VC.Verify (verify.cu).  One proof: result word 0 = 0 if accepted.
+// ---- VC.Verify (verify.cu), on s and on side streams that are joined back to it before the call returns
+// (independent checks run beside each other).  One proof: result word 0 = 0 if accepted.
 size_t verify_scratch_bytes(uint32_t b, int lr, int lc);
 void verify_one(const void* proof, const void* C_be, const void* mi_be, uint32_t nk, int lr, int lc, uint32_t b,
                 uint64_t i, uint32_t M, uint32_t k, uint32_t lo, const void* g1beta, const void* g2tau, void* scratch,
-                uint32_t* result, cudaStream_t s);
+                uint32_t* result, cudaStream_t s, cudaStream_t side, cudaStream_t side2);
 // FC.BVerify of one block: blk = its nk row commitments, fc = pi_{C_k}; result word 0 = 0 if accepted
 size_t verify_block_scratch_bytes(uint32_t b, int lr);
 void verify_block(const void* blk, const void* fc, const void* C_be, uint32_t nk, int lr, uint32_t b, uint32_t k,
-                  uint32_t lo, const void* g1beta, void* scratch, uint32_t* result, cudaStream_t s);
+                  uint32_t lo, const void* g1beta, void* scratch, uint32_t* result, cudaStream_t s, cudaStream_t side);
 // The evaluation proof at r (proof = y | C_F | pi_FC | pi_PST, r log_n x 32 B big-endian); result
 // word 0 = 0 if accepted
 size_t verify_eval_scratch_bytes(uint32_t R, int lr, int lc, int log_n);
 void verify_eval(const void* proof, const void* C_be, const void* r_be, int log_n, int lr, int lc, uint32_t R,
-                 const void* g1beta, const void* g2tau, void* scratch, uint32_t* result, cudaStream_t s);
+                 const void* g1beta, const void* g2tau, void* scratch, uint32_t* result, cudaStream_t s,
+                 cudaStream_t side, cudaStream_t side2);
 // All N proofs of an OpenAll output (its shared pieces as stored by vc_prove_all) against the
 // claimed values m (device, N x 4 little-endian u64): ok_out (host, N bytes, may be null) gets 1
 // per accepted proof; returns the number accepted.  each = 1: no PST check is shared.  Synchronises.
 size_t verify_all_scratch_bytes(const ProofLayout& L);
 uint64_t verify_all(const ProofLayout& L, const void* C_be, const void* m, const void* rows_ser, const void* blocks,
                     const void* row_tree, const void* top_tree, const void* D_ser, const void* g, const void* pst_ser,
-                    const void* g1beta, const void* g2tau, int each, void* scratch, void* ok_out, cudaStream_t s);
+                    const void* g1beta, const void* g2tau, int each, void* scratch, void* ok_out, cudaStream_t s,
+                    cudaStream_t side, cudaStream_t side2);
 
 }  // namespace fpk

@@ -1027,8 +1027,9 @@ fp_status vc_verify(const fp_pp* pp, const uint8_t* C, uint32_t b, uint64_t i, c
             res = dalloc(sizeof(uint32_t), s);
             check(cudaMemcpyAsync(dbuf, host.data(), host.size(), cudaMemcpyHostToDevice, s), "H2D proof");
             const uint8_t* d = (const uint8_t*)dbuf;
+            const Streams st = streams(s);
             verify_one(d, d + len, d + len + GT_SER, nk, lr, lc, b, i, pp->M, k, lo, pp->g1beta, pp->g2tau, scr,
-                       (uint32_t*)res, s);
+                       (uint32_t*)res, s, st.sp, st.la[0]);
             check_launch("vc_verify kernels");
             check(cudaMemcpyAsync(&hres, res, sizeof hres, cudaMemcpyDeviceToHost, s), "D2H result");
             dfree(dbuf, s); dfree(scr, s); dfree(res, s);
@@ -1065,8 +1066,9 @@ fp_status vc_verify_all(const fp_pp* pp, const uint8_t* C, const uint64_t* m, in
                 md = dm;
             }
             scr = dalloc(verify_all_scratch_bytes(L), s);
+            const Streams st = streams(s);
             const uint64_t good = verify_all(L, dC, md, pf->rows_ser, pf->blocks, pf->row_tree, pf->top_tree, pf->D_ser,
-                                             pf->g, pf->pst_ser, pp->g1beta, pp->g2tau, flags & 1, scr, ok, s);
+                                             pf->g, pf->pst_ser, pp->g1beta, pp->g2tau, flags & 1, scr, ok, s, st.sp, st.la[0]);
             check_launch("vc_verify_all kernels");
             dfree(dC, s); dfree(dm, s); dfree(scr, s);
             check(cudaStreamSynchronize(s), "vc_verify_all");
@@ -1192,8 +1194,9 @@ fp_status vc_eval_verify(const fp_pp* pp, const uint8_t* C, const uint8_t* r, co
             res = dalloc(sizeof(uint32_t), s);
             check(cudaMemcpyAsync(dbuf, host.data(), host.size(), cudaMemcpyHostToDevice, s), "H2D");
             const uint8_t* d = (const uint8_t*)dbuf;
+            const Streams st = streams(s);
             verify_eval(d, d + len, d + len + GT_SER, ln, (int)pp->log_r, (int)pp->log_c, pp->R, pp->g1beta,
-                        pp->g2tau, scr, (uint32_t*)res, s);
+                        pp->g2tau, scr, (uint32_t*)res, s, st.sp, st.la[0]);
             check_launch("vc_eval_verify kernels");
             check(cudaMemcpyAsync(&hres, res, sizeof hres, cudaMemcpyDeviceToHost, s), "D2H result");
             dfree(dbuf, s); dfree(scr, s); dfree(res, s);
@@ -1281,7 +1284,7 @@ fp_status vc_verify_segment(const fp_pp* pp, const uint8_t* C, uint32_t b, uint3
             uint32_t* o = (uint32_t*)out;
             load_vector(d + len + GT_SER, M, mc, mm, o + 1, s);
             msm_g1(pp->lam_tab, mc, sh, mscr, cj, o + 2, s);       // C_j from m_j (VC.Commit's row MSM)
-            verify_block(d, d + (size_t)nk * G1_SER, d + len, nk, lr, b, k, lo, pp->g1beta, vscr, o, s);
+            verify_block(d, d + (size_t)nk * G1_SER, d + len, nk, lr, b, k, lo, pp->g1beta, vscr, o, s, streams(s).sp);
             check_launch("vc_verify_segment kernels");
             check(cudaMemcpyAsync(hout, out, sizeof hout, cudaMemcpyDeviceToHost, s), "D2H");
             dfree(dbuf, s); dfree(vscr, s); dfree(mscr, s); dfree(mc, s); dfree(mm, s); dfree(cj, s); dfree(out, s);

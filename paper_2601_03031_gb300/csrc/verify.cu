@@ -27,6 +27,7 @@
 
 #include "group_ec.cuh"
 #include "k_common.cuh"
+#include "limb_ec.cuh"
 #include "limb_miller.cuh"
 #include "warp12.cuh"
 
@@ -103,27 +104,32 @@ FPG_DEV bool digest_same(const uint8_t* a, const uint8_t* b) {
     return true;
 }
 FPG_DEV g2a g2a_negate(const g2a& p) { return g2a_is_inf(p) ? p : g2a{p.x, fq2_neg(p.y)}; }
-// homogeneous projective (X : Y : Z) -> Jacobian (X Z, Y Z^2, Z)
-FPG_DEV g1j proj_to_jac(const GPt<fq>& r) {
-    g1j o;
-    o.X = fq_mul(r.X, r.Z);
-    o.Y = fq_mul(r.Y, fq_sqr(r.Z));
-    o.Z = r.Z;
-    return o;
-}
-FPG_DEV g2j proj_to_jac(const GPt<fq2>& r) {
-    g2j o;
-    o.X = fq2_mul(r.X, r.Z);
-    o.Y = fq2_mul(r.Y, fq2_sqr(r.Z));
-    o.Z = r.Z;
-    return o;
-}
-// k P on one 8-lane group (GLV, 2-bit joint windows); every lane of the group must call it
-FPG_DEV g1j g1_mul8(GEc<fq>& sm, int lane, const g1a& P, const fr& k_mont) {
+// k P + Q as an affine point on 96 threads, one limb per lane (limb_ec.cuh): x and y on the first lanes
+// of slots 0 and 1
+FPG_DEV fq g1_lin(LimbEc& S, const LecLane& c, const g1a& P, const fr& k_mont, const g1a& Q) {
     uint32_t kw[8];
     fr_canon_words(kw, k_mont);
-    return proj_to_jac(gec_g1_mul_proj_w2(sm, lane, P, kw));
+    lec_g1_mul(S, c, P, kw);
+    lec_add_affine(S, c, Q);
+    return lec_affine(S, c);
 }
+FPG_DEV void g1_lin_put(const LecLane& c, g1a* out, const fq& v) {
+    if (c.k.l == 0 && c.slot < 2) reinterpret_cast<fq*>(out)[c.slot] = v;
+}
+// k_mont P + sum_h D_h (n <= 16 serialised points at dser + 96 off(h)) into S.acc, on 96 threads; the
+// return value is false on a thread that met a malformed point
+template <class Off>
+FPG_DEV bool g1_mul_sum(LimbEc& S, const LecLane& c, g1a* D, const g1a& P, const fr& k_mont, const uint8_t* dser, int n,
+                        Off&& off) {
+    bool ok = true;
+    if (lec_thread() < n) ok = g1_decode(dser + off(lec_thread()), D[lec_thread()]);
+    uint32_t kw[8];
+    fr_canon_words(kw, k_mont);
+    lec_g1_mul(S, c, P, kw);
+    for (int h = 0; h < n; h++) lec_add_affine(S, c, D[h]);
+    return ok;
+}
+FPG_DEV g1a g1_neg_gen() { return g1a_neg(g1_generator()); }
 // r_j = HFr("FP-rho", root || u32be(j))
 FPG_DEV fr row_rho(const uint8_t* root, uint32_t j) {
     uint8_t rb[36];
@@ -162,13 +168,10 @@ FPG_DEV void row_leaf_hash(uint8_t* cur, const uint8_t* Cj_be) {
 // FC.BVerify state of one block
 struct VBlk {
     uint32_t bad;
-    uint8_t hstmt[32];
     fr x[32], xinv[32];            // Montgomery
     fr z, Pz, bl;                  // Montgomery
     g1a Al;
     g2a vl, W;
-    g1j blA, zg;
-    g2j Pzg;
 };
 
 // blocks q = 0 .. nb - 1 (block k0 + q): row commitments at blk + q blk_stride, pi_{C_k} at
@@ -189,136 +192,103 @@ __global__ void k_v_cdec(const uint8_t* C_be, fq12* Cd, uint32_t* cbad) {
     *cbad = fq12_decode(C_be, *Cd) ? 0u : 1u;
 }
 
-// D_k, the tree root over the nk >= 1 row commitments at blk (96 bytes each), on one thread: the
-// leaves SHA256("FP-sleaf" || C_a) go in order onto a stack of subtree roots, two subtrees of equal
-// height merge as SHA256("FP-snode" || left || right) as soon as they meet, and the stack is then
-// folded from the top; this is the level-by-level tree with an odd last node carried up
-FPG_DEV void stmt_rows_root(const uint8_t* blk, uint32_t nk, uint8_t* out) {
-    uint8_t st[33][32];
-    int hgt[33];
-    int sp = 0;
-    auto node = [&](int l) {                           // st[l] <- H(st[l] || st[l + 1])
-        sha256_ctx c;
-        sha256_init(c);
-        sha256_update(c, (const uint8_t*)"FP-snode", 8);
-        sha256_update(c, st[l], 32);
-        sha256_update(c, st[l + 1], 32);
-        sha256_final(c, st[l]);
-    };
-    for (uint32_t t = 0; t < nk; t++) {
-        sha256_ctx c;
-        sha256_init(c);
-        sha256_update(c, (const uint8_t*)"FP-sleaf", 8);
-        sha256_update(c, blk + (size_t)t * 96, 96);
-        sha256_final(c, st[sp]);
-        hgt[sp++] = 0;
-        while (sp >= 2 && hgt[sp - 1] == hgt[sp - 2]) {
-            node(sp - 2);
-            hgt[sp - 2]++;
-            sp--;
-        }
-    }
-    while (sp >= 2) {
-        node(sp - 2);
-        sp--;
-    }
-    for (int q = 0; q < 32; q++) out[q] = st[0][q];
-}
-
-// statement hash, x_j and x_j^-1, A_l, v_l, W, z and P(z) = prod_j (1 + x_j^-1 z^(2^(l - j + 1)))
-__global__ void k_vb_transcript(VSrc S, const uint8_t* C_be, VBlk* st) {
-    const uint64_t q = gtid();
-    if (q >= S.nb) return;
+// x_j and x_j^-1, A_l, v_l, W, z and P(z) = prod_j (1 + x_j^-1 z^(2^(l - j + 1))), one warp per block: the
+// two SHA-256 halves of HFr on two lanes (the chain of the x_j is serial), then the inverses on one lane
+// each and the three points' checks beside each other: 0.55 ms at l = 8.  (On one thread, with the
+// statement's tree, 1.1 ms; the tree is k_stmt_hash's now.)
+__global__ void __launch_bounds__(32) k_vb_transcript(VSrc S, VBlk* st) {
+    __shared__ uint8_t wide[64], xp[32];
+    const uint64_t q = blockIdx.x;
+    const int L = threadIdx.x, lr = S.lr;
     VBlk& B = st[q];
-    const uint32_t k = S.k0 + (uint32_t)q, nk = S.nk((uint32_t)q);
-    const uint8_t* blk = S.blk + q * S.blk_stride;
     const uint8_t* fc = S.fc + q * S.fc_stride;
-    const int lr = S.lr;
-    uint32_t bad = 0;
-    if (S.blk) {                                       // the evaluation proof has no block statement
-        sha256_ctx c;
-        sha256_init(c);
-        sha256_update(c, C_be, 576);
-        uint8_t hdr[12];
-        put_be32(hdr, k); put_be32(hdr + 4, S.b); put_be32(hdr + 8, nk);
-        sha256_update(c, hdr, 12);
-        uint8_t root[32];
-        stmt_rows_root(blk, nk, root);
-        sha256_update(c, root, 32);
-        sha256_final(c, B.hstmt);
-    }
-    uint8_t xprev[32];
+    auto absorb = [&](const char* tag, bool with_x, const uint8_t* d, uint32_t n) {
+        if (L < 2) {
+            sha256_ctx c;
+            sha256_init(c);
+            sha256_update(c, (const uint8_t*)tag, 4);
+            sha256_byte(c, (uint8_t)L);
+            if (with_x) sha256_update(c, xp, 32);
+            sha256_update(c, d, n);
+            sha256_final(c, wide + 32 * L);
+        }
+        __syncwarp();
+    };
     for (int j = 1; j <= lr; j++) {
         const uint8_t* rd = fc + (size_t)(j - 1) * ROUND_BYTES;
-        const fr x = hash_to_fr_nonzero("FP-x", 4, xprev, j > 1 ? 32 : 0, rd, ROUND_BYTES, nullptr, 0);
-        B.x[j - 1] = x;
-        B.xinv[j - 1] = fr_inv(x);
-        fr_to_be(xprev, x);
+        absorb("FP-x", j > 1, rd, ROUND_BYTES);
+        if (L == 0) {
+            fr x = fr_from_be64(wide);
+            if (fr_is_zero(x)) x = hash_to_fr_nonzero("FP-x", 4, xp, j > 1 ? 32 : 0, rd, ROUND_BYTES, nullptr, 0);
+            B.x[j - 1] = x;
+            fr_to_be(xp, x);
+        }
+        __syncwarp();
     }
     const uint8_t* tail = fc + (size_t)lr * ROUND_BYTES;
-    if (!g1_decode(tail, B.Al) || !g2_decode(tail + G1_SER, B.vl) || !g2_decode(tail + G1_SER + G2_SER, B.W))
-        bad |= 2;
-    const fr z = hash_to_fr("FP-z", 4, xprev, 32, tail + G1_SER, G2_SER, nullptr, 0);
-    B.z = z;
-    fr zp[34];
-    zp[0] = z;
-    for (int e = 1; e <= lr + 1; e++) zp[e] = fr_mul(zp[e - 1], zp[e - 1]);
-    fr one, Pz;
-    fr_one(one);
-    Pz = one;
-    for (int j = 1; j <= lr; j++) Pz = fr_mul(Pz, fr_add(one, fr_mul(B.xinv[j - 1], zp[lr - j + 1])));
-    B.Pz = Pz;
-    B.bad = bad;
+    absorb("FP-z", true, tail + G1_SER, G2_SER);
+    if (L < lr) B.xinv[L] = fr_inv(B.x[L]);
+    bool ok = true;
+    if (L == 0) ok = g1_decode(tail, B.Al);
+    else if (L <= 2) ok = g2_decode(tail + G1_SER + (L == 1 ? 0 : G2_SER), L == 1 ? B.vl : B.W);
+    const unsigned all = __ballot_sync(0xffffffffu, ok);
+    __syncwarp();
+    if (L == 0) {
+        const fr z = fr_from_be64(wide);
+        B.z = z;
+        fr zp[34];
+        zp[0] = z;
+        for (int e = 1; e <= lr + 1; e++) zp[e] = fr_mul(zp[e - 1], zp[e - 1]);
+        fr one, Pz;
+        fr_one(one);
+        Pz = one;
+        for (int j = 1; j <= lr; j++) Pz = fr_mul(Pz, fr_add(one, fr_mul(B.xinv[j - 1], zp[lr - j + 1])));
+        B.Pz = Pz;
+        B.bad = all == 0xffffffffu ? 0u : 2u;
+    }
 }
 
-// per block tpb term slots (a power of two): r_a C_a for its nk rows, then x_j L_j.1 and
-// x_j^-1 R_j.1; the b_l summands r_a prod_k x_k^-(bit l - k of a) at wt[q b + t].  One 8-lane
-// group per slot (16 per block); unused slots keep the identity the caller cleared them to.
-__global__ void __launch_bounds__(128) k_vb_terms(VSrc S, VBlk* st, uint32_t tpb, g1j* T, fr* wt) {
-    __shared__ GEc<fq> sm[16];
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
-    const uint64_t t = (uint64_t)blockIdx.x * 16 + grp;
+// per block tpb term slots (a power of two), point and factor each: r_a C_a for its nk rows, then
+// x_j L_j.1 and x_j^-1 R_j.1, then b_l (-A_l) (the factor by k_vb_scalars), so that the sum is the
+// identity if the folded G1 part is b_l A_l; unused slots have factor zero.  The b_l summands
+// r_a prod_k x_k^-(bit l - k of a) at wt[q b + u].
+__global__ void __launch_bounds__(64) k_vb_terms(VSrc S, VBlk* st, const uint8_t* hstmt, uint32_t tpb, g1a* tP, fr* tk,
+                                                 fr* wt) {
+    const uint64_t t = gtid();
+    if (t >= (uint64_t)S.nb * tpb) return;
     const int lr = S.lr;
-    uint32_t q = 0, u = 0, nk = 0;
-    bool valid = t < (uint64_t)S.nb * tpb;
-    if (valid) {
-        q = (uint32_t)(t / tpb);
-        u = (uint32_t)(t % tpb);
-        nk = S.nk(q);
-        valid = u < nk + 2 * (uint32_t)lr;
-    }
-    g1a P;                                             // identity and k = 0 for the idle groups
+    const uint32_t q = (uint32_t)(t / tpb), u = (uint32_t)(t % tpb), nk = S.nk(q);
+    VBlk& B = st[q];
+    g1a P;
     fq_zero(P.x);
     fq_zero(P.y);
     fr k;
     fr_zero(k);
-    if (valid) {
-        VBlk& B = st[q];
-        if (u < nk) {
-            const uint32_t a = S.lo(q) + u;
-            if (!g1_decode(S.blk + q * S.blk_stride + 96 * (size_t)u, P) && lane == 0) atomicOr(&B.bad, 32u);
-            uint8_t buf[36];
-            for (int c = 0; c < 32; c++) buf[c] = B.hstmt[c];
-            put_be32(buf + 32, a);
-            k = hash_to_fr("FP-r", 4, buf, 36, nullptr, 0, nullptr, 0);
-            if (lane == 0) {
-                fr w = k;
-                for (int kk = 1; kk <= lr; kk++)
-                    if ((a >> (lr - kk)) & 1) w = fr_mul(w, B.xinv[kk - 1]);
-                wt[(size_t)q * S.b + u] = w;
-            }
-        } else {
-            const int v = (int)(u - nk), jj = v >> 1, side = v & 1;
-            const uint8_t* rd = S.fc + q * S.fc_stride + (size_t)jj * ROUND_BYTES;
-            if (!g1_decode(rd + (side ? GT_SER + G1_SER + GT_SER : GT_SER), P) && lane == 0) atomicOr(&B.bad, 64u);
-            k = side ? B.xinv[jj] : B.x[jj];
-        }
+    if (u < nk) {
+        const uint32_t a = S.lo(q) + u;
+        if (!g1_decode(S.blk + q * S.blk_stride + 96 * (size_t)u, P)) atomicOr(&B.bad, 32u);
+        uint8_t buf[36];
+        for (int c = 0; c < 32; c++) buf[c] = hstmt[32 * (size_t)q + c];
+        put_be32(buf + 32, a);
+        k = hash_to_fr("FP-r", 4, buf, 36, nullptr, 0, nullptr, 0);
+        fr w = k;
+        for (int kk = 1; kk <= lr; kk++)
+            if ((a >> (lr - kk)) & 1) w = fr_mul(w, B.xinv[kk - 1]);
+        wt[(size_t)q * S.b + u] = w;
+    } else if (u < nk + 2 * (uint32_t)lr) {
+        const int v = (int)(u - nk), jj = v >> 1, side = v & 1;
+        const uint8_t* rd = S.fc + q * S.fc_stride + (size_t)jj * ROUND_BYTES;
+        if (!g1_decode(rd + (side ? GT_SER + G1_SER + GT_SER : GT_SER), P)) atomicOr(&B.bad, 64u);
+        k = side ? B.xinv[jj] : B.x[jj];
+    } else if (u == nk + 2 * (uint32_t)lr) {
+        P = g1a_neg(B.Al);
     }
-    const g1j r = g1_mul8(sm[grp], lane, P, k);
-    if (valid && lane == 0) T[t] = r;
+    tP[t] = P;
+    tk[t] = k;
 }
 
-__global__ void k_vb_scalars(VSrc S, const fr* wt, VBlk* st) {
+// b_l, also as the factor of block q's slot `slot` (or after its nk + 2 l_R terms for slot 0)
+__global__ void k_vb_scalars(VSrc S, const fr* wt, VBlk* st, uint32_t tpb, uint32_t slot, fr* tk) {
     const uint64_t q = gtid();
     if (q >= S.nb) return;
     fr s;
@@ -326,53 +296,58 @@ __global__ void k_vb_scalars(VSrc S, const fr* wt, VBlk* st) {
     const uint32_t nk = S.nk((uint32_t)q);
     for (uint32_t u = 0; u < nk; u++) s = fr_add(s, wt[q * S.b + u]);
     st[q].bl = s;
+    tk[q * tpb + (slot ? slot : nk + 2 * (uint32_t)S.lr)] = s;
 }
 
-// per block: P(z) g2 on one warp (the first nb2 CTAs, four blocks each), b_l A_l and z g1 on
-// 8-lane groups (16 per CTA)
+// Every scalar multiplication of the block checks in one launch, one limb per lane (limb_ec.cuh).  Blocks
+// [0, nb): v_l - P(z) g2 of block q, and its pairs at 3q: (A_l, v_l), (g1^beta - z g1, W),
+// (-g1, v_l - P(z) g2); the others two G1 multiplications each: the nt terms (Jacobian), then g1^beta - z g1
+// of every block.  0.25 ms for one proof (8 lanes per G1 and a warp per G2 point: 0.82 + 0.86 ms in two
+// launches, and 0.25 ms for the conversions to affine on one thread).
 union VMulSmem {
-    GEcW g2[4];
-    GEc<fq> g1[16];
+    LimbEc2 g2;
+    LimbEc g1[2];
 };
-__global__ void __launch_bounds__(128) k_vb_muls(VBlk* st, uint32_t nb, uint32_t nb2) {
+__global__ void __launch_bounds__(LEC2_THREADS) k_vb_muls(VBlk* st, uint32_t nb, const g1a* tP, const fr* tk, uint64_t nt,
+                                                          const g1a* g1beta, g1j* T, g1a* P, g2a* Q) {
     __shared__ VMulSmem sm;
-    if (blockIdx.x < nb2) {
-        const int w = threadIdx.x >> 5, L = threadIdx.x & 31;
-        const uint64_t q = (uint64_t)blockIdx.x * 4 + w;
-        if (q >= nb) return;                                  // warp-uniform
+    if (blockIdx.x < nb) {
+        const uint64_t q = blockIdx.x;
         VBlk& B = st[q];
         uint32_t kw[8];
         fr_canon_words(kw, B.Pz);
-        const GPt<fq2> r = gecw_g2_mul_proj(sm.g2[w], L, g2_generator(), kw);
-        if (L == 0) B.Pzg = proj_to_jac(r);
+        const Lec2Lane c = lec2_lane();
+        lec2_g2_mul(sm.g2, c, g2a_negate(g2_generator()), kw);
+        lec2_add_affine(sm.g2, c, B.vl);
+        const fq v = lec2_affine(sm.g2, c);
+        if (c.k.l == 0 && c.slot < 4) reinterpret_cast<fq*>(&Q[3 * q + 2])[c.slot] = v;
+        if (threadIdx.x == 0) {
+            P[3 * q] = B.Al;
+            Q[3 * q] = B.vl;
+            Q[3 * q + 1] = B.W;
+            P[3 * q + 2] = g1_neg_gen();
+        }
         return;
     }
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
-    const uint64_t t0 = (uint64_t)(blockIdx.x - nb2) * 16 + grp;
-    const bool valid = t0 < 2 * (uint64_t)nb;
-    const uint64_t t = valid ? t0 : 0;
-    VBlk& B = st[t >> 1];
-    const bool zg = t & 1;
-    const g1j r = g1_mul8(sm.g1[grp], lane, zg ? g1_generator() : B.Al, zg ? B.z : B.bl);
-    if (valid && lane == 0) {
-        if (zg) B.zg = r;
-        else B.blA = r;
+    const int half = (int)(threadIdx.x / LEC_THREADS);
+    const uint64_t t = (blockIdx.x - nb) * (uint64_t)2 + half;
+    if (t >= nt + nb) return;                                 // three whole warps, with a barrier of their own
+    const LecLane c = lec_lane();
+    if (t >= nt) {
+        const uint64_t q = t - nt;
+        g1_lin_put(c, &P[3 * q + 1], g1_lin(sm.g1[half], c, g1_neg_gen(), st[q].z, g1beta[0]));
+        return;
     }
-}
-
-// block q's pairs at 3q: (A_l, v_l), (g1^beta - z g1, W), (-g1, v_l - P(z) g2); and b_l A_l
-// against the folded G1 part c1[q]
-__global__ void k_vb_pairs(uint32_t nb, const g1a* g1beta, const g1j* c1, VBlk* st, g1a* P, g2a* Q) {
-    const uint64_t q = gtid();
-    if (q >= nb) return;
-    VBlk& B = st[q];
-    if (!jac_eq(c1[q], B.blA)) atomicOr(&B.bad, 128u);
-    P[3 * q] = B.Al;
-    Q[3 * q] = B.vl;
-    P[3 * q + 1] = g1_affine(g1_madd(g1j_neg(B.zg), g1beta[0]));
-    Q[3 * q + 1] = B.W;
-    P[3 * q + 2] = g1a_neg(g1_generator());
-    Q[3 * q + 2] = g2_affine(g2_madd(g2j{B.Pzg.X, fq2_neg(B.Pzg.Y), B.Pzg.Z}, B.vl));
+    const fr k = tk[t];
+    if (fr_is_zero(k)) {
+        if (lec_thread() == 0) jac_set_inf(T[t]);
+        return;
+    }
+    uint32_t kw[8];
+    fr_canon_words(kw, k);
+    lec_g1_mul(sm.g1[half], c, tP[t], kw);
+    const fq v = lec_jacobian(sm.g1[half], c);
+    if (c.k.l == 0 && c.slot < 3) reinterpret_cast<fq*>(&T[t])[c.slot] = v;
 }
 
 // one block per pair, one limb per lane (limb_miller.cuh)
@@ -384,51 +359,63 @@ __global__ void __launch_bounds__(LM_THREADS, 2) k_v_miller(const g1a* P, const 
     if (!c.point && c.k.l == 0) reinterpret_cast<fq*>(&out[j])[2 * w_tower_pos(c.kc) + c.e] = v;
 }
 
-// L_j.T^(x_j) and R_j.T^(1/x_j) of block q at 2 lr q + 2 (j - 1) + side
-__global__ void __launch_bounds__(128) k_vb_gt(VSrc S, VBlk* st, fq12* out) {
-    __shared__ W12 W;
-    const int L = threadIdx.x;
+// L_j.T^(x_j) and R_j.T^(1/x_j) of block q at 2 lr q + 2 (j - 1) + side, one limb per lane (limb12.cuh).  The
+// values come from the proof and may lie outside the cyclotomic subgroup, so a squaring is a product:
+// 3-bit windows, 255 squarings and ~80 products, 0.53 ms for one proof's sixteen, beside the block's G1 and
+// pairing work (one Fq product per lane on 128 threads: 0.84 ms on the same stream).
+__global__ void __launch_bounds__(L12_THREADS) k_vb_gt(VSrc S, VBlk* st, fq12* out) {
+    __shared__ L12 W;
+    const L12Lane c = l12_lane();
     const int per = 2 * S.lr;
     const uint32_t q = blockIdx.x / per;
     const int jj = (blockIdx.x % per) >> 1, side = blockIdx.x & 1;
     VBlk& B = st[q];
     const uint8_t* rd = S.fc + q * S.fc_stride + (size_t)jj * ROUND_BYTES + (side ? GT_SER + G1_SER : 0);
-    if (L < 12) {
-        const int pos = 2 * w_tower_pos(L >> 1) + (L & 1);
-        fq v;
-        if (!fq_from_be48(rd + 48 * pos, v)) {
-            atomicOr(&B.bad, 1024u);
-            fq_zero(v);
-        }
-        W.s[0][L] = v;
+    const int tp = w_tower_pos(c.kc);
+    fq in;
+    if (!fq_from_be48(rd + 48 * (2 * tp + c.e), in)) {
+        atomicOr(&B.bad, 1024u);
+        fq_zero(in);
     }
-    __syncthreads();
-    uint32_t kw[8];
+    uint32_t kw[9];
     fr_canon_words(kw, side ? B.xinv[jj] : B.x[jj]);
-    w_exp<4>(W, W.s[1], W.s[0], kw, 256);
-    if (L < 12) reinterpret_cast<fq*>(&out[blockIdx.x])[2 * w_tower_pos(L >> 1) + (L & 1)] = W.s[1][L];
+    kw[8] = 0;
+    l12_load(W, c, W.v[1], W.v[8], in);                       // W.v[d] <- the value to the d-th, d < 8
+    for (int d = 2; d < 8; d++) l12_mul(W, c, W.v[d], W.v[d - 1], W.v[1], false);
+    int cur = -1, nxt = 8, oth = 0;                           // buffers 8 and 0 alternate
+    for (int i = 84; i >= 0; i--) {
+        const int bit = 3 * i, w = bit >> 5;
+        const int d = (int)(__funnelshift_r(kw[w], kw[w + 1], bit & 31) & 7);
+        if (cur >= 0) {
+            for (int n = 0; n < 4; n++) {                     // three squarings, then the digit's product
+                if (n == 3 && !d) break;
+                l12_mul(W, c, W.v[nxt], W.v[cur], n < 3 ? W.v[cur] : W.v[d], false);
+                cur = nxt;
+                nxt = oth;
+                oth = cur;
+            }
+        } else if (d) {
+            cur = d;                                          // (the first product replaces it by a buffer)
+        }
+    }
+    fq v;
+    if (cur < 0) {                                            // the zeroth power
+        fq_zero(v);
+        if (c.o == 0) fq_one(v);
+    } else {
+        v = l12_store(W, c, W.v[cur], W.v[nxt]);
+    }
+    if (c.k.l == 0) reinterpret_cast<fq*>(&out[blockIdx.x])[2 * tp + c.e] = v;
 }
 
-// per block: the folded C, and the inputs of its two final exponentiations (e(A_l, v_l) and the
-// fast-verification product) at fe_in[2q], fe_in[2q + 1]
-__global__ void k_vb_prod(const fq12* ml, const fq12* ge, const fq12* Cd, uint32_t nb, int lr, fq12* fe_in,
-                          fq12* cT) {
-    const uint64_t q = gtid();
-    if (q >= nb) return;
-    fq12 c = *Cd;
-    for (int t = 0; t < 2 * lr; t++) c = fq12_mul(c, ge[q * 2 * lr + t]);
-    cT[q] = c;
-    fe_in[2 * q] = ml[3 * q];
-    fe_in[2 * q + 1] = fq12_mul(ml[3 * q + 1], ml[3 * q + 2]);
-}
-
-__global__ void k_vb_check(const fq12* fe_out, const fq12* cT, const uint32_t* cbad, const VBlk* st, uint32_t nb,
-                           uint32_t* res) {
+__global__ void k_vb_check(const fq12* fe_out, const fq12* cT, const g1j* c1, const uint32_t* cbad, const VBlk* st,
+                           uint32_t nb, uint32_t* res) {
     const uint64_t q = gtid();
     if (q >= nb) return;
     fq12 one;
     fq12_one(one);
     uint32_t bad = st[q].bad | *cbad;
+    if (!fq_is_zero(c1[q].Z)) bad |= 128;                     // the folded G1 part minus b_l A_l
     if (!fq12_eq(fe_out[2 * q], cT[q])) bad |= 2048;
     if (!fq12_eq(fe_out[2 * q + 1], one)) bad |= 4096;
     res[q] = bad;
@@ -475,15 +462,6 @@ __global__ void k_vp_pairs(PiSrc pi, const uint32_t* job_a, uint32_t a0, const g
     Q[t] = v;
 }
 
-// out[q] = prod_{u < per} ml[per q + u]
-__global__ void k_vp_prod(const fq12* ml, uint32_t per, uint32_t nj, fq12* out) {
-    const uint64_t q = gtid();
-    if (q >= nj) return;
-    fq12 p = ml[q * per];
-    for (uint32_t u = 1; u < per; u++) p = fq12_mul(p, ml[q * per + u]);
-    out[q] = p;
-}
-
 // job q's result (decode failures | the pairing check) at res[idx ? idx[q0 + q] : q]
 __global__ void k_vp_check(const fq12* fe_out, const uint32_t* job_bad, uint32_t nj, const uint32_t* idx, uint32_t q0,
                            uint32_t* res) {
@@ -501,7 +479,6 @@ struct VElem {
     uint32_t bad;
     fr rj, ys;
     g1a Cj;
-    g1j ysg, rjCj;
 };
 
 // offsets inside a proof of block size nk: block | pi_Ck | path | siblings | pst
@@ -543,29 +520,33 @@ __global__ void k_v_elem(const uint8_t* proof, const uint8_t* mi_be, VLayout Ly,
     e->bad = bad;
 }
 
-// group 0: y* g1, group 1: r_j C_j (groups 2 and 3 idle)
-__global__ void __launch_bounds__(32) k_v_elem_muls(VElem* e) {
-    __shared__ GEc<fq> sm[4];
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
-    const bool yg = grp == 0;
-    const g1j r = g1_mul8(sm[grp], lane, yg ? g1_generator() : e->Cj, yg ? e->ys : e->rj);
-    if (lane == 0 && grp < 2) {
-        if (yg) e->ysg = r;
-        else e->rjCj = r;
+// r_j C_j + sum_w D_w - y* g1, one block: the first half of its threads r_j C_j and the D_w, the second
+// y* (-g1), one limb per lane
+struct VESmem {
+    LimbEc g1[2];
+    g1a D[16];
+};
+template <class Off>
+FPG_DEV void v_point_E(VESmem& sm, const g1a& Cj, const fr& rj, const fr& ys, const uint8_t* dser, int n, Off&& off,
+                       g1a* E, uint32_t* bad) {
+    const int half = (int)(threadIdx.x / LEC_THREADS);
+    const LecLane c = lec_lane();
+    if (half == 0) {
+        if (!g1_mul_sum(sm.g1[0], c, sm.D, Cj, rj, dser, n, off) && bad) atomicOr(bad, 256u);
+    } else {
+        uint32_t kw[8];
+        fr_canon_words(kw, ys);
+        lec_g1_mul(sm.g1[1], c, g1_neg_gen(), kw);
     }
+    __syncthreads();
+    if (half) return;
+    lec_step<false>(sm.g1[0], c, sm.g1[1].acc[0], sm.g1[1].acc[1], sm.g1[1].acc[2]);
+    g1_lin_put(c, E, lec_affine(sm.g1[0], c));
 }
-
 // E = D* - y* g1 with D* = r_j C_j + sum_w D_w
-__global__ void k_v_elem_E(const uint8_t* proof, VLayout Ly, VElem* e, g1a* E) {
-    if (gtid() != 0) return;
-    g1j Ds = e->rjCj;
-    const uint8_t* sib = proof + Ly.sib();
-    for (int h = 0; h < Ly.lr; h++) {
-        g1a D;
-        if (!g1_decode(sib + 128 * h, D)) atomicOr(&e->bad, 256u);
-        Ds = g1_madd(Ds, D);
-    }
-    E[0] = g1_affine(jac_add(Ds, g1j_neg(e->ysg)));
+__global__ void __launch_bounds__(2 * LEC_THREADS) k_v_elem_E(const uint8_t* proof, VLayout Ly, VElem* e, g1a* E) {
+    __shared__ VESmem sm;
+    v_point_E(sm, e->Cj, e->rj, e->ys, proof + Ly.sib(), Ly.lr, [](int h) { return 128 * (size_t)h; }, E, &e->bad);
 }
 
 __global__ void k_v_result(const uint32_t* blk_res, const VElem* e, const uint32_t* pst_res, uint32_t* result) {
@@ -598,14 +579,22 @@ uint32_t pow2_at_least(uint64_t n) {
     return p;
 }
 
+// term slots of a block of size b: its rows, the rounds' G1 parts and b_l A_l
+uint32_t vb_slots(uint32_t b, int lr) { return pow2_at_least(b + 2 * (uint64_t)lr + 1); }
+
 // scratch of the checks of nb blocks of size b
 template <class A>
 struct BlockBufs {
-    VBlk* st; g1j* T; g1j* T2; fr* wt; g1a* P; g2a* Q; fq12* ml; fq12* ge; fq12* fe_in; fq12* fe_out; fq12* cT;
-    uint32_t* res;
+    VBlk* st; uint8_t* hstmt; uint8_t* hscr; g1a* tP; fr* tk; g1j* T; g1j* T2; fr* wt; g1a* P; g2a* Q; fq12* ml;
+    fq12* ge; fq12* fe_in; fq12* fe_out; fq12* cT; uint32_t* res;
+    const g1j* c1 = nullptr;       // the blocks' sums of terms, in T or T2
     BlockBufs(A& ar, uint32_t nb, uint32_t b, int lr) {
-        const uint64_t tpb = pow2_at_least(b + 2 * (uint64_t)lr);
+        const uint64_t tpb = vb_slots(b, lr);
         st = (VBlk*)ar.take(nb * sizeof(VBlk));
+        hstmt = (uint8_t*)ar.take(32 * (size_t)nb);
+        hscr = (uint8_t*)ar.take(stmt_hash_scratch_bytes(nb, nb * b, b));
+        tP = (g1a*)ar.take(nb * tpb * G1A_BYTES);
+        tk = (fr*)ar.take(nb * tpb * FR_BYTES);
         T = (g1j*)ar.take(nb * tpb * G1J_BYTES);
         T2 = (g1j*)ar.take((nb * tpb / 2 + 1) * G1J_BYTES);
         wt = (fr*)ar.take((size_t)nb * b * FR_BYTES);
@@ -637,24 +626,62 @@ struct JobBufs {
     }
 };
 
-// the block checks up to their pairs (at Bb.P / Bb.Q, three per block)
+// the blocks' statement hashes, their transcripts and, on the side stream after them, the GT part of the
+// folded commitment (cT); the caller joins the side stream
+void vb_join(cudaStream_t from, cudaStream_t to) {
+    cudaEvent_t e = nullptr;
+    cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
+    cudaEventRecord(e, from);
+    cudaStreamWaitEvent(to, e, 0);
+    cudaEventDestroy(e);
+}
 template <class A>
-void block_checks_front(const VSrc& S, const uint8_t* C_be, const g1a* g1beta, BlockBufs<A>& Bb, cudaStream_t s) {
-    const uint32_t tpb = pow2_at_least(S.b + 2 * (uint64_t)S.lr);
+void block_transcripts(const VSrc& S, const uint8_t* C_be, const fq12* Cd, BlockBufs<A>& Bb, cudaStream_t s,
+                       cudaStream_t side) {
+    // the rows of block k0 + q start at S.blk + q S.blk_stride; k_stmt_hash indexes them from row 0
+    if (S.blk)
+        step1_stmt_hash(C_be, S.blk - 96 * (size_t)S.lo(0), S.k0, S.nb, S.R, S.b, Bb.hscr, Bb.hstmt, s);
+    FP_KERNEL("k_vb_transcript", s, k_vb_transcript<<<S.nb, 32, 0, s>>>(S, Bb.st));
+    vb_join(s, side);
+    FP_KERNEL("k_vb_gt", side, k_vb_gt<<<2 * S.lr * S.nb, L12_THREADS, 0, side>>>(S, Bb.st, Bb.ge));
+    fq12_products(Cd, Bb.ge, 2 * S.lr, 2 * S.lr, Bb.cT, 1, S.nb, side);
+}
+// the terms' multiplications and their sums (c1), and the pairs (at Bb.P / Bb.Q, three per block)
+template <class A>
+void block_muls(const VSrc& S, uint32_t tpb, const g1a* g1beta, BlockBufs<A>& Bb, cudaStream_t s) {
     const uint64_t nt = (uint64_t)S.nb * tpb;
-    cudaMemsetAsync(Bb.T, 0, nt * G1J_BYTES, s);
-    FP_KERNEL("k_vb_transcript", s, k_vb_transcript<<<grid_for(S.nb, 32), 32, 0, s>>>(S, C_be, Bb.st));
-    FP_KERNEL("k_vb_terms", s, k_vb_terms<<<grid_for(nt, 16), 128, 0, s>>>(S, Bb.st, tpb, Bb.T, Bb.wt));
+    FP_KERNEL("k_vb_muls", s, k_vb_muls<<<(unsigned)(S.nb + (nt + S.nb + 1) / 2), LEC2_THREADS, 0, s>>>(
+                                  Bb.st, S.nb, Bb.tP, Bb.tk, nt, g1beta, Bb.T, Bb.P, Bb.Q));
     g1j* x = Bb.T;
     g1j* y = Bb.T2;
-    for (uint64_t n = nt; n > S.nb; n /= 2) {            // per-block sums: tpb is a power of two
-        g1_pair_reduce(x, y, n / 2, s);
+    for (uint64_t n = nt; n > S.nb;) {                   // per-block sums: tpb is a power of two
+        if (n > 8192) {
+            g1_pair_reduce(x, y, n / 2, s);
+            n /= 2;
+        } else {
+            const uint32_t gs = (uint32_t)std::min<uint64_t>(32, n / S.nb);
+            g1_tree_reduce(x, y, n, gs, s);
+            n /= gs;
+        }
         std::swap(x, y);
     }
-    FP_KERNEL("k_vb_scalars", s, k_vb_scalars<<<grid_for(S.nb, 64), 64, 0, s>>>(S, Bb.wt, Bb.st));
-    const uint32_t nb2 = (S.nb + 3) / 4;
-    FP_KERNEL("k_vb_muls", s, k_vb_muls<<<nb2 + grid_for(2 * (uint64_t)S.nb, 16), 128, 0, s>>>(Bb.st, S.nb, nb2));
-    FP_KERNEL("k_vb_pairs", s, k_vb_pairs<<<grid_for(S.nb, 64), 64, 0, s>>>(S.nb, g1beta, x, Bb.st, Bb.P, Bb.Q));
+    Bb.c1 = x;
+}
+template <class A>
+void block_checks_front(const VSrc& S, const uint8_t* C_be, const fq12* Cd, const g1a* g1beta, BlockBufs<A>& Bb,
+                        cudaStream_t s, cudaStream_t side) {
+    const uint32_t tpb = vb_slots(S.b, S.lr);
+    block_transcripts(S, C_be, Cd, Bb, s, side);
+    FP_KERNEL("k_vb_terms", s, k_vb_terms<<<grid_for((uint64_t)S.nb * tpb, 64), 64, 0, s>>>(S, Bb.st, Bb.hstmt, tpb, Bb.tP,
+                                                                                          Bb.tk, Bb.wt));
+    FP_KERNEL("k_vb_scalars", s, k_vb_scalars<<<grid_for(S.nb, 64), 64, 0, s>>>(S, Bb.wt, Bb.st, tpb, 0, Bb.tk));
+    block_muls(S, tpb, g1beta, Bb, s);
+}
+// the inputs of the blocks' two final exponentiations: e(A_l, v_l) and the fast-verification product
+template <class A>
+void block_fe_inputs(BlockBufs<A>& Bb, uint32_t nb, fq12* fe_in, cudaStream_t s) {
+    fq12_products(nullptr, Bb.ml, 3, 1, fe_in, 2, nb, s);
+    fq12_products(nullptr, Bb.ml + 1, 3, 2, fe_in + 1, 2, nb, s);
 }
 
 // verify_one's scratch: the block's buffers, the element state, and the pairs of the block's
@@ -685,7 +712,7 @@ struct OneBufs {
 
 void verify_one(const void* proof, const void* C_be, const void* mi_be, uint32_t nk, int lr, int lc, uint32_t b,
                 uint64_t i, uint32_t M, uint32_t k, uint32_t lo, const void* g1beta, const void* g2tau, void* scratch,
-                uint32_t* result, cudaStream_t s) {
+                uint32_t* result, cudaStream_t s, cudaStream_t side, cudaStream_t side2) {
     const VLayout Ly{nk, lr, lc};
     const uint8_t* pr = (const uint8_t*)proof;
     const VSrc S{pr, 0, pr + Ly.fc(), 0, k, 1, b, lo + nk, lr};   // R = lo + nk gives nk(0) = nk
@@ -694,19 +721,20 @@ void verify_one(const void* proof, const void* C_be, const void* mi_be, uint32_t
     const int np = 3 + lc + 1;
     cudaMemsetAsync(O.job_bad, 0, 4, s);
     FP_KERNEL("k_v_cdec", s, k_v_cdec<<<1, 32, 0, s>>>((const uint8_t*)C_be, O.Cd, O.cbad));
-    FP_KERNEL("k_v_elem", s, k_v_elem<<<1, 32, 0, s>>>(pr, (const uint8_t*)mi_be, Ly, i, M, lo, O.e));
-    block_checks_front(S, (const uint8_t*)C_be, (const g1a*)g1beta, O.Bb, s);
-    FP_KERNEL("k_v_elem_muls", s, k_v_elem_muls<<<1, 32, 0, s>>>(O.e));
-    FP_KERNEL("k_v_elem_E", s, k_v_elem_E<<<1, 32, 0, s>>>(pr, Ly, O.e, O.E));
+    vb_join(s, side2);                                         // the element's checks beside the block's
+    FP_KERNEL("k_v_elem", side2, k_v_elem<<<1, 32, 0, side2>>>(pr, (const uint8_t*)mi_be, Ly, i, M, lo, O.e));
+    FP_KERNEL("k_v_elem_E", side2, k_v_elem_E<<<1, 2 * LEC_THREADS, 0, side2>>>(pr, Ly, O.e, O.E));
     const PiSrc pi{pr + Ly.pst(), 0, M, lc};
-    FP_KERNEL("k_vp_pairs", s, k_vp_pairs<<<1, 32, 0, s>>>(pi, nullptr, (uint32_t)(i % M), O.E, 1,
-                                                           (const g2a*)g2tau, O.job_bad, O.P + 3, O.Q + 3));
+    FP_KERNEL("k_vp_pairs", side2, k_vp_pairs<<<1, 32, 0, side2>>>(pi, nullptr, (uint32_t)(i % M), O.E, 1,
+                                                                 (const g2a*)g2tau, O.job_bad, O.P + 3, O.Q + 3));
+    block_checks_front(S, (const uint8_t*)C_be, O.Cd, (const g1a*)g1beta, O.Bb, s, side);
+    vb_join(side2, s);
     FP_KERNEL("k_v_miller", s, k_v_miller<<<np, LM_THREADS, 0, s>>>(O.P, O.Q, O.ml));
-    FP_KERNEL("k_vb_gt", s, k_vb_gt<<<2 * lr, 128, 0, s>>>(S, O.Bb.st, O.Bb.ge));
-    FP_KERNEL("k_vb_prod", s, k_vb_prod<<<1, 32, 0, s>>>(O.ml, O.Bb.ge, O.Cd, 1, lr, O.fe_in, O.Bb.cT));
-    FP_KERNEL("k_vp_prod", s, k_vp_prod<<<1, 32, 0, s>>>(O.ml + 3, lc + 1, 1, O.fe_in + 2));
+    block_fe_inputs(O.Bb, 1, O.fe_in, s);
+    fq12_products(nullptr, O.ml + 3, lc + 1, lc + 1, O.fe_in + 2, 1, 1, s);
     final_exp_group(O.fe_in, 3, O.fe_out, nullptr, 1, 0, 0, s);
-    FP_KERNEL("k_vb_check", s, k_vb_check<<<1, 32, 0, s>>>(O.fe_out, O.Bb.cT, O.cbad, O.Bb.st, 1, O.Bb.res));
+    vb_join(side, s);
+    FP_KERNEL("k_vb_check", s, k_vb_check<<<1, 32, 0, s>>>(O.fe_out, O.Bb.cT, O.Bb.c1, O.cbad, O.Bb.st, 1, O.Bb.res));
     FP_KERNEL("k_vp_check", s, k_vp_check<<<1, 32, 0, s>>>(O.fe_out + 2, O.job_bad, 1, nullptr, 0, O.pst_res));
     FP_KERNEL("k_v_result", s, k_v_result<<<1, 32, 0, s>>>(O.Bb.res, O.e, O.pst_res, result));
 }
@@ -737,17 +765,17 @@ size_t verify_block_scratch_bytes(uint32_t b, int lr) {
 }
 
 void verify_block(const void* blk, const void* fc, const void* C_be, uint32_t nk, int lr, uint32_t b, uint32_t k,
-                  uint32_t lo, const void* g1beta, void* scratch, uint32_t* result, cudaStream_t s) {
+                  uint32_t lo, const void* g1beta, void* scratch, uint32_t* result, cudaStream_t s, cudaStream_t side) {
     const VSrc S{(const uint8_t*)blk, 0, (const uint8_t*)fc, 0, k, 1, b, lo + nk, lr};
     Arena ar{(uint8_t*)scratch};
     BlockOnlyBufs<Arena> O(ar, b, lr);
     FP_KERNEL("k_v_cdec", s, k_v_cdec<<<1, 32, 0, s>>>((const uint8_t*)C_be, O.Cd, O.cbad));
-    block_checks_front(S, (const uint8_t*)C_be, (const g1a*)g1beta, O.Bb, s);
+    block_checks_front(S, (const uint8_t*)C_be, O.Cd, (const g1a*)g1beta, O.Bb, s, side);
     FP_KERNEL("k_v_miller", s, k_v_miller<<<3, LM_THREADS, 0, s>>>(O.Bb.P, O.Bb.Q, O.Bb.ml));
-    FP_KERNEL("k_vb_gt", s, k_vb_gt<<<2 * lr, 128, 0, s>>>(S, O.Bb.st, O.Bb.ge));
-    FP_KERNEL("k_vb_prod", s, k_vb_prod<<<1, 32, 0, s>>>(O.Bb.ml, O.Bb.ge, O.Cd, 1, lr, O.Bb.fe_in, O.Bb.cT));
+    block_fe_inputs(O.Bb, 1, O.Bb.fe_in, s);
     final_exp_group(O.Bb.fe_in, 2, O.Bb.fe_out, nullptr, 1, 0, 0, s);
-    FP_KERNEL("k_vb_check", s, k_vb_check<<<1, 32, 0, s>>>(O.Bb.fe_out, O.Bb.cT, O.cbad, O.Bb.st, 1, result));
+    vb_join(side, s);
+    FP_KERNEL("k_vb_check", s, k_vb_check<<<1, 32, 0, s>>>(O.Bb.fe_out, O.Bb.cT, O.Bb.c1, O.cbad, O.Bb.st, 1, result));
 }
 
 // ------------------------------------------------------------------------------ evaluation proof
@@ -761,31 +789,30 @@ __global__ void k_ve_decode(const uint8_t* proof, fr* y, g1a* CF, uint32_t* bad)
     if (!fr_from_be32(proof, *y) || !g1_decode(proof + 32, *CF)) atomicOr(bad, 1u);
 }
 
-// slot 0: r_0 C_F; slots 1 .. 2 l_R: x_j L_j.1 and x_j^-1 R_j.1 (one 8-lane group each)
-__global__ void __launch_bounds__(128) k_ve_terms(VSrc S, VBlk* st, const g1a* CF, const fr* r0, uint32_t tpb,
-                                                  g1j* T) {
-    __shared__ GEc<fq> sm[16];
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
-    const uint64_t u = (uint64_t)blockIdx.x * 16 + grp;
-    const int lr = S.lr;
-    const bool valid = u < 1 + 2 * (uint64_t)lr && u < tpb;
+// slot 0: r_0 C_F; slots 1 .. 2 l_R: x_j L_j.1 and x_j^-1 R_j.1; slot 2 l_R + 1: -A_l, its factor by k_vb_scalars
+__global__ void __launch_bounds__(64) k_ve_terms(VSrc S, VBlk* st, const g1a* CF, const fr* r0, uint32_t tpb, g1a* tP,
+                                                 fr* tk) {
+    const uint64_t u = gtid();
+    if (u >= tpb) return;
     VBlk& B = st[0];
     g1a P;
     fq_zero(P.x);
     fq_zero(P.y);
     fr k;
     fr_zero(k);
-    if (valid && u == 0) {
+    if (u == 0) {
         P = *CF;
         k = *r0;
-    } else if (valid) {
+    } else if (u < 1 + 2 * (uint64_t)S.lr) {
         const int v = (int)(u - 1), jj = v >> 1, side = v & 1;
         const uint8_t* rd = S.fc + (size_t)jj * ROUND_BYTES;
-        if (!g1_decode(rd + (side ? GT_SER + G1_SER + GT_SER : GT_SER), P) && lane == 0) atomicOr(&B.bad, 64u);
+        if (!g1_decode(rd + (side ? GT_SER + G1_SER + GT_SER : GT_SER), P)) atomicOr(&B.bad, 64u);
         k = side ? B.xinv[jj] : B.x[jj];
+    } else if (u == 1 + 2 * (uint64_t)S.lr) {
+        P = g1a_neg(B.Al);
     }
-    const g1j r = g1_mul8(sm[grp], lane, P, k);
-    if (valid && lane == 0) T[u] = r;
+    tP[u] = P;
+    tk[u] = k;
 }
 
 // b_l summands w_a prod_k x_k^-(bit l - k of a), a < R
@@ -798,38 +825,32 @@ __global__ void k_ve_wt(VSrc S, const VBlk* st, const fr* w, fr* wt) {
     wt[a] = v;
 }
 
-// E = C_F - y g1 on one 8-lane group
-__global__ void __launch_bounds__(32) k_ve_E(const g1a* CF, const fr* y, g1a* E) {
-    __shared__ GEc<fq> sm[4];
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
-    const g1j yg = g1_mul8(sm[grp], lane, g1_generator(), *y);
-    if (threadIdx.x == 0) *E = g1_affine(g1_madd(g1j_neg(yg), *CF));
-}
-
-// PST pairs at r: idx < l_c: (-pi_idx, g2^{tau_t} - r_t g2), t = l_c - 1 - idx (r_t g2 on one warp);
-// idx = l_c: (E, g2)
-__global__ void __launch_bounds__(32) k_ve_pst_pairs(const uint8_t* pst, const fr* r_mont, const g2a* g2tau, int lc,
-                                                     const g1a* E, uint32_t* bad, g1a* P, g2a* Q) {
-    __shared__ GEcW sm;
-    const int idx = blockIdx.x, L = threadIdx.x;
+// PST pairs at r, one block each: idx < l_c: (-pi_idx, g2^{tau_t} - r_t g2), t = l_c - 1 - idx;
+// idx = l_c: (C_F - y g1, g2)
+__global__ void __launch_bounds__(LEC2_THREADS) k_ve_pst_pairs(const uint8_t* pst, const fr* r_mont, const g2a* g2tau,
+                                                               int lc, const g1a* CF, const fr* y, uint32_t* bad, g1a* P,
+                                                               g2a* Q) {
+    __shared__ VMulSmem sm;
+    const int idx = blockIdx.x;
     if (idx == lc) {
-        if (L == 0) {
-            P[idx] = *E;
-            Q[idx] = g2_generator();
-        }
+        if (threadIdx.x >= LEC_THREADS) return;
+        const LecLane c = lec_lane();
+        g1_lin_put(c, &P[idx], g1_lin(sm.g1[0], c, g1_neg_gen(), *y, *CF));
+        if (threadIdx.x == 0) Q[idx] = g2_generator();
         return;
     }
     const int t = lc - 1 - idx;
     uint32_t kw[8];
     fr_canon_words(kw, r_mont[t]);
-    const GPt<fq2> rg = gecw_g2_mul_proj(sm, L, g2_generator(), kw);
-    if (L == 0) {
+    const Lec2Lane c = lec2_lane();
+    lec2_g2_mul(sm.g2, c, g2a_negate(g2_generator()), kw);
+    lec2_add_affine(sm.g2, c, g2tau[t]);
+    const fq v = lec2_affine(sm.g2, c);
+    if (c.k.l == 0 && c.slot < 4) reinterpret_cast<fq*>(&Q[idx])[c.slot] = v;
+    if (threadIdx.x == 0) {
         g1a p;
         if (!g1_decode(pst + 96 * (size_t)idx, p)) atomicOr(bad, 512u);
         P[idx] = g1a_neg(p);
-        g2a ra;
-        gec_to_affine(ra.x, ra.y, rg);
-        Q[idx] = g2_affine(g2_madd(g2_from_affine(g2tau[t]), g2a_negate(ra)));
     }
 }
 
@@ -843,7 +864,7 @@ namespace {
 template <class A>
 struct EvalBufs {
     fq12* Cd; uint32_t* cbad; BlockBufs<A> Bb; fr* r_mont; uint32_t* err; fr* Tm; fr* Tc; fr* w; fr* r0; fr* y;
-    g1a* CF; g1a* E; uint32_t* dec_bad; g1a* P; g2a* Q; fq12* ml; fq12* fe_in; fq12* fe_out; uint32_t* blk_res;
+    g1a* CF; uint32_t* dec_bad; g1a* P; g2a* Q; fq12* ml; fq12* fe_in; fq12* fe_out; uint32_t* blk_res;
     uint32_t* pst_res;
     EvalBufs(A& ar, uint32_t R, int lr, int lc, int log_n)
         : Cd((fq12*)ar.take(FQ12_BYTES)), cbad((uint32_t*)ar.take(4)), Bb(ar, 1, R, lr) {
@@ -855,7 +876,6 @@ struct EvalBufs {
         r0 = (fr*)ar.take(FR_BYTES);
         y = (fr*)ar.take(FR_BYTES);
         CF = (g1a*)ar.take(G1A_BYTES);
-        E = (g1a*)ar.take(G1A_BYTES);
         dec_bad = (uint32_t*)ar.take(4);
         P = (g1a*)ar.take((size_t)(lc + 1) * G1A_BYTES);
         Q = (g2a*)ar.take((size_t)(lc + 1) * G2A_BYTES);
@@ -876,7 +896,8 @@ size_t verify_eval_scratch_bytes(uint32_t R, int lr, int lc, int log_n) {
 }
 
 void verify_eval(const void* proof, const void* C_be, const void* r_be, int log_n, int lr, int lc, uint32_t R,
-                 const void* g1beta, const void* g2tau, void* scratch, uint32_t* result, cudaStream_t s) {
+                 const void* g1beta, const void* g2tau, void* scratch, uint32_t* result, cudaStream_t s,
+                 cudaStream_t side, cudaStream_t side2) {
     const uint8_t* pr = (const uint8_t*)proof;
     const size_t blen = (size_t)lr * ROUND_BYTES + G1_SER + 2 * G2_SER;
     const VSrc S{nullptr, 0, pr + 128, 0, 0, 1, R, R, lr};
@@ -889,33 +910,26 @@ void verify_eval(const void* proof, const void* C_be, const void* r_be, int log_
     FP_KERNEL("k_ve_decode", s, k_ve_decode<<<1, 32, 0, s>>>(pr, O.y, O.CF, O.dec_bad));
     eval_bvec(C_be, r_be, log_n, pr + 32, O.Tm, R, O.r0, O.w, s);          // r_0 and w = r_0 T
     FP_KERNEL("k_v_cdec", s, k_v_cdec<<<1, 32, 0, s>>>((const uint8_t*)C_be, O.Cd, O.cbad));
-    // FC.BVerify front: transcript, the G1 part of C_0 and the rounds, b_l, the three pairs
-    const uint32_t tpb = pow2_at_least(1 + 2 * (uint64_t)lr);
-    cudaMemsetAsync(O.Bb.T, 0, (size_t)tpb * G1J_BYTES, s);
-    FP_KERNEL("k_vb_transcript", s, k_vb_transcript<<<1, 32, 0, s>>>(S, (const uint8_t*)C_be, O.Bb.st));
-    FP_KERNEL("k_ve_terms", s, k_ve_terms<<<grid_for(tpb, 16), 128, 0, s>>>(S, O.Bb.st, O.CF, O.r0, tpb, O.Bb.T));
+    // PST.Verify's pairs at r_R on a side stream beside FC.BVerify's front
+    vb_join(s, side2);
+    FP_KERNEL("k_ve_pst_pairs", side2, k_ve_pst_pairs<<<lc + 1, LEC2_THREADS, 0, side2>>>(
+                                           pr + 128 + blen, O.r_mont, (const g2a*)g2tau, lc, O.CF, O.y, O.dec_bad, O.P, O.Q));
+    FP_KERNEL("k_v_miller", side2, k_v_miller<<<lc + 1, LM_THREADS, 0, side2>>>(O.P, O.Q, O.ml));
+    fq12_products(nullptr, O.ml, lc + 1, lc + 1, O.fe_in, 1, 1, side2);
+    final_exp_group(O.fe_in, 1, O.fe_out, nullptr, 1, 0, 0, side2);
+    // FC.BVerify: transcript, the G1 part of C_0 and the rounds, b_l, the three pairs
+    const uint32_t tpb = pow2_at_least(2 + 2 * (uint64_t)lr);
+    block_transcripts(S, (const uint8_t*)C_be, O.Cd, O.Bb, s, side);
+    FP_KERNEL("k_ve_terms", s, k_ve_terms<<<grid_for(tpb, 64), 64, 0, s>>>(S, O.Bb.st, O.CF, O.r0, tpb, O.Bb.tP, O.Bb.tk));
     FP_KERNEL("k_ve_wt", s, k_ve_wt<<<grid_for(R, 64), 64, 0, s>>>(S, O.Bb.st, O.w, O.Bb.wt));
-    g1j* x = O.Bb.T;
-    g1j* yb = O.Bb.T2;
-    for (uint64_t n = tpb; n > 1; n /= 2) {
-        g1_pair_reduce(x, yb, n / 2, s);
-        std::swap(x, yb);
-    }
-    FP_KERNEL("k_vb_scalars", s, k_vb_scalars<<<1, 64, 0, s>>>(S, O.Bb.wt, O.Bb.st));
-    FP_KERNEL("k_vb_muls", s, k_vb_muls<<<2, 128, 0, s>>>(O.Bb.st, 1, 1));
-    FP_KERNEL("k_vb_pairs", s, k_vb_pairs<<<1, 64, 0, s>>>(1, (const g1a*)g1beta, x, O.Bb.st, O.Bb.P, O.Bb.Q));
+    FP_KERNEL("k_vb_scalars", s, k_vb_scalars<<<1, 64, 0, s>>>(S, O.Bb.wt, O.Bb.st, tpb, 1 + 2 * (uint32_t)lr, O.Bb.tk));
+    block_muls(S, tpb, (const g1a*)g1beta, O.Bb, s);
     FP_KERNEL("k_v_miller", s, k_v_miller<<<3, LM_THREADS, 0, s>>>(O.Bb.P, O.Bb.Q, O.Bb.ml));
-    FP_KERNEL("k_vb_gt", s, k_vb_gt<<<2 * lr, 128, 0, s>>>(S, O.Bb.st, O.Bb.ge));
-    FP_KERNEL("k_vb_prod", s, k_vb_prod<<<1, 32, 0, s>>>(O.Bb.ml, O.Bb.ge, O.Cd, 1, lr, O.Bb.fe_in, O.Bb.cT));
+    block_fe_inputs(O.Bb, 1, O.Bb.fe_in, s);
     final_exp_group(O.Bb.fe_in, 2, O.Bb.fe_out, nullptr, 1, 0, 0, s);
-    FP_KERNEL("k_vb_check", s, k_vb_check<<<1, 32, 0, s>>>(O.Bb.fe_out, O.Bb.cT, O.cbad, O.Bb.st, 1, O.blk_res));
-    // PST.Verify at r_R
-    FP_KERNEL("k_ve_E", s, k_ve_E<<<1, 32, 0, s>>>(O.CF, O.y, O.E));
-    FP_KERNEL("k_ve_pst_pairs", s, k_ve_pst_pairs<<<lc + 1, 32, 0, s>>>(pr + 128 + blen, O.r_mont, (const g2a*)g2tau,
-                                                                       lc, O.E, O.dec_bad, O.P, O.Q));
-    FP_KERNEL("k_v_miller", s, k_v_miller<<<lc + 1, LM_THREADS, 0, s>>>(O.P, O.Q, O.ml));
-    FP_KERNEL("k_vp_prod", s, k_vp_prod<<<1, 32, 0, s>>>(O.ml, lc + 1, 1, O.fe_in));
-    final_exp_group(O.fe_in, 1, O.fe_out, nullptr, 1, 0, 0, s);
+    vb_join(side, s);
+    FP_KERNEL("k_vb_check", s, k_vb_check<<<1, 32, 0, s>>>(O.Bb.fe_out, O.Bb.cT, O.Bb.c1, O.cbad, O.Bb.st, 1, O.blk_res));
+    vb_join(side2, s);
     cudaMemsetAsync(O.pst_res, 0, 4, s);
     FP_KERNEL("k_vp_check", s, k_vp_check<<<1, 32, 0, s>>>(O.fe_out, O.pst_res, 1, nullptr, 0, O.pst_res));
     FP_KERNEL("k_ve_result", s, k_ve_result<<<1, 32, 0, s>>>(O.blk_res, O.pst_res, O.dec_bad, O.err, result));
@@ -949,29 +963,28 @@ __global__ void k_va_paths(ProofLayout L, const uint64_t* m, const uint8_t* row_
     for (int q = 0; q < 32; q++) roots[32 * i + q] = cur[q];
 }
 
-// per row, with the root of proof 0: r_j and D*_j = r_j C_j + sum_w D_w (affine); one 8-lane
-// group per row
-__global__ void __launch_bounds__(128) k_va_rows(ProofLayout L, const uint8_t* roots, const uint8_t* rows_ser,
-                                                 const uint8_t* D_ser, fr* rj, g1a* Dstar, uint32_t* row_bad) {
-    __shared__ GEc<fq> sm[16];
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
-    const uint64_t j0 = (uint64_t)blockIdx.x * 16 + grp;
-    const bool valid = j0 < L.R;
-    const uint32_t j = valid ? (uint32_t)j0 : 0;
+// per row, with the root of proof 0: r_j and D*_j = r_j C_j + sum_w D_w (affine), one limb per lane, two
+// rows per block
+__global__ void __launch_bounds__(2 * LEC_THREADS) k_va_rows(ProofLayout L, const uint8_t* roots, const uint8_t* rows_ser,
+                                                             const uint8_t* D_ser, fr* rj, g1a* Dstar, uint32_t* row_bad) {
+    __shared__ LimbEc sm[2];
+    __shared__ g1a D[2][16];
+    const int half = (int)(threadIdx.x / LEC_THREADS);
+    const uint64_t j0 = blockIdx.x * (uint64_t)2 + half;
+    if (j0 >= L.R) return;                                    // three whole warps, with a barrier of their own
+    const uint32_t j = (uint32_t)j0;
+    const LecLane c = lec_lane();
     const fr r = row_rho(roots, j);
     g1a Cj;
     const bool cok = g1_decode(rows_ser + 96 * (size_t)j, Cj);
-    g1j Ds = g1_mul8(sm[grp], lane, Cj, r);
-    if (!valid || lane != 0) return;
-    uint32_t bad = cok ? 0u : 16u;
-    for (int h = 0; h < L.log_r; h++) {
-        g1a D;
-        if (!g1_decode(D_ser + G1_SER * (tree_off(L.R, h) + ((j >> h) ^ 1)), D)) bad |= 256;
-        Ds = g1_madd(Ds, D);
-    }
-    rj[j] = r;
-    Dstar[j] = g1_affine(Ds);
-    row_bad[j] = bad;
+    if (lec_thread() == 0) row_bad[j] = cok ? 0u : 16u;
+    lec_sync();
+    const bool dok = g1_mul_sum(sm[half], c, D[half], Cj, r, D_ser, L.log_r, [&](int h) {
+        return G1_SER * (size_t)(tree_off(L.R, h) + ((j >> h) ^ 1));
+    });
+    if (!dok) atomicOr(&row_bad[j], 256u);
+    if (lec_thread() == 0) rj[j] = r;
+    g1_lin_put(c, &Dstar[j], lec_affine(sm[half], c));
 }
 
 // y* = r_j m_i + sum_w g_w[a] of every proof, r_j from the proof's own root
@@ -1009,41 +1022,29 @@ __global__ void k_va_class(ProofLayout L, const uint8_t* roots, const g1a* Dstar
     if (!sh) irr[atomicAdd(nirr, 1u)] = (uint32_t)i;
 }
 
-// column jobs: E_a = D*_0 - y*_a g1, one 8-lane group each
-__global__ void __launch_bounds__(128) k_va_colE(const g1a* Dstar, const fr* ys, uint32_t M, g1a* E) {
-    __shared__ GEc<fq> sm[16];
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
-    const uint64_t a0 = (uint64_t)blockIdx.x * 16 + grp;
-    const bool valid = a0 < M;
-    const uint64_t a = valid ? a0 : 0;
-    const g1j yg = g1_mul8(sm[grp], lane, g1_generator(), ys[a]);
-    if (valid && lane == 0) E[a] = g1_affine(g1_madd(g1j_neg(yg), Dstar[0]));
+// column jobs: E_a = D*_0 - y*_a g1, two per block
+__global__ void __launch_bounds__(2 * LEC_THREADS) k_va_colE(const g1a* Dstar, const fr* ys, uint32_t M, g1a* E) {
+    __shared__ LimbEc sm[2];
+    const int half = (int)(threadIdx.x / LEC_THREADS);
+    const uint64_t a = blockIdx.x * (uint64_t)2 + half;
+    if (a >= M) return;
+    const LecLane c = lec_lane();
+    g1_lin_put(c, &E[a], g1_lin(sm[half], c, g1_neg_gen(), ys[a], Dstar[0]));
 }
 
 // jobs of the listed proofs irr[q0 .. q0 + nj): E = r_j C_j + sum_w D_w - y* g1, r_j from the
-// proof's own root; one 8-lane group each
-__global__ void __launch_bounds__(128) k_va_irrE(ProofLayout L, const uint32_t* irr, uint32_t q0, uint32_t nj,
-                                                 const uint8_t* roots, const fr* ys, const uint8_t* rows_ser,
-                                                 const uint8_t* D_ser, g1a* E, uint32_t* job_a) {
-    __shared__ GEc<fq> sm[16];
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
-    const uint64_t q0g = (uint64_t)blockIdx.x * 16 + grp;
-    const bool valid = q0g < nj;
-    const uint64_t q = valid ? q0g : 0;
-    const uint64_t i = irr[q0 + q];
+// proof's own root; one block each
+__global__ void __launch_bounds__(2 * LEC_THREADS) k_va_irrE(ProofLayout L, const uint32_t* irr, uint32_t q0,
+                                                             const uint8_t* roots, const fr* ys, const uint8_t* rows_ser,
+                                                             const uint8_t* D_ser, g1a* E, uint32_t* job_a) {
+    __shared__ VESmem sm;
+    const uint64_t q = blockIdx.x, i = irr[q0 + q];
     const uint32_t j = (uint32_t)(i / L.M);
     g1a Cj;
     g1_decode(rows_ser + 96 * (size_t)j, Cj);         // a bad C_j or D_w fails the row's check
-    g1j Ds = g1_mul8(sm[grp], lane, Cj, row_rho(roots + 32 * i, j));
-    const g1j yg = g1_mul8(sm[grp], lane, g1_generator(), ys[i]);
-    if (!valid || lane != 0) return;
-    for (int h = 0; h < L.log_r; h++) {
-        g1a D;
-        g1_decode(D_ser + G1_SER * (tree_off(L.R, h) + ((j >> h) ^ 1)), D);
-        Ds = g1_madd(Ds, D);
-    }
-    job_a[q] = (uint32_t)(i % L.M);
-    E[q] = g1_affine(jac_add(Ds, g1j_neg(yg)));
+    if (threadIdx.x == 0) job_a[q] = (uint32_t)(i % L.M);
+    v_point_E(sm, Cj, row_rho(roots + 32 * i, j), ys[i], D_ser, L.log_r,
+              [&](int h) { return G1_SER * (size_t)(tree_off(L.R, h) + ((j >> h) ^ 1)); }, &E[q], nullptr);
 }
 
 __global__ void k_va_result(ProofLayout L, const uint32_t* blk_res, const uint32_t* row_bad, const uint8_t* mbad,
@@ -1103,7 +1104,7 @@ void pst_jobs(const ProofLayout& L, JobBufs<A>& J, uint32_t nj, const uint32_t* 
     FP_KERNEL("k_vp_pairs", s, k_vp_pairs<<<grid_for(np, 64), 64, 0, s>>>(pi, job_a, 0, J.E, nj, g2tau, J.bad, J.P,
                                                                         J.Q));
     FP_KERNEL("k_v_miller", s, k_v_miller<<<(unsigned)np, LM_THREADS, 0, s>>>(J.P, J.Q, J.ml));
-    FP_KERNEL("k_vp_prod", s, k_vp_prod<<<grid_for(nj, 64), 64, 0, s>>>(J.ml, lc + 1, nj, J.fe_in));
+    fq12_products(nullptr, J.ml, lc + 1, lc + 1, J.fe_in, 1, nj, s);
     final_exp_group(J.fe_in, nj, J.fe_out, nullptr, 1, 0, 0, s);
     FP_KERNEL("k_vp_check", s, k_vp_check<<<grid_for(nj, 64), 64, 0, s>>>(J.fe_out, J.bad, nj, idx, q0, res));
 }
@@ -1121,7 +1122,8 @@ size_t verify_all_scratch_bytes(const ProofLayout& L) {
 
 uint64_t verify_all(const ProofLayout& L, const void* C_be, const void* m, const void* rows_ser, const void* blocks,
                     const void* row_tree, const void* top_tree, const void* D_ser, const void* g, const void* pst_ser,
-                    const void* g1beta, const void* g2tau, int each, void* scratch, void* ok_out, cudaStream_t s) {
+                    const void* g1beta, const void* g2tau, int each, void* scratch, void* ok_out, cudaStream_t s,
+                    cudaStream_t side, cudaStream_t side2) {
     const uint64_t N = (uint64_t)L.R * L.M;
     Arena ar{(uint8_t*)scratch};
     AllBufs<Arena> Ab(ar, L);
@@ -1134,37 +1136,38 @@ uint64_t verify_all(const ProofLayout& L, const void* C_be, const void* m, const
     const uint8_t* ps = (const uint8_t*)pst_ser;
     cudaMemsetAsync(Ab.nirr, 0, 8, s);
     cudaMemsetAsync(Ab.n_ok, 0, 8, s);
+    // element checks and the sharing classes, on a side stream beside the blocks' checks
+    vb_join(s, side2);
+    const uint64_t* md = (const uint64_t*)m;
+    FP_KERNEL("k_va_paths", side2, k_va_paths<<<grid_for(N, 64), 64, 0, side2>>>(L, md, (const uint8_t*)row_tree,
+                                                                       (const uint8_t*)top_tree, rs, Ab.roots,
+                                                                       Ab.mbad));
+    FP_KERNEL("k_va_rows", side2, k_va_rows<<<(L.R + 1) / 2, 2 * LEC_THREADS, 0, side2>>>(L, Ab.roots, rs, Ds, Ab.rj, Ab.Dstar,
+                                                                       Ab.row_bad));
+    FP_KERNEL("k_va_y", side2, k_va_y<<<grid_for(N), TPB, 0, side2>>>(L, md, Ab.roots, Ab.rj, (const fr*)g, Ab.mbad, Ab.ys));
+    FP_KERNEL("k_va_class", side2, k_va_class<<<grid_for(N), TPB, 0, side2>>>(L, Ab.roots, Ab.Dstar, Ab.ys, each, Ab.shared,
+                                                                      Ab.irr, Ab.nirr));
+    // one PST check per column
+    FP_KERNEL("k_va_colE", side2, k_va_colE<<<(L.M + 1) / 2, 2 * LEC_THREADS, 0, side2>>>(Ab.Dstar, Ab.ys, L.M, J.E));
+    pst_jobs(L, J, L.M, nullptr, ps, (const g2a*)g2tau, nullptr, 0, Ab.col_res, side2);
     // the checks of all K blocks
     const VSrc S{rs, (size_t)L.b * G1_SER, (const uint8_t*)blocks, L.bopen_len, 0, L.K, L.b, L.R, L.log_r};
     FP_KERNEL("k_v_cdec", s, k_v_cdec<<<1, 32, 0, s>>>(Cb, Ab.Cd, Ab.cbad));
-    block_checks_front(S, Cb, (const g1a*)g1beta, Bb, s);
+    block_checks_front(S, Cb, Ab.Cd, (const g1a*)g1beta, Bb, s, side);
     FP_KERNEL("k_v_miller", s, k_v_miller<<<3 * L.K, LM_THREADS, 0, s>>>(Bb.P, Bb.Q, Bb.ml));
-    FP_KERNEL("k_vb_gt", s, k_vb_gt<<<2 * L.log_r * L.K, 128, 0, s>>>(S, Bb.st, Bb.ge));
-    FP_KERNEL("k_vb_prod", s, k_vb_prod<<<grid_for(L.K, 64), 64, 0, s>>>(Bb.ml, Bb.ge, Ab.Cd, L.K, L.log_r, Bb.fe_in,
-                                                                       Bb.cT));
+    block_fe_inputs(Bb, L.K, Bb.fe_in, s);
     final_exp_group(Bb.fe_in, 2 * L.K, Bb.fe_out, nullptr, 1, 0, 0, s);
-    FP_KERNEL("k_vb_check", s, k_vb_check<<<grid_for(L.K, 64), 64, 0, s>>>(Bb.fe_out, Bb.cT, Ab.cbad, Bb.st, L.K,
+    vb_join(side, s);
+    FP_KERNEL("k_vb_check", s, k_vb_check<<<grid_for(L.K, 64), 64, 0, s>>>(Bb.fe_out, Bb.cT, Bb.c1, Ab.cbad, Bb.st, L.K,
                                                                          Bb.res));
-    // element checks and the sharing classes
-    const uint64_t* md = (const uint64_t*)m;
-    FP_KERNEL("k_va_paths", s, k_va_paths<<<grid_for(N, 64), 64, 0, s>>>(L, md, (const uint8_t*)row_tree,
-                                                                       (const uint8_t*)top_tree, rs, Ab.roots,
-                                                                       Ab.mbad));
-    FP_KERNEL("k_va_rows", s, k_va_rows<<<grid_for(L.R, 16), 128, 0, s>>>(L, Ab.roots, rs, Ds, Ab.rj, Ab.Dstar,
-                                                                       Ab.row_bad));
-    FP_KERNEL("k_va_y", s, k_va_y<<<grid_for(N), TPB, 0, s>>>(L, md, Ab.roots, Ab.rj, (const fr*)g, Ab.mbad, Ab.ys));
-    FP_KERNEL("k_va_class", s, k_va_class<<<grid_for(N), TPB, 0, s>>>(L, Ab.roots, Ab.Dstar, Ab.ys, each, Ab.shared,
-                                                                      Ab.irr, Ab.nirr));
-    // one PST check per column
-    FP_KERNEL("k_va_colE", s, k_va_colE<<<grid_for(L.M, 16), 128, 0, s>>>(Ab.Dstar, Ab.ys, L.M, J.E));
-    pst_jobs(L, J, L.M, nullptr, ps, (const g2a*)g2tau, nullptr, 0, Ab.col_res, s);
     // and one for each proof outside the shared classes
+    vb_join(side2, s);
     uint32_t nirr = 0;
     cudaMemcpyAsync(&nirr, Ab.nirr, 4, cudaMemcpyDeviceToHost, s);
     cudaStreamSynchronize(s);
     for (uint32_t q0 = 0; q0 < nirr; q0 += chunk) {
         const uint32_t nj = std::min(chunk, nirr - q0);
-        FP_KERNEL("k_va_irrE", s, k_va_irrE<<<grid_for(nj, 16), 128, 0, s>>>(L, Ab.irr, q0, nj, Ab.roots, Ab.ys, rs,
+        FP_KERNEL("k_va_irrE", s, k_va_irrE<<<nj, 2 * LEC_THREADS, 0, s>>>(L, Ab.irr, q0, Ab.roots, Ab.ys, rs,
                                                                           Ds, J.E, J.a));
         pst_jobs(L, J, nj, J.a, ps, (const g2a*)g2tau, Ab.irr, q0, Ab.irr_res, s);
     }
