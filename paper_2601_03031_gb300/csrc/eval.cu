@@ -8,7 +8,7 @@
 //   with t = 1: r_0 = HFr("FP-r", SHA256("FP-eval" || C || u32be(log N) || r || C_F) || u32be(0)),
 //   b = r_0 T, through the Step-1 round chain), and PST.Eval(F, r_R): for t = l_c - 1 .. 0,
 //   q_t[c] = F[2^t + c] - F[c], pi_t = sum_c q_t[c] Lambda_t[c], F[c] <- F[c] + r_t q_t[c].
-#include "group_ec.cuh"
+#include "limb_ec.cuh"
 #include "k_common.cuh"
 
 namespace fpk {
@@ -93,26 +93,21 @@ __global__ void __launch_bounds__(1024) k_eval_fold(fr* F, const fr* r_mont, int
     if (threadIdx.x == 0) fr_to_be(y_out, F[0]);
 }
 
-// terms q_t[c] Lambda_t[c] (flat index e = 2^t - 1 + c for both tables), one 8-lane group each,
-// written to out[t (M/2) + c] as Jacobian (the other slots of a level stay the identity)
-__global__ void __launch_bounds__(128) k_eval_pst_terms(const fr* q, const g1a* lam, uint32_t M, g1j* out) {
-    __shared__ GEc<fq> sm[16];
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
-    const uint64_t e0 = (uint64_t)blockIdx.x * 16 + grp;
-    const bool valid = e0 < M - 1;
-    const uint64_t e = valid ? e0 : 0;
+// terms q_t[c] Lambda_t[c] (flat index e = 2^t - 1 + c for both tables), one limb per lane, half a block
+// each, written to out[t (M/2) + c], c < 2^t, as Jacobian
+__global__ void __launch_bounds__(2 * LEC_THREADS) k_eval_pst_terms(const fr* q, const g1a* lam, uint32_t M, g1j* out) {
+    __shared__ LimbEc sm[2];
+    const int half = (int)(threadIdx.x / LEC_THREADS);
+    const uint64_t e = blockIdx.x * (uint64_t)2 + half;
+    if (e >= M - 1) return;                                   // three whole warps, with a barrier of their own
     const int t = 31 - __clz((uint32_t)(e + 1));
     const uint64_t c = e + 1 - (1ull << t);
     uint32_t kw[8];
     fr_canon_words(kw, q[e]);
-    const GPt<fq> r = gec_g1_mul_proj_w2(sm[grp], lane, lam[e], kw);
-    if (valid && lane == 0) {
-        g1j o;
-        o.X = fq_mul(r.X, r.Z);
-        o.Y = fq_mul(r.Y, fq_sqr(r.Z));
-        o.Z = r.Z;
-        out[(uint64_t)t * (M / 2) + c] = o;
-    }
+    const LecLane k = lec_lane();
+    lec_g1_mul(sm[half], k, lam[e], kw);
+    const fq v = lec_jacobian(sm[half], k);
+    if (k.k.l == 0 && k.slot < 3) reinterpret_cast<fq*>(&out[(uint64_t)t * (M / 2) + c])[k.slot] = v;
 }
 
 void eval_point(const void* r_be, int log_n, void* r_mont, uint32_t* err, cudaStream_t s) {
@@ -139,7 +134,7 @@ void eval_pst_fold(void* F, const void* r_mont, int log_c, void* q, void* y_out,
 }
 void eval_pst_terms(const void* q, const void* lam, uint32_t M, void* out, cudaStream_t s) {
     if (M < 2) return;
-    FP_KERNEL("k_eval_pst_terms", s, k_eval_pst_terms<<<grid_for(M - 1, 16), 128, 0, s>>>((const fr*)q,
+    FP_KERNEL("k_eval_pst_terms", s, k_eval_pst_terms<<<M / 2, 2 * LEC_THREADS, 0, s>>>((const fr*)q,
                                                                                         (const g1a*)lam, M,
                                                                                         (g1j*)out));
 }

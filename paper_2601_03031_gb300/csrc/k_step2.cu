@@ -2,6 +2,7 @@
 // tree of Sec. 4.2) and the assembly of individual proofs.
 // Stored trees keep every level: leaves first, then each parent level (offset 2L - 2L/2^l).
 #include "k_common.cuh"
+#include "limb_ec.cuh"
 
 namespace fpk {
 
@@ -66,14 +67,34 @@ __global__ void k_randomize(const fr* m_mont, const fr* rj, uint32_t R, uint32_t
     g[i] = fr_mul(rj[i / M], m_mont[i]);
 }
 
-// D_j = C_j^{r_j} (Eq. ProverRand)
-__global__ void __launch_bounds__(64) k_d0(const g1a* rows, const fr* rj, uint32_t R, g1a* D) {
+// D_j = C_j^{r_j} (Eq. ProverRand), Jacobian
+__global__ void __launch_bounds__(64) k_d0(const g1a* rows, const fr* rj, uint32_t R, g1j* D) {
     uint64_t j = gtid();
     if (j >= R) return;
     uint32_t kw[8];
     fr_canon_words(kw, rj[j]);
-    D[j] = g1_affine(g1_mul(rows[j], kw));
+    D[j] = g1_mul(rows[j], kw);
 }
+// k P as Jacobian on 96 threads, one limb per lane (limb_ec.cuh)
+FPG_DEV void mul_limb(LimbEc& S, const g1a& P, const fr& k_mont, g1j* out) {
+    uint32_t kw[8];
+    fr_canon_words(kw, k_mont);
+    const LecLane c = lec_lane();
+    lec_g1_mul(S, c, P, kw);
+    const fq v = lec_jacobian(S, c);
+    if (c.k.l == 0 && c.slot < 3) reinterpret_cast<fq*>(out)[c.slot] = v;
+}
+// the same, half a block per row.  Few rows are one scalar multiplication's latency: 0.22 ms, on one thread
+// each 2.8 ms (256 rows).  Up to STEP2_LIMB_MAX multiplications the limb lanes also finish before the
+// threads' latency; beyond, the threads do less work in total.
+__global__ void __launch_bounds__(2 * LEC_THREADS) k_d0_l(const g1a* rows, const fr* rj, uint32_t R, g1j* D) {
+    __shared__ LimbEc sm[2];
+    const int half = (int)(threadIdx.x / LEC_THREADS);
+    const uint64_t j = blockIdx.x * (uint64_t)2 + half;
+    if (j >= R) return;                                       // three whole warps, with a barrier of their own
+    mul_limb(sm[half], rows[j], rj[j], &D[j]);
+}
+constexpr uint64_t STEP2_LIMB_MAX = 8 * 152;
 
 // Sub-protocol: g_w = g_wl + g_wr for every node at level h (all nodes kept)
 __global__ void k_fold_g(fr* g, uint32_t R, uint32_t M, int h) {
@@ -84,12 +105,12 @@ __global__ void k_fold_g(fr* g, uint32_t R, uint32_t M, int h) {
     uint64_t w = tree_off(R, h) + s, wl = tree_off(R, h - 1) + 2 * s;
     g[w * M + a] = fr_add(g[wl * M + a], g[(wl + 1) * M + a]);
 }
-// D_w = D_wl D_wr
-__global__ void __launch_bounds__(64) k_fold_d(g1a* D, uint32_t R, int h) {
+// D_w = D_wl D_wr, Jacobian (every node is converted once, after the last level)
+__global__ void __launch_bounds__(64) k_fold_d(g1j* D, uint32_t R, int h) {
     uint64_t s = gtid();
     if (s >= (R >> h)) return;
     uint64_t w = tree_off(R, h) + s, wl = tree_off(R, h - 1) + 2 * s;
-    D[w] = g1_affine(g1_madd(g1_from_affine(D[wl]), D[wl + 1]));
+    D[w] = jac_add(D[wl], D[wl + 1]);
 }
 
 // HyperEval on g* (PST at every hypercube point): level t, prefix p < M/2^(t+1), c < 2^t:
@@ -113,6 +134,19 @@ __global__ void __launch_bounds__(64) k_pst_terms(const fr* g, const g1a* lam, u
         res = g1_mul(lam[(1ull << t) - 1 + c], kw);
     }
     out[idx] = res;
+}
+
+// the same terms with one limb per lane, half a block each
+__global__ void __launch_bounds__(2 * LEC_THREADS) k_pst_terms_l(const fr* g, const g1a* lam, uint32_t R, uint32_t M,
+                                                                 int log_c, g1j* out) {
+    __shared__ LimbEc sm[2];
+    const int half = (int)(threadIdx.x / LEC_THREADS);
+    const uint64_t idx = blockIdx.x * (uint64_t)2 + half, hm = M / 2;
+    if (idx >= (uint64_t)log_c * hm) return;
+    const int t = (int)(idx / hm);
+    const uint64_t rem = idx % hm, p = rem >> t, c = rem & ((1ull << t) - 1), w = 1ull << t;
+    const fr* gs = g + (2 * (uint64_t)R - 2) * M;
+    mul_limb(sm[half], lam[w - 1 + c], fr_sub(gs[(2 * p + 1) * w + c], gs[2 * p * w + c]), &out[idx]);
 }
 
 __global__ void k_gstar_ser(const fr* g, uint32_t R, uint32_t M, uint8_t* out) {
@@ -140,16 +174,24 @@ void step2_randomize(const void* m_mont, const void* rj, uint32_t R, uint32_t M,
     FP_KERNEL("k_randomize", s, k_randomize<<<grid_for((uint64_t)R * M), TPB, 0, s>>>((const fr*)m_mont, (const fr*)rj, R, M, (fr*)g));
 }
 void step2_d0(const void* rows, const void* rj, uint32_t R, void* D, cudaStream_t s) {
-    FP_KERNEL("k_d0", s, k_d0<<<grid_for(R, 64), 64, 0, s>>>((const g1a*)rows, (const fr*)rj, R, (g1a*)D));
+    if (R <= STEP2_LIMB_MAX)
+        FP_KERNEL("k_d0", s, k_d0_l<<<(R + 1) / 2, 2 * LEC_THREADS, 0, s>>>((const g1a*)rows, (const fr*)rj, R, (g1j*)D));
+    else
+        FP_KERNEL("k_d0", s, k_d0<<<grid_for(R, 64), 64, 0, s>>>((const g1a*)rows, (const fr*)rj, R, (g1j*)D));
 }
 void step2_fold_g(void* g, uint32_t R, uint32_t M, int h, cudaStream_t s) {
     FP_KERNEL("k_fold_g", s, k_fold_g<<<grid_for((uint64_t)(R >> h) * M), TPB, 0, s>>>((fr*)g, R, M, h));
 }
 void step2_fold_d(void* D, uint32_t R, int h, cudaStream_t s) {
-    FP_KERNEL("k_fold_d", s, k_fold_d<<<grid_for(R >> h, 64), 64, 0, s>>>((g1a*)D, R, h));
+    FP_KERNEL("k_fold_d", s, k_fold_d<<<grid_for(R >> h, 64), 64, 0, s>>>((g1j*)D, R, h));
 }
 void step2_pst_terms(const void* g, const void* lam, uint32_t R, uint32_t M, int log_c, void* out, cudaStream_t s) {
     uint64_t n = (uint64_t)log_c * (M / 2);
+    if (n <= STEP2_LIMB_MAX) {
+        FP_KERNEL("k_pst_terms", s, k_pst_terms_l<<<(unsigned)((n + 1) / 2), 2 * LEC_THREADS, 0, s>>>(
+                                        (const fr*)g, (const g1a*)lam, R, M, log_c, (g1j*)out));
+        return;
+    }
     FP_KERNEL("k_pst_terms", s, k_pst_terms<<<grid_for(n, 64), 64, 0, s>>>((const fr*)g, (const g1a*)lam, R, M, log_c, (g1j*)out));
 }
 void step2_gstar_ser(const void* g, uint32_t R, uint32_t M, void* out, cudaStream_t s) {

@@ -156,9 +156,9 @@ void step2_row_leaves(const void* row_tree, const void* rows_ser, uint32_t R, ui
                       cudaStream_t s);
 void step2_rj(const void* top_tree, uint32_t R, void* rj, cudaStream_t s);
 void step2_randomize(const void* m_mont, const void* rj, uint32_t R, uint32_t M, void* g, cudaStream_t s);
-void step2_d0(const void* rows_g1a, const void* rj, uint32_t R, void* D_g1a, cudaStream_t s);
+void step2_d0(const void* rows_g1a, const void* rj, uint32_t R, void* D_g1j, cudaStream_t s);
 void step2_fold_g(void* g, uint32_t R, uint32_t M, int h, cudaStream_t s);
-void step2_fold_d(void* D_g1a, uint32_t R, int h, cudaStream_t s);
+void step2_fold_d(void* D_g1j, uint32_t R, int h, cudaStream_t s);
 void step2_pst_terms(const void* g, const void* lam, uint32_t R, uint32_t M, int log_c, void* out_g1j,
                      cudaStream_t s);
 void step2_gstar_ser(const void* g, uint32_t R, uint32_t M, void* out, cudaStream_t s);

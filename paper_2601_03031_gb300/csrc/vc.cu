@@ -745,7 +745,7 @@ fp_proofs* prove_impl(const fp_pp* pp, const fp_commit* cm, uint32_t b, uint32_t
             blocks1 = (uint8_t*)pf->blocks + (size_t)k0 * blen;
             // Step 2 depends only on the commitment: it runs on a second stream, concurrently with Step 1
             const uint64_t half = M / 2;
-            void *pt = nullptr, *pt2 = nullptr;
+            void *pt = nullptr, *pt2 = nullptr, *pj = nullptr, *Dj = nullptr;
             if (with_step2) {
                 pf->row_tree = dalloc((size_t)R * (2 * M - 1) * DIGEST, s);
                 pf->top_tree = dalloc((2 * (size_t)R - 1) * DIGEST, s);
@@ -756,6 +756,8 @@ fp_proofs* prove_impl(const fp_pp* pp, const fp_commit* cm, uint32_t b, uint32_t
                 pf->pst_ser = dalloc(((size_t)M - 1) * G1_SER, s);
                 pt = T((size_t)lc * half * G1J_BYTES);
                 pt2 = T((half / 2 + 1) * G1J_BYTES);
+                pj = T((size_t)M * G1J_BYTES);
+                Dj = T((2 * (size_t)R - 1) * G1J_BYTES);
             }
             // every buffer is allocated (stream-ordered on s) before the fork to the internal streams
             const Step1Bufs B = step1_bufs(pp, Kc, T);
@@ -777,21 +779,27 @@ fp_proofs* prove_impl(const fp_pp* pp, const fp_commit* cm, uint32_t b, uint32_t
                 for (int l = 1; l <= lr; l++) tree_level(pf->top_tree, 1, R, l, s2);
                 step2_rj(pf->top_tree, R, pf->rj, s2);
                 step2_randomize(cm->m_mont, pf->rj, R, M, pf->g, s2);
-                step2_d0(cm->rows, pf->rj, R, pf->D, s2);
+                step2_d0(cm->rows, pf->rj, R, Dj, s2);
                 for (int h = 1; h <= lr; h++) {
                     step2_fold_g(pf->g, R, M, h, s2);
-                    step2_fold_d(pf->D, R, h, s2);
+                    step2_fold_d(Dj, R, h, s2);
                 }
-                g1a_serialize(pf->D, pf->D_ser, G1_SER, 2 * (uint64_t)R - 1, s2);
+                g1j_to_affine(Dj, pf->D, pf->D_ser, G1_SER, 2 * (uint64_t)R - 1, s2);
                 step2_pst_terms(pf->g, pp->lam, R, M, lc, pt, s2);
-                size_t pst_off = 0;
+                // level t's sums of 2^t terms into their places pst_off .. of the proofs' order, then one
+                // conversion of all M - 1
+                uint64_t pst_off = 0;
                 for (int t = 0; t < lc; t++) {
                     void* lvl = (uint8_t*)pt + (size_t)t * half * G1J_BYTES;
-                    uint64_t nseg = half >> t;
-                    void* res = reduce_pairs(lvl, pt2, half, nseg, g1_pair_reduce, s2);
-                    g1j_to_affine(res, nullptr, (uint8_t*)pf->pst_ser + pst_off * G1_SER, G1_SER, nseg, s2);
+                    const uint64_t nseg = half >> t;
+                    void* res = half <= TREE_REDUCE_MAX
+                                    ? reduce_tree(lvl, pt2, half, nseg, 32, g1_tree_reduce, s2)
+                                    : reduce_pairs(lvl, pt2, half, nseg, g1_pair_reduce, s2);
+                    check(cudaMemcpyAsync((uint8_t*)pj + pst_off * G1J_BYTES, res, nseg * G1J_BYTES,
+                                          cudaMemcpyDeviceToDevice, s2), "D2D");
                     pst_off += nseg;
                 }
+                g1j_to_affine(pj, nullptr, pf->pst_ser, G1_SER, (uint64_t)M - 1, s2);
             }
             check(cudaEventRecord(ev_join, s2), "event");
 
@@ -1121,18 +1129,38 @@ fp_status vc_eval_prove(const fp_pp* pp, const fp_commit* cm, const uint8_t* r, 
             void* r0 = T(FR_BYTES);
             void* terms = T((size_t)(lc ? lc : 1) * half * G1J_BYTES);
             void* terms2 = T((half / 2 + 1) * G1J_BYTES);
+            void* sums = T((size_t)(lc ? lc : 1) * G1J_BYTES);
             const Step1Bufs B = step1_bufs(pp, 1, T);
             const bool la = lookahead_on((int)pp->log_r);
             const LaBufs L = la ? la_bufs(pp, 1, T) : LaBufs{};
             const Streams st = streams(s);
-            cudaStream_t s1 = st.hi, s3 = st.sp;
-            cudaEvent_t ev_fork = new_event(), ev_bvec = new_event(), ev_join = new_event();
+            cudaStream_t s1 = st.hi, s3 = st.sp, s2 = st.lo;
+            cudaEvent_t ev_fork = new_event(), ev_bvec = new_event(), ev_join = new_event(), ev_wts = new_event(),
+                        ev_pst = new_event();
             check(cudaEventRecord(ev_fork, s), "event");
             check(cudaStreamWaitEvent(s1, ev_fork, 0), "wait");
             check(cudaMemsetAsync(err, 0, 4, s1), "memset");
             check(cudaMemcpyAsync(r_be, r, 32 * (size_t)ln, cudaMemcpyHostToDevice, s1), "H2D r");
             eval_point(r_be, ln, r_mont, err, s1);
             eval_weights(r_mont, lr, lc, Tm, Tc, s1);
+            // PST.Eval of F = sum_j T_j f_j at r_R needs the weights only: on a stream beside the FC rounds
+            check(cudaEventRecord(ev_wts, s1), "event");
+            check(cudaStreamWaitEvent(s2, ev_wts, 0), "wait");
+            eval_ftable(cm->m_mont, Tm, R, M, F, s2);
+            eval_pst_fold(F, r_mont, lc, q, proof, s2);
+            if (lc) {
+                eval_pst_terms(q, pp->lam, M, terms, s2);
+                for (int t = 0; t < lc; t++) {
+                    void* lvl = (uint8_t*)terms + (size_t)t * half * G1J_BYTES;
+                    const uint64_t n = 1ull << t;                  // level t's terms (one sum)
+                    void* res = n <= TREE_REDUCE_MAX ? reduce_tree(lvl, terms2, n, 1, 32, g1_tree_reduce, s2)
+                                                     : reduce_pairs(lvl, terms2, n, 1, g1_pair_reduce, s2);
+                    check(cudaMemcpyAsync((uint8_t*)sums + (size_t)(lc - 1 - t) * G1J_BYTES, res, G1J_BYTES,
+                                          cudaMemcpyDeviceToDevice, s2), "D2D");
+                }
+                g1j_to_affine(sums, nullptr, proof + 128 + blen, G1_SER, lc, s2);
+            }
+            check(cudaEventRecord(ev_pst, s2), "event");
             // step 1: C_F = sum_j T_j C_j over the row commitments (and their GLV partners)
             check(cudaMemcpyAsync(tab, cm->rows, (size_t)R * G1A_BYTES, cudaMemcpyDeviceToDevice, s1), "D2D");
             msm_bases_endo(tab, R, s1);
@@ -1144,18 +1172,7 @@ fp_status vc_eval_prove(const fp_pp* pp, const fp_commit* cm, const uint8_t* r, 
             check(cudaStreamWaitEvent(s3, ev_bvec, 0), "wait");
             if (la) step1_rounds_la(pp, 0, 1, R, B, L, proof + 128, blen, s1, s3, st.la, st.fold);
             else step1_rounds(pp, 0, 1, R, B, proof + 128, blen, s1, s3);
-            // step 3: PST.Eval of F = sum_j T_j f_j at r_R
-            eval_ftable(cm->m_mont, Tm, R, M, F, s1);
-            eval_pst_fold(F, r_mont, lc, q, proof, s1);
-            if (lc) {
-                check(cudaMemsetAsync(terms, 0, (size_t)lc * half * G1J_BYTES, s1), "memset");
-                eval_pst_terms(q, pp->lam, M, terms, s1);
-                for (int t = 0; t < lc; t++) {
-                    void* lvl = (uint8_t*)terms + (size_t)t * half * G1J_BYTES;
-                    void* res = reduce_pairs(lvl, terms2, half, 1, g1_pair_reduce, s1);
-                    g1j_to_affine(res, nullptr, proof + 128 + blen + G1_SER * (size_t)(lc - 1 - t), G1_SER, 1, s1);
-                }
-            }
+            check(cudaStreamWaitEvent(s1, ev_pst, 0), "wait");
             check_launch("vc_eval_prove kernels");
             check(cudaMemcpyAsync(out, proof, need, cudaMemcpyDeviceToHost, s1), "D2H proof");
             check(cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, s1), "D2H err");
@@ -1164,6 +1181,7 @@ fp_status vc_eval_prove(const fp_pp* pp, const fp_commit* cm, const uint8_t* r, 
             for (void* p : tmp) cudaFreeAsync(p, s);
             tmp.clear();
             cudaEventDestroy(ev_fork); cudaEventDestroy(ev_bvec); cudaEventDestroy(ev_join);
+            cudaEventDestroy(ev_wts); cudaEventDestroy(ev_pst);
             check(cudaStreamSynchronize(s), "vc_eval_prove");
         } catch (...) {
             for (void* p : tmp) cudaFreeAsync(p, s);
