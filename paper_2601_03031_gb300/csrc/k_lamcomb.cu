@@ -108,31 +108,43 @@ void lam_comb_tables(const void* bases_g1a, uint32_t M, void* scratch, void* tab
     FP_KERNEL("k_lamc_rows", s, k_lamc_rows<<<grid_for((uint64_t)M * LAMC_W * 15, 64), 64, 0, s>>>(M, (g1a*)tab));
 }
 
-// partial[(j M + a) Q + q] = sum over the windows w in [8 q, 8 q + 8) of T[a][w][digit_w(m[j M + a])],
-// one thread per (j, a, q); an entry with digit 0 is the identity and is skipped
-__global__ void __launch_bounds__(128) k_lamc_sum(const g1a* tab, const fr* m_canon, uint32_t R, uint32_t M,
+// partial[((j M + a0) / G) Q + q] = sum over the bases a in [a0, a0 + G) and the windows w in [8 q, 8 q + 8)
+// of T[a][w][digit_w(m[j M + a])], one thread per (j, a0, q), G | M; an entry with digit 0 is the identity
+// and is skipped.  G is as large as still leaves 2^18 threads (lam_comb_group), which fill the GPU: the
+// partial sums are then 38 MB however long the vector is, and what is added beyond here (a Jacobian
+// addition per partial sum, through DRAM) does not grow.  N = 2^20: this kernel and the pairwise sums
+// after it 11.6 + 3.6 ms with G = 1, 13.6 ms and no pairwise sums with G = 16.
+__global__ void __launch_bounds__(128) k_lamc_sum(const g1a* tab, const fr* m_canon, uint32_t R, uint32_t M, uint32_t G,
                                                   g1j* partial) {
     const uint64_t u = gtid();
-    if (u >= (uint64_t)R * M * LAMC_Q) return;
-    const uint64_t ja = u / LAMC_Q;
+    if (u >= (uint64_t)R * (M / G) * LAMC_Q) return;
     const int q = (int)(u % LAMC_Q);
-    const uint32_t a = (uint32_t)(ja % M);
-    uint32_t k1[5], k0[4];
-    div_by_const<4, 5>(k1, k0, m_canon[ja].v, GLV_D, GLV_BARRETT);
-    const g1a* T = tab + (uint64_t)a * LAMC_W * LAMC_E;
+    const uint64_t ja0 = u / LAMC_Q * G;
+    const uint32_t a0 = (uint32_t)(ja0 % M);
     g1j acc;
     jac_set_inf(acc);
-    for (int w = 8 * q; w < 8 * q + 8; w++) {
-        const int e = (int)(((k0[w >> 3] >> (4 * (w & 7))) & 15) | (((k1[w >> 3] >> (4 * (w & 7))) & 15) << 4));
-        if (e) acc = g1_madd(acc, T[(uint64_t)w * LAMC_E + e]);
+    for (uint32_t i = 0; i < G; i++) {
+        uint32_t k1[5], k0[4];
+        div_by_const<4, 5>(k1, k0, m_canon[ja0 + i].v, GLV_D, GLV_BARRETT);
+        const g1a* T = tab + (uint64_t)(a0 + i) * LAMC_W * LAMC_E;
+        for (int w = 8 * q; w < 8 * q + 8; w++) {
+            const int e = (int)(((k0[w >> 3] >> (4 * (w & 7))) & 15) | (((k1[w >> 3] >> (4 * (w & 7))) & 15) << 4));
+            if (e) acc = g1_madd(acc, T[(uint64_t)w * LAMC_E + e]);
+        }
     }
     partial[u] = acc;
 }
 
-void lam_comb_partials(const void* tab, const void* m_canon, uint32_t R, uint32_t M, void* partial, cudaStream_t s) {
-    FP_KERNEL("k_lamc_sum", s, k_lamc_sum<<<grid_for((uint64_t)R * M * LAMC_Q, 128), 128, 0, s>>>(
-                                   (const g1a*)tab, (const fr*)m_canon, R, M, (g1j*)partial));
+uint32_t lam_comb_group(uint32_t R, uint32_t M) {
+    uint32_t G = 1;
+    while (G < M && (uint64_t)R * (M / G) * LAMC_Q > (1u << 18)) G *= 2;
+    return G;
 }
-uint32_t lam_comb_parts() { return LAMC_Q; }
+void lam_comb_partials(const void* tab, const void* m_canon, uint32_t R, uint32_t M, void* partial, cudaStream_t s) {
+    const uint32_t G = lam_comb_group(R, M);
+    FP_KERNEL("k_lamc_sum", s, k_lamc_sum<<<grid_for((uint64_t)R * (M / G) * LAMC_Q, 128), 128, 0, s>>>(
+                                   (const g1a*)tab, (const fr*)m_canon, R, M, G, (g1j*)partial));
+}
+uint64_t lam_comb_parts(uint32_t R, uint32_t M) { return (uint64_t)(M / lam_comb_group(R, M)) * LAMC_Q; }
 
 }  // namespace fpk

@@ -24,12 +24,16 @@ FPG_DEV void fq2_zero(fq2& a) { fq_zero(a.c0); fq_zero(a.c1); }
 FPG_DEV void fq2_one(fq2& a) { fq_one(a.c0); fq_zero(a.c1); }
 FPG_DEV bool fq2_is_zero(const fq2& a) { return fq_is_zero(a.c0) && fq_is_zero(a.c1); }
 FPG_DEV bool fq2_eq(const fq2& a, const fq2& b) { return fq_eq(a.c0, b.c0) && fq_eq(a.c1, b.c1); }
-FPG_NOINL fq2 fq2_mul(const fq2& a, const fq2& b) {
+// Operands and results of the Fq2 products travel in registers (by value): by reference they go through
+// local memory, which bounds the one-thread pairings (65% L1 hits at two warps per sub-partition; more
+// warps miss more and are slower).  By value a Miller loop's frame is 2.3 instead of 3.9 KB: 131,072 loops
+// 50.6 -> 49.0 ms, 32,768 14.4 -> 12.3 ms (one GB300).
+FPG_NOINL fq2 fq2_mul(const fq2 a, const fq2 b) {
     fq t0 = fq_mul(a.c0, b.c0), t1 = fq_mul(a.c1, b.c1);
     fq s = fq_mul(fq_add(a.c0, a.c1), fq_add(b.c0, b.c1));
     return {fq_sub(t0, t1), fq_sub(fq_sub(s, t0), t1)};
 }
-FPG_NOINL fq2 fq2_sqr(const fq2& a) {
+FPG_NOINL fq2 fq2_sqr(const fq2 a) {
     fq t = fq_mul(a.c0, a.c1);
     return {fq_mul(fq_add(a.c0, a.c1), fq_sub(a.c0, a.c1)), fq_dbl(t)};
 }

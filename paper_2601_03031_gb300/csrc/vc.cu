@@ -357,10 +357,10 @@ fp_commit* commit_enqueue(const fp_pp* pp, const uint64_t* m, int on_device, cud
         }
         load_vector(msrc, N, cm->m_canon, cm->m_mont, cm->err, s);
         // C_j = sum_a m[jM + a] Lambda_{l_c}[a]: R sums of M terms over the shared bases, from their
-        // comb tables when the setup has them (partial sums per base and quarter of the windows,
+        // comb tables when the setup has them (partial sums over bases and quarters of the windows,
         // reduced pairwise and then by block trees), else R MSMs
         if (pp->lam_comb) {
-            const uint64_t np = (uint64_t)R * M * lam_comb_parts();
+            const uint64_t np = (uint64_t)R * lam_comb_parts(R, M);
             t1 = dalloc(np * G1J_BYTES, s);
             t2 = dalloc((np / 2 + 1) * G1J_BYTES, s);
             lam_comb_partials(pp->lam_comb, cm->m_canon, R, M, t1, s);
