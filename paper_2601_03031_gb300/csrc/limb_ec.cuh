@@ -70,17 +70,18 @@ FPG_DEV int32_t lec_mul1(LimbEc& S, const LecLane& c, const int32_t* y, const in
 
 // acc <- acc + Q for Q's windows qx, qy, qz, or 2 acc for DBL (the windows are then acc's own)
 template <bool DBL>
-FPG_DEV void lec_step(LimbEc& S, const LecLane& c, const int32_t* qx, const int32_t* qy, const int32_t* qz) {
+FPG_DEV void lec_step_on(LimbEc& S, const LecLane& c, int32_t (*acc)[LIMB_WIN], const int32_t* qx, const int32_t* qy,
+                         const int32_t* qz) {
     const int l = c.k.l, s = c.slot;
     {
         const int32_t* qi = c.i == 0 ? qx : c.i == 1 ? qy : qz;
         const int32_t* qj = c.j == 0 ? qx : c.j == 1 ? qy : qz;
         int64_t lo, hi;
         if (s < 2) {                               // warp 0: squares of coordinates, one product each
-            const int32_t *row[1] = {S.acc[c.i]}, *win[1] = {qi};
+            const int32_t *row[1] = {acc[c.i]}, *win[1] = {qi};
             limb_dot<1>(c.k, lo, hi, row, win);
         } else {
-            const int32_t *row[2] = {S.acc[c.i], S.acc[c.j]}, *win[2] = {qj, s == 2 ? S.zero : qi};
+            const int32_t *row[2] = {acc[c.i], acc[c.j]}, *win[2] = {qj, s == 2 ? S.zero : qi};
             limb_dot<2>(c.k, lo, hi, row, win);
         }
         lo *= c.scale;
@@ -110,9 +111,14 @@ FPG_DEV void lec_step(LimbEc& S, const LecLane& c, const int32_t* qx, const int3
         int64_t lo, hi;
         limb_dot<2>(c.k, lo, hi, row, win);
         const int32_t v = limb_carry(limb_reduce(c.k, lo, hi, S.u[s]), l);
-        if (s < 3) limb_put_window(S.acc[s], l, v);
+        if (s < 3) limb_put_window(acc[s], l, v);
     }
     lec_sync();
+}
+
+template <bool DBL>
+FPG_DEV void lec_step(LimbEc& S, const LecLane& c, const int32_t* qx, const int32_t* qy, const int32_t* qz) {
+    lec_step_on<DBL>(S, c, S.acc, qx, qy, qz);
 }
 
 // the width-4 NAF of a 128-bit k, least significant first, into the zeroed d (one lane)

@@ -24,7 +24,7 @@
 #include <cmath>
 #include <type_traits>
 
-#include "group_ec.cuh"
+#include "limb_ec.cuh"
 #include "k_common.cuh"
 
 namespace fpk {
@@ -372,6 +372,110 @@ __global__ void __launch_bounds__(64) k_msm_final(MsmShape sh, const GPt<F>* win
     }
 }
 
+// ---- G1 with one limb per lane (limb_ec.cuh), for latency: 96 threads per running sum.  A point enters as
+// its homogeneous residues' limbs: the common factor between the residues' Montgomery form and the
+// engine's scales all three coordinates and leaves the point the same.
+constexpr int MSM_L_BUCKETS = 16, MSM_L_GROUPS = 4;        // buckets per running sum, sums per block
+constexpr uint64_t MSM_L_MAX = 16384;                      // buckets in all up to which the sums run on limb lanes
+struct MsmPart { int32_t c[3][LIMB_ROW]; };                // X, Y, Z as limbs
+uint32_t msm_l_parts(const MsmShape& sh) {                 // partial sums per window
+    const uint32_t per = MSM_L_BUCKETS * MSM_L_GROUPS;
+    return (sh.buckets(0) + per - 1) / per;
+}
+
+// Window sums: group g of window w of batch j adds its buckets b in [16 g, 16 g + 16) from the top,
+// run += B_b, sum += run, then sum += 16 g run; the block's four groups are added up.  0.106 ms for a
+// 3000-term sum, where one thread per 4 buckets took 0.42 ms and the pairwise sums after it 0.18.
+struct MsmWinSmem {
+    LimbEc g[MSM_L_GROUPS];
+    alignas(16) int32_t sum[MSM_L_GROUPS][3][LIMB_WIN];
+};
+__global__ void __launch_bounds__(MSM_L_GROUPS * LEC_THREADS) k_msm_window_l(MsmShape sh, uint32_t parts,
+                                                                            const GPt<fq>* buckets, MsmPart* out) {
+    __shared__ MsmWinSmem sm;
+    const int gi = (int)(threadIdx.x / LEC_THREADS);
+    LimbEc& S = sm.g[gi];
+    const LecLane c = lec_lane();
+    const int l = c.k.l, s = c.slot;
+    const uint64_t jw = blockIdx.x / parts;
+    const uint32_t part = (uint32_t)(blockIdx.x % parts);
+    const uint64_t j = jw / sh.W;
+    const int w = (int)(jw % sh.W);
+    const uint32_t B = sh.buckets(w), lo = (part * MSM_L_GROUPS + gi) * MSM_L_BUCKETS;
+    const uint32_t n = lo < B ? min(B - lo, (uint32_t)MSM_L_BUCKETS) : 0;
+    const GPt<fq>* bk = buckets + j * sh.KW + sh.off(w) + lo;
+    if (s == 5) limb_put_window(S.zero, l, 0);
+    if (s < 3) {                                           // run and sum start at the identity (0 : 1 : 0)
+        const int32_t v = s == 1 ? LIMB_FROB2[0][l] : 0;
+        limb_put_window(S.acc[s], l, v);
+        limb_put_window(sm.sum[gi][s], l, v);
+    }
+    const int co = s < 3 ? s : 0;
+    int32_t next = n ? limb_of_words(reinterpret_cast<const fq*>(&bk[n - 1])[co].v, l) : 0;
+    for (int b = (int)n - 1; b >= 0; b--) {
+        if (s < 3) limb_put_window(S.two[s], l, next);
+        lec_sync();
+        if (b) next = limb_of_words(reinterpret_cast<const fq*>(&bk[b - 1])[co].v, l);
+        lec_step<false>(S, c, S.two[0], S.two[1], S.two[2]);
+        lec_step_on<false>(S, c, sm.sum[gi], S.acc[0], S.acc[1], S.acc[2]);
+    }
+    lec_sync();
+    if (n && lo) {                                         // sum += lo run
+        if (s < 3) limb_put_window(S.two[s], l, S.acc[s][l]);
+        lec_sync();
+        for (int b = 30 - __clz(lo); b >= 0; b--) {
+            lec_step<true>(S, c, S.acc[0], S.acc[1], S.acc[2]);
+            if ((lo >> b) & 1) lec_step<false>(S, c, S.two[0], S.two[1], S.two[2]);
+        }
+        lec_step_on<false>(S, c, sm.sum[gi], S.acc[0], S.acc[1], S.acc[2]);
+    }
+    __syncthreads();
+    if (gi) return;
+    for (int g = 1; g < MSM_L_GROUPS; g++)
+        lec_step_on<false>(S, c, sm.sum[0], sm.sum[g][0], sm.sum[g][1], sm.sum[g][2]);
+    if (s < 3) out[blockIdx.x].c[s][l] = sm.sum[0][s][l];
+}
+
+// per batch, on 96 threads: sum_w 2^(lo_w) S_w by Horner from the top window, S_w the sum of `parts` partial
+// sums (limbs) or one window sum (residues), then affine.  129 doublings and the additions: 0.14 ms for 9 windows
+// of one sum each (an 8-lane group 0.45), 0.30 for a 3000-term sum's windows of several partial sums (0.48).
+template <typename In>
+__global__ void __launch_bounds__(2 * LEC_THREADS) k_msm_final_l(MsmShape sh, uint32_t parts, const In* win, g1a* out,
+                                                                 uint8_t* ser, size_t ser_stride) {
+    __shared__ LimbEc sm[2];
+    const int half = (int)(threadIdx.x / LEC_THREADS);
+    const uint64_t j = blockIdx.x * (uint64_t)2 + half;
+    if (j >= sh.nbatch) return;                            // three whole warps, with a barrier of their own
+    LimbEc& S = sm[half];
+    const LecLane c = lec_lane();
+    const int l = c.k.l, s = c.slot, co = s < 3 ? s : 0;
+    if (s == 5) limb_put_window(S.zero, l, 0);
+    if (s == 4) limb_put_window(S.back, l, LIMB_CONV[1][l]);
+    if (s < 3) limb_put_window(S.acc[s], l, s == 1 ? LIMB_FROB2[0][l] : 0);
+    const In* W = win + j * sh.W * parts;
+    auto limb = [&](uint64_t q) -> int32_t {
+        if constexpr (std::is_same<In, MsmPart>::value) return W[q].c[co][l];
+        else return limb_of_words(reinterpret_cast<const fq*>(&W[q])[co].v, l);
+    };
+    lec_sync();
+    for (int w = sh.W - 1; w >= 0; w--) {
+        int32_t next = limb((uint64_t)w * parts);
+        if (w < sh.W - 1)
+            for (int q = 0; q < sh.bits(w); q++) lec_step<true>(S, c, S.acc[0], S.acc[1], S.acc[2]);
+        for (uint32_t p = 0; p < parts; p++) {
+            if (s < 3) limb_put_window(S.two[s], l, next);
+            lec_sync();
+            if (p + 1 < parts) next = limb((uint64_t)w * parts + p + 1);
+            lec_step<false>(S, c, S.two[0], S.two[1], S.two[2]);
+        }
+    }
+    const fq v = lec_affine(S, c);
+    if (l == 0 && s < 2) {
+        if (out) reinterpret_cast<fq*>(&out[j])[s] = v;
+        if (ser) fq_to_be(ser + j * ser_stride + 48 * s, v);
+    }
+}
+
 // ---------------------------------------------------------------------------- bases
 // first half of the bases table from serialised affine points; err |= 1 for a point that is not
 // canonical, not on y^2 = x^3 + 4 or not in the order-r subgroup (all-zero bytes = identity)
@@ -485,6 +589,10 @@ MsmShape msm_shape(uint64_t n, uint32_t nbatch, uint64_t npts, int c, int parts,
     return sh;
 }
 
+// G1 sums with few buckets in all: their reduction on limb lanes
+template <typename F>
+static bool msm_l_sums(const MsmShape& sh) { return std::is_same<F, fq>::value && sh.nkeys() <= MSM_L_MAX; }
+
 template <typename F>
 static size_t scratch_bytes(const MsmShape& sh) {
     const uint64_t nk = sh.nkeys();
@@ -496,6 +604,7 @@ static size_t scratch_bytes(const MsmShape& sh) {
     b += 2 * r(nchunks * sizeof(xyzz_t<F>));
     b += 2 * r(sh.nsegs() * sizeof(xyzz_t<F>));
     b += r((uint64_t)sh.nbatch * sh.W * sizeof(GPt<F>));
+    if (msm_l_sums<F>(sh)) b += r(nk * sizeof(GPt<F>)) + r((uint64_t)sh.nbatch * sh.W * msm_l_parts(sh) * sizeof(MsmPart));
     return b;
 }
 size_t msm_scratch_bytes(const MsmShape& sh) { return scratch_bytes<fq>(sh); }
@@ -575,6 +684,19 @@ static void msm_run(const void* bases, const void* k_canon, const MsmShape& sh, 
                   k_msm_fixup<F><<<grid_for(nchunks, 128), 128, 0, s>>>(keys, offsets, counts, nk, T, head, tail,
                                                                        buckets));
     }
+    if constexpr (!g2) {
+        if (msm_l_sums<F>(sh)) {
+            const uint32_t parts = msm_l_parts(sh);
+            GPt<F>* bp = (GPt<F>*)take(nk * sizeof(GPt<F>));
+            MsmPart* ps = (MsmPart*)take(nwin * parts * sizeof(MsmPart));
+            FP_KERNEL("k_msm_to_proj", s, k_msm_to_proj<F><<<grid_for(nk, 128), 128, 0, s>>>(buckets, bp, nk));
+            FP_KERNEL("k_msm_segment", s, k_msm_window_l<<<(unsigned)(nwin * parts), MSM_L_GROUPS * LEC_THREADS, 0,
+                                                          s>>>(sh, parts, bp, ps));
+            FP_KERNEL("k_msm_final", s, k_msm_final_l<MsmPart><<<(sh.nbatch + 1) / 2, 2 * LEC_THREADS, 0, s>>>(
+                                            sh, parts, ps, (g1a*)out_aff, (uint8_t*)ser_out, ser_stride));
+            return;
+        }
+    }
     FP_KERNEL(g2 ? "k_msm_segment_g2" : "k_msm_segment", s, k_msm_segment<F><<<grid_for(nseg, 128), 128, 0, s>>>(sh, buckets, seg_a));
     X* a = seg_a;
     X* b = seg_b;
@@ -583,6 +705,11 @@ static void msm_run(const void* bases, const void* k_canon, const MsmShape& sh, 
         std::swap(a, b);
     }
     FP_KERNEL(g2 ? "k_msm_to_proj_g2" : "k_msm_to_proj", s, k_msm_to_proj<F><<<grid_for(nwin, 128), 128, 0, s>>>(a, proj, nwin));
+    if constexpr (!g2) {
+        FP_KERNEL("k_msm_final", s, k_msm_final_l<GPt<fq>><<<(sh.nbatch + 1) / 2, 2 * LEC_THREADS, 0, s>>>(
+                                        sh, 1, proj, (g1a*)out_aff, (uint8_t*)ser_out, ser_stride));
+        return;
+    }
     FP_KERNEL(g2 ? "k_msm_final_g2" : "k_msm_final", s,
               k_msm_final<F><<<grid_for(sh.nbatch, 8), 64, 0, s>>>(sh, proj, (typename Aff<F>::T*)out_aff,
                                                                   (uint8_t*)ser_out, ser_stride));
