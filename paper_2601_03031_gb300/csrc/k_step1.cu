@@ -124,17 +124,21 @@ __global__ void __launch_bounds__(64) k_round_g1_out(const g1j* sp, uint32_t K, 
 
 // Both folds of round j with one limb per lane (limb_ec.cuh): blocks [0, n) fold a point of v each, the
 // remaining blocks two points of A (96 threads each) and their entries of b, n = K h points t = (k, i).
-// Latency-bound up to about one block per SM: 0.25 ms for 1 to 64 points, 0.31 ms for 128, 0.79 for 512,
-// 2.8 for 2048, 5.5 for 4096 (one GB300).  A warp per G2 point and 8 lanes per G1 point took 1.21 ms for
-// 512 points and 6.1 for 4096; one thread per point (k_fold) takes 4.5 ms for 8192, which is where the
-// default limit leaves off.  It replaces comb tables of the round's bases formed beside the pairings
-// (0.16 ms for 64 points after the challenge, but 0.96 ms of chains and tables per round before it).
+// Latency-bound up to about one block per SM: 0.155 ms for 1 to 64 points and 0.19 for 128 from tables of the
+// bases' shifts formed beside the round's pairings (k_fold_pre, 0.13 ms), 0.25 and 0.31 without them; 0.79 ms
+// for 512 points, 2.8 for 2048, 5.5 for 4096 (one GB300).  A warp per G2 point and 8 lanes per G1 point took
+// 1.21 ms for 512 points and 6.1 for 4096; one thread per point (k_fold) takes 4.5 ms for 8192, which is where
+// the default limit leaves off.  Full comb tables of the bases (0.16 ms for 64 points after the challenge)
+// took 0.96 ms of chains and tables per round beside the pairings.
 union FoldSmemW {
     LimbEc2 g2;
     LimbEc g1[2];
 };
+// PRE: from the tables of the points' shifts (fold_pre_bytes, by k_fold_pre)
+template <bool PRE>
 __global__ void __launch_bounds__(LEC2_THREADS) k_fold_w(g1a* A, g2a* v, fr* bvec, const fr* x_mont,
-                                                         const fr* xinv_mont, uint32_t K, uint32_t R, uint32_t h) {
+                                                         const fr* xinv_mont, uint32_t K, uint32_t R, uint32_t h,
+                                                         const int32_t* pre) {
     __shared__ FoldSmemW sm;
     const uint64_t n = (uint64_t)K * h;
     uint32_t kw[8];
@@ -143,7 +147,8 @@ __global__ void __launch_bounds__(LEC2_THREADS) k_fold_w(g1a* A, g2a* v, fr* bve
         const uint64_t lo = k * R + (uint32_t)(t % h), hi = lo + h;
         fr_canon_words(kw, xinv_mont[k]);
         const Lec2Lane c = lec2_lane();
-        lec2_g2_mul(sm.g2, c, v[hi], kw);
+        if (PRE) lec2_g2_mul_pre(sm.g2, c, pre + n * LEC_PRE_INTS + t * LEC2_PRE_INTS, kw);
+        else lec2_g2_mul(sm.g2, c, v[hi], kw);
         lec2_add_affine(sm.g2, c, v[lo]);
         const fq r = lec2_affine(sm.g2, c);
         if (c.k.l == 0 && c.slot < 4) reinterpret_cast<fq*>(&v[lo])[c.slot] = r;
@@ -156,12 +161,30 @@ __global__ void __launch_bounds__(LEC2_THREADS) k_fold_w(g1a* A, g2a* v, fr* bve
     const uint64_t lo = k * R + (uint32_t)(t % h), hi = lo + h;
     fr_canon_words(kw, x_mont[k]);
     const LecLane c = lec_lane();
-    lec_g1_mul(sm.g1[half], c, A[hi], kw);
+    if (PRE) lec_g1_mul_pre(sm.g1[half], c, pre + t * LEC_PRE_INTS, kw);
+    else lec_g1_mul(sm.g1[half], c, A[hi], kw);
     lec_add_affine(sm.g1[half], c, A[lo]);
     const fq r = lec_affine(sm.g1[half], c);
     if (c.k.l == 0 && c.slot < 2) reinterpret_cast<fq*>(&A[lo])[c.slot] = r;
     if (c.k.l == 0 && c.slot == 2) bvec[lo] = fr_add(bvec[lo], fr_mul(bvec[hi], xinv_mont[k]));
 }
+// The fold's bases A[h + i], v[h + i] are known a round before its challenge: their tables of shifts
+// (lec_pre, lec2_pre) are formed beside the round's pairings, for rounds of few points
+__global__ void __launch_bounds__(LEC2_THREADS) k_fold_pre(const g1a* A, const g2a* v, uint32_t K, uint32_t R,
+                                                           uint32_t h, int32_t* pre) {
+    __shared__ FoldSmemW sm;
+    const uint64_t n = (uint64_t)K * h;
+    if (blockIdx.x < n) {
+        const uint64_t t = blockIdx.x;
+        lec2_pre(sm.g2, lec2_lane(), v[t / h * R + h + (uint32_t)(t % h)], pre + n * LEC_PRE_INTS + t * LEC2_PRE_INTS);
+        return;
+    }
+    const int half = (int)(threadIdx.x / LEC_THREADS);
+    const uint64_t t = (blockIdx.x - n) * 2 + half;
+    if (t >= n) return;
+    lec_pre(sm.g1[half], lec_lane(), A[t / h * R + h + (uint32_t)(t % h)], pre + t * LEC_PRE_INTS);
+}
+size_t fold_pre_bytes(uint32_t n) { return (size_t)n * (LEC_PRE_INTS + LEC2_PRE_INTS) * sizeof(int32_t); }
 
 // L_j.1 and R_j.1 terms at the support of b only, one block per term (limb_ec.cuh), for the blocks
 // k0 .. k0 + K - 1 (local index k - k0).  Block k's vector b is
@@ -470,12 +493,22 @@ uint64_t step1_miller_g(const void* A, const void* v, uint32_t K, uint32_t R, ui
     round_miller_w(A, v, K, R, h, ml_out, s);      // few pairs: one warp or block each, for latency
     return n;
 }
+void step1_fold_pre(const void* A, const void* v, uint32_t K, uint32_t R, uint32_t h, void* pre, cudaStream_t s) {
+    const uint32_t n = K * h;
+    FP_KERNEL("k_fold_pre", s, k_fold_pre<<<n + (n + 1) / 2, LEC2_THREADS, 0, s>>>((const g1a*)A, (const g2a*)v, K, R, h,
+                                                                                  (int32_t*)pre));
+}
 void step1_fold(void* A, void* v, void* bvec, const void* x_mont, const void* xinv_mont, uint32_t K, uint32_t R,
-                uint32_t h, cudaStream_t s) {
+                uint32_t h, const void* pre, cudaStream_t s) {
     const uint64_t n = (uint64_t)K * h;
-    if (n <= engine_limits().fold_warp_max) {          // few points: a block per G2 point, half a block per G1
-        FP_KERNEL("k_fold_w", s, k_fold_w<<<(unsigned)(n + (n + 1) / 2), LEC2_THREADS, 0, s>>>(
-                                     (g1a*)A, (g2a*)v, (fr*)bvec, (const fr*)x_mont, (const fr*)xinv_mont, K, R, h));
+    if (pre || n <= engine_limits().fold_warp_max) {   // few points: a block per G2 point, half a block per G1
+        const unsigned nb = (unsigned)(n + (n + 1) / 2);
+        if (pre)
+            FP_KERNEL("k_fold_w", s, k_fold_w<true><<<nb, LEC2_THREADS, 0, s>>>((g1a*)A, (g2a*)v, (fr*)bvec,
+                                         (const fr*)x_mont, (const fr*)xinv_mont, K, R, h, (const int32_t*)pre));
+        else
+            FP_KERNEL("k_fold_w", s, k_fold_w<false><<<nb, LEC2_THREADS, 0, s>>>((g1a*)A, (g2a*)v, (fr*)bvec,
+                                         (const fr*)x_mont, (const fr*)xinv_mont, K, R, h, nullptr));
         return;
     }
     uint32_t nb = grid_for((uint64_t)K * h, 64);

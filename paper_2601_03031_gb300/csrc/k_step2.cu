@@ -85,8 +85,10 @@ FPG_DEV void mul_limb(LimbEc& S, const g1a& P, const fr& k_mont, g1j* out) {
     if (c.k.l == 0 && c.slot < 3) reinterpret_cast<fq*>(out)[c.slot] = v;
 }
 // the same, half a block per row.  Few rows are one scalar multiplication's latency: 0.22 ms, on one thread
-// each 2.8 ms (256 rows).  Up to STEP2_LIMB_MAX multiplications the limb lanes also finish before the
-// threads' latency; beyond, the threads do less work in total.
+// each 2.8 ms (256 rows).  Up to STEP2_LIMB_MAX multiplications the limb lanes are quicker
+// and Step 2 can bound the call; beyond, Step 1's rounds bound it and the threads take less issue from them
+// (1024 quotient terms at N = 2^16: 0.67 ms on limb lanes, but round 2's Miller loops 0.33 -> 0.67 ms beside
+// them; 2.6 ms on threads).
 __global__ void __launch_bounds__(2 * LEC_THREADS) k_d0_l(const g1a* rows, const fr* rj, uint32_t R, g1j* D) {
     __shared__ LimbEc sm[2];
     const int half = (int)(threadIdx.x / LEC_THREADS);
@@ -94,7 +96,7 @@ __global__ void __launch_bounds__(2 * LEC_THREADS) k_d0_l(const g1a* rows, const
     if (j >= R) return;                                       // three whole warps, with a barrier of their own
     mul_limb(sm[half], rows[j], rj[j], &D[j]);
 }
-constexpr uint64_t STEP2_LIMB_MAX = 8 * 152;
+constexpr uint64_t STEP2_LIMB_MAX = 4 * 152;
 
 // Sub-protocol: g_w = g_wl + g_wr for every node at level h (all nodes kept)
 __global__ void k_fold_g(fr* g, uint32_t R, uint32_t M, int h) {

@@ -109,8 +109,13 @@ void step1_g1_out(const void* sp_g1j, uint32_t K, int j, void* blocks, size_t bo
 void step1_gt_out(const void* ml_fq12, uint32_t K, int j, void* blocks, size_t bopen_len, cudaStream_t s);
 // Round j's folds: at most fold_warp_max points on the limb lanes (a block per G2 point, half a block per
 // G1 point), more on one thread per point.
+// For rounds of at most FOLD_PRE_MAX points, step1_fold_pre forms tables of the bases' shifts in `pre`
+// (fold_pre_bytes(K h)) before the challenge and step1_fold uses them (pre = nullptr: none).
+constexpr uint32_t FOLD_PRE_MAX = 152;
+size_t fold_pre_bytes(uint32_t n);
+void step1_fold_pre(const void* A, const void* v, uint32_t K, uint32_t R, uint32_t h, void* pre, cudaStream_t s);
 void step1_fold(void* A, void* v, void* bvec, const void* x_mont, const void* xinv_mont, uint32_t K, uint32_t R,
-                uint32_t h, cudaStream_t s);
+                uint32_t h, const void* pre, cudaStream_t s);
 // Look-ahead rounds (lookahead.cuh): round j's record from round j-1's state (half-length h = 2 h2)
 // and challenge.  Before the challenge: la_miller (the 8 K h2 Miller values by class; then pairwise
 // products to 8 K and their final exponentiations, fe), la_sparse (the 6 K (4 h2) G1 terms; then

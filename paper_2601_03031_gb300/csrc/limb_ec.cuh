@@ -32,6 +32,8 @@ struct LimbEc {
     alignas(16) int32_t zero[LIMB_WIN], one[LIMB_WIN], back[LIMB_WIN], omega[LIMB_WIN];
     fq x[2];
     signed char d[2][LEC_DIGITS];
+    int nops;
+    unsigned char ops[192];
 };
 
 // Barrier of a multiplication's 96 threads: a block may hold several, each on three whole warps.
@@ -147,10 +149,10 @@ FPG_DEV void lec_naf(signed char* d, const uint32_t* k) {
     }
 }
 
-// S.acc <- k P for a canonical k < r (8 words) and an affine P (Montgomery residues, (0, 0) the identity)
-FPG_DEV void lec_g1_mul(LimbEc& S, const LecLane& c, const g1a& P, const uint32_t* kw) {
+// constant windows and an affine P (Montgomery residues, (0, 0) the identity) into the accumulator and the
+// table's first entry
+FPG_DEV void lec_enter(LimbEc& S, const LecLane& c, const g1a& P) {
     const int l = c.k.l, s = c.slot;
-    for (int i = lec_thread(); i < 2 * LEC_DIGITS; i += LEC_THREADS) (&S.d[0][0])[i] = 0;
     if (s == 0) limb_put_window(S.zero, l, 0);
     if (s == 1) limb_put_window(S.one, l, LIMB_FROB2[0][l]);
     if (s == 2) limb_put_window(S.back, l, LIMB_CONV[1][l]);
@@ -159,27 +161,34 @@ FPG_DEV void lec_g1_mul(LimbEc& S, const LecLane& c, const g1a& P, const uint32_
     if (s < 2) limb_put_window(S.acc[s], l, LIMB_CONV[0][l]);
     limb_put(S.t[s], l, s < 2 ? limb_of_words(s == 0 ? P.x.v : P.y.v, l) : 0);
     lec_sync();
-    if (l == 0 && (s == 0 || s == 2)) {            // one lane of warps 0 and 1
-        uint32_t k1[5], k0[4];
-        div_by_const<4, 5>(k1, k0, kw, GLV_D, GLV_BARRETT);
-        lec_naf(S.d[s >> 1], s ? k1 : k0);
-    }
-    __syncwarp();
     const bool inf = g1a_is_inf(P);
-    {
-        int32_t v = lec_mul1(S, c, S.t[s], S.acc[s < 2 ? s : 0]);
-        const int32_t one = LIMB_FROB2[0][l];
-        if (s == 1 && inf) v = one;                // the identity is (0 : 1 : 0)
-        lec_sync();                           // reads of S.acc are over
-        if (s == 2) v = inf ? 0 : one;
-        if (s < 3) {
-            limb_put_window(S.acc[s], l, v);
-            limb_put_window(S.tab[0][s == 2 ? 3 : s], l, v);
-            if (s == 1) limb_put_window(S.tab[0][2], l, -v);
-        }
+    int32_t v = lec_mul1(S, c, S.t[s], S.acc[s < 2 ? s : 0]);
+    const int32_t one = LIMB_FROB2[0][l];
+    if (s == 1 && inf) v = one;                    // the identity is (0 : 1 : 0)
+    lec_sync();                                    // reads of S.acc are over
+    if (s == 2) v = inf ? 0 : one;
+    if (s < 3) {
+        limb_put_window(S.acc[s], l, v);
+        limb_put_window(S.tab[0][s == 2 ? 3 : s], l, v);
+        if (s == 1) limb_put_window(S.tab[0][2], l, -v);
     }
     lec_sync();
-    // step 0: 2P; steps 1 .. 3: 3P = 2P + P, 5P = 3P + 2P, 7P = 5P + 2P
+}
+// the digits of the GLV halves of a canonical k < r (8 words) into S.d (visible after the next barrier)
+FPG_DEV void lec_digits(LimbEc& S, const LecLane& c, const uint32_t* kw) {
+    for (int i = lec_thread(); i < 2 * LEC_DIGITS; i += LEC_THREADS) (&S.d[0][0])[i] = 0;
+    lec_sync();
+    if (c.k.l == 0 && (c.slot == 0 || c.slot == 2)) {   // one lane of warps 0 and 1
+        uint32_t k1[5], k0[4];
+        div_by_const<4, 5>(k1, k0, kw, GLV_D, GLV_BARRETT);
+        lec_naf(S.d[c.slot >> 1], c.slot ? k1 : k0);
+    }
+    __syncwarp();
+}
+// from P in the accumulator and the table's first entry: 2P in S.two, 3P = 2P + P, 5P = 3P + 2P,
+// 7P = 5P + 2P in the table, and omega X of the four entries
+FPG_DEV void lec_table(LimbEc& S, const LecLane& c) {
+    const int l = c.k.l, s = c.slot;
     lec_step<true>(S, c, S.acc[0], S.acc[1], S.acc[2]);
     if (s < 3) limb_put_window(S.two[s], l, S.acc[s][l]);
     lec_sync();
@@ -193,13 +202,21 @@ FPG_DEV void lec_g1_mul(LimbEc& S, const LecLane& c, const g1a& P, const uint32_
         }
         lec_sync();
     }
-    {
-        const int e = s < 4 ? s : 0;
-        const int32_t v = lec_mul1(S, c, S.tab[e][0], S.omega);
-        if (s < 4) limb_put_window(S.phix[s], l, v);
-        if (s < 3) limb_put_window(S.acc[s], l, s == 1 ? LIMB_FROB2[0][l] : 0);
-    }
+    const int32_t v = lec_mul1(S, c, S.tab[s < 4 ? s : 0][0], S.omega);
+    if (s < 4) limb_put_window(S.phix[s], l, v);
     lec_sync();
+}
+FPG_DEV void lec_set_identity(LimbEc& S, const LecLane& c) {
+    if (c.slot < 3) limb_put_window(S.acc[c.slot], c.k.l, c.slot == 1 ? LIMB_FROB2[0][c.k.l] : 0);
+    lec_sync();
+}
+
+// S.acc <- k P for a canonical k < r (8 words) and an affine P
+FPG_DEV void lec_g1_mul(LimbEc& S, const LecLane& c, const g1a& P, const uint32_t* kw) {
+    lec_digits(S, c, kw);
+    lec_enter(S, c, P);
+    lec_table(S, c);
+    lec_set_identity(S, c);
     int i = LEC_DIGITS - 1;
     while (i >= 0 && !S.d[0][i] && !S.d[1][i]) i--;
     for (bool first = true; i >= 0; i--) {
@@ -212,6 +229,83 @@ FPG_DEV void lec_g1_mul(LimbEc& S, const LecLane& c, const g1a& P, const uint32_
             // the half k1 multiplies -phi(P) = (omega x, -y)
             lec_step<false>(S, c, h ? S.phix[e] : S.tab[e][0], S.tab[e][(d < 0) != (h == 1) ? 2 : 1], S.tab[e][3]);
         }
+    }
+}
+
+// ---- Bases known before their scalar: the chain of doublings is cut into LEC_CUTS pieces.  The tables of
+// 2^(CH i) P, i < 4, are formed ahead (lec_pre, lec2_pre: limbs in global memory), and k P is then one
+// chain of CH doublings in which every piece's digits are added: ~83 (G1, CH = 32) or ~68 operations (G2,
+// CH = 16) instead of ~182 and ~121.  The order of operations is listed first, so that the next table
+// entry's limbs are loaded while an operation runs.
+constexpr int LEC_CUTS = 4, LEC_CH = 32, LEC2_CH = 16;
+constexpr int LEC_PRE_INTS = LEC_CUTS * 4 * 4 * LIMB_ROW;        // (cut, entry, X Y Z omega-X)
+constexpr int LEC2_PRE_INTS = LEC_CUTS * 16 * 6 * LIMB_ROW;      // (cut, 4 h + entry, X Y Z parts)
+
+// operations in order: 0 a doubling, else 0x80 | sign 0x40 | (cut, half or digit string h, entry); at most
+// one digit in any four of a string is nonzero, so there are at most 2 33 + 36 (G1), 4 17 + 20 (G2).  One lane.
+template <int NH, int CH, int LIM>
+FPG_DEV int lec_list(unsigned char* ops, const signed char (*d)[LEC_DIGITS]) {
+    int n = 0;
+    for (int pos = LIM - 1 - 3 * CH; pos >= 0; pos--) {
+        if (n) ops[n++] = 0;
+#pragma unroll
+        for (int q = 0; q < LEC_CUTS * NH; q++) {
+            const int cut = q / NH, h = q % NH;
+            if (pos >= CH && cut < LEC_CUTS - 1) continue;
+            const int v = d[h][CH * cut + pos];
+            if (v) ops[n++] = (unsigned char)(0x80 | (v < 0 ? 0x40 : 0) | (cut << 4) | (h << 2) | ((v < 0 ? -v : v) >> 1));
+        }
+    }
+    return n;
+}
+
+FPG_DEV void lec_pre(LimbEc& S, const LecLane& c, const g1a& P, int32_t* T) {
+    const int l = c.k.l, s = c.slot;
+    lec_enter(S, c, P);
+    for (int cut = 0; cut < LEC_CUTS; cut++) {
+        lec_table(S, c);
+        if (s < 4)
+            for (int e = 0; e < 4; e++) {
+                const int32_t* w = s == 3 ? S.phix[e] : S.tab[e][s == 2 ? 3 : s];
+                T[((cut * 4 + e) * 4 + s) * LIMB_ROW + l] = l < LIMB_N ? w[l] : 0;
+            }
+        if (cut == LEC_CUTS - 1) break;
+        if (s < 3) limb_put_window(S.acc[s], l, S.two[s][l]);
+        lec_sync();
+        for (int i = 1; i < LEC_CH; i++) lec_step<true>(S, c, S.acc[0], S.acc[1], S.acc[2]);
+        if (s < 3) {
+            const int32_t v = S.acc[s][l];
+            limb_put_window(S.tab[0][s == 2 ? 3 : s], l, v);
+            if (s == 1) limb_put_window(S.tab[0][2], l, -v);
+        }
+        lec_sync();
+    }
+}
+// S.acc <- k P from lec_pre's tables of P
+FPG_DEV void lec_g1_mul_pre(LimbEc& S, const LecLane& c, const int32_t* T, const uint32_t* kw) {
+    const int l = c.k.l, s = c.slot;
+    if (s == 5) limb_put_window(S.zero, l, 0);
+    if (s == 4) limb_put_window(S.back, l, LIMB_CONV[1][l]);
+    lec_digits(S, c, kw);
+    lec_sync();
+    if (lec_thread() == 0) S.nops = lec_list<2, LEC_CH, LEC_DIGITS>(S.ops, S.d);
+    lec_set_identity(S, c);
+    auto limb = [&](int op) -> int32_t {           // slot s < 3's coordinate of the entry
+        const int h = (op >> 2) & 1, row = ((op >> 4) & 3) * 16 + (op & 3) * 4 + (s == 0 && h ? 3 : s < 3 ? s : 0);
+        const int32_t v = T[row * LIMB_ROW + l];
+        return s == 1 && (((op & 0x40) != 0) != (h == 1)) ? -v : v;
+    };
+    const int n = S.nops;
+    int32_t next = n && S.ops[0] ? limb(S.ops[0]) : 0;
+    for (int i = 0; i < n; i++) {
+        const int op = S.ops[i], nx = i + 1 < n ? S.ops[i + 1] : 0;
+        if (op) {
+            if (s < 3) limb_put_window(S.two[s], l, next);
+            lec_sync();
+        }
+        if (nx) next = limb(nx);
+        if (op) lec_step<false>(S, c, S.two[0], S.two[1], S.two[2]);
+        else lec_step<true>(S, c, S.acc[0], S.acc[1], S.acc[2]);
     }
 }
 
@@ -311,6 +405,8 @@ struct LimbEc2 {
     alignas(16) int32_t cst[12][2 * LIMB_WIN + 16];   // slots' constant windows
     fq x[6];
     signed char d[4][LEC_DIGITS];
+    int nops;
+    unsigned char ops[192];
 };
 
 FPG_DEV const int32_t* lec2_win(const int32_t* pair, int e) { return pair + (e ? LIMB_WIN + 16 : 0); }
@@ -464,10 +560,9 @@ FPG_DEV int32_t lec2_load(LimbEc2& S, const Lec2Lane& c, const fq& w) {
 // the component of an affine point that slot s loads
 FPG_DEV const fq& lec2_comp(const g2a& P, int s) { return s == 0 ? P.x.c0 : s == 1 ? P.x.c1 : s == 2 ? P.y.c0 : P.y.c1; }
 
-// S.acc <- k P for a canonical k < r (8 words) and an affine P (Montgomery residues, (0, 0) the identity)
-FPG_DEV void lec2_g2_mul(LimbEc2& S, const Lec2Lane& c, const g2a& P, const uint32_t* kw) {
+// an affine P into the accumulator and the table's first entry
+FPG_DEV void lec2_enter(LimbEc2& S, const Lec2Lane& c, const g2a& P) {
     const int l = c.k.l, s = c.slot;
-    for (int i = (int)threadIdx.x; i < 4 * LEC_DIGITS; i += LEC2_THREADS) (&S.d[0][0])[i] = 0;
     const bool inf = g2a_is_inf(P);
     const int32_t one = LIMB_FROB2[0][l];
     int32_t v = lec2_load(S, c, lec2_comp(P, s));
@@ -479,8 +574,14 @@ FPG_DEV void lec2_g2_mul(LimbEc2& S, const Lec2Lane& c, const g2a& P, const uint
         limb_put_window(lec2_win(S.tab[0][i == 2 ? 3 : i], c.e), l, v);
         if (i == 1) limb_put_window(lec2_win(S.tab[0][2], c.e), l, -v);
     }
-    __syncthreads();                               // d is zero
-    if (l == 0 && c.e == 0 && s < 8) {             // one lane of warps 0 .. 3
+    __syncthreads();
+}
+// the digits of the four GLS parts of a canonical k < r (visible after the next barrier)
+FPG_DEV void lec2_digits(LimbEc2& S, const Lec2Lane& c, const uint32_t* kw) {
+    const int s = c.slot;
+    for (int i = (int)threadIdx.x; i < 4 * LEC_DIGITS; i += LEC2_THREADS) (&S.d[0][0])[i] = 0;
+    __syncthreads();
+    if (c.k.l == 0 && c.e == 0 && s < 8) {         // one lane of warps 0 .. 3
         uint32_t dg[4][2], w[4] = {0, 0, 0, 0};
         gls_digits(dg, kw);
         const int h = s >> 1;
@@ -489,7 +590,11 @@ FPG_DEV void lec2_g2_mul(LimbEc2& S, const Lec2Lane& c, const g2a& P, const uint
         lec_naf(S.d[h], w);
     }
     __syncwarp();
-    // 2P, then 3P = 2P + P, 5P = 3P + 2P, 7P = 5P + 2P
+}
+// from P in the accumulator and the table's first entry: 2P in S.two, 3P, 5P, 7P, and the four entries'
+// images B_{i + 1} = -psi(B_i)
+FPG_DEV void lec2_table(LimbEc2& S, const Lec2Lane& c) {
+    const int l = c.k.l, s = c.slot;
     lec2_step<true>(S, c, S.win[0], S.win[1], S.win[2]);
     if (s < 6) limb_put_window(lec2_win(S.two[s >> 1], c.e), l, S.acc[s >> 1][c.e][l]);
     __syncthreads();
@@ -504,38 +609,46 @@ FPG_DEV void lec2_g2_mul(LimbEc2& S, const Lec2Lane& c, const g2a& P, const uint
         }
         __syncthreads();
     }
-    // B_{i + 1} = -psi(B_i): (cx conj(X) : -cy conj(Y) : conj(Z)); conj(a) g: a0 g0 + a1 g1, a0 g1 - a1 g0.
+    // -psi: (cx conj(X) : -cy conj(Y) : conj(Z)); conj(a) g: a0 g0 + a1 g1, a0 g1 - a1 g0.
     // Warp w: entry w / 2 of a pass's three, X or Y by w % 2
-    {
-        const int w = s >> 1, xy = w & 1;
-        const int32_t g0 = LIMB_PSI[2 * xy][l], g1 = LIMB_PSI[2 * xy + 1][l];
-        int32_t* cw = S.cst[s];
-        limb_put_window(cw, l, c.e ? g1 : g0);
-        limb_put_window(cw + LIMB_WIN, l, c.e ? -g0 : g1);
-        __syncwarp();
-        for (int i = 0; i < 3; i++) {
-            for (int pass = 0; pass < 2; pass++) {
-                const int m = 3 * pass + (w >> 1), mm = m < 4 ? m : 0;
-                const int32_t(*src)[LEC2_PAIR] = S.tab[4 * i + mm];
-                const int32_t *row[2] = {lec2_win(src[xy], 0), lec2_win(src[xy], 1)}, *win[2] = {cw, cw + LIMB_WIN};
-                int64_t lo, hi;
-                limb_dot<2>(c.k, lo, hi, row, win);
-                const int32_t x = limb_carry(limb_reduce(c.k, lo, hi, S.u[s]), l);
-                if (m < 4) {
-                    int32_t(*dst)[LEC2_PAIR] = S.tab[4 * i + 4 + m];
-                    limb_put_window(lec2_win(dst[xy], c.e), l, xy ? -x : x);
-                    if (xy) limb_put_window(lec2_win(dst[2], c.e), l, x);
-                    else {
-                        const int32_t z = lec2_win(src[3], c.e)[l];
-                        limb_put_window(lec2_win(dst[3], c.e), l, c.e ? -z : z);
-                    }
+    const int w = s >> 1, xy = w & 1;
+    const int32_t g0 = LIMB_PSI[2 * xy][l], g1 = LIMB_PSI[2 * xy + 1][l];
+    int32_t* cw = S.cst[s];
+    limb_put_window(cw, l, c.e ? g1 : g0);
+    limb_put_window(cw + LIMB_WIN, l, c.e ? -g0 : g1);
+    __syncwarp();
+    for (int i = 0; i < 3; i++) {
+        for (int pass = 0; pass < 2; pass++) {
+            const int m = 3 * pass + (w >> 1), mm = m < 4 ? m : 0;
+            const int32_t(*src)[LEC2_PAIR] = S.tab[4 * i + mm];
+            const int32_t *row[2] = {lec2_win(src[xy], 0), lec2_win(src[xy], 1)}, *win[2] = {cw, cw + LIMB_WIN};
+            int64_t lo, hi;
+            limb_dot<2>(c.k, lo, hi, row, win);
+            const int32_t x = limb_carry(limb_reduce(c.k, lo, hi, S.u[s]), l);
+            if (m < 4) {
+                int32_t(*dst)[LEC2_PAIR] = S.tab[4 * i + 4 + m];
+                limb_put_window(lec2_win(dst[xy], c.e), l, xy ? -x : x);
+                if (xy) limb_put_window(lec2_win(dst[2], c.e), l, x);
+                else {
+                    const int32_t z = lec2_win(src[3], c.e)[l];
+                    limb_put_window(lec2_win(dst[3], c.e), l, c.e ? -z : z);
                 }
             }
-            __syncthreads();
         }
+        __syncthreads();
     }
-    if (s < 6) lec2_put_acc(S, s >> 1, c.e, l, s == 2 ? one : 0);
+}
+FPG_DEV void lec2_set_identity(LimbEc2& S, const Lec2Lane& c) {
+    if (c.slot < 6) lec2_put_acc(S, c.slot >> 1, c.e, c.k.l, c.slot == 2 ? LIMB_FROB2[0][c.k.l] : 0);
     __syncthreads();
+}
+
+// S.acc <- k P for a canonical k < r (8 words) and an affine P (Montgomery residues, (0, 0) the identity)
+FPG_DEV void lec2_g2_mul(LimbEc2& S, const Lec2Lane& c, const g2a& P, const uint32_t* kw) {
+    lec2_digits(S, c, kw);
+    lec2_enter(S, c, P);
+    lec2_table(S, c);
+    lec2_set_identity(S, c);
     int i = LEC_DIGITS - 1;
     while (i >= 0 && !S.d[0][i] && !S.d[1][i] && !S.d[2][i] && !S.d[3][i]) i--;
     for (bool first = true; i >= 0; i--) {
@@ -547,6 +660,55 @@ FPG_DEV void lec2_g2_mul(LimbEc2& S, const Lec2Lane& c, const g2a& P, const uint
             const int32_t(*t)[LEC2_PAIR] = S.tab[4 * h + ((d < 0 ? -d : d) >> 1)];
             lec2_step<false>(S, c, t[0], t[d < 0 ? 2 : 1], t[3]);
         }
+    }
+}
+
+// tables of 2^(16 i) P, i < 4 (see lec_pre)
+FPG_DEV void lec2_pre(LimbEc2& S, const Lec2Lane& c, const g2a& P, int32_t* T) {
+    const int l = c.k.l, s = c.slot;
+    lec2_enter(S, c, P);
+    for (int cut = 0; cut < LEC_CUTS; cut++) {
+        lec2_table(S, c);
+        if (s < 6)
+            for (int e = 0; e < 16; e++) {
+                const int i = s >> 1;
+                T[((cut * 16 + e) * 6 + s) * LIMB_ROW + l] = l < LIMB_N ? lec2_win(S.tab[e][i == 2 ? 3 : i], c.e)[l] : 0;
+            }
+        if (cut == LEC_CUTS - 1) break;
+        if (s < 6) lec2_put_acc(S, s >> 1, c.e, l, lec2_win(S.two[s >> 1], c.e)[l]);
+        __syncthreads();
+        for (int i = 1; i < LEC2_CH; i++) lec2_step<true>(S, c, S.win[0], S.win[1], S.win[2]);
+        if (s < 6) {
+            const int i = s >> 1;
+            const int32_t v = S.acc[i][c.e][l];
+            limb_put_window(lec2_win(S.tab[0][i == 2 ? 3 : i], c.e), l, v);
+            if (i == 1) limb_put_window(lec2_win(S.tab[0][2], c.e), l, -v);
+        }
+        __syncthreads();
+    }
+}
+// S.acc <- k P from lec2_pre's tables of P
+FPG_DEV void lec2_g2_mul_pre(LimbEc2& S, const Lec2Lane& c, const int32_t* T, const uint32_t* kw) {
+    const int l = c.k.l, s = c.slot;
+    lec2_digits(S, c, kw);
+    __syncthreads();
+    if (threadIdx.x == 0) S.nops = lec_list<4, LEC2_CH, 68>(S.ops, S.d);
+    lec2_set_identity(S, c);
+    auto limb = [&](int op) -> int32_t {           // slot s < 6's part of the entry
+        const int32_t v = T[((((op >> 4) & 3) * 16 + (op & 15)) * 6 + (s < 6 ? s : 0)) * LIMB_ROW + l];
+        return (s >> 1) == 1 && (op & 0x40) ? -v : v;
+    };
+    const int n = S.nops;
+    int32_t next = n && S.ops[0] ? limb(S.ops[0]) : 0;
+    for (int i = 0; i < n; i++) {
+        const int op = S.ops[i], nx = i + 1 < n ? S.ops[i + 1] : 0;
+        if (op) {
+            if (s < 6) limb_put_window(lec2_win(S.two[s >> 1], c.e), l, next);
+            __syncthreads();
+        }
+        if (nx) next = limb(nx);
+        if (op) lec2_step<false>(S, c, S.two[0], S.two[1], S.two[2]);
+        else lec2_step<true>(S, c, S.win[0], S.win[1], S.win[2]);
     }
 }
 

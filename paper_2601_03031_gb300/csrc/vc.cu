@@ -148,14 +148,14 @@ constexpr uint64_t TREE_REDUCE_MAX = 8192;
 
 size_t bopen_len(uint32_t log_r) { return (size_t)log_r * ROUND_BYTES + G1_SER + 2 * G2_SER; }
 
-// Internal non-blocking streams: OpenAll's latency-bound Step 1 runs on two high-priority
-// streams (the round chain, and beside it the sparse G1 terms), the
+// Internal non-blocking streams: OpenAll's latency-bound Step 1 runs on three high-priority
+// streams (the round chain, and beside it the sparse G1 terms and the fold bases' tables), the
 // throughput-bound Step 2 on a low-priority stream; all are forked from and joined back to the caller's stream with events
 // created per call.  Each caller stream (per device) gets its own set, so calls on different caller
 // streams run concurrently; past 256 caller streams the sets are shared (still correct, less
 // concurrent).
 struct Streams {
-    cudaStream_t hi = nullptr, sp = nullptr, la[2] = {nullptr, nullptr}, fold = nullptr, lo = nullptr;
+    cudaStream_t hi = nullptr, sp = nullptr, pre = nullptr, la[2] = {nullptr, nullptr}, fold = nullptr, lo = nullptr;
     cudaStream_t tail = nullptr;   // Commit's pairings of the row commitments (high priority)
 };
 struct StreamKey { int dev; cudaStream_t user; Streams set; };
@@ -167,6 +167,7 @@ Streams make_set() {
     check(cudaDeviceGetStreamPriorityRange(&lo, &hi), "priority range");
     check(cudaStreamCreateWithPriority(&a.hi, cudaStreamNonBlocking, hi), "cudaStreamCreate");
     check(cudaStreamCreateWithPriority(&a.sp, cudaStreamNonBlocking, hi), "cudaStreamCreate");
+    check(cudaStreamCreateWithPriority(&a.pre, cudaStreamNonBlocking, hi), "cudaStreamCreate");
     check(cudaStreamCreateWithPriority(&a.la[0], cudaStreamNonBlocking, hi), "cudaStreamCreate");
     check(cudaStreamCreateWithPriority(&a.la[1], cudaStreamNonBlocking, hi), "cudaStreamCreate");
     check(cudaStreamCreateWithPriority(&a.fold, cudaStreamNonBlocking, hi), "cudaStreamCreate");
@@ -502,6 +503,8 @@ namespace {
 // outputs, the challenges and the fast-verification proof of v_l
 struct Step1Bufs {
     void *A, *v, *bvec, *xprev, *x_mont, *xinv_mont, *xinv_all, *ml, *ml2, *sp, *sp2, *pcoef, *q;
+    void* pre = nullptr;                 // the bases' tables of rounds with few fold points (step1_fold_pre)
+    uint32_t pre_n = 0;                  // points they hold
     void *wt = nullptr, *wt2 = nullptr, *wscr = nullptr;
     MsmShape wsh{};
     bool w_msm = false;
@@ -524,6 +527,9 @@ Step1Bufs step1_bufs(const fp_pp* pp, uint32_t Kc, Alloc&& T) {
     B.sp2 = T((KR / 2 + 1) * G1J_BYTES);
     B.pcoef = T((size_t)Kc * (2 * R - 1) * FR_BYTES);
     B.q = T((size_t)Kc * 2 * R * FR_BYTES);
+    B.pre_n = (uint32_t)std::min<uint64_t>(FOLD_PRE_MAX, KR / 2);
+    B.pre_n -= B.pre_n % Kc;             // a round folds Kc h points
+    if (B.pre_n) B.pre = T(fold_pre_bytes(B.pre_n));
     // W proofs: one batched G2 MSM over the shared bases g2^{beta^i} when many blocks share them,
     // else one scalar multiplication per term and pairwise sums (with few batches the MSM's bucket
     // reduction runs nearly serially per window)
@@ -569,16 +575,23 @@ LaBufs la_bufs(const fp_pp* pp, uint32_t Kc, Alloc&& T) {
 
 // FC.BOpen rounds (Sec. 3, Eq. folding) and the fast-verification proof of v_l for the Kc blocks
 // k0 .. k0 + Kc - 1 of size b, whose combined vectors are in B.bvec (their support is the block):
-// the round chain on s1, each round's G1 parts on s3 (joined before the challenge); the records go to
+// the round chain on s1, each round's G1 parts on s3 (joined before the challenge) and, in rounds with few
+// points, the tables of the fold's bases on s4 (joined before the fold); the records go to
 // blocks1 (stride blen).  s3 must already be ordered after whatever filled B.bvec.
 void step1_rounds(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, const Step1Bufs& B, uint8_t* blocks1,
-                  size_t blen, cudaStream_t s1, cudaStream_t s3) {
+                  size_t blen, cudaStream_t s1, cudaStream_t s3, cudaStream_t s4) {
     const uint32_t R = pp->R;
     const int lr = (int)pp->log_r;
-    cudaEvent_t ev_folded = new_event(), ev_sparse = new_event();
+    cudaEvent_t ev_folded = new_event(), ev_sparse = new_event(), ev_pre = new_event();
     for (int j = 1; j <= lr; j++) {
         const uint32_t h = R >> j;
         check(cudaEventRecord(ev_folded, s1), "event");
+        const bool pre = (uint64_t)Kc * h <= std::min(B.pre_n, engine_limits().fold_warp_max);
+        if (pre) {
+            check(cudaStreamWaitEvent(s4, ev_folded, 0), "wait");
+            step1_fold_pre(B.A, B.v, Kc, R, h, B.pre, s4);
+            check(cudaEventRecord(ev_pre, s4), "event");
+        }
         check(cudaStreamWaitEvent(s3, ev_folded, 0), "wait");
         step1_sparse_terms(B.A, B.bvec, k0, Kc, R, h, b, B.sp, s3);
         void* spr = (uint64_t)Kc * 2 * h <= TREE_REDUCE_MAX
@@ -591,7 +604,8 @@ void step1_rounds(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, const S
         step1_gt_out(mlr, Kc, j, blocks1, blen, s1);
         check(cudaStreamWaitEvent(s1, ev_sparse, 0), "wait");
         step1_challenge(blocks1, blen, Kc, j, B.xprev, B.x_mont, B.xinv_mont, B.xinv_all, lr, s1);
-        step1_fold(B.A, B.v, B.bvec, B.x_mont, B.xinv_mont, Kc, R, h, s1);
+        if (pre) check(cudaStreamWaitEvent(s1, ev_pre, 0), "wait");
+        step1_fold(B.A, B.v, B.bvec, B.x_mont, B.xinv_mont, Kc, R, h, pre ? B.pre : nullptr, s1);
     }
     step1_kzg(B.A, B.v, B.xprev, B.xinv_all, Kc, R, lr, blocks1, blen, B.pcoef, B.q, s1);
     uint8_t* w_out = blocks1 + (size_t)lr * ROUND_BYTES + G1_SER + G2_SER;
@@ -607,6 +621,7 @@ void step1_rounds(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, const S
     }
     cudaEventDestroy(ev_folded);
     cudaEventDestroy(ev_sparse);
+    cudaEventDestroy(ev_pre);
 }
 
 // The rounds with look-ahead (lookahead.cuh): round 1 as in step1_rounds; for j >= 2 round j's record
@@ -659,7 +674,7 @@ void step1_rounds_la(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, cons
         const uint32_t h = R >> j;
         wait(sF, ev_x[j]);
         if (j + 1 <= lr) wait(sF, ev_snap[j + 1]);
-        step1_fold(B.A, B.v, B.bvec, xm(j), xim(j), Kc, R, h, sF);
+        step1_fold(B.A, B.v, B.bvec, xm(j), xim(j), Kc, R, h, nullptr, sF);
         ev_S[j + 1] = rec(sF);
     };
     cudaEvent_t ev_a = rec(s1), ev_b = rec(s3);     // S_1: A, v (s1) and b (s3)
@@ -816,7 +831,7 @@ fp_proofs* prove_impl(const fp_pp* pp, const fp_commit* cm, uint32_t b, uint32_t
             step1_stmt_hash(cm->C_ser, cm->rows_ser, k0, Kc, R, b, hscr, hstmt, s3);
             step1_block_r(hstmt, k0, Kc, R, b, B.bvec, s3);
             if (la) step1_rounds_la(pp, k0, Kc, b, B, L, blocks1, blen, s1, s3, st.la, st.fold);
-            else step1_rounds(pp, k0, Kc, b, B, blocks1, blen, s1, s3);
+            else step1_rounds(pp, k0, Kc, b, B, blocks1, blen, s1, s3, st.pre);
             check(cudaEventRecord(ev_join1, s1), "event");
             check(cudaStreamWaitEvent(s, ev_join1, 0), "join");
             cudaEventDestroy(ev_init);
@@ -1171,7 +1186,7 @@ fp_status vc_eval_prove(const fp_pp* pp, const fp_commit* cm, const uint8_t* r, 
             check(cudaEventRecord(ev_bvec, s1), "event");
             check(cudaStreamWaitEvent(s3, ev_bvec, 0), "wait");
             if (la) step1_rounds_la(pp, 0, 1, R, B, L, proof + 128, blen, s1, s3, st.la, st.fold);
-            else step1_rounds(pp, 0, 1, R, B, proof + 128, blen, s1, s3);
+            else step1_rounds(pp, 0, 1, R, B, proof + 128, blen, s1, s3, st.pre);
             check(cudaStreamWaitEvent(s1, ev_pst, 0), "wait");
             check_launch("vc_eval_prove kernels");
             check(cudaMemcpyAsync(out, proof, need, cudaMemcpyDeviceToHost, s1), "D2H proof");

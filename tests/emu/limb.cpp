@@ -84,7 +84,7 @@ void emu_limb_g1_mul(const uint8_t* p, const uint32_t* k, uint8_t* out) {
     fq_to_be(out + 48, a.y);
 }
 // k P + Q on G2 (192 bytes each)
-void emu_limb_g2_mul_add(const uint8_t* p, const uint32_t* k, const uint8_t* q, uint8_t* out) {
+void emu_limb_g2_mul_add(int pre, const uint8_t* p, const uint32_t* k, const uint8_t* q, uint8_t* out) {
     auto pt = [](const uint8_t* b) {
         g2a P;
         P.x.c0 = be_fq(b); P.x.c1 = be_fq(b + 48); P.y.c0 = be_fq(b + 96); P.y.c1 = be_fq(b + 144);
@@ -93,19 +93,33 @@ void emu_limb_g2_mul_add(const uint8_t* p, const uint32_t* k, const uint8_t* q, 
     const g2a P = pt(p), Q = pt(q);
     lanes(LEC2_THREADS, [&] {
         const Lec2Lane c = lec2_lane();
-        lec2_g2_mul(g_ec2, c, P, k);
+        if (pre) {
+            static int32_t T[LEC2_PRE_INTS];
+            lec2_pre(g_ec2, c, P, T);
+            __syncthreads();
+            lec2_g2_mul_pre(g_ec2, c, T, k);
+        } else {
+            lec2_g2_mul(g_ec2, c, P, k);
+        }
         lec2_add_affine(g_ec2, c, Q);
         const fq v = lec2_affine(g_ec2, c);
         if (c.k.l == 0 && c.slot < 4) fq_to_be(out + 48 * c.slot, v);
     });
 }
 // k P + Q on G1, affine
-void emu_limb_g1_mul_add(const uint8_t* p, const uint32_t* k, const uint8_t* q, uint8_t* out) {
+void emu_limb_g1_mul_add(int pre, const uint8_t* p, const uint32_t* k, const uint8_t* q, uint8_t* out) {
     g1a P, Q;
     P.x = be_fq(p); P.y = be_fq(p + 48); Q.x = be_fq(q); Q.y = be_fq(q + 48);
     lanes(LEC_THREADS, [&] {
         const LecLane c = lec_lane();
-        lec_g1_mul(g_ec, c, P, k);
+        if (pre) {
+            static int32_t T[LEC_PRE_INTS];
+            lec_pre(g_ec, c, P, T);
+            __syncthreads();
+            lec_g1_mul_pre(g_ec, c, T, k);
+        } else {
+            lec_g1_mul(g_ec, c, P, k);
+        }
         lec_add_affine(g_ec, c, Q);
         const fq v = lec_affine(g_ec, c);
         if (c.k.l == 0 && c.slot < 2) fq_to_be(out + 48 * c.slot, v);

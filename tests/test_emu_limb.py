@@ -72,8 +72,9 @@ def test_g1_scalar_mul_against_oracle(emu):
             assert out.raw == O.g1_mul(pt, k % r), hex(k)
 
 
-def test_g2_scalar_mul_and_add_against_oracle(emu):
-    """k P + Q for edge and random k, with P = Q, P = -Q sums and identities among them."""
+@pytest.mark.parametrize("pre", [0, 1])
+def test_g2_scalar_mul_and_add_against_oracle(emu, pre):
+    """k P + Q, directly and from tables of P's shifts, for edge and random k, with P = Q, P = -Q sums and identities among them."""
     rnd = random.Random(6)
     r, x = ref.R, 0xD201000000010000
     P = O.g2_mul(O.g2_gen(), 777)
@@ -83,18 +84,21 @@ def test_g2_scalar_mul_and_add_against_oracle(emu):
              (P, x**3 + x**2 - 1, Q)] + [(P, rnd.randrange(r), Q) for _ in range(2)]
     out = ctypes.create_string_buffer(192)
     for p, k, q in cases:
-        emu.emu_limb_g2_mul_add(p, (ctypes.c_uint32 * 8)(*[(k >> (32 * i)) & 0xFFFFFFFF for i in range(8)]), q, out)
+        emu.emu_limb_g2_mul_add(pre, p, (ctypes.c_uint32 * 8)(*[(k >> (32 * i)) & 0xFFFFFFFF for i in range(8)]), q, out)
         assert out.raw == O.g2_add(O.g2_mul(p, k), q), hex(k)
 
 
-def test_g1_scalar_mul_and_add_against_oracle(emu):
+@pytest.mark.parametrize("pre", [0, 1])
+def test_g1_scalar_mul_and_add_against_oracle(emu, pre):
     rnd = random.Random(7)
     r = ref.R
     P, Q, inf = O.g1_mul(O.g1_gen(), 777), O.g1_mul(O.g1_gen(), 4242), bytes(96)
-    cases = [(P, 0, Q), (P, 1, P), (P, r - 1, P), (P, 8, inf), (inf, 5, Q), (inf, 3, inf), (P, rnd.randrange(r), Q)]
+    x2 = 0xD201000000010000 ** 2
+    cases = [(P, 0, Q), (P, 1, P), (P, r - 1, P), (P, 8, inf), (inf, 5, Q), (inf, 3, inf), (P, x2 - 1, Q),
+             (P, (1 << 96) - 1, Q), (P, rnd.randrange(r), Q)]
     out = ctypes.create_string_buffer(96)
     for p, k, q in cases:
-        emu.emu_limb_g1_mul_add(p, (ctypes.c_uint32 * 8)(*[(k >> (32 * i)) & 0xFFFFFFFF for i in range(8)]), q, out)
+        emu.emu_limb_g1_mul_add(pre, p, (ctypes.c_uint32 * 8)(*[(k >> (32 * i)) & 0xFFFFFFFF for i in range(8)]), q, out)
         assert out.raw == O.g1_add(O.g1_mul(p, k), q), hex(k)
 
 
