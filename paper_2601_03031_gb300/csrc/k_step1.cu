@@ -209,27 +209,22 @@ __global__ void __launch_bounds__(LEC_THREADS) k_sparse_g(const g1a* A, const fr
     if (c.k.l == 0 && c.slot < 3) reinterpret_cast<fq*>(&out[k * 2 * h + p])[c.slot] = v;
 }
 
-// the same with the two SHA-256 halves of HFr on two lanes of a warp per block (they are
-// independent); lane 0 finishes (a zero challenge falls back to the serial re-hash)
+// x_j = HFr("FP-x", x_{j-1} || L_j || R_j) and its inverse, one warp per block: the hash on the warp
+// (hfr_wide_warp), the inverse on a quad (a zero challenge falls back to the serial re-hash): 0.052 ms (0.077
+// with the hash's halves on two lanes)
+constexpr uint32_t CHAL_MSG = (5 + 32 + ROUND_BYTES + 9 + 63) / 64 * 64;
 __global__ void __launch_bounds__(64) k_challenge2(const uint8_t* blocks, size_t bopen_len, uint32_t K, int j,
                                                    uint8_t* xprev, fr* x_mont, fr* xinv_mont, fr* xinv_all,
                                                    int log_r) {
+    __shared__ __align__(16) uint8_t msg[2][CHAL_MSG];
+    __shared__ uint32_t wk[2][64 * 32];
     __shared__ uint8_t wide[2][64];
     const int w = threadIdx.x >> 5, L = threadIdx.x & 31;
     const uint64_t k = (uint64_t)blockIdx.x * 2 + w;
     if (k >= K) return;                                       // warp-uniform
     const uint8_t* rec = blocks + k * bopen_len + (size_t)(j - 1) * ROUND_BYTES;
     uint8_t* xp = xprev + k * 32;
-    if (L < 2) {
-        sha256_ctx c;
-        sha256_init(c);
-        sha256_update(c, (const uint8_t*)"FP-x", 4);
-        sha256_byte(c, (uint8_t)L);
-        if (j > 1) sha256_update(c, xp, 32);
-        sha256_update(c, rec, ROUND_BYTES);
-        sha256_final(c, wide[w] + 32 * L);
-    }
-    __syncwarp();
+    hfr_wide_warp(msg[w], wk[w], wide[w], "FP-x", j > 1 ? xp : nullptr, rec, ROUND_BYTES);
     if (L < 4) {                                              // the inverse on the quad of lanes 0 .. 3
         fr x = fr_from_be64(wide[w]);
         if (fr_is_zero(x)) x = hash_to_fr_nonzero("FP-x", 4, xp, j > 1 ? 32 : 0, rec, ROUND_BYTES, nullptr, 0);
@@ -433,37 +428,81 @@ void g2_comb_tables(const void* pts_g2a, uint32_t n, void* chain_scratch, void* 
                                       (uint64_t)n * 64, (const GPt<fq2>*)chain_scratch, (GPt<fq2>*)tab));
 }
 
-// W terms q_i g2^{beta^i} from the comb tables: one 128-thread block per term (k, i < 2R), 16 8-lane
-// groups on G2 (group_ec.cuh with F = Fq2) each adding the entries of positions g, g + 16, g + 32,
-// g + 48 of the GLS digits of q_i, then a tree over the groups; term 2R - 1 is the identity
-__global__ void __launch_bounds__(128) k_w_comb(const GPt<fq2>* tab, const fr* q_canon, uint32_t R, g2j* out) {
-    __shared__ GEcs<fq2> e[16];
-    __shared__ GPt<fq2> part[16];
-    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
+// W = sum_i q_i g2^{beta^i} from the comb tables, one limb per lane (limb_ec.cuh): a block per term (k, i < 2R)
+// adds the entries of its 64 positions in a row, the next entry's limbs loaded while an addition runs; then
+// blocks of up to 16 terms each, the last with the conversion to affine.  A point is kept as the limbs of
+// its homogeneous coordinates (residues' limbs as they are: a common factor leaves the point the same).
+// The term 2R - 1 and zero factors are the identity.
+// 2R = 512 terms: 8-lane groups, their trees and the conversion took 0.25 + 0.21 + 0.055 ms in five launches.
+struct WPart { int32_t c[6][LIMB_ROW]; };
+FPG_DEV void w_put(LimbEc2& S, const Lec2Lane& c, int32_t v, bool first) {   // slot s < 6's coordinate part
+    if (c.slot < 6) {
+        if (first) lec2_put_acc(S, c.slot >> 1, c.e, c.k.l, v);
+        else limb_put_window(lec2_win(S.two[c.slot >> 1], c.e), c.k.l, v);
+    }
+    __syncthreads();
+}
+__global__ void __launch_bounds__(LEC2_THREADS) k_w_comb(const GPt<fq2>* tab, const fr* q_canon, uint32_t R, WPart* out) {
+    __shared__ LimbEc2 S;
+    __shared__ unsigned char dg[64];
+    const Lec2Lane c = lec2_lane();
+    const int l = c.k.l, s = c.slot;
     const uint64_t t = blockIdx.x;
     const uint32_t i = (uint32_t)(t % (2 * R));
-    const bool live = i < 2 * R - 1;
-    uint32_t d[4][2];
-    gls_digits(d, q_canon[t].v);
-    const GPt<fq2>* tb = tab + (size_t)(live ? i : 0) * 64 * 16;
-    const GPt<fq2> id = gec_identity<fq2>();
-    GPt<fq2> acc = live ? tb[grp * 16 + gls_position(d, grp)] : id;
-    for (int j = 1; j < 4; j++) {
-        const int pos = grp + 16 * j;
-        acc = gec_add(e[grp], lane, acc, live ? tb[pos * 16 + gls_position(d, pos)] : id);
+    if (threadIdx.x < 64) {
+        uint32_t d[4][2];
+        gls_digits(d, q_canon[t].v);
+        dg[threadIdx.x] = i < 2 * R - 1 ? (unsigned char)gls_position(d, (int)threadIdx.x) : 0;
     }
-    for (int sh = 8; sh >= 1; sh >>= 1) {
-        __syncthreads();
-        if (lane == 0) part[grp] = acc;
-        __syncthreads();
-        const GPt<fq2> r = gec_add(e[grp], lane, acc, part[grp < sh ? grp + sh : grp]);
-        if (grp < sh) acc = r;
+    lec2_set_identity(S, c);                                  // (and the digits are visible)
+    const GPt<fq2>* tb = tab + (size_t)(i < 2 * R - 1 ? i : 0) * 64 * 16;
+    auto limb = [&](int pos) -> int32_t {
+        return limb_of_words(reinterpret_cast<const fq*>(&tb[pos * 16 + dg[pos]])[s < 6 ? s : 0].v, l);
+    };
+    int pos = 0;
+    while (pos < 64 && !dg[pos]) pos++;
+    int32_t next = pos < 64 ? limb(pos) : 0;
+    for (bool first = true; pos < 64; first = false) {
+        w_put(S, c, next, first);
+        do pos++;
+        while (pos < 64 && !dg[pos]);
+        if (pos < 64) next = limb(pos);
+        if (!first) lec2_step<false>(S, c, S.two[0], S.two[1], S.two[2]);
     }
-    if (grp == 0 && lane == 0) out[t] = proj_to_jac(acc);
+    if (s < 6) out[t].c[s][l] = l < LIMB_N ? S.acc[s >> 1][c.e][l] : 0;
 }
-void step1_w_comb(const void* tab, const void* q_canon, uint32_t K, uint32_t R, void* out, cudaStream_t s) {
-    FP_KERNEL("k_w_comb", s, k_w_comb<<<(unsigned)((uint64_t)K * 2 * R), 128, 0, s>>>((const GPt<fq2>*)tab,
-                                                                                    (const fr*)q_canon, R, (g2j*)out));
+// out[b] = sum of in[gs b .. gs b + gs); with ser the affine sum's serialisation at ser + b stride instead
+__global__ void __launch_bounds__(LEC2_THREADS) k_w_sum(const WPart* in, uint32_t gs, WPart* out, uint8_t* ser,
+                                                        size_t stride) {
+    __shared__ LimbEc2 S;
+    const Lec2Lane c = lec2_lane();
+    const int l = c.k.l, s = c.slot, co = s < 6 ? s : 0;
+    const WPart* p = in + blockIdx.x * (uint64_t)gs;
+    int32_t next = p[0].c[co][l];
+    for (uint32_t u = 0; u < gs; u++) {
+        w_put(S, c, next, u == 0);
+        if (u + 1 < gs) next = p[u + 1].c[co][l];
+        if (u) lec2_step<false>(S, c, S.two[0], S.two[1], S.two[2]);
+    }
+    if (ser) {
+        const fq v = lec2_affine(S, c);
+        if (l == 0 && s < 4) fq_to_be(ser + blockIdx.x * stride + 48 * s, v);
+    } else if (s < 6) {
+        out[blockIdx.x].c[s][l] = S.acc[s >> 1][c.e][l];
+    }
+}
+size_t w_comb_bytes(uint32_t K, uint32_t R) { return (size_t)K * 2 * R * sizeof(WPart); }
+void step1_w_comb(const void* tab, const void* q_canon, uint32_t K, uint32_t R, void* buf, void* buf2, void* ser,
+                  size_t stride, cudaStream_t s) {
+    uint64_t n = (uint64_t)K * 2 * R;
+    WPart *a = (WPart*)buf, *b = (WPart*)buf2;
+    FP_KERNEL("k_w_comb", s, k_w_comb<<<(unsigned)n, LEC2_THREADS, 0, s>>>((const GPt<fq2>*)tab, (const fr*)q_canon, R, a));
+    while (n > K) {
+        const uint32_t gs = (uint32_t)std::min<uint64_t>(16, n / K);
+        n /= gs;
+        FP_KERNEL("k_w_sum", s, k_w_sum<<<(unsigned)n, LEC2_THREADS, 0, s>>>(a, gs, b, n == K ? (uint8_t*)ser : nullptr, stride));
+        std::swap(a, b);
+    }
 }
 
 void step1_w_terms(const void* g2pow, const void* q_canon, uint32_t K, uint32_t R, void* out, cudaStream_t s) {

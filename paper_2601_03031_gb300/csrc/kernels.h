@@ -136,7 +136,10 @@ void step1_kzg(const void* A, const void* v, const void* xprev, const void* xinv
                int log_r, void* blocks, size_t bopen_len, void* pcoef, void* q_canon, cudaStream_t s);
 void step1_w_terms(const void* g2pow, const void* q_canon, uint32_t K, uint32_t R, void* out_g2j, cudaStream_t s);
 // the same terms from the comb tables of g2pow (g2_comb_tables): one table entry per position
-void step1_w_comb(const void* tab, const void* q_canon, uint32_t K, uint32_t R, void* out_g2j, cudaStream_t s);
+// the whole sums, serialised at ser + k stride, through two buffers of w_comb_bytes
+size_t w_comb_bytes(uint32_t K, uint32_t R);
+void step1_w_comb(const void* tab, const void* q_canon, uint32_t K, uint32_t R, void* buf, void* buf2, void* ser,
+                  size_t stride, cudaStream_t s);
 // comb tables of n fixed G2 points (64 positions x 16 entries each, g2_comb_bytes(n) bytes), through
 // a scratch of n 64 projective points
 constexpr uint32_t G2_COMB_MAX_R = 1024;        // setups with R <= this keep the W proofs' comb tables

@@ -143,6 +143,21 @@ void* reduce_tree(void* a, void* b, uint64_t n, uint64_t target, uint32_t gmax, 
     }
     return a;
 }
+// products of consecutive Fq12 values down to `target`: by eights, one block each, once few are left
+void* reduce_fq12(void* a, void* b, uint64_t n, uint64_t target, cudaStream_t s) {
+    while (n > target) {
+        uint32_t gs = 2;
+        if (n <= 4096) {
+            gs = (uint32_t)std::min<uint64_t>(8, n / target);
+            fq12_products(nullptr, a, gs, gs, b, 1, n / gs, s);
+        } else {
+            fq12_pair_reduce(a, b, n / 2, s);
+        }
+        std::swap(a, b);
+        n /= gs;
+    }
+    return a;
+}
 // sums of few points (one block per sum is enough to fill the GPU's share the round leaves free)
 constexpr uint64_t TREE_REDUCE_MAX = 8192;
 
@@ -383,7 +398,7 @@ fp_commit* commit_enqueue(const fp_pp* pp, const uint64_t* m, int on_device, cud
         cudaStream_t st = streams(s).tail;
         check(cudaStreamWaitEvent(st, cm->rows_done, 0), "wait");
         commit_miller(cm->rows, pp->g2pow, R, ml, st);
-        void* prod = reduce_pairs(ml, ml2, R, 1, fq12_pair_reduce, st);
+        void* prod = reduce_fq12(ml, ml2, R, 1, st);
         final_exp_group(prod, 1, cm->C, cm->C_ser, 1, GT_SER, 0, st);
         check_launch("vc_commit kernels");
         dfree(src, s); dfree(t1, s); dfree(t2, s); dfree(ml, st); dfree(ml2, st);
@@ -537,6 +552,9 @@ Step1Bufs step1_bufs(const fp_pp* pp, uint32_t Kc, Alloc&& T) {
     if (B.w_msm) {
         B.wsh = msm_shape(2 * R, Kc, 2 * R, fp_msm_window_g2(2 * R, Kc), 4, 65);
         B.wscr = T(msm_scratch_bytes_g2(B.wsh));
+    } else if (pp->g2comb) {
+        B.wt = T(w_comb_bytes(Kc, R));
+        B.wt2 = T(w_comb_bytes(Kc, R));
     } else {
         B.wt = T((size_t)Kc * 2 * R * G2J_BYTES);
         B.wt2 = T(((size_t)Kc * R + 1) * G2J_BYTES);
@@ -600,7 +618,7 @@ void step1_rounds(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, const S
         step1_g1_out(spr, Kc, j, blocks1, blen, s3);
         check(cudaEventRecord(ev_sparse, s3), "event");
         const uint64_t nml = step1_miller_g(B.A, B.v, Kc, R, h, B.ml, s1);
-        void* mlr = reduce_pairs(B.ml, B.ml2, nml, (uint64_t)Kc * 2, fq12_pair_reduce, s1);
+        void* mlr = reduce_fq12(B.ml, B.ml2, nml, (uint64_t)Kc * 2, s1);
         step1_gt_out(mlr, Kc, j, blocks1, blen, s1);
         check(cudaStreamWaitEvent(s1, ev_sparse, 0), "wait");
         step1_challenge(blocks1, blen, Kc, j, B.xprev, B.x_mont, B.xinv_mont, B.xinv_all, lr, s1);
@@ -611,9 +629,10 @@ void step1_rounds(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, const S
     uint8_t* w_out = blocks1 + (size_t)lr * ROUND_BYTES + G1_SER + G2_SER;
     if (B.w_msm) {
         msm_g2(pp->g2w_tab, B.q, B.wsh, B.wscr, nullptr, w_out, blen, s1);
+    } else if (pp->g2comb) {
+        step1_w_comb(pp->g2comb, B.q, Kc, R, B.wt, B.wt2, w_out, blen, s1);
     } else {
-        if (pp->g2comb) step1_w_comb(pp->g2comb, B.q, Kc, R, B.wt, s1);
-        else step1_w_terms(pp->g2pow, B.q, Kc, R, B.wt, s1);
+        step1_w_terms(pp->g2pow, B.q, Kc, R, B.wt, s1);
         void* wr = (uint64_t)Kc * 2 * R <= TREE_REDUCE_MAX
                        ? reduce_tree(B.wt, B.wt2, (uint64_t)Kc * 2 * R, Kc, 16, g2_tree_reduce, s1)
                        : reduce_pairs(B.wt, B.wt2, (uint64_t)Kc * 2 * R, Kc, g2_pair_reduce, s1);
@@ -692,7 +711,7 @@ void step1_rounds_la(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, cons
         step1_g1_out(spr, Kc, 1, blocks1, blen, s3);
         cudaEvent_t ev_sp = rec(s3);
         const uint64_t nml = step1_miller_g(B.A, B.v, Kc, R, h, B.ml, s1);
-        void* mlr = reduce_pairs(B.ml, B.ml2, nml, (uint64_t)Kc * 2, fq12_pair_reduce, s1);
+        void* mlr = reduce_fq12(B.ml, B.ml2, nml, (uint64_t)Kc * 2, s1);
         step1_gt_out(mlr, Kc, 1, blocks1, blen, s1);
         wait(s1, ev_sp);
         step1_challenge(blocks1, blen, Kc, 1, B.xprev, xm(1), xim(1), B.xinv_all, lr, s1);
@@ -716,9 +735,10 @@ void step1_rounds_la(const fp_pp* pp, uint32_t k0, uint32_t Kc, uint32_t b, cons
     uint8_t* w_out = blocks1 + (size_t)lr * ROUND_BYTES + G1_SER + G2_SER;
     if (B.w_msm) {
         msm_g2(pp->g2w_tab, B.q, B.wsh, B.wscr, nullptr, w_out, blen, s1);
+    } else if (pp->g2comb) {
+        step1_w_comb(pp->g2comb, B.q, Kc, R, B.wt, B.wt2, w_out, blen, s1);
     } else {
-        if (pp->g2comb) step1_w_comb(pp->g2comb, B.q, Kc, R, B.wt, s1);
-        else step1_w_terms(pp->g2pow, B.q, Kc, R, B.wt, s1);
+        step1_w_terms(pp->g2pow, B.q, Kc, R, B.wt, s1);
         void* wr = (uint64_t)Kc * 2 * R <= TREE_REDUCE_MAX
                        ? reduce_tree(B.wt, B.wt2, (uint64_t)Kc * 2 * R, Kc, 16, g2_tree_reduce, s1)
                        : reduce_pairs(B.wt, B.wt2, (uint64_t)Kc * 2 * R, Kc, g2_pair_reduce, s1);

@@ -193,30 +193,20 @@ __global__ void k_v_cdec(const uint8_t* C_be, fq12* Cd, uint32_t* cbad) {
 }
 
 // x_j and x_j^-1, A_l, v_l, W, z and P(z) = prod_j (1 + x_j^-1 z^(2^(l - j + 1))), one warp per block: the
-// two SHA-256 halves of HFr on two lanes (the chain of the x_j is serial), then the inverses on one lane
-// each and the three points' checks beside each other: 0.55 ms at l = 8.  (On one thread, with the
+// hashes on the warp (hfr_wide_warp; the chain of the x_j is serial), then the inverses on one lane
+// each and the three points' checks beside each other: 0.34 ms at l = 8.  (On one thread, with the
 // statement's tree, 1.1 ms; the tree is k_stmt_hash's now.)
 __global__ void __launch_bounds__(32) k_vb_transcript(VSrc S, VBlk* st) {
+    __shared__ __align__(16) uint8_t msg[(5 + 32 + ROUND_BYTES + 9 + 63) / 64 * 64];
+    __shared__ uint32_t wk[64 * 32];
     __shared__ uint8_t wide[64], xp[32];
     const uint64_t q = blockIdx.x;
     const int L = threadIdx.x, lr = S.lr;
     VBlk& B = st[q];
     const uint8_t* fc = S.fc + q * S.fc_stride;
-    auto absorb = [&](const char* tag, bool with_x, const uint8_t* d, uint32_t n) {
-        if (L < 2) {
-            sha256_ctx c;
-            sha256_init(c);
-            sha256_update(c, (const uint8_t*)tag, 4);
-            sha256_byte(c, (uint8_t)L);
-            if (with_x) sha256_update(c, xp, 32);
-            sha256_update(c, d, n);
-            sha256_final(c, wide + 32 * L);
-        }
-        __syncwarp();
-    };
     for (int j = 1; j <= lr; j++) {
         const uint8_t* rd = fc + (size_t)(j - 1) * ROUND_BYTES;
-        absorb("FP-x", j > 1, rd, ROUND_BYTES);
+        hfr_wide_warp(msg, wk, wide, "FP-x", j > 1 ? xp : nullptr, rd, ROUND_BYTES);
         if (L == 0) {
             fr x = fr_from_be64(wide);
             if (fr_is_zero(x)) x = hash_to_fr_nonzero("FP-x", 4, xp, j > 1 ? 32 : 0, rd, ROUND_BYTES, nullptr, 0);
@@ -226,7 +216,7 @@ __global__ void __launch_bounds__(32) k_vb_transcript(VSrc S, VBlk* st) {
         __syncwarp();
     }
     const uint8_t* tail = fc + (size_t)lr * ROUND_BYTES;
-    absorb("FP-z", true, tail + G1_SER, G2_SER);
+    hfr_wide_warp(msg, wk, wide, "FP-z", xp, tail + G1_SER, G2_SER);
     if (L < lr) B.xinv[L] = fr_inv(B.x[L]);
     bool ok = true;
     if (L == 0) ok = g1_decode(tail, B.Al);
