@@ -38,7 +38,8 @@ FQ_MULS = {
     "g2_mul": 3300,          # GLS: 64 doublings + ~60 mixed additions over Fq2, 15-point table
     "msm_madd": 10,          # XYZZ mixed addition (8M + 2S), one per bucket entry
     # one pair of a 4-pair multi-Miller loop: the 62 Fq12 squarings (36 Fq products each) are shared
-    # by the 4 pairs, so a pair costs 7135 - 3/4 x 62 x 36
+    # by the 4 pairs, so a pair costs 7135 - 3/4 x 62 x 36 (pairs by two, 7135 - 1/2 x 62 x 36, are
+    # counted the same: an undercount of their work)
     "miller_loop_multi4": 7135 - 3 * 62 * 36 // 4,
     "g2_msm_madd": 30,       # XYZZ mixed addition over Fq2 (8M + 2S), 3 Fq products per Fq2 product
     # comb folds of a point of A and of v (k_step1.cu): 64 table entries and the L half added with
@@ -120,6 +121,19 @@ NCU_TRAFFIC = {
 }
 
 
+MILLER_WAVE = 152 * 256       # threads of the thread-per-pair Miller kernels that run at once
+
+
+def miller_group(n: int, h: int, group_min: int) -> int:
+    """Pairs per thread of a thread-engine launch of n Miller loops, as the library chooses them."""
+    if h >= 4 and n >= group_min:
+        return 4
+    if n < group_min // 4:
+        return 1
+    return min((g for g in (1, 2, 4) if g <= h),
+               key=lambda g: -(-(n // g) // MILLER_WAVE) * {1: 126, 2: 214, 4: 383}[g])
+
+
 def step_units(log_n: int, b: int, msm_window: int, msm_window_g2: int = 16, lim: dict | None = None) -> dict:
     """Per kernel: (unit, units processed per step) for one Commit + OpenAll step.  `lim` is the
     library's engine-choice limits (fp_get_engine_limits: the launch sizes at which a kernel moves
@@ -147,7 +161,7 @@ def step_units(log_n: int, b: int, msm_window: int, msm_window_g2: int = 16, lim
     for h in hs:
         n = K * 2 * h
         e = engine(n, mb, mw)
-        miller["t4" if e == "t" and h >= 4 and n >= mg else e] += n
+        miller["t4" if e == "t" and miller_group(n, h, mg) > 1 else e] += n
     fe = {"c": 0, "w": 0, "t": 0}
     fe[engine(1, lim["fe_block_max"], lim["fe_warp_max"])] += 1                  # Commit's one
     fe[engine(2 * K, lim["fe_block_max"], lim["fe_warp_max"])] += 2 * K * lr     # two per block and round

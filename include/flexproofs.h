@@ -323,7 +323,8 @@ typedef enum { FP_SCHEDULE_DIRECT = 0, FP_SCHEDULE_LOOKAHEAD = 1 } fp_schedule;
  *                                        (profiled as k_round_miller_c up to block_max, as
  *                                        k_round_miller_w above), else a thread each (1024 / 16383)
  *   miller_group_min                     from this many (and h >= 4), a thread runs 4 pairs of one
- *                                        product with shared squarings (default 2^18)
+ *                                        product with shared squarings (default 2^18); from a
+ *                                        quarter of it 1, 2 or 4, whichever fills whole waves best
  *   commit_block_max / commit_warp_max   Commit's R Miller loops, the same way (default 1024 / 16384)
  *   fe_block_max / fe_warp_max           final exponentiations: block / warp / thread (256 / 2^32-1;
  *                                        unless block_max is 0, blocks also up to 912)

@@ -223,19 +223,39 @@ void commit_miller(const void* rows, const void* g2pow, uint32_t R, void* out, c
     FP_KERNEL(R <= lim.commit_block_max ? "k_commit_miller_c" : "k_commit_miller_w", s,
               k_commit_miller_c<<<R, LM_THREADS, 0, s>>>((const g1a*)rows, (const g2a*)g2pow, (fq12*)out));
 }
-// grouping pays once the grouped threads still fill the GPU several times over (2^16 threads)
+// Pairs per thread of a launch of n pairs.  These kernels hold 255 registers a thread, so the GPU takes
+// 152 x 256 threads at once and a launch costs whole waves: measured per wave 12.6 ms with one pair per
+// thread, 21.4 with two sharing the squarings, 38.3 with four.  From miller_group_min on four (fewer
+// products; 2^18 pairs 77 ms against 88).  Down to a quarter of it the fewest ms by waves: 2^17 pairs
+// one wave of four, 38.3 ms against 42.5 (two waves of two) and 47.7 (four of one); 2^16 pairs one wave of
+// two, 21.4 against 25.2 and 27.9; 87552 pairs 36 ms each way.  2^15 pairs and fewer fit one wave as
+// they are (12.7 ms; pairs of them 15.4).  Eight per thread gained 6 ms at 2^18 pairs, lost 5 at 2^20 and
+// doubled the local memory.
+constexpr uint64_t MILLER_WAVE = 152 * 256;
 uint32_t step1_miller_group(uint64_t n, uint32_t h, const EngineLimits& lim) {
-    return (h >= 4 && n >= lim.miller_group_min) ? 4 : 1;
+    if (h >= 4 && n >= lim.miller_group_min) return 4;
+    uint32_t best = 1;
+    if (n < lim.miller_group_min / 4) return best;
+    const uint32_t wave_ms10[3] = {126, 214, 383};
+    uint64_t best_ms = ~0ull;
+    for (uint32_t i = 0; i < 3 && (1u << i) <= h; i++) {
+        const uint64_t ms = ((n >> i) + MILLER_WAVE - 1) / MILLER_WAVE * wave_ms10[i];
+        if (ms < best_ms) { best_ms = ms; best = 1u << i; }
+    }
+    return best;
+}
+template <int G>
+static void launch_miller_multi(const void* A, const void* v, uint32_t K, uint32_t R, uint32_t h, void* out,
+                                cudaStream_t s) {
+    const uint64_t n = (uint64_t)K * 2 * (h / G);
+    FP_KERNEL("k_step1_miller_multi", s,
+              k_step1_miller_multi<G><<<grid_for(n, 64), 64, 0, s>>>((const g1a*)A, (const g2a*)v, K, R, h,
+                                                                    (fq12*)out));
 }
 void step1_miller(const void* A, const void* v, uint32_t K, uint32_t R, uint32_t h, uint32_t group, void* out,
                   cudaStream_t s) {
-    if (group == 4) {                                   // 4 pairs per thread share the squarings
-        const uint64_t n = (uint64_t)K * 2 * (h / 4);
-        FP_KERNEL("k_step1_miller_multi", s,
-                  k_step1_miller_multi<4><<<grid_for(n, 64), 64, 0, s>>>((const g1a*)A, (const g2a*)v, K, R, h,
-                                                                        (fq12*)out));
-        return;
-    }
+    if (group == 4) return launch_miller_multi<4>(A, v, K, R, h, out, s);   // pairs sharing the squarings
+    if (group == 2) return launch_miller_multi<2>(A, v, K, R, h, out, s);
     uint64_t n = (uint64_t)K * 2 * h;
     FP_KERNEL("k_step1_miller", s, k_step1_miller<<<grid_for(n, 64), 64, 0, s>>>((const g1a*)A, (const g2a*)v, K, R, h, (fq12*)out));
 }

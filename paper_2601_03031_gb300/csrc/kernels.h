@@ -27,7 +27,8 @@ void prof_end(cudaStream_t s);
 struct EngineLimits {
     uint32_t miller_block_max = 1024;       // Step-1 Miller loops per launch: <= this, a block each
     uint32_t miller_warp_max = 16383;       //   <= this, a block each too; above, a thread each
-    uint32_t miller_group_min = 1u << 18;   //   from this many (h >= 4), 4 pairs of a product per thread
+    uint32_t miller_group_min = 1u << 18;   //   from this many (h >= 4), 4 pairs of a product per thread;
+                                            //   from a quarter of it 1, 2 or 4 by full waves
     uint32_t commit_block_max = 1024;       // Commit's Miller loops: <= this, a block each
     uint32_t commit_warp_max = 16384;       //   <= this, a block each too; above, a thread each
     uint32_t fe_block_max = 256;            // final exponentiations per launch: <= this, a block each

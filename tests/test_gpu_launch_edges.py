@@ -1,0 +1,45 @@
+"""Launch rules that depend on the number of pairs, fold points or buckets, at the sizes where they change:
+the bytes equal those of the thread-per-item kernels (held to the oracle by the engine tests) or, for
+the MSM, the oracle's."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+import oracle as O  # noqa: E402
+from paper_2601_03031_gb300 import _lib as F  # noqa: E402
+from paper_2601_03031_gb300 import inputs as I  # noqa: E402
+
+BIG = 0xFFFFFFFF
+
+
+@pytest.mark.parametrize("log_r,b,plain", [
+    # 2^17 then 2^16 Miller loops: four, then two per thread; against one per thread
+    (9, 2, {"miller_group_min": BIG}),
+    # 19 blocks: 152 fold points in the fifth round (the largest with tables of the shifts), 304 before it
+    (8, 14, {"fold_warp_max": 0}),
+    # 16 blocks of 16 rows: 128 fold points in the first round, 256 Miller outputs reduced by eights
+    (4, 1, {"fold_warp_max": 0, "miller_block_max": 0, "miller_warp_max": 0, "pair_block_max": 0}),
+])
+def test_openall_equal_across_launch_rules(log_r, b, plain):
+    pp = F.PP(log_r + 1, b, 5, log_r=log_r)
+    m = I.vector(17, log_r + 1)
+    out = []
+    try:
+        for lim in ({}, plain):
+            F.set_engine_limits(None)
+            if lim:
+                F.set_engine_limits(lim)
+            cm = F.Commitment(pp, m)
+            pf = F.vc_open_segments(pp, cm, b)
+            out.append((cm.get(), [pf.segment_proof(j) for j in range(0, pp.R, b)]))
+    finally:
+        F.set_engine_limits(None)
+    assert out[0] == out[1]
+
+
+@pytest.mark.parametrize("window", [11, 12])       # 12 x 1024 buckets: one limb per lane; 11 x 2048: threads
+def test_msm_bucket_count_edge(window):
+    n = 40
+    pts = b"".join(O.g1_mul(O.g1_gen(), 3 * v + 1) for v in range(n))
+    k = I.vector(23, 6)[:n]
+    assert F.msm_g1(F.G1Bases(points=pts), k, 1, window) == O.g1_msm(pts, I.to_ints(k))
