@@ -79,35 +79,28 @@ def _wnaf4_exp_rounds(e: int) -> int:
 
 X_ABS = 0xd201000000010000                   # |x| of BLS12-381 (x < 0)
 H1 = (X_ABS + 1) ** 2 // 3                   # h1 = (x - 1)^2 / 3
-# Sequential Fq-product rounds on one launch's critical path in the lane-parallel engines: every
-# round waits for one dependent Montgomery product, so rounds x the measured product latency is a
-# lower bound on the launch time (the linear combinations between rounds and the one-lane
-# binary-gcd inversions are left out, so the bound is optimistic).
+# Sequential rounds on one launch's critical path.  In the engines that give a limb to a lane a round is one
+# sum of products per value with one reduction; rounds x the latency of one lane's dependent product is
+# the yardstick they are reported against (what the same chain would take at one product per lane and
+# round with nothing in between), so a fraction above 1 says that such a round is the shorter one.
 CRITICAL_ROUNDS = {
     # easy part 8 rounds (n, two Frobenius^2, u, n u, c^2, c^2 u, t) + 5 products of the Fq2 inverse,
-    # g 2, hard part: h1 on its width-4 NAF and 3 |x| exponentiations (cyclotomic squarings split over
-    # the block's warps, products one per lane) + 6 Frobenius / product rounds
+    # g 2, hard part: h1 on its width-4 NAF and 3 |x| exponentiations + 6 Frobenius / product rounds
     "k_final_exp_c": 8 + 5 + 2 + _wnaf4_exp_rounds(H1) + 3 * _cyc_exp_rounds(X_ABS) + 6,
     # pipelined Miller loop: a priming round, 63 doubling steps of 2 rounds, 5 addition steps of 4
     # each followed by a priming round
     "k_round_miller_c": 1 + 63 * 2 + 5 * (4 + 1),
     "k_commit_miller_c": 1 + 63 * 2 + 5 * (4 + 1),
-    # G1 by 8-lane groups, 2-bit joint GLV windows: 13 table formulas + 64 x (2 doublings + 1 addition),
-    # 2 phases each, then the addition of A_L and the conversion (longer than the warp G2 chain)
-    "k_fold_w": (13 + 64 * 3) * 2 + 2 + 3,
-    # comb folds (rounds of at most 256 points): the G2 warp's 7 additions of table entries, 3 tree
-    # levels and the addition of v_L, 2 phases each, then the conversion (the G1 groups' 3 + 4 + 1
-    # additions are shorter)
-    "k_fold_c": (7 + 3 + 1) * 2 + 3,
-    # comb chains beside the round: 127 G1 doublings of 2 phases
-    "k_comb_chain": 127 * 2,
-    "k_sparse_g": (13 + 64 * 3) * 2 + 2,
+    # G1 from the tables of the point's shifts: about 83 operations of 2 rounds, then the addition of
+    # A_L and the conversion (the G2 chain has about 68); without tables about 182
+    "k_fold_w": 83 * 2 + 2 + 3,
+    # 128 doublings and about 51 additions of width-4 NAF digits, 3 table additions, 2 rounds each
+    "k_sparse_g": (128 + 51 + 3) * 2,
 }
-# of those rounds, the ones whose product is split over a block's four warps (fq_split.cuh): the
-# cyclotomic squarings (h1's NAF has one digit more than h1 has bits: base^2 and one per lower digit)
-SPLIT_ROUNDS = {"k_final_exp_c": (H1.bit_length() + 1) + 3 * (X_ABS.bit_length() - 1)}
+# rounds whose product is split over a block's four warps (fq_split.cuh): none in these engines
+SPLIT_ROUNDS = {"k_final_exp_c": 0}
 # the kernels of Step 1's round chain (the rest of a round runs beside it)
-CHAIN_KERNELS = ("k_final_exp_c", "k_round_miller_c", "k_fold_c", "k_challenge2")
+CHAIN_KERNELS = ("k_final_exp_c", "k_round_miller_c", "k_fold_w", "k_challenge2")
 
 
 LAM_COMB_MAX_M = 1024         # setups with M <= this commit by the fixed-base combs of their bases
@@ -115,10 +108,7 @@ G2_COMB_MAX_R = 1024          # setups with R <= this keep the W proofs' comb ta
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu capture of the
 # kernel at this workload, keyed by (log N, b, kernel); an entry is removed when its kernel changes
-NCU_TRAFFIC = {
-    (16, 256, "k_round_miller_c"): 277e3,
-    (16, 256, "k_lamc_sum"): 310e6,
-}
+NCU_TRAFFIC = {}
 
 
 MILLER_WAVE = 152 * 256       # threads of the thread-per-pair Miller kernels that run at once
@@ -236,9 +226,9 @@ def roofline_report(prof: dict, units: dict, peak: float, t_lane: float, t_split
         if r:
             roof_all[kname] = {"frac": round(r["frac"], 4), "avg_launch_ms": round(r["avg_launch_ms"], 4),
                                "units_per_step": r["units_per_step"], "unit_op": r["unit_op"]}
-    # latency bound of every round-structured kernel: rounds x the measured latency of one dependent
-    # product (one lane; for the split rounds, the block's four warps together); the headline is the
-    # round chain's kernel with the most time per step
+    # latency yardstick of every round-structured kernel: rounds x the measured latency of one dependent
+    # product (one lane; for split rounds, a block's four warps together); the headline is the round
+    # chain's kernel with the most time per step
     lat_all = {}
     for kname, (kc, kt) in prof.items():
         if kname in CRITICAL_ROUNDS and kc and kt > 0:
@@ -253,10 +243,9 @@ def roofline_report(prof: dict, units: dict, peak: float, t_lane: float, t_split
     if chain:
         top = max(chain, key=lambda k: lat_all[k]["ms_per_step"])
         lat = dict(kernel=top, **lat_all[top], fq_mul_ns=t_lane, fq_mul_split_ns=t_split,
-                   note="sequential Fq-product rounds of the round chain's largest kernel x the measured "
-                        "latency of one dependent product (one lane, or split over a block's four warps for "
-                        "the split rounds); combines and inversions excluded; every such kernel in "
-                        "latency_rooflines")
+                   note="sequential rounds of the round chain's largest kernel x the measured latency of one "
+                        "dependent product on one lane; the kernel's rounds run one limb per lane, so the "
+                        "fraction can exceed 1; every such kernel in latency_rooflines")
     share = {k: round(v[1] / (total_ms if total_ms else 1), 4) for k, v in
              sorted(prof.items(), key=lambda kv: -kv[1][1])[:8]}
     # every kernel: launches per step and mean CUDA-event time per launch (ms)

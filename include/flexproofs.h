@@ -370,7 +370,8 @@ size_t fp_profile_report(char* out, size_t cap);
  * only by a call that writes it out (out != NULL, cap > 0). */
 size_t fp_profile_launches(char* out, size_t cap);
 /* Measured rate of the 32-bit integer multiply-add pipe on the current device (lane operations
- * per second, independent chains, all SMs), the denominator of the integer roofline.  Returns a
+ * per second, independent chains, all SMs; a 32 x 32 + 64 bit multiply-add counts as two, the low
+ * and the high half of its product), the denominator of the integer roofline.  Returns a
  * fp_status code. */
 int fp_imad_probe(double* ops_per_s, double* ms);
 
@@ -378,8 +379,7 @@ int fp_imad_probe(double* ops_per_s, double* ms);
  * current device, CUDA-event timed), in ns: the unit of the latency bound of the lane-parallel
  * engines, whose every round waits for one product.  Returns a fp_status code. */
 int fp_fq_mul_latency(double* ns_per_product);
-/* The same for one Fq product computed by the four warps of a 128-thread block together (the block
- * engine's cyclotomic squarings), in ns.  Returns a fp_status code. */
+/* The same for one Fq product computed by the four warps of a 128-thread block together, in ns.  Returns a fp_status code. */
 int fp_fq_mul_split_latency(double* ns_per_product);
 
 const char* fp_strerror(fp_status s);

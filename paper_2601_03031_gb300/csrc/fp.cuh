@@ -22,7 +22,6 @@ FPG_DEV uint32_t subc_cc(uint32_t a, uint32_t b) { uint32_t r; asm volatile("sub
 FPG_DEV uint32_t subc(uint32_t a, uint32_t b) { uint32_t r; asm volatile("subc.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b)); return r; }
 FPG_DEV uint32_t mad_lo_cc(uint32_t a, uint32_t b, uint32_t c) { uint32_t r; asm volatile("mad.lo.cc.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c)); return r; }
 FPG_DEV uint32_t madc_lo_cc(uint32_t a, uint32_t b, uint32_t c) { uint32_t r; asm volatile("madc.lo.cc.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c)); return r; }
-FPG_DEV uint32_t mad_hi_cc(uint32_t a, uint32_t b, uint32_t c) { uint32_t r; asm volatile("mad.hi.cc.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c)); return r; }
 FPG_DEV uint32_t madc_hi_cc(uint32_t a, uint32_t b, uint32_t c) { uint32_t r; asm volatile("madc.hi.cc.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c)); return r; }
 }  // namespace ptx
 #endif
@@ -57,8 +56,9 @@ FPG_DEV void mac_chain(uint32_t* acc, const uint32_t* v, uint32_t b) {
 // Dividing by 2^32 swaps the two: O becomes the new E, and E without its lowest word (zero) and the
 // word above it (added to the new E, its carry starting the next O chain) the new O.  Both stay in
 // N words: E + 2^32 O < a + P + 2^32 (a + P) before the shift, so O < 2^(32 N); E's carries go to O.
-// 384-bit product, one GB300 at 2070 MHz, separate half chains -> this form: latency on one lane
-// 3.5 k -> 2.0 k cycles; 152 SMs x 32 warps 18.8 -> 30.4 G products/s, 88% of the pipe's 4 cycles per
+// 384-bit product, one GB300 at 2070 MHz, separate half chains -> this form: latency of a full warp
+// 3.5 k -> 2.0 k cycles (a lone lane 2.86 k -> 1.11 k); 152 SMs x 32 warps 18.8 -> 30.4 G products/s,
+// 88% of the pipe at 4 cycles per
 // product and warp.  (Column-wise sums in 96 bits: 28.5 G/s; radix 2^30 or 2^28 without carries: 21
 // and 19 G/s, the pipe takes 4 cycles per 64-bit multiply-add with or without a carry; Karatsuba over
 // 6 + 6 limbs with a separate reduction: 28.8 G/s, its additions cost what its 36 products save.)
@@ -420,7 +420,7 @@ FPG_DEV void fq_from_const(fq& a, const uint32_t* c) {
 #pragma unroll
     for (int j = 0; j < 12; j++) a.v[j] = c[j];
 }
-// The Montgomery products are out of line: one copy of the ~700-instruction body per translation
+// The Montgomery products are out of line: one copy of the ~500-instruction body per translation
 // unit instead of one per call site.  Inlined, a group operation's dozen products overflow the
 // instruction cache and every product runs about three times slower; the call costs a few moves
 // (arguments and result travel in registers).

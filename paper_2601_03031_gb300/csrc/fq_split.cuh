@@ -1,7 +1,7 @@
 // One Fq Montgomery product computed by the four warps of a 128-thread block together.
 //
-// A single lane's CIOS product (fp.cuh) is one warp's instruction stream of ~700 carry-chain
-// multiply-adds; however many lanes take part, that stream runs on one of the SM's four
+// A single lane's product (fp.cuh) is one warp's instruction stream of 300 wide multiply-adds and
+// their carries; however many lanes take part, that stream runs on one of the SM's four
 // sub-partitions, and it sets the latency of every round of the latency-bound engines.  Here lane
 // t of each of the four warps (one warp per sub-partition) takes a quarter of product t, so a round
 // of up to 32 products costs about a quarter of the multiply-adds per sub-partition plus two block

@@ -1,7 +1,7 @@
 // Fq arithmetic with one limb per lane, for latency: sums of products of Fq values on 16 lanes each.
 //
-// A product on one lane is a chain of 288 multiply-adds (fp.cuh), about 2.0 k cycles however idle the
-// GPU is, and every addition around it another 24 carries.  Here a value is 15 signed limbs of 26 bits
+// A product per lane is a chain of 300 multiply-adds (fp.cuh), about 2.0 k cycles for a warp however idle
+// the GPU is, and every addition around it another 24 carries.  Here a value is 15 signed limbs of 26 bits
 // on 15 of the 16 lanes of a slot, so an addition is one instruction without carries, and a lane forms
 // one column of a product with 15 multiply-adds into a 64-bit sum.  What is computed is
 //     out = sum_{t < n} x_t y_t  2^-390  +  addend   (mod p)

@@ -121,24 +121,23 @@ size_t fp_profile_launches(char* out, size_t cap) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Peak of the integer multiply-add pipe: every thread runs 8 independent chains of 32-bit
-// multiply-adds (alternating low and high halves, the two kinds every Montgomery product issues),
-// so the pipe, not latency, bounds the rate.  ops = lanes x iterations x 8.
+// Peak of the integer multiply-add pipe: every thread runs 4 independent chains of 32 x 32 + 64 bit
+// multiply-adds, the form the Montgomery products issue, so the pipe, not latency, bounds the rate.  One
+// counts as two operations (a product's low and its high half): ops = lanes x iterations x 8.  (Halves
+// as instructions of their own, a low half 2 and a high half 4 cycles per warp, reach 12.6 T a second.)
 // ---------------------------------------------------------------------------------------
 __global__ void k_imad_probe(uint32_t iters, uint32_t seed, uint32_t* sink) {
-    uint32_t a[8];
-    for (int k = 0; k < 8; k++) a[k] = seed + threadIdx.x * 8 + k;
-    const uint32_t m = 0x9e3779b9u + blockIdx.x, c = 0x7f4a7c15u;
+    uint64_t a[4];
+    for (int k = 0; k < 4; k++) a[k] = seed + threadIdx.x * 4 + k;
+    const uint32_t m = 0x9e3779b9u + blockIdx.x;
     for (uint32_t it = 0; it < iters; it++) {
 #pragma unroll
-        for (int k = 0; k < 8; k += 2) {
-            asm volatile("mad.lo.u32 %0, %0, %1, %2;" : "+r"(a[k]) : "r"(m), "r"(c));
-            asm volatile("mad.hi.u32 %0, %0, %1, %2;" : "+r"(a[k + 1]) : "r"(m), "r"(c));
-        }
+        for (int k = 0; k < 4; k++)
+            asm volatile("{ .reg .u32 lo, hi; mov.b64 {lo, hi}, %0; mad.wide.u32 %0, lo, %1, %0; }" : "+l"(a[k]) : "r"(m));
     }
-    uint32_t x = 0;
-    for (int k = 0; k < 8; k++) x ^= a[k];
-    if (x == 0x12345678u) sink[0] = x;
+    uint64_t x = 0;
+    for (int k = 0; k < 4; k++) x ^= a[k];
+    if (x == 0x12345678u) sink[0] = (uint32_t)x;
 }
 
 extern "C" int fp_imad_probe(double* ops_per_s, double* ms_out) {

@@ -1,8 +1,10 @@
 // Fq12 arithmetic on one warp: the Fq products of an operation are spread one per lane and round.
 //
-// A Montgomery product is ~700 multiply-add instructions that one warp issues at the integer
-// pipe's rate whatever their dependency structure, so a single lane cannot make one faster; what
-// shortens a chain of Fq12 operations is doing all of an operation's products at once.  Values
+// A Montgomery product is 300 wide multiply-adds that one warp issues at the integer pipe's rate
+// whatever their dependency structure, so a single lane cannot make one faster; what shortens a
+// chain of Fq12 operations is doing all of an operation's products at once.  (Where a launch is a few
+// blocks, a value with one limb per lane is faster still: limb12.cuh and limb_miller.cuh run the final
+// exponentiations and Miller loops that this file's blocks ran.)  Values
 // live in shared memory, flat as Fq2[w]/(w^6 - xi) (xi = 1 + u): Fq index 2k + e holds component
 // e (0 = real, 1 = u) of the coefficient of w^k, k = 0..5 (w^2 = v, so flat k = 0,2,4 are the tower's
 // c0.c0, c0.c1, c0.c2 and k = 1,3,5 are c1.c0, c1.c1, c1.c2).  Every operation is
@@ -971,28 +973,4 @@ FPG_NOINL void w_miller(WMill& S, g1a P, g2a Q) {
         S.f[L] = fq_select(inf, fq_select(L == 0, one, z), v);
     }
     wsync<NW>();
-}
-
-// acc = base^e for any base (e little-endian words, squarings as products); acc != base
-template <int NW>
-FPG_NOINL void w_exp(W12& W, fq* acc, const fq* base, const uint32_t* e, int bits) {
-    const int L = w_lane<NW>();
-    int i = bits - 1;
-    while (i >= 0 && !((e[i >> 5] >> (i & 31)) & 1)) i--;
-    if (i < 0) {                                   // e = 0: acc = 1
-        wsync<NW>();
-        if (L < 12) {
-            fq v;
-            if (L == 0) fq_one(v);
-            else fq_zero(v);
-            acc[L] = v;
-        }
-        wsync<NW>();
-        return;
-    }
-    w_copy<NW>(acc, base);
-    for (i = i - 1; i >= 0; i--) {
-        w_mul<NW>(W, acc, acc, acc);
-        if ((e[i >> 5] >> (i & 31)) & 1) w_mul<NW>(W, acc, acc, base);
-    }
 }
