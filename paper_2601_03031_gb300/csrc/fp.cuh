@@ -58,8 +58,7 @@ FPG_DEV void mac_chain(uint32_t* acc, const uint32_t* v, uint32_t b) {
 // N words: E + 2^32 O < a + P + 2^32 (a + P) before the shift, so O < 2^(32 N); E's carries go to O.
 // 384-bit product, one GB300 at 2070 MHz, separate half chains -> this form: latency of a full warp
 // 3.5 k -> 2.0 k cycles (a lone lane 2.86 k -> 1.11 k); 152 SMs x 32 warps 18.8 -> 30.4 G products/s,
-// 88% of the pipe at 4 cycles per
-// product and warp.  (Column-wise sums in 96 bits: 28.5 G/s; radix 2^30 or 2^28 without carries: 21
+// 88% of the pipe at 4 cycles per product and warp.  (Column-wise sums in 96 bits: 28.5 G/s; radix 2^30 or 2^28 without carries: 21
 // and 19 G/s, the pipe takes 4 cycles per 64-bit multiply-add with or without a carry; Karatsuba over
 // 6 + 6 limbs with a separate reduction: 28.8 G/s, its additions cost what its 36 products save.)
 template <int N>

@@ -121,23 +121,30 @@ size_t fp_profile_launches(char* out, size_t cap) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Peak of the integer multiply-add pipe: every thread runs 4 independent chains of 32 x 32 + 64 bit
-// multiply-adds, the form the Montgomery products issue, so the pipe, not latency, bounds the rate.  One
-// counts as two operations (a product's low and its high half): ops = lanes x iterations x 8.  (Halves
-// as instructions of their own, a low half 2 and a high half 4 cycles per warp, reach 12.6 T a second.)
+// Peak of the integer multiply-add pipe in the form the Montgomery products use it: every thread adds rows
+// of six 32 x 32 bit products to two accumulators (mac_chain), a new factor for each row so that nothing
+// can be formed outside the loop.  A product counts as two operations (its low and its high half):
+// ops = lanes x iterations x 48.  (Halves as instructions of their own reach 12.6 T a second;
+// multiply-adds without carry whose factor is another sum's low word 15.8 T.)
 // ---------------------------------------------------------------------------------------
 __global__ void k_imad_probe(uint32_t iters, uint32_t seed, uint32_t* sink) {
-    uint64_t a[4];
-    for (int k = 0; k < 4; k++) a[k] = seed + threadIdx.x * 4 + k;
-    const uint32_t m = 0x9e3779b9u + blockIdx.x;
+    uint32_t v[12], E[12], O[12], b = seed ^ threadIdx.x;
+    for (int k = 0; k < 12; k++) {
+        v[k] = 0x9e3779b9u * (k + 1) + blockIdx.x;
+        E[k] = v[k] + threadIdx.x;
+        O[k] = v[k] ^ threadIdx.x;
+    }
     for (uint32_t it = 0; it < iters; it++) {
 #pragma unroll
-        for (int k = 0; k < 4; k++)
-            asm volatile("{ .reg .u32 lo, hi; mov.b64 {lo, hi}, %0; mad.wide.u32 %0, lo, %1, %0; }" : "+l"(a[k]) : "r"(m));
+        for (int u = 0; u < 2; u++) {
+            mp::mac_chain<12, false>(E, v, b);
+            mp::mac_chain<12, false>(O, v + 1, b);
+            b += 0x7f4a7c15u ^ E[11];
+        }
     }
-    uint64_t x = 0;
-    for (int k = 0; k < 4; k++) x ^= a[k];
-    if (x == 0x12345678u) sink[0] = (uint32_t)x;
+    uint32_t x = 0;
+    for (int k = 0; k < 12; k++) x ^= E[k] ^ O[k];
+    if (x == 0x12345678u) sink[0] = x;
 }
 
 extern "C" int fp_imad_probe(double* ops_per_s, double* ms_out) {
@@ -146,7 +153,7 @@ extern "C" int fp_imad_probe(double* ops_per_s, double* ms_out) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     uint32_t* sink = nullptr;
     if (cudaMalloc(&sink, 4) != cudaSuccess) return 2;
-    const uint32_t iters = 4096, threads = 256, blocks = (uint32_t)sms * 8;
+    const uint32_t iters = 1024, threads = 256, blocks = (uint32_t)sms * 8;
     cudaEvent_t a, b;
     cudaEventCreate(&a); cudaEventCreate(&b);
     k_imad_probe<<<blocks, threads>>>(64, 1, sink);      // warm-up
@@ -158,7 +165,7 @@ extern "C" int fp_imad_probe(double* ops_per_s, double* ms_out) {
     cudaEventElapsedTime(&ms, a, b);
     cudaEventDestroy(a); cudaEventDestroy(b); cudaFree(sink);
     if (e != cudaSuccess) return 3;
-    *ops_per_s = (double)blocks * threads * iters * 8 / (ms * 1e-3);
+    *ops_per_s = (double)blocks * threads * iters * 48 / (ms * 1e-3);
     if (ms_out) *ms_out = ms;
     return 0;
 }
