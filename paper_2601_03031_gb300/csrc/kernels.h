@@ -41,6 +41,7 @@ struct EngineLimits {
     uint32_t msm_segment_threads = 1u << 15;  // MSM bucket reduction: at most about this many segments
 };
 EngineLimits engine_limits();              // a snapshot of the current limits
+void require(cudaError_t e, const char* what);   // throws what the library's entry points turn into their status
 
 constexpr size_t FR_BYTES = 32;     // fr: 8 x u32, Montgomery or canonical as documented
 constexpr size_t G1A_BYTES = 96;    // affine G1, Montgomery, (0,0) = identity

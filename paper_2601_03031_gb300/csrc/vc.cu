@@ -82,6 +82,7 @@ struct CudaError {
 
 void check(cudaError_t e, const char* what) {
     if (e != cudaSuccess) {
+        cudaGetLastError();                          // reported here, not by the next call's check_launch
         g_last_error = std::string(what) + ": " + cudaGetErrorString(e);
         throw CudaError{e == cudaErrorMemoryAllocation ? FP_ENOMEM : FP_EDEVICE};
     }
@@ -213,6 +214,14 @@ cudaEvent_t new_event() {
     check(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "cudaEventCreate");
     return e;
 }
+// waits for what a failed call has enqueued on its stream and on the internal ones it took (null: none yet),
+// whose joins may be missing, before its buffers are given back
+void drain(cudaStream_t s, const Streams& st) {
+    for (cudaStream_t x : {st.hi, st.sp, st.pre, st.la[0], st.la[1], st.fold, st.lo, st.tail})
+        if (x) cudaStreamSynchronize(x);
+    cudaStreamSynchronize(s);
+    cudaGetLastError();
+}
 
 }  // namespace
 
@@ -226,6 +235,7 @@ EngineLimits engine_limits() {
     std::lock_guard<std::mutex> lk(g_limits_mu);
     return g_limits;
 }
+void require(cudaError_t e, const char* what) { check(e, what); }
 const void* pp_lambda_top(const fp_pp* pp) { return (const uint8_t*)pp->lam + ((size_t)pp->M - 1) * G1A_BYTES; }
 }  // namespace fpk
 
@@ -1064,13 +1074,14 @@ fp_status vc_verify(const fp_pp* pp, const uint8_t* C, uint32_t b, uint64_t i, c
             for (int q = 0; q < 8; q++) host[len + GT_SER + 8 * (3 - w) + q] = (uint8_t)(m_i[w] >> (56 - 8 * q));
         void *dbuf = nullptr, *scr = nullptr, *res = nullptr;
         uint32_t hres = 1;
+        Streams st;
         try {
             dbuf = dalloc(host.size(), s);
             scr = dalloc(verify_scratch_bytes(b, lr, lc), s);
             res = dalloc(sizeof(uint32_t), s);
             check(cudaMemcpyAsync(dbuf, host.data(), host.size(), cudaMemcpyHostToDevice, s), "H2D proof");
             const uint8_t* d = (const uint8_t*)dbuf;
-            const Streams st = streams(s);
+            st = streams(s);
             verify_one(d, d + len, d + len + GT_SER, nk, lr, lc, b, i, pp->M, k, lo, pp->g1beta, pp->g2tau, scr,
                        (uint32_t*)res, s, st.sp, st.la[0]);
             check_launch("vc_verify kernels");
@@ -1078,7 +1089,7 @@ fp_status vc_verify(const fp_pp* pp, const uint8_t* C, uint32_t b, uint64_t i, c
             dfree(dbuf, s); dfree(scr, s); dfree(res, s);
             check(cudaStreamSynchronize(s), "vc_verify");
         } catch (...) {
-            cudaStreamSynchronize(s);
+            drain(s, st);
             dfree(dbuf, s); dfree(scr, s); dfree(res, s);
             throw;
         }
@@ -1095,6 +1106,7 @@ fp_status vc_verify_all(const fp_pp* pp, const uint8_t* C, const uint64_t* m, in
         const uint64_t N = (uint64_t)L.R * L.M;
         void *dC = nullptr, *dm = nullptr, *scr = nullptr;
         cudaEvent_t ready = nullptr;
+        Streams st;
         try {
             // the proof pieces are written on the handle's stream
             check(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming), "cudaEventCreate");
@@ -1109,7 +1121,7 @@ fp_status vc_verify_all(const fp_pp* pp, const uint8_t* C, const uint64_t* m, in
                 md = dm;
             }
             scr = dalloc(verify_all_scratch_bytes(L), s);
-            const Streams st = streams(s);
+            st = streams(s);
             const uint64_t good = verify_all(L, dC, md, pf->rows_ser, pf->blocks, pf->row_tree, pf->top_tree, pf->D_ser,
                                              pf->g, pf->pst_ser, pp->g1beta, pp->g2tau, flags & 1, scr, ok, s, st.sp, st.la[0]);
             check_launch("vc_verify_all kernels");
@@ -1118,7 +1130,7 @@ fp_status vc_verify_all(const fp_pp* pp, const uint8_t* C, const uint64_t* m, in
             cudaEventDestroy(ready);
             if (n_ok) *n_ok = good;
         } catch (...) {
-            cudaStreamSynchronize(s);
+            drain(s, st);
             dfree(dC, s); dfree(dm, s); dfree(scr, s);
             if (ready) cudaEventDestroy(ready);
             throw;
@@ -1241,13 +1253,14 @@ fp_status vc_eval_verify(const fp_pp* pp, const uint8_t* C, const uint8_t* r, co
         memcpy(host.data() + len + GT_SER, r, 32 * (size_t)ln);
         void *dbuf = nullptr, *scr = nullptr, *res = nullptr;
         uint32_t hres = 1;
+        Streams st;
         try {
             dbuf = dalloc(host.size(), s);
             scr = dalloc(verify_eval_scratch_bytes(pp->R, (int)pp->log_r, (int)pp->log_c, ln), s);
             res = dalloc(sizeof(uint32_t), s);
             check(cudaMemcpyAsync(dbuf, host.data(), host.size(), cudaMemcpyHostToDevice, s), "H2D");
             const uint8_t* d = (const uint8_t*)dbuf;
-            const Streams st = streams(s);
+            st = streams(s);
             verify_eval(d, d + len, d + len + GT_SER, ln, (int)pp->log_r, (int)pp->log_c, pp->R, pp->g1beta,
                         pp->g2tau, scr, (uint32_t*)res, s, st.sp, st.la[0]);
             check_launch("vc_eval_verify kernels");
@@ -1255,7 +1268,7 @@ fp_status vc_eval_verify(const fp_pp* pp, const uint8_t* C, const uint8_t* r, co
             dfree(dbuf, s); dfree(scr, s); dfree(res, s);
             check(cudaStreamSynchronize(s), "vc_eval_verify");
         } catch (...) {
-            cudaStreamSynchronize(s);
+            drain(s, st);
             dfree(dbuf, s); dfree(scr, s); dfree(res, s);
             throw;
         }
@@ -1323,6 +1336,7 @@ fp_status vc_verify_segment(const fp_pp* pp, const uint8_t* C, uint32_t b, uint3
         void *dbuf = nullptr, *vscr = nullptr, *mscr = nullptr, *mc = nullptr, *mm = nullptr, *cj = nullptr,
              *out = nullptr;
         uint32_t hout[2 + 24] = {};
+        Streams st;
         try {
             dbuf = dalloc(host.size(), s);
             vscr = dalloc(verify_block_scratch_bytes(b, lr), s);
@@ -1337,13 +1351,14 @@ fp_status vc_verify_segment(const fp_pp* pp, const uint8_t* C, uint32_t b, uint3
             uint32_t* o = (uint32_t*)out;
             load_vector(d + len + GT_SER, M, mc, mm, o + 1, s);
             msm_g1(pp->lam_tab, mc, sh, mscr, cj, o + 2, s);       // C_j from m_j (VC.Commit's row MSM)
-            verify_block(d, d + (size_t)nk * G1_SER, d + len, nk, lr, b, k, lo, pp->g1beta, vscr, o, s, streams(s).sp);
+            st = streams(s);
+            verify_block(d, d + (size_t)nk * G1_SER, d + len, nk, lr, b, k, lo, pp->g1beta, vscr, o, s, st.sp);
             check_launch("vc_verify_segment kernels");
             check(cudaMemcpyAsync(hout, out, sizeof hout, cudaMemcpyDeviceToHost, s), "D2H");
             dfree(dbuf, s); dfree(vscr, s); dfree(mscr, s); dfree(mc, s); dfree(mm, s); dfree(cj, s); dfree(out, s);
             check(cudaStreamSynchronize(s), "vc_verify_segment");
         } catch (...) {
-            cudaStreamSynchronize(s);
+            drain(s, st);
             dfree(dbuf, s); dfree(vscr, s); dfree(mscr, s); dfree(mc, s); dfree(mm, s); dfree(cj, s); dfree(out, s);
             throw;
         }

@@ -616,15 +616,18 @@ struct JobBufs {
     }
 };
 
-// the blocks' statement hashes, their transcripts and, on the side stream after them, the GT part of the
-// folded commitment (cT); the caller joins the side stream
+// what is enqueued on `to` from here on comes after what is on `from`; a join that cannot be made ends the call
+// before anything unordered is launched (its entry point then waits for both streams)
 void vb_join(cudaStream_t from, cudaStream_t to) {
     cudaEvent_t e = nullptr;
-    cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
-    cudaEventRecord(e, from);
-    cudaStreamWaitEvent(to, e, 0);
+    require(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "cudaEventCreate");
+    cudaError_t st = cudaEventRecord(e, from);
+    if (st == cudaSuccess) st = cudaStreamWaitEvent(to, e, 0);
     cudaEventDestroy(e);
+    require(st, "join");
 }
+// the blocks' statement hashes, their transcripts and, on the side stream after them, the GT part of the
+// folded commitment (cT); the caller joins the side stream
 template <class A>
 void block_transcripts(const VSrc& S, const uint8_t* C_be, const fq12* Cd, BlockBufs<A>& Bb, cudaStream_t s,
                        cudaStream_t side) {

@@ -1,0 +1,98 @@
+"""The library's host path on the CPU, its object files linked against a CUDA runtime that runs nothing
+(tests/emu/fake_cudart.cpp): the order of work over streams and what a failing event call leaves behind."""
+import ctypes
+import glob
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+vp, u32, u64, sz = ctypes.c_void_p, ctypes.c_uint32, ctypes.c_uint64, ctypes.c_size_t
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    from paper_2601_03031_gb300 import build as B
+    gxx = shutil.which("g++")
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B.nvcc()))), "include")
+    if not gxx or not os.path.exists(os.path.join(inc, "cuda_runtime_api.h")):
+        pytest.skip("g++ or the CUDA headers not available")
+    B.build()
+    objs = [os.path.join(B.BUILD_DIR, os.path.basename(s) + ".o") for s in B.sources()]
+    if any(not os.path.exists(o) for o in objs):
+        B.build(force=True)
+    out = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    subprocess.check_call([gxx, "-std=c++17", "-O1", "-shared", "-fPIC", f"-I{inc}", "-o", out,
+                           os.path.join(ROOT, "tests", "emu", "fake_cudart.cpp"), *objs])
+    L = ctypes.CDLL(out)
+    for f in ("fake_event_calls", "fake_bad_frees", "fake_late_launches"):
+        getattr(L, f).restype = ctypes.c_long
+    L.fake_log.restype = ctypes.c_char_p
+    for f in ("vc_proof_len", "vc_segment_proof_len", "vc_eval_proof_len"):
+        getattr(L, f).restype = sz
+    return L
+
+
+@pytest.fixture(scope="module")
+def pp(lib):
+    lib.fake_reset(ctypes.c_long(-1))
+    h = vp()
+    assert lib.vc_setup(u32(8), u32(3), u64(1), None, ctypes.byref(h)) == 0
+    return h
+
+
+@pytest.fixture(scope="module")
+def cm(lib, pp):
+    h = vp()
+    assert lib.vc_commit(pp, ctypes.create_string_buffer(32 << 8), 0, None, ctypes.byref(h)) == 0
+    return h
+
+
+C = ctypes.create_string_buffer(576)
+B = 3
+
+
+def verify_one(lib, pp, cm):
+    n = lib.vc_proof_len(pp, u32(B), u64(5))
+    return lib.vc_verify(pp, C, u32(B), u64(5), (u64 * 4)(), ctypes.create_string_buffer(n), sz(n), None)
+
+
+def verify_segment(lib, pp, cm):
+    n = lib.vc_segment_proof_len(pp, u32(B), u32(4))
+    return lib.vc_verify_segment(pp, C, u32(B), u32(4), (u64 * 64)(), ctypes.create_string_buffer(n), sz(n), None)
+
+
+def verify_eval(lib, pp, cm):
+    n = lib.vc_eval_proof_len(pp)
+    return lib.vc_eval_verify(pp, C, ctypes.create_string_buffer(256), ctypes.create_string_buffer(n), sz(n), None)
+
+
+def verify_all(lib, pp, cm):
+    return lib.vc_verify_all(pp, C, ctypes.create_string_buffer(32 << 8), 0, verify_all.pf, 0, None, None, None)
+
+
+def run(lib, pp, cm, call, fail_at):
+    """Status of the call whose fail_at-th event call fails (-1: none), how many event calls it made, buffers it
+    freed under running work, and launches after the failure."""
+    if call is verify_all:
+        lib.fake_reset(ctypes.c_long(-1))
+        verify_all.pf = vp()
+        assert lib.vc_prove_all(pp, cm, u32(B), None, ctypes.byref(verify_all.pf)) == 0
+    lib.fake_reset(ctypes.c_long(fail_at))
+    st = call(lib, pp, cm)
+    return st, lib.fake_event_calls(), lib.fake_bad_frees(), lib.fake_late_launches()
+
+
+@pytest.mark.parametrize("call", [verify_one, verify_segment, verify_eval, verify_all])
+def test_failed_joins_of_the_verifier(lib, pp, cm, call):
+    """Whichever event call of a verification fails, the call says so (FP_EDEVICE), launches nothing after it
+    and gives no buffer back that a side stream may still use."""
+    st, calls, bad, _ = run(lib, pp, cm, call, -1)
+    assert (st, bad) == (0, 0) and calls > 0
+    for n in range(calls):
+        st, _, bad, late = run(lib, pp, cm, call, n)
+        assert (st, bad, late) == (3, 0, 0), n
+        st, _, bad, _ = run(lib, pp, cm, call, -1)          # and the failure is not reported again
+        assert (st, bad) == (0, 0), n
