@@ -778,6 +778,7 @@ fp_proofs* prove_impl(const fp_pp* pp, const fp_commit* cm, uint32_t b, uint32_t
         const size_t blen = pf->L.bopen_len;
         uint8_t* blocks1 = nullptr;
         std::vector<void*> tmp;
+        Streams st;
         auto T = [&](size_t bytes) { void* p = dalloc(bytes, s); tmp.push_back(p); return p; };
         try {
             // the commitment may have been made on another stream: order after its rows (C, which only
@@ -810,7 +811,7 @@ fp_proofs* prove_impl(const fp_pp* pp, const fp_commit* cm, uint32_t b, uint32_t
             const LaBufs L = la ? la_bufs(pp, Kc, T) : LaBufs{};
             void* hstmt = T(Kc * DIGEST);
             void* hscr = T(stmt_hash_scratch_bytes(Kc, R, b));
-            const Streams st = streams(s);
+            st = streams(s);
             cudaStream_t s2 = st.lo, s1 = st.hi, s3 = st.sp;
             cudaEvent_t ev_fork = new_event(), ev_join = new_event(), ev_join1 = new_event();
             check(cudaEventRecord(ev_fork, s), "event");
@@ -880,8 +881,8 @@ fp_proofs* prove_impl(const fp_pp* pp, const fp_commit* cm, uint32_t b, uint32_t
             for (void* p : tmp) cudaFreeAsync(p, s);
             tmp.clear();
         } catch (...) {
+            drain(s, st);
             for (void* p : tmp) cudaFreeAsync(p, s);
-            cudaStreamSynchronize(s);
             fp_proofs_free(pf);
             throw;
         }
@@ -1159,6 +1160,7 @@ fp_status vc_eval_prove(const fp_pp* pp, const fp_commit* cm, const uint8_t* r, 
         const uint64_t half = M / 2 ? M / 2 : 1;
         const MsmShape sh = msm_shape(R, 1, R, fp_msm_window(R, 1));
         std::vector<void*> tmp;
+        Streams st;
         auto T = [&](size_t bytes) { void* p = dalloc(bytes, s); tmp.push_back(p); return p; };
         uint32_t herr = 0;
         try {
@@ -1180,7 +1182,7 @@ fp_status vc_eval_prove(const fp_pp* pp, const fp_commit* cm, const uint8_t* r, 
             const Step1Bufs B = step1_bufs(pp, 1, T);
             const bool la = lookahead_on((int)pp->log_r);
             const LaBufs L = la ? la_bufs(pp, 1, T) : LaBufs{};
-            const Streams st = streams(s);
+            st = streams(s);
             cudaStream_t s1 = st.hi, s3 = st.sp, s2 = st.lo;
             cudaEvent_t ev_fork = new_event(), ev_bvec = new_event(), ev_join = new_event(), ev_wts = new_event(),
                         ev_pst = new_event();
@@ -1231,8 +1233,8 @@ fp_status vc_eval_prove(const fp_pp* pp, const fp_commit* cm, const uint8_t* r, 
             cudaEventDestroy(ev_wts); cudaEventDestroy(ev_pst);
             check(cudaStreamSynchronize(s), "vc_eval_prove");
         } catch (...) {
+            drain(s, st);
             for (void* p : tmp) cudaFreeAsync(p, s);
-            cudaStreamSynchronize(s);
             throw;
         }
         return herr ? FP_ERANGE : FP_OK;

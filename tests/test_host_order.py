@@ -96,3 +96,39 @@ def test_failed_joins_of_the_verifier(lib, pp, cm, call):
         assert (st, bad, late) == (3, 0, 0), n
         st, _, bad, _ = run(lib, pp, cm, call, -1)          # and the failure is not reported again
         assert (st, bad) == (0, 0), n
+
+
+def prove_all(lib, pp, cm):
+    pf = vp()
+    st = lib.vc_prove_all(pp, cm, u32(B), None, ctypes.byref(pf))
+    if st == 0:
+        lib.fp_proofs_free(pf)
+    return st
+
+
+def prove_one(lib, pp, cm):
+    n = lib.vc_proof_len(pp, u32(B), u64(5))
+    return lib.vc_prove_one(pp, cm, u32(B), u64(5), None, ctypes.create_string_buffer(n), sz(n), ctypes.byref(sz()))
+
+
+def eval_prove(lib, pp, cm):
+    n = lib.vc_eval_proof_len(pp)
+    return lib.vc_eval_prove(pp, cm, ctypes.create_string_buffer(256), None, ctypes.create_string_buffer(n), sz(n),
+                             ctypes.byref(sz()))
+
+
+@pytest.mark.parametrize("schedule", [0, 1])
+@pytest.mark.parametrize("call", [prove_all, prove_one, eval_prove])
+def test_failed_events_of_the_prover(lib, pp, cm, call, schedule):
+    """The same for the proving calls, which work on up to seven internal streams, under both schedules."""
+    lib.fp_set_schedule(schedule)
+    try:
+        st, calls, bad, _ = run(lib, pp, cm, call, -1)
+        assert (st, bad) == (0, 0) and calls > 0
+        for n in range(calls):
+            st, _, bad, late = run(lib, pp, cm, call, n)
+            assert (st, bad, late) == (3, 0, 0), n
+            st, _, bad, _ = run(lib, pp, cm, call, -1)
+            assert (st, bad) == (0, 0), n
+    finally:
+        lib.fp_set_schedule(0)
