@@ -328,7 +328,8 @@ typedef enum { FP_SCHEDULE_DIRECT = 0, FP_SCHEDULE_LOOKAHEAD = 1 } fp_schedule;
  *   commit_block_max / commit_warp_max   Commit's R Miller loops, the same way (default 1024 / 16384)
  *   fe_block_max / fe_warp_max           final exponentiations: block / warp / thread (256 / 2^32-1;
  *                                        unless block_max is 0, blocks also up to 912)
- *   pair_block_max                       pairwise Fq12 products: <= a block each, above a thread (2048)
+ *   pair_block_max                       pairwise Fq12 products: <= blocks (of up to eight values, in the
+ *                                        look-ahead schedule of two), above a thread per pair (2048)
  *   fold_warp_max                        fold points of a round: <= a block (G2) and half a block (G1)
  *                                        each, above a thread (4096)
  *   wterm_warp_max                       terms of the v_l proof W when not by MSM: <= a warp each,

@@ -33,7 +33,8 @@ struct EngineLimits {
     uint32_t commit_warp_max = 16384;       //   <= this, a block each too; above, a thread each
     uint32_t fe_block_max = 256;            // final exponentiations per launch: <= this, a block each
     uint32_t fe_warp_max = 0xffffffffu;     //   <= this, a warp each; above, a thread each
-    uint32_t pair_block_max = 2048;         // pairwise Fq12 products: <= this, a block each; above, a thread
+    uint32_t pair_block_max = 2048;         // pairwise Fq12 products: <= this, by eights with a block each (by
+                                            //   pairs in the look-ahead schedule); above, a thread per pair
     uint32_t fold_warp_max = 4096;          // fold points: <= this, a block per G2 point and half a block per G1
                                             //   per point; above, a thread per point
     uint32_t wterm_warp_max = 4096;         // W terms: <= this, a warp per term; above, a thread per term

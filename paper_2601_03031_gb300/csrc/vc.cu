@@ -144,11 +144,13 @@ void* reduce_tree(void* a, void* b, uint64_t n, uint64_t target, uint32_t gmax, 
     }
     return a;
 }
-// products of consecutive Fq12 values down to `target`: by eights, one block each, once few are left
+// products of consecutive Fq12 values down to `target`: by eights, one block each, once the pairwise products
+// left are at most pair_block_max, until then pairwise
 void* reduce_fq12(void* a, void* b, uint64_t n, uint64_t target, cudaStream_t s) {
+    const uint32_t blocks_max = engine_limits().pair_block_max;
     while (n > target) {
         uint32_t gs = 2;
-        if (n <= 4096) {
+        if (n / 2 <= blocks_max) {
             gs = (uint32_t)std::min<uint64_t>(8, n / target);
             fq12_products(nullptr, a, gs, gs, b, 1, n / gs, s);
         } else {

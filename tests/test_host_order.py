@@ -132,3 +132,34 @@ def test_failed_events_of_the_prover(lib, pp, cm, call, schedule):
             assert (st, bad) == (0, 0), n
     finally:
         lib.fp_set_schedule(0)
+
+
+LIMITS = ["miller_block_max", "miller_warp_max", "miller_group_min", "commit_block_max", "commit_warp_max", "fe_block_max",
+          "fe_warp_max", "pair_block_max", "fold_warp_max", "wterm_warp_max", "msm_chunks", "msm_segment_threads"]
+
+
+def launches(lib, fn, **limits):
+    """[(kernel's mangled name, grid, block)] of fn() under the given engine limits."""
+    lim = (u32 * len(LIMITS))()
+    lib.fp_engine_limits_default(lim)
+    for k, v in limits.items():
+        lim[LIMITS.index(k)] = v
+    lib.fp_set_engine_limits(lim)
+    try:
+        lib.fake_reset(ctypes.c_long(-1))
+        assert fn() == 0
+        return [(w[0], int(w[1]), int(w[2])) for w in (x.split() for x in lib.fake_log().decode().splitlines())]
+    finally:
+        lib.fp_set_engine_limits(None)
+
+
+@pytest.mark.parametrize("pair_block_max", [0, 2, 1 << 16])
+def test_fq12_products_keep_to_their_limit(lib, pp, cm, pair_block_max):
+    """pair_block_max: rounds with more pairwise products than that run them one per thread."""
+    log = launches(lib, lambda: prove_all(lib, pp, cm), pair_block_max=pair_block_max)
+    threads = [g for n, g, _ in log if "k_fq12_pairE" in n]
+    blocks = [g for n, g, _ in log if "k_fq12_prod" in n]
+    # R = 16, six blocks of up to 3 rows: 96, 48, 24 and 12 Miller values in the rounds, reduced to 12: halved 3, 2, 1
+    # and 0 times, or by eights, fours and twos
+    want = {0: (6, 0), 2: (6, 0), 1 << 16: (0, 3)}[pair_block_max]
+    assert (len(threads), len(blocks)) == want, (threads, blocks)
