@@ -28,7 +28,7 @@ sys.path.insert(0, ROOT)
 os.environ.setdefault("CUDA_DEVICE_MAX_CONNECTIONS", "32")
 
 # Fq multiplications per unit operation, from the operation counts of efficient textbook formulas
-# (an Fq multiplication is one 12-limb CIOS Montgomery product = 4 * 12^2 = 576 32-bit
+# (an Fq multiplication is one 12-limb Montgomery product = 4 * 12^2 = 576 32-bit
 # multiply-adds).  These are ALGORITHMIC counts: the kernels' own formulas may do more.
 FQ_MUL_IMAD = 4 * 12 * 12
 FQ_MULS = {
@@ -111,6 +111,7 @@ G2_COMB_MAX_R = 1024          # setups with R <= this keep the W proofs' comb ta
 NCU_TRAFFIC = {}
 
 
+FE_LIMB_MAX = 6 * 152         # final exponentiations on blocks although warps are allowed
 MILLER_WAVE = 152 * 256       # threads of the thread-per-pair Miller kernels that run at once
 
 
@@ -146,17 +147,18 @@ def step_units(log_n: int, b: int, msm_window: int, msm_window_g2: int = 16, lim
             return "t"
         return "c" if n <= block_max else "w"
 
-    mb, mw, mg = lim["miller_block_max"], lim["miller_warp_max"], lim["miller_group_min"]
-    miller = {"c": 0, "w": 0, "t": 0, "t4": 0}
+    mb, mg = max(lim["miller_block_max"], lim["miller_warp_max"]), lim["miller_group_min"]
+    miller = {"c": 0, "t": 0, "t4": 0}
     for h in hs:
         n = K * 2 * h
-        e = engine(n, mb, mw)
-        miller["t4" if e == "t" and miller_group(n, h, mg) > 1 else e] += n
+        miller["c" if n <= mb else "t4" if miller_group(n, h, mg) > 1 else "t"] += n
     fe = {"c": 0, "w": 0, "t": 0}
-    fe[engine(1, lim["fe_block_max"], lim["fe_warp_max"])] += 1                  # Commit's one
-    fe[engine(2 * K, lim["fe_block_max"], lim["fe_warp_max"])] += 2 * K * lr     # two per block and round
-    cm = {"c": 0, "w": 0, "t": 0}
-    cm[engine(R, lim["commit_block_max"], lim["commit_warp_max"])] += R
+    fb, fw = lim["fe_block_max"], lim["fe_warp_max"]
+    for n, launches in ((1, 1), (2 * K, lr)):           # Commit's one, then two per block and round
+        e = engine(n, fb, fw)
+        fe["c" if e == "w" and fb and n <= FE_LIMB_MAX else e] += n * launches
+    cm = {"c": 0, "t": 0}
+    cm["c" if R <= max(lim["commit_block_max"], lim["commit_warp_max"]) else "t"] += R
     fw = lim["fold_warp_max"]
     w_terms = K * (2 * R - 2) if not w_msm and R > G2_COMB_MAX_R else 0
     return {
@@ -164,11 +166,9 @@ def step_units(log_n: int, b: int, msm_window: int, msm_window_g2: int = 16, lim
         "k_final_exp_w": ("final_exp", fe["w"]),
         "k_final_exp_t": ("final_exp", fe["t"]),
         "k_round_miller_c": ("miller_loop", miller["c"]),
-        "k_round_miller_w": ("miller_loop", miller["w"]),
         "k_step1_miller_multi": ("miller_loop_multi4", miller["t4"]),
         "k_step1_miller": ("miller_loop", miller["t"]),
         "k_commit_miller_c": ("miller_loop", cm["c"]),
-        "k_commit_miller_w": ("miller_loop", cm["w"]),
         "k_commit_miller": ("miller_loop", cm["t"]),
         "k_sparse_g": ("g1_mul", sum(K * min(b, 2 * h) for h in hs)),
         # folds by comb tables of the round's bases: none (every fold is a scalar multiplication)

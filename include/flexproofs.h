@@ -316,18 +316,17 @@ typedef enum { FP_SCHEDULE_DIRECT = 0, FP_SCHEDULE_LOOKAHEAD = 1 } fp_schedule;
 
 /* Engine choice by size (no counterpart in the paper: how the device work is laid out).  Each launch
  * runs its pairings, final exponentiations, fold points or terms either on a latency engine (one
- * 128-thread block or one warp per item: shortest chain, few items) or on a throughput engine (one
- * thread per item: least total work, many items); every engine computes the same values, so these
- * limits change which kernels run and how fast, never the bytes.  Counts are per launch.
- *   miller_block_max / miller_warp_max   Step-1 Miller loops: <= the larger of the two a block each
- *                                        (profiled as k_round_miller_c up to block_max, as
- *                                        k_round_miller_w above), else a thread each (1024 / 16383)
+ * block with one limb per lane, or one warp, per item: shortest chain, few items) or on a throughput
+ * engine (one thread per item: least total work, many items); every engine computes the same values,
+ * so these limits change which kernels run and how fast, never the bytes.  Counts are per launch.
+ *   miller_block_max / miller_warp_max   Step-1 Miller loops: <= the larger of the two a block each,
+ *                                        else a thread each (1024 / 16383)
  *   miller_group_min                     from this many (and h >= 4), a thread runs 4 pairs of one
  *                                        product with shared squarings (default 2^18); from a
  *                                        quarter of it 1, 2 or 4, whichever fills whole waves best
  *   commit_block_max / commit_warp_max   Commit's R Miller loops, the same way (default 1024 / 16384)
  *   fe_block_max / fe_warp_max           final exponentiations: block / warp / thread (256 / 2^32-1;
- *                                        unless block_max is 0, blocks also up to 912)
+ *                                        unless block_max is 0, blocks also for up to 912 of the warps')
  *   pair_block_max                       pairwise Fq12 products: <= blocks (of up to eight values, in the
  *                                        look-ahead schedule of two), above a thread per pair (2048)
  *   fold_warp_max                        fold points of a round: <= a block (G2) and half a block (G1)

@@ -22,14 +22,14 @@ from . import _lib as F
 
 UNLIMITED = 0xFFFFFFFF
 
-# settings of each group of limits: latency engines up to the default sizes, fewer latency engines,
-# and one thread per item (0: no launch is small enough for a block or a warp)
+# settings of each group of limits, every one launching other kernels somewhere: latency engines up to the
+# default sizes, fewer latency engines, and one thread per item (0: no launch is small enough for a block
+# or a warp).  Miller loops have one latency engine, up to the larger of their two limits.
 GROUPS = {
-    "miller": [{}, {"miller_block_max": 256, "miller_warp_max": 4096}, {"miller_block_max": 0, "miller_warp_max": 0},
-               {"miller_block_max": 0}],
+    "miller": [{}, {"miller_block_max": 256, "miller_warp_max": 4096}, {"miller_block_max": 0, "miller_warp_max": 0}],
     "final_exp": [{}, {"fe_block_max": 0}, {"fe_block_max": 0, "fe_warp_max": 64}, {"fe_block_max": 0, "fe_warp_max": 0}],
     "folds": [{}, {"fold_warp_max": 1024, "wterm_warp_max": 1024}, {"fold_warp_max": 0, "wterm_warp_max": 0}],
-    "commit": [{}, {"commit_block_max": 0}, {"commit_block_max": 0, "commit_warp_max": 0}],
+    "commit": [{}, {"commit_block_max": 0, "commit_warp_max": 0}],
     "pairs": [{}, {"pair_block_max": 256}, {"pair_block_max": 0}],
 }
 MSM_CHUNKS = [1 << 15, 1 << 16, 1 << 17, 1 << 18]

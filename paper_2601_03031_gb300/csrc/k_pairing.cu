@@ -112,8 +112,8 @@ void final_exp_group(const void* in, uint32_t n, void* out, void* ser, uint32_t 
     // limb lanes also beyond the block limit (if there is one) up to six blocks per SM: 512 take 0.8 ms, 1024
     // 1.56 ms; a warp each takes 1.48 ms for 257 to 1024
     if (n <= lim.fe_block_max || (lim.fe_block_max && n <= FE_LIMB_MAX)) {
-        FP_KERNEL(n <= lim.fe_block_max ? "k_final_exp_c" : "k_final_exp_w", s, k_final_exp_c<<<n, L12_THREADS, 0, s>>>((const fq12*)in, n, (fq12*)out, (uint8_t*)ser, per,
-                                                                     stride_a, stride_b));
+        FP_KERNEL("k_final_exp_c", s, k_final_exp_c<<<n, L12_THREADS, 0, s>>>((const fq12*)in, n, (fq12*)out,
+                                                                             (uint8_t*)ser, per, stride_a, stride_b));
         return;
     }
     FP_KERNEL("k_final_exp_w", s, k_final_exp_w<<<(n + 3) / 4, 128, 0, s>>>((const fq12*)in, n, (fq12*)out,
@@ -205,11 +205,10 @@ __global__ void __launch_bounds__(LM_THREADS, 2) k_commit_miller_c(const g1a* ro
     const uint64_t j = blockIdx.x;
     miller_block(rows[j], g2pow[2 * j], &out[j]);
 }
-// (the two names keep the ranges of the engine limits apart in profiles)
-void round_miller_w(const void* A, const void* v, uint32_t K, uint32_t R, uint32_t h, void* out, cudaStream_t s) {
+void round_miller(const void* A, const void* v, uint32_t K, uint32_t R, uint32_t h, void* out, cudaStream_t s) {
     const uint64_t n = (uint64_t)K * 2 * h;
-    FP_KERNEL(n <= engine_limits().miller_block_max ? "k_round_miller_c" : "k_round_miller_w", s,
-              k_round_miller_c<<<(unsigned)n, LM_THREADS, 0, s>>>((const g1a*)A, (const g2a*)v, K, R, h, (fq12*)out));
+    FP_KERNEL("k_round_miller_c", s, k_round_miller_c<<<(unsigned)n, LM_THREADS, 0, s>>>((const g1a*)A, (const g2a*)v, K,
+                                                                                        R, h, (fq12*)out));
 }
 
 void commit_miller(const void* rows, const void* g2pow, uint32_t R, void* out, cudaStream_t s) {
@@ -220,8 +219,8 @@ void commit_miller(const void* rows, const void* g2pow, uint32_t R, void* out, c
                                                                                        (fq12*)out));
         return;
     }
-    FP_KERNEL(R <= lim.commit_block_max ? "k_commit_miller_c" : "k_commit_miller_w", s,
-              k_commit_miller_c<<<R, LM_THREADS, 0, s>>>((const g1a*)rows, (const g2a*)g2pow, (fq12*)out));
+    FP_KERNEL("k_commit_miller_c", s, k_commit_miller_c<<<R, LM_THREADS, 0, s>>>((const g1a*)rows, (const g2a*)g2pow,
+                                                                                (fq12*)out));
 }
 // Pairs per thread of a launch of n pairs.  These kernels hold 255 registers a thread, so the GPU takes
 // 152 x 256 threads at once and a launch costs whole waves: measured per wave 12.6 ms with one pair per

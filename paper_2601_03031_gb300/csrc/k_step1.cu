@@ -524,12 +524,12 @@ uint64_t step1_miller_g(const void* A, const void* v, uint32_t K, uint32_t R, ui
                         cudaStream_t s) {
     uint64_t n = (uint64_t)K * 2 * h;
     const EngineLimits lim = engine_limits();
-    if (n > lim.miller_warp_max && n > lim.miller_block_max) {   // many pairs: threads, less work than warps
+    if (n > lim.miller_warp_max && n > lim.miller_block_max) {   // many pairs: threads, less work in all
         const uint32_t group = step1_miller_group(n, h, lim);
         step1_miller(A, v, K, R, h, group, ml_out, s);
         return n / group;
     }
-    round_miller_w(A, v, K, R, h, ml_out, s);      // few pairs: one warp or block each, for latency
+    round_miller(A, v, K, R, h, ml_out, s);        // few pairs: one block each, for latency
     return n;
 }
 void step1_fold_pre(const void* A, const void* v, uint32_t K, uint32_t R, uint32_t h, void* pre, cudaStream_t s) {

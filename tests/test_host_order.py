@@ -3,6 +3,7 @@
 import ctypes
 import glob
 import os
+import re
 import shutil
 import subprocess
 
@@ -138,8 +139,13 @@ LIMITS = ["miller_block_max", "miller_warp_max", "miller_group_min", "commit_blo
           "fe_warp_max", "pair_block_max", "fold_warp_max", "wterm_warp_max", "msm_chunks", "msm_segment_threads"]
 
 
+def kernel(mangled):
+    m = re.match(r"_ZN3fpk(\d+)", mangled)
+    return mangled[m.end():m.end() + int(m.group(1))] if m else mangled
+
+
 def launches(lib, fn, **limits):
-    """[(kernel's mangled name, grid, block)] of fn() under the given engine limits."""
+    """[(kernel, grid, block)] of fn() under the given engine limits."""
     lim = (u32 * len(LIMITS))()
     lib.fp_engine_limits_default(lim)
     for k, v in limits.items():
@@ -148,7 +154,7 @@ def launches(lib, fn, **limits):
     try:
         lib.fake_reset(ctypes.c_long(-1))
         assert fn() == 0
-        return [(w[0], int(w[1]), int(w[2])) for w in (x.split() for x in lib.fake_log().decode().splitlines())]
+        return [(kernel(w[0]), int(w[1]), int(w[2])) for w in (x.split() for x in lib.fake_log().decode().splitlines())]
     finally:
         lib.fp_set_engine_limits(None)
 
@@ -157,9 +163,39 @@ def launches(lib, fn, **limits):
 def test_fq12_products_keep_to_their_limit(lib, pp, cm, pair_block_max):
     """pair_block_max: rounds with more pairwise products than that run them one per thread."""
     log = launches(lib, lambda: prove_all(lib, pp, cm), pair_block_max=pair_block_max)
-    threads = [g for n, g, _ in log if "k_fq12_pairE" in n]
-    blocks = [g for n, g, _ in log if "k_fq12_prod" in n]
+    threads = [g for n, g, _ in log if n == "k_fq12_pair"]
+    blocks = [g for n, g, _ in log if n == "k_fq12_prod"]
     # R = 16, six blocks of up to 3 rows: 96, 48, 24 and 12 Miller values in the rounds, reduced to 12: halved 3, 2, 1
     # and 0 times, or by eights, fours and twos
     want = {0: (6, 0), 2: (6, 0), 1 << 16: (0, 3)}[pair_block_max]
     assert (len(threads), len(blocks)) == want, (threads, blocks)
+
+
+@pytest.mark.parametrize("limits", [{}, {"miller_block_max": 0, "commit_block_max": 0}, {"fe_block_max": 1},
+                                    {"fe_block_max": 0}, {"fe_block_max": 0, "fe_warp_max": 0},
+                                    {"miller_block_max": 0, "miller_warp_max": 0, "miller_group_min": 64,
+                                     "commit_block_max": 0, "commit_warp_max": 0}])
+def test_pairing_launches_are_profiled_by_the_kernel_that_runs(lib, pp, limits):
+    def work():
+        h, pf = vp(), vp()
+        st = lib.vc_commit(pp, ctypes.create_string_buffer(32 << 8), 0, None, ctypes.byref(h))
+        st = st or lib.vc_prove_all(pp, h, u32(1), None, ctypes.byref(pf))
+        if st == 0:
+            lib.fp_proofs_free(pf)
+            lib.fp_commit_free(h)
+        return st
+
+    def counts(names):
+        return {n: sum(1 for x in names if x == n) for n in names if "miller" in n or "final_exp" in n}
+
+    lib.fp_profile_report.restype = sz
+    buf = ctypes.create_string_buffer(1 << 16)
+    lib.fp_profile_enable(1)
+    try:
+        log = launches(lib, work, **limits)
+    finally:
+        lib.fp_profile_enable(0)
+        lib.fp_profile_report(buf, sz(len(buf)))
+    labels = {w[0]: int(w[1]) for w in (x.split() for x in buf.value.decode().splitlines())
+              if "miller" in w[0] or "final_exp" in w[0]}
+    assert labels == counts([n for n, _, _ in log])
