@@ -186,12 +186,13 @@ __global__ void __launch_bounds__(LEC2_THREADS) k_fold_pre(const g1a* A, const g
 }
 size_t fold_pre_bytes(uint32_t n) { return (size_t)n * (LEC_PRE_INTS + LEC2_PRE_INTS) * sizeof(int32_t); }
 
-// L_j.1 and R_j.1 terms at the support of b only, one block per term (limb_ec.cuh), for the blocks
+// L_j.1 and R_j.1 terms at the support of b only, for the blocks
 // k0 .. k0 + K - 1 (local index k - k0).  Block k's vector b is
 // non-zero only at its statement indices S_k = [k b, k b + |S_k|) folded mod the current length 2h:
 // term t < min(|S_k|, 2h) sits at p = (k b + t) mod 2h (all p < 2h when |S_k| > 2h); p < h is an
 // L_j.1 term b[p] A[h + p], p >= h an R_j.1 term b[p] A[p - h].  Results go to the dense per-block
 // layout out[k 2h + p] (Jacobian), whose other entries the caller has zeroed (Z = 0: identity).
+// Few terms: a block each, one limb per lane (limb_ec.cuh), for the latency the challenge waits for.
 __global__ void __launch_bounds__(LEC_THREADS) k_sparse_g(const g1a* A, const fr* bvec, uint32_t k0, uint32_t K,
                                                           uint32_t R, uint32_t h, uint32_t b, uint32_t cmax,
                                                           g1j* out) {
@@ -207,6 +208,29 @@ __global__ void __launch_bounds__(LEC_THREADS) k_sparse_g(const g1a* A, const fr
     lec_g1_mul(S, c, A[k * R + (p < h ? h + p : p - h)], kw);
     const fq v = lec_jacobian(S, c);
     if (c.k.l == 0 && c.slot < 3) reinterpret_cast<fq*>(&out[k * 2 * h + p])[c.slot] = v;
+}
+// Many terms: 8 lanes each (group_ec.cuh), which issue less per term.  A launch beside the pairings of the same
+// round (one GB300), blocks against groups: 512 terms 0.6 and 0.9 ms, 1024 0.55-0.65 and 1.0, 2048 1.1 and
+// 0.9, 4096 2.0 and 1.1, 8192 3.8 and 2.1.  Whole openings of sub-arrays with the line at 1024 against blocks
+// at every size: 8192 rows in one block 46.8 and 49.9 ms, in 16 blocks 174 and 184, 4096 in one 29.3 and 30.5,
+// 2048 in one 20.8 and 21.1; with the line at 512 1024 rows in one block take 12.1 instead of 12.0.
+constexpr uint64_t SPARSE_LIMB_MAX = 1024;
+__global__ void __launch_bounds__(128) k_sparse_g8(const g1a* A, const fr* bvec, uint32_t k0, uint32_t K, uint32_t R,
+                                                   uint32_t h, uint32_t b, uint32_t cmax, g1j* out) {
+    __shared__ GEc<fq> sm[16];
+    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
+    const uint64_t u = (uint64_t)blockIdx.x * 16 + grp;
+    uint64_t k = u / cmax;
+    uint32_t t = (uint32_t)(u % cmax);
+    bool valid = k < K;
+    uint32_t sk = valid ? min(b, R - (k0 + (uint32_t)k) * b) : 1;
+    valid = valid && t < min(sk, 2 * h);
+    if (!valid) { k = 0; t = 0; sk = min(b, R - k0 * b); }    // idle groups repeat a term, store nothing
+    const uint32_t p = sk <= 2 * h ? (uint32_t)(((uint64_t)(k0 + k) * b + t) % (2 * h)) : t;
+    uint32_t kw[8];
+    fr_canon_words(kw, bvec[k * R + p]);
+    const GPt<fq> r = gec_g1_mul_proj_w2(sm[grp], lane, A[k * R + (p < h ? h + p : p - h)], kw);
+    if (valid && lane == 0) out[k * 2 * h + p] = proj_to_jac(r);
 }
 
 // x_j = HFr("FP-x", x_{j-1} || L_j || R_j) and its inverse, one warp per block: the hash on the warp
@@ -373,8 +397,13 @@ void step1_sparse_terms(const void* A, const void* bvec, uint32_t k0, uint32_t K
                         void* out, cudaStream_t s) {
     const uint32_t cmax = std::min(b, 2 * h);
     cudaMemsetAsync(out, 0, (size_t)K * 2 * h * G1J_BYTES, s);
-    FP_KERNEL("k_sparse_g", s, k_sparse_g<<<(unsigned)((uint64_t)K * cmax), LEC_THREADS, 0, s>>>(
-                                   (const g1a*)A, (const fr*)bvec, k0, K, R, h, b, cmax, (g1j*)out));
+    const uint64_t n = (uint64_t)K * cmax;
+    if (n > SPARSE_LIMB_MAX)
+        FP_KERNEL("k_sparse_g", s, k_sparse_g8<<<grid_for(n, 16), 128, 0, s>>>((const g1a*)A, (const fr*)bvec, k0, K, R, h,
+                                                                              b, cmax, (g1j*)out));
+    else
+        FP_KERNEL("k_sparse_g", s, k_sparse_g<<<(unsigned)n, LEC_THREADS, 0, s>>>((const g1a*)A, (const fr*)bvec, k0, K, R,
+                                                                                 h, b, cmax, (g1j*)out));
 }
 void step1_gt_out(const void* ml, uint32_t K, int j, void* blocks, size_t bopen_len, cudaStream_t s) {
     final_exp_group(ml, 2 * K, nullptr, (uint8_t*)blocks + (size_t)(j - 1) * ROUND_BYTES, 2, bopen_len,

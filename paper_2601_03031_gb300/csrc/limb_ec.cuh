@@ -11,10 +11,11 @@
 // On an 8-lane group with one Fq product per lane (group_ec.cuh) an operation is two rounds of products
 // and about twenty field additions in sequence, 8.6 k cycles; here the additions are lane-wise.
 // A multiplication by k: GLV halves k0, k1 (curve.cuh) in width-4 NAF, P, 3P, 5P, 7P, one accumulator:
-// 128 doublings and ~51 additions.  Alone on the GPU's idle SMs it takes 0.20 ms (8-lane groups: 0.80),
-// about 2.2 k cycles per operation, half of it in the two reductions.  256 of them beside a round's
-// Miller loops take 0.52 ms (1.07), 1024 of them 2.4 ms (1.5: the groups issue less per term, but
-// nothing waits for them at that size, where the pairings take four times as long).
+// 128 doublings and ~51 additions.  Alone on the GPU's idle SMs it takes 0.19 ms (8-lane groups: 0.78),
+// about 2.2 k cycles per operation, half of it in the two reductions.  It issues more than a group does, so with
+// many of them the groups win.  A launch of n multiplications, two per block / one per block / groups, in ms:
+// 512: 0.26 / 0.26 / 0.79, 1024: 0.42 / 0.51 / 0.79, 2048: 0.74 / 0.97 / 0.79, 4096: 1.39 / 1.76 / 0.99,
+// 8192: 2.62 / 3.43 / 1.97, 65536: 20.4 / 26.6 / 13.4.
 #pragma once
 #include "group_ec.cuh"
 #include "limb.cuh"

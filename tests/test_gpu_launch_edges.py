@@ -43,3 +43,26 @@ def test_msm_bucket_count_edge(window):
     pts = b"".join(O.g1_mul(O.g1_gen(), 3 * v + 1) for v in range(n))
     k = I.vector(23, 6)[:n]
     assert F.msm_g1(F.G1Bases(points=pts), k, 1, window) == O.g1_msm(pts, I.to_ints(k))
+
+
+@pytest.mark.parametrize("log_r,b,some", [
+    (11, 37, 8),        # 56 blocks, the last of 13 rows: 2072 terms in the early rounds on 8 lanes each
+    (11, 3, 128),       # 683 blocks: more than 1024 terms also where three rows meet two or four values
+    (11, 2048, 1),      # one block: 2048 terms in the first round alone
+])
+def test_sparse_terms_equal_on_groups_and_blocks(log_r, b, some):
+    """A call over all blocks (more than 1024 terms in a round) against calls over a few of them (at most 1024), or,
+    for one block, the verifier; four rows commit to zeros."""
+    pp = F.PP(log_r + 1, b, 5, log_r=log_r)
+    m = I.vector(17, log_r + 1)
+    m[6:12] = 0
+    m[-2:] = 0
+    cm = F.Commitment(pp, m)
+    C, R, K = cm.get()[0], pp.R, -(-pp.R // b)
+    pf = F.vc_open_segments(pp, cm, b)
+    for k in ([0] if K == 1 else [0, K // 2, K - some]):
+        if K > 1:
+            few = F.vc_open_segments(pp, cm, b, k, some)
+            for j in range(k * b, min((k + some) * b, R), b):
+                assert pf.segment_proof(j) == few.segment_proof(j), j
+        assert F.vc_verify_segment(pp, C, b, k * b, m[2 * k * b:2 * k * b + 2], pf.segment_proof(k * b))

@@ -199,3 +199,27 @@ def test_pairing_launches_are_profiled_by_the_kernel_that_runs(lib, pp, limits):
     labels = {w[0]: int(w[1]) for w in (x.split() for x in buf.value.decode().splitlines())
               if "miller" in w[0] or "final_exp" in w[0]}
     assert labels == counts([n for n, _, _ in log])
+
+
+@pytest.mark.parametrize("log_r,b,groups", [(10, 1024, 0), (11, 2048, 1), (11, 37, 7)])
+def test_many_sparse_terms_take_the_groups(lib, log_r, b, groups):
+    """L_j.1 / R_j.1 terms of a round: a block each up to 1024, above that 8 lanes each (16 terms per block)."""
+    p, h = vp(), vp()
+    assert lib.vc_setup_split(u32(log_r), u32(1), u32(b), u64(1), None, ctypes.byref(p)) == 0
+    assert lib.vc_commit(p, ctypes.create_string_buffer(64 << log_r), 0, None, ctypes.byref(h)) == 0
+
+    def work():
+        pf = vp()
+        st = lib.vc_open_segments(p, h, u32(b), u32(0), u32(0), None, ctypes.byref(pf))
+        if st == 0:
+            lib.fp_proofs_free(pf)
+        return st
+
+    R = 1 << log_r
+    K = -(-R // b)
+    terms = [K * min(b, R >> j) for j in range(log_r)]
+    got = [(g, t) for n, g, t in launches(lib, work) if n.startswith("k_sparse_g")]
+    assert got == [(n, 96) if n <= 1024 else (-(-n // 16), 128) for n in terms]
+    assert sum(n > 1024 for n in terms) == groups
+    lib.fp_commit_free(h)
+    lib.fp_pp_free(p)
