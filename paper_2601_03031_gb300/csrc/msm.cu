@@ -439,6 +439,9 @@ __global__ void __launch_bounds__(MSM_L_GROUPS * LEC_THREADS) k_msm_window_l(Msm
 // per batch, on 96 threads: sum_w 2^(lo_w) S_w by Horner from the top window, S_w the sum of `parts` partial
 // sums (limbs) or one window sum (residues), then affine.  129 doublings and the additions: 0.14 ms for 9 windows
 // of one sum each (an 8-lane group 0.45), 0.30 for a 3000-term sum's windows of several partial sums (0.48).
+// Up to 1024 sums; above, k_msm_final's groups issue less per sum: 256 sums 0.21 and 0.57 ms, 1024 0.57 and
+// 0.61, 1536 0.65 and 0.58, 4096 1.46 and 0.73, 8192 2.78 and 1.44 (one GB300).
+constexpr uint32_t MSM_FINAL_L_MAX = 1024;
 template <typename In>
 __global__ void __launch_bounds__(2 * LEC_THREADS) k_msm_final_l(MsmShape sh, uint32_t parts, const In* win, g1a* out,
                                                                  uint8_t* ser, size_t ser_stride) {
@@ -706,9 +709,11 @@ static void msm_run(const void* bases, const void* k_canon, const MsmShape& sh, 
     }
     FP_KERNEL(g2 ? "k_msm_to_proj_g2" : "k_msm_to_proj", s, k_msm_to_proj<F><<<grid_for(nwin, 128), 128, 0, s>>>(a, proj, nwin));
     if constexpr (!g2) {
-        FP_KERNEL("k_msm_final", s, k_msm_final_l<GPt<fq>><<<(sh.nbatch + 1) / 2, 2 * LEC_THREADS, 0, s>>>(
-                                        sh, 1, proj, (g1a*)out_aff, (uint8_t*)ser_out, ser_stride));
-        return;
+        if (sh.nbatch <= MSM_FINAL_L_MAX) {
+            FP_KERNEL("k_msm_final", s, k_msm_final_l<GPt<fq>><<<(sh.nbatch + 1) / 2, 2 * LEC_THREADS, 0, s>>>(
+                                            sh, 1, proj, (g1a*)out_aff, (uint8_t*)ser_out, ser_stride));
+            return;
+        }
     }
     FP_KERNEL(g2 ? "k_msm_final_g2" : "k_msm_final", s,
               k_msm_final<F><<<grid_for(sh.nbatch, 8), 64, 0, s>>>(sh, proj, (typename Aff<F>::T*)out_aff,

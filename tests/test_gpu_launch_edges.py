@@ -66,3 +66,14 @@ def test_sparse_terms_equal_on_groups_and_blocks(log_r, b, some):
             for j in range(k * b, min((k + some) * b, R), b):
                 assert pf.segment_proof(j) == few.segment_proof(j), j
         assert F.vc_verify_segment(pp, C, b, k * b, m[2 * k * b:2 * k * b + 2], pf.segment_proof(k * b))
+
+
+def test_msm_batches_equal_on_groups_and_blocks():
+    """1025 sums in one call (8 lanes each at the end) against the same sums in two calls (half a block each)."""
+    n, nb = 3, 1025
+    bases = F.G1Bases(points=b"".join(O.g1_mul(O.g1_gen(), 5 * v + 2) for v in range(n)))
+    k = I.fr_uniform(29, n * nb)
+    k[3 * 700:3 * 701] = 0                             # one sum is the identity
+    whole = F.msm_g1(bases, k, nb)
+    assert whole == F.msm_g1(bases, k[:3 * 600], 600) + F.msm_g1(bases, k[3 * 600:], 425)
+    assert whole[:96] == O.g1_msm(b"".join(O.g1_mul(O.g1_gen(), 5 * v + 2) for v in range(n)), I.to_ints(k[:3]))

@@ -223,3 +223,15 @@ def test_many_sparse_terms_take_the_groups(lib, log_r, b, groups):
     assert sum(n > 1024 for n in terms) == groups
     lib.fp_commit_free(h)
     lib.fp_pp_free(p)
+
+
+@pytest.mark.parametrize("nbatch", [1024, 1025])
+def test_many_msm_batches_take_the_groups(lib, nbatch):
+    """Horner over the windows of a sum: half a block each up to 1024 sums, above that 8 lanes each."""
+    lib.fake_reset(ctypes.c_long(-1))
+    bases = vp()
+    assert lib.fp_g1_bases_from_scalars(vp(4096), u64(2), 1, None, ctypes.byref(bases)) == 0
+    log = launches(lib, lambda: lib.fp_msm_g1(bases, vp(4096), u64(2), u32(nbatch), 1, 0, None, vp(8192)))
+    got = [(n, g, t) for n, g, t in log if n.startswith("k_msm_final")]
+    assert got == ([("k_msm_final_l", 512, 192)] if nbatch == 1024 else [("k_msm_final", 129, 64)])
+    lib.fp_g1_bases_free(bases)
