@@ -77,3 +77,20 @@ def test_msm_batches_equal_on_groups_and_blocks():
     whole = F.msm_g1(bases, k, nb)
     assert whole == F.msm_g1(bases, k[:3 * 600], 600) + F.msm_g1(bases, k[3 * 600:], 425)
     assert whole[:96] == O.g1_msm(b"".join(O.g1_mul(O.g1_gen(), 5 * v + 2) for v in range(n)), I.to_ints(k[:3]))
+
+
+@pytest.mark.parametrize("log_c", [11, 12])        # 2047 terms: half a block each; 4095: 8 lanes each
+def test_evaluation_proof_verifies_on_either_side_of_the_term_limit(log_c):
+    """Its PST proofs are the only points that satisfy the oracle's check (pairing by pairing over every level)."""
+    pp = F.PP(1 + log_c, 1, 9, log_r=1)
+    m = I.vector(31, 1 + log_c)
+    m[:1 << (log_c - 1)] = 0                       # and zero factors
+    cm = F.Commitment(pp, m)
+    C = cm.get()[0]
+    for r in (I.to_ints(I.fr_uniform(37, 1 + log_c)), [1] + [0] * log_c):
+        proof = F.vc_eval_prove(pp, cm, r)
+        assert O.eval_verify(O.PP(1 + log_c, 9, log_r=1), C, r, proof)
+        assert F.vc_eval_verify(pp, C, r, proof)
+        bad = bytearray(proof)
+        bad[-1] ^= 1
+        assert not F.vc_eval_verify(pp, C, r, bytes(bad))

@@ -67,7 +67,7 @@ def verify_segment(lib, pp, cm):
 
 def verify_eval(lib, pp, cm):
     n = lib.vc_eval_proof_len(pp)
-    return lib.vc_eval_verify(pp, C, ctypes.create_string_buffer(256), ctypes.create_string_buffer(n), sz(n), None)
+    return lib.vc_eval_verify(pp, C, ctypes.create_string_buffer(1024), ctypes.create_string_buffer(n), sz(n), None)
 
 
 def verify_all(lib, pp, cm):
@@ -114,7 +114,7 @@ def prove_one(lib, pp, cm):
 
 def eval_prove(lib, pp, cm):
     n = lib.vc_eval_proof_len(pp)
-    return lib.vc_eval_prove(pp, cm, ctypes.create_string_buffer(256), None, ctypes.create_string_buffer(n), sz(n),
+    return lib.vc_eval_prove(pp, cm, ctypes.create_string_buffer(1024), None, ctypes.create_string_buffer(n), sz(n),
                              ctypes.byref(sz()))
 
 
@@ -235,3 +235,16 @@ def test_many_msm_batches_take_the_groups(lib, nbatch):
     got = [(n, g, t) for n, g, t in log if n.startswith("k_msm_final")]
     assert got == ([("k_msm_final_l", 512, 192)] if nbatch == 1024 else [("k_msm_final", 129, 64)])
     lib.fp_g1_bases_free(bases)
+
+
+@pytest.mark.parametrize("log_c", [11, 12])
+def test_many_evaluation_proof_terms_take_the_groups(lib, log_c):
+    """The PST terms of an evaluation proof: half a block each up to 2048, above that 8 lanes each."""
+    p, h = vp(), vp()
+    assert lib.vc_setup_split(u32(1), u32(log_c), u32(1), u64(1), None, ctypes.byref(p)) == 0
+    assert lib.vc_commit(p, ctypes.create_string_buffer(64 << log_c), 0, None, ctypes.byref(h)) == 0
+    log = launches(lib, lambda: eval_prove(lib, p, h))
+    assert [x for x in log if x[0].startswith("k_eval_pst_terms")] == \
+        [("k_eval_pst_terms", 1024, 192) if log_c == 11 else ("k_eval_pst_terms8", 256, 128)]
+    lib.fp_commit_free(h)
+    lib.fp_pp_free(p)
