@@ -90,9 +90,7 @@ FPG_DEV bool fq12_decode(const uint8_t* b, fq12& f) {
         if (!fq_from_be48(b + 48 * t, c[t])) return false;
     return true;
 }
-FPG_DEV g1j g1j_neg(const g1j& p) { g1j r = p; r.Y = fq_neg(p.Y); return r; }
 FPG_DEV bool g1a_same(const g1a& a, const g1a& b) { return fq_eq(a.x, b.x) && fq_eq(a.y, b.y); }
-FPG_DEV bool jac_eq(const g1j& p, const g1j& q) { return g1a_same(g1_affine(p), g1_affine(q)); }
 FPG_DEV bool fr_same(const fr& a, const fr& b) {
     for (int w = 0; w < 8; w++)
         if (a.v[w] != b.v[w]) return false;
@@ -115,6 +113,13 @@ FPG_DEV fq g1_lin(LimbEc& S, const LecLane& c, const g1a& P, const fr& k_mont, c
 }
 FPG_DEV void g1_lin_put(const LecLane& c, g1a* out, const fq& v) {
     if (c.k.l == 0 && c.slot < 2) reinterpret_cast<fq*>(out)[c.slot] = v;
+}
+// k P on one 8-lane group (group_ec.cuh); every lane of the warp must call it.  The launches of more than
+// LEC_MULS_MAX multiplications use it: they issue less per multiplication than one limb per lane.
+FPG_DEV GPt<fq> g1_mul8(GEc<fq>& sm, int lane, const g1a& P, const fr& k_mont) {
+    uint32_t kw[8];
+    fr_canon_words(kw, k_mont);
+    return gec_g1_mul_proj_w2(sm, lane, P, kw);
 }
 // k_mont P + sum_h D_h (n <= 16 serialised points at dser + 96 off(h)) into S.acc, on 96 threads; the
 // return value is false on a thread that met a malformed point
@@ -338,6 +343,22 @@ __global__ void __launch_bounds__(LEC2_THREADS) k_vb_muls(VBlk* st, uint32_t nb,
     lec_g1_mul(sm.g1[half], c, tP[t], kw);
     const fq v = lec_jacobian(sm.g1[half], c);
     if (c.k.l == 0 && c.slot < 3) reinterpret_cast<fq*>(&T[t])[c.slot] = v;
+}
+
+// the G1 multiplications of k_vb_muls for many of them: the first `used` slots of every block (the others are
+// cleared by the caller), then g1^beta - z g1 of every block.  One block of 8219 terms (R = 2^13, b = R): 3.4 ms in
+// k_vb_muls, 0.24 + 2.0 with the groups; 1024 blocks of 22 terms: 6.0 ms here
+__global__ void __launch_bounds__(128) k_vb_muls8(const VBlk* st, uint32_t nb, uint32_t tpb, uint32_t used, const g1a* tP,
+                                                  const fr* tk, const g1a* g1beta, g1j* T, g1a* P) {
+    __shared__ GEc<fq> sm[16];
+    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
+    const uint64_t i = (uint64_t)blockIdx.x * 16 + grp, nt = (uint64_t)nb * used;
+    const bool valid = i < nt + nb, term = i < nt;
+    const uint64_t t = term ? i / used * tpb + i % used : 0, q = valid && !term ? i - nt : 0;
+    const GPt<fq> r = g1_mul8(sm[grp], lane, term ? tP[t] : g1_neg_gen(), term ? tk[t] : st[q].z);
+    if (term && lane == 0) T[t] = proj_to_jac(r);
+    const GPt<fq> z = gec_add(sm[grp], lane, r, gec_from_affine_or_inf(g1beta[0].x, g1beta[0].y));
+    if (valid && !term && lane == 0) gec_to_affine(P[3 * q + 1].x, P[3 * q + 1].y, z);
 }
 
 // one block per pair, one limb per lane (limb_miller.cuh)
@@ -639,12 +660,19 @@ void block_transcripts(const VSrc& S, const uint8_t* C_be, const fq12* Cd, Block
     FP_KERNEL("k_vb_gt", side, k_vb_gt<<<2 * S.lr * S.nb, L12_THREADS, 0, side>>>(S, Bb.st, Bb.ge));
     fq12_products(Cd, Bb.ge, 2 * S.lr, 2 * S.lr, Bb.cT, 1, S.nb, side);
 }
-// the terms' multiplications and their sums (c1), and the pairs (at Bb.P / Bb.Q, three per block)
+// the terms' multiplications (`used` of a block's tpb slots) and their sums (c1), and the pairs (at Bb.P / Bb.Q,
+// three per block)
 template <class A>
-void block_muls(const VSrc& S, uint32_t tpb, const g1a* g1beta, BlockBufs<A>& Bb, cudaStream_t s) {
-    const uint64_t nt = (uint64_t)S.nb * tpb;
-    FP_KERNEL("k_vb_muls", s, k_vb_muls<<<(unsigned)(S.nb + (nt + S.nb + 1) / 2), LEC2_THREADS, 0, s>>>(
+void block_muls(const VSrc& S, uint32_t tpb, uint32_t used, const g1a* g1beta, BlockBufs<A>& Bb, cudaStream_t s) {
+    const uint64_t nt = (uint64_t)S.nb * tpb, muls = (uint64_t)S.nb * used + S.nb;
+    const bool groups = muls > LEC_MULS_MAX;
+    FP_KERNEL("k_vb_muls", s, k_vb_muls<<<(unsigned)(S.nb + (groups ? 0 : (nt + S.nb + 1) / 2)), LEC2_THREADS, 0, s>>>(
                                   Bb.st, S.nb, Bb.tP, Bb.tk, nt, g1beta, Bb.T, Bb.P, Bb.Q));
+    if (groups) {
+        cudaMemsetAsync(Bb.T, 0, nt * G1J_BYTES, s);          // Z = 0: the identity
+        FP_KERNEL("k_vb_muls8", s, k_vb_muls8<<<grid_for(muls, 16), 128, 0, s>>>(Bb.st, S.nb, tpb, used, Bb.tP, Bb.tk,
+                                                                                g1beta, Bb.T, Bb.P));
+    }
     g1j* x = Bb.T;
     g1j* y = Bb.T2;
     for (uint64_t n = nt; n > S.nb;) {                   // per-block sums: tpb is a power of two
@@ -668,7 +696,7 @@ void block_checks_front(const VSrc& S, const uint8_t* C_be, const fq12* Cd, cons
     FP_KERNEL("k_vb_terms", s, k_vb_terms<<<grid_for((uint64_t)S.nb * tpb, 64), 64, 0, s>>>(S, Bb.st, Bb.hstmt, tpb, Bb.tP,
                                                                                           Bb.tk, Bb.wt));
     FP_KERNEL("k_vb_scalars", s, k_vb_scalars<<<grid_for(S.nb, 64), 64, 0, s>>>(S, Bb.wt, Bb.st, tpb, 0, Bb.tk));
-    block_muls(S, tpb, g1beta, Bb, s);
+    block_muls(S, tpb, S.b + 2 * (uint32_t)S.lr + 1, g1beta, Bb, s);
 }
 // the inputs of the blocks' two final exponentiations: e(A_l, v_l) and the fast-verification product
 template <class A>
@@ -916,7 +944,7 @@ void verify_eval(const void* proof, const void* C_be, const void* r_be, int log_
     FP_KERNEL("k_ve_terms", s, k_ve_terms<<<grid_for(tpb, 64), 64, 0, s>>>(S, O.Bb.st, O.CF, O.r0, tpb, O.Bb.tP, O.Bb.tk));
     FP_KERNEL("k_ve_wt", s, k_ve_wt<<<grid_for(R, 64), 64, 0, s>>>(S, O.Bb.st, O.w, O.Bb.wt));
     FP_KERNEL("k_vb_scalars", s, k_vb_scalars<<<1, 64, 0, s>>>(S, O.Bb.wt, O.Bb.st, tpb, 1 + 2 * (uint32_t)lr, O.Bb.tk));
-    block_muls(S, tpb, (const g1a*)g1beta, O.Bb, s);
+    block_muls(S, tpb, 2 + 2 * (uint32_t)lr, (const g1a*)g1beta, O.Bb, s);
     FP_KERNEL("k_v_miller", s, k_v_miller<<<3, LM_THREADS, 0, s>>>(O.Bb.P, O.Bb.Q, O.Bb.ml));
     block_fe_inputs(O.Bb, 1, O.Bb.fe_in, s);
     final_exp_group(O.Bb.fe_in, 2, O.Bb.fe_out, nullptr, 1, 0, 0, s);
@@ -980,6 +1008,30 @@ __global__ void __launch_bounds__(2 * LEC_THREADS) k_va_rows(ProofLayout L, cons
     g1_lin_put(c, &Dstar[j], lec_affine(sm[half], c));
 }
 
+// the same on 8 lanes per row, for more than LEC_MULS_MAX rows: R = 2^12 2.4 ms on blocks, 1.4 on groups;
+// R = 2^13 4.7 and 2.8
+__global__ void __launch_bounds__(128) k_va_rows8(ProofLayout L, const uint8_t* roots, const uint8_t* rows_ser,
+                                                  const uint8_t* D_ser, fr* rj, g1a* Dstar, uint32_t* row_bad) {
+    __shared__ GEc<fq> sm[16];
+    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
+    const uint64_t j0 = (uint64_t)blockIdx.x * 16 + grp;
+    const bool valid = j0 < L.R;
+    const uint32_t j = valid ? (uint32_t)j0 : 0;              // idle groups repeat row 0, store nothing
+    const fr r = row_rho(roots, j);
+    g1a Cj;
+    uint32_t bad = g1_decode(rows_ser + 96 * (size_t)j, Cj) ? 0u : 16u;
+    g1j Ds = proj_to_jac(g1_mul8(sm[grp], lane, Cj, r));
+    if (!valid || lane != 0) return;
+    for (int h = 0; h < L.log_r; h++) {
+        g1a D;
+        if (!g1_decode(D_ser + G1_SER * (size_t)(tree_off(L.R, h) + ((j >> h) ^ 1)), D)) bad |= 256u;
+        Ds = g1_madd(Ds, D);
+    }
+    rj[j] = r;
+    Dstar[j] = g1_affine(Ds);
+    row_bad[j] = bad;
+}
+
 // y* = r_j m_i + sum_w g_w[a] of every proof, r_j from the proof's own root
 __global__ void k_va_y(ProofLayout L, const uint64_t* m, const uint8_t* roots, const fr* rj, const fr* g,
                        const uint8_t* mbad, fr* ys) {
@@ -1025,6 +1077,19 @@ __global__ void __launch_bounds__(2 * LEC_THREADS) k_va_colE(const g1a* Dstar, c
     g1_lin_put(c, &E[a], g1_lin(sm[half], c, g1_neg_gen(), ys[a], Dstar[0]));
 }
 
+// the same on 8 lanes each, for more than LEC_MULS_MAX columns: M = 2^13 3.4 ms on blocks, 2.1 on groups;
+// M = 2^16 26.7 and 14.2
+__global__ void __launch_bounds__(128) k_va_colE8(const g1a* Dstar, const fr* ys, uint32_t M, g1a* E) {
+    __shared__ GEc<fq> sm[16];
+    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
+    const uint64_t a0 = (uint64_t)blockIdx.x * 16 + grp;
+    const bool valid = a0 < M;
+    const uint64_t a = valid ? a0 : 0;
+    const GPt<fq> r = gec_add(sm[grp], lane, g1_mul8(sm[grp], lane, g1_neg_gen(), ys[a]),
+                              gec_from_affine_or_inf(Dstar[0].x, Dstar[0].y));
+    if (valid && lane == 0) gec_to_affine(E[a].x, E[a].y, r);
+}
+
 // jobs of the listed proofs irr[q0 .. q0 + nj): E = r_j C_j + sum_w D_w - y* g1, r_j from the
 // proof's own root; one block each
 __global__ void __launch_bounds__(2 * LEC_THREADS) k_va_irrE(ProofLayout L, const uint32_t* irr, uint32_t q0,
@@ -1038,6 +1103,33 @@ __global__ void __launch_bounds__(2 * LEC_THREADS) k_va_irrE(ProofLayout L, cons
     if (threadIdx.x == 0) job_a[q] = (uint32_t)(i % L.M);
     v_point_E(sm, Cj, row_rho(roots + 32 * i, j), ys[i], D_ser, L.log_r,
               [&](int h) { return G1_SER * (size_t)(tree_off(L.R, h) + ((j >> h) ^ 1)); }, &E[q], nullptr);
+}
+
+// the same on 8 lanes each, for more than LEC_MULS_MAX multiplications (two a job): 8192 jobs 8.7 ms on blocks,
+// 4.6 on groups
+__global__ void __launch_bounds__(128) k_va_irrE8(ProofLayout L, const uint32_t* irr, uint32_t q0, uint32_t nj,
+                                                  const uint8_t* roots, const fr* ys, const uint8_t* rows_ser,
+                                                  const uint8_t* D_ser, g1a* E, uint32_t* job_a) {
+    __shared__ GEc<fq> sm[16];
+    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 7;
+    const uint64_t qg = (uint64_t)blockIdx.x * 16 + grp;
+    const bool valid = qg < nj;
+    const uint64_t q = valid ? qg : 0, i = irr[q0 + q];
+    const uint32_t j = (uint32_t)(i / L.M);
+    g1a Cj;
+    g1_decode(rows_ser + 96 * (size_t)j, Cj);         // a bad C_j or D_w fails the row's check
+    const GPt<fq> yg = g1_mul8(sm[grp], lane, g1_neg_gen(), ys[i]);
+    const GPt<fq> rC = g1_mul8(sm[grp], lane, Cj, row_rho(roots + 32 * i, j));
+    const GPt<fq> r = gec_add(sm[grp], lane, rC, yg);
+    if (!valid || lane != 0) return;
+    g1j Ds = proj_to_jac(r);
+    for (int h = 0; h < L.log_r; h++) {
+        g1a D;
+        g1_decode(D_ser + G1_SER * (size_t)(tree_off(L.R, h) + ((j >> h) ^ 1)), D);
+        Ds = g1_madd(Ds, D);
+    }
+    job_a[q] = (uint32_t)(i % L.M);
+    E[q] = g1_affine(Ds);
 }
 
 __global__ void k_va_result(ProofLayout L, const uint32_t* blk_res, const uint32_t* row_bad, const uint8_t* mbad,
@@ -1135,13 +1227,20 @@ uint64_t verify_all(const ProofLayout& L, const void* C_be, const void* m, const
     FP_KERNEL("k_va_paths", side2, k_va_paths<<<grid_for(N, 64), 64, 0, side2>>>(L, md, (const uint8_t*)row_tree,
                                                                        (const uint8_t*)top_tree, rs, Ab.roots,
                                                                        Ab.mbad));
-    FP_KERNEL("k_va_rows", side2, k_va_rows<<<(L.R + 1) / 2, 2 * LEC_THREADS, 0, side2>>>(L, Ab.roots, rs, Ds, Ab.rj, Ab.Dstar,
+    if (L.R > LEC_MULS_MAX)
+        FP_KERNEL("k_va_rows", side2, k_va_rows8<<<grid_for(L.R, 16), 128, 0, side2>>>(L, Ab.roots, rs, Ds, Ab.rj, Ab.Dstar,
+                                                                       Ab.row_bad));
+    else
+        FP_KERNEL("k_va_rows", side2, k_va_rows<<<(L.R + 1) / 2, 2 * LEC_THREADS, 0, side2>>>(L, Ab.roots, rs, Ds, Ab.rj, Ab.Dstar,
                                                                        Ab.row_bad));
     FP_KERNEL("k_va_y", side2, k_va_y<<<grid_for(N), TPB, 0, side2>>>(L, md, Ab.roots, Ab.rj, (const fr*)g, Ab.mbad, Ab.ys));
     FP_KERNEL("k_va_class", side2, k_va_class<<<grid_for(N), TPB, 0, side2>>>(L, Ab.roots, Ab.Dstar, Ab.ys, each, Ab.shared,
                                                                       Ab.irr, Ab.nirr));
     // one PST check per column
-    FP_KERNEL("k_va_colE", side2, k_va_colE<<<(L.M + 1) / 2, 2 * LEC_THREADS, 0, side2>>>(Ab.Dstar, Ab.ys, L.M, J.E));
+    if (L.M > LEC_MULS_MAX)
+        FP_KERNEL("k_va_colE", side2, k_va_colE8<<<grid_for(L.M, 16), 128, 0, side2>>>(Ab.Dstar, Ab.ys, L.M, J.E));
+    else
+        FP_KERNEL("k_va_colE", side2, k_va_colE<<<(L.M + 1) / 2, 2 * LEC_THREADS, 0, side2>>>(Ab.Dstar, Ab.ys, L.M, J.E));
     pst_jobs(L, J, L.M, nullptr, ps, (const g2a*)g2tau, nullptr, 0, Ab.col_res, side2);
     // the checks of all K blocks
     const VSrc S{rs, (size_t)L.b * G1_SER, (const uint8_t*)blocks, L.bopen_len, 0, L.K, L.b, L.R, L.log_r};
@@ -1160,8 +1259,12 @@ uint64_t verify_all(const ProofLayout& L, const void* C_be, const void* m, const
     cudaStreamSynchronize(s);
     for (uint32_t q0 = 0; q0 < nirr; q0 += chunk) {
         const uint32_t nj = std::min(chunk, nirr - q0);
-        FP_KERNEL("k_va_irrE", s, k_va_irrE<<<nj, 2 * LEC_THREADS, 0, s>>>(L, Ab.irr, q0, Ab.roots, Ab.ys, rs,
-                                                                          Ds, J.E, J.a));
+        if (2 * (uint64_t)nj > LEC_MULS_MAX)
+            FP_KERNEL("k_va_irrE", s, k_va_irrE8<<<grid_for(nj, 16), 128, 0, s>>>(L, Ab.irr, q0, nj, Ab.roots, Ab.ys, rs,
+                                                                                 Ds, J.E, J.a));
+        else
+            FP_KERNEL("k_va_irrE", s, k_va_irrE<<<nj, 2 * LEC_THREADS, 0, s>>>(L, Ab.irr, q0, Ab.roots, Ab.ys, rs,
+                                                                              Ds, J.E, J.a));
         pst_jobs(L, J, nj, J.a, ps, (const g2a*)g2tau, Ab.irr, q0, Ab.irr_res, s);
     }
     FP_KERNEL("k_va_result", s, k_va_result<<<grid_for(N), TPB, 0, s>>>(L, Bb.res, Ab.row_bad, Ab.mbad, Ab.shared,

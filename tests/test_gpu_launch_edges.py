@@ -94,3 +94,31 @@ def test_evaluation_proof_verifies_on_either_side_of_the_term_limit(log_c):
         bad = bytearray(proof)
         bad[-1] ^= 1
         assert not F.vc_eval_verify(pp, C, r, bytes(bad))
+
+
+@pytest.mark.parametrize("log_r,log_c,b", [
+    (9, 1, 3),         # 171 blocks of up to 22 terms, the last of two rows: block terms on 8 lanes each
+    (12, 1, 64),       # 4096 rows
+    (1, 12, 2),        # 4096 columns
+    (5, 6, 32),        # everything on half a block each, but the 2048 single checks of `each`
+])
+def test_verify_all_equal_on_groups_and_blocks(log_r, log_c, b):
+    """Acceptance of every proof, by shared and by single checks, against the claimed values that are wrong, and the
+    single verifier (half a block per multiplication) at some positions."""
+    pp = F.PP(log_r + log_c, b, 7, log_r=log_r)
+    m = I.vector(41, log_r + log_c)
+    m[: 1 << log_c] = 0                                # row 0 commits to the identity
+    cm = F.Commitment(pp, m)
+    C = cm.get()[0]
+    pf = F.vc_prove_all(pp, cm, b)
+    claim, wrong = m.copy(), [1, pp.N // 2 + 1, pp.N - 1]
+    for i in wrong:
+        claim[i, 0] ^= 1
+    for each in (False, True):
+        ok, n_ok = F.vc_verify_all(pf, C, claim, each=each)
+        assert n_ok == pp.N - 3 and [i for i in range(pp.N) if not ok[i]] == wrong
+    for i in [0] + wrong:
+        v = I.to_ints(claim[i:i + 1])[0]
+        assert F.vc_verify(pp, C, b, i, v, pf.proof(i)) == (i not in wrong)
+    ok, n_ok = F.vc_verify_all(pf, F.Commitment(pp, claim).get()[0], m)
+    assert n_ok == 0 and not any(ok)

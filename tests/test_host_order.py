@@ -248,3 +248,29 @@ def test_many_evaluation_proof_terms_take_the_groups(lib, log_c):
         [("k_eval_pst_terms", 1024, 192) if log_c == 11 else ("k_eval_pst_terms8", 256, 128)]
     lib.fp_commit_free(h)
     lib.fp_pp_free(p)
+
+
+@pytest.mark.parametrize("log_r,log_c,b,groups", [(5, 6, 32, set()), (9, 1, 3, {"k_vb_muls8"}), (8, 1, 2, {"k_vb_muls8"}),
+                                                  (12, 1, 1024, {"k_vb_muls8", "k_va_rows8"}), (1, 12, 2, {"k_va_colE8"})])
+def test_many_multiplications_of_the_verifier_take_the_groups(lib, log_r, log_c, b, groups):
+    """Block terms, rows and columns: half a block each up to 2048 per launch, above that 8 lanes each."""
+    p, h, pf = vp(), vp(), vp()
+    N = 1 << (log_r + log_c)
+    assert lib.vc_setup_split(u32(log_r), u32(log_c), u32(b), u64(1), None, ctypes.byref(p)) == 0
+    assert lib.vc_commit(p, ctypes.create_string_buffer(32 * N), 0, None, ctypes.byref(h)) == 0
+    assert lib.vc_prove_all(p, h, u32(b), None, ctypes.byref(pf)) == 0
+    log = launches(lib, lambda: lib.vc_verify_all(p, C, ctypes.create_string_buffer(32 * N), 0, pf, 0, None, None, None))
+    K, tpb = -(-(1 << log_r) // b), 1
+    used = b + 2 * log_r + 1
+    while tpb < used:
+        tpb *= 2
+    at = {n: g for n, g, _ in log}
+    assert {n for n in at if n in ("k_vb_muls8", "k_va_rows8", "k_va_colE8")} == groups
+    assert at["k_vb_muls"] == K + (0 if "k_vb_muls8" in groups else (K * tpb + K + 1) // 2)
+    if "k_vb_muls8" in groups:
+        assert at["k_vb_muls8"] == -(-(K * used + K) // 16)
+    assert at.get("k_va_rows8") == ((1 << log_r) // 16 if "k_va_rows8" in groups else None)
+    assert at.get("k_va_colE8") == ((1 << log_c) // 16 if "k_va_colE8" in groups else None)
+    lib.fp_proofs_free(pf)
+    lib.fp_commit_free(h)
+    lib.fp_pp_free(p)
