@@ -100,6 +100,7 @@ def test_evaluation_proof_verifies_on_either_side_of_the_term_limit(log_c):
     (9, 1, 3),         # 171 blocks of up to 22 terms, the last of two rows: block terms on 8 lanes each
     (12, 1, 64),       # 4096 rows
     (1, 12, 2),        # 4096 columns
+    (1, 14, 2),        # 16384 columns: products of a thread each
     (5, 6, 32),        # everything on half a block each, but the 2048 single checks of `each`
 ])
 def test_verify_all_equal_on_groups_and_blocks(log_r, log_c, b):
