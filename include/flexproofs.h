@@ -336,7 +336,8 @@ typedef enum { FP_SCHEDULE_DIRECT = 0, FP_SCHEDULE_LOOKAHEAD = 1 } fp_schedule;
  *   msm_chunks                           MSM bucket pass: about this many chunks of the sorted entry
  *                                        list, one thread each (2^17; > 0)
  *   msm_segment_threads                  MSM bucket reduction: at most about this many segment
- *                                        threads (2^15; > 0)
+ *                                        threads (2^15; > 0); G1 sums with at most 16384 buckets in
+ *                                        all are reduced by blocks instead
  * A process-wide setting read when a call enqueues its work (set it between calls: a call enqueued
  * concurrently may see either setting).  fp_set_engine_limits(NULL) restores the defaults;
  * FP_EINVAL for a zero msm_chunks or msm_segment_threads. */

@@ -127,8 +127,9 @@ __global__ void __launch_bounds__(64) k_round_g1_out(const g1j* sp, uint32_t K, 
 // Latency-bound up to about one block per SM: 0.155 ms for 1 to 64 points and 0.19 for 128 from tables of the
 // bases' shifts formed beside the round's pairings (k_fold_pre, 0.13 ms), 0.25 and 0.31 without them; 0.79 ms
 // for 512 points, 2.8 for 2048, 5.5 for 4096 (one GB300).  A warp per G2 point and 8 lanes per G1 point took
-// 1.21 ms for 512 points and 6.1 for 4096; one thread per point (k_fold) takes 4.5 ms for 8192, which is where
-// the default limit leaves off.  Full comb tables of the bases (0.16 ms for 64 points after the challenge)
+// 1.21 ms for 512 points and 6.1 for 4096.  One thread per point (k_fold) takes 4.2 ms for any number up to 8192
+// and 5.7 for 16384, so the two meet at about 3200 points: the default limit is right for 2048 points (2.8) and
+// 8192 (10.7), and 1.2 ms dear at 4096 (5.4), which a fold_warp_max of 3000 saves.  Full comb tables of the bases (0.16 ms for 64 points after the challenge)
 // took 0.96 ms of chains and tables per round beside the pairings.
 union FoldSmemW {
     LimbEc2 g2;

@@ -616,7 +616,9 @@ size_t msm_scratch_bytes_g2(const MsmShape& sh) { return scratch_bytes<fq2>(sh);
 // Window size from a cost model: per phase the larger of the throughput time (about 1.9e10 Fq
 // products/s over the GPU) and the latency of one thread's dependent chain (about 2.7 us per
 // product); mixed addition 10 field products, addition 14, group doubling/addition about
-// 2 x 1.5 (fmul = Fq products per field product: 1 on G1, 3 on G2).
+// 2 x 1.5 (fmul = Fq products per field product: 1 on G1, 3 on G2).  The rates are those of products with
+// separate half chains (now 3.0e10 and about 1 us) and the phases those of the thread and 8-lane kernels: it does
+// not know the limb-lane reduction of at most MSM_L_MAX buckets.  fp_msm_autotune times the windows around its choice.
 int msm_window_model(uint64_t n, uint32_t nbatch, int parts, int part_bits, double fmul) {
     const double tp = fmul / 1.9e10, lat = fmul * 2.7e-6;
     int best = 8;
