@@ -25,7 +25,7 @@ def lib(tmp_path_factory):
     if any(not os.path.exists(o) for o in objs):
         B.build(force=True)
     out = str(tmp_path_factory.mktemp("fake") / "libfake.so")
-    subprocess.check_call([gxx, "-std=c++17", "-O1", "-shared", "-fPIC", f"-I{inc}", "-o", out,
+    subprocess.check_call([gxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", f"-I{inc}", "-o", out,
                            os.path.join(ROOT, "tests", "emu", "fake_cudart.cpp"), *objs])
     L = ctypes.CDLL(out)
     for f in ("fake_event_calls", "fake_bad_frees", "fake_late_launches"):
