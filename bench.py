@@ -108,7 +108,10 @@ G2_COMB_MAX_R = 1024          # setups with R <= this keep the W proofs' comb ta
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu capture of the
 # kernel at this workload, keyed by (log N, b, kernel); an entry is removed when its kernel changes
-NCU_TRAFFIC = {}
+# (profiles/dram_traffic_proveall_n16_b256.md: means over the step's launches)
+NCU_TRAFFIC = {(16, 256, "k_lamc_sum"): 301.7e6, (16, 256, "k_fold_w"): 829.6e3, (16, 256, "k_pst_terms"): 243.7e3,
+               (16, 256, "k_commit_miller_c"): 1243.4e3, (16, 256, "k_round_miller_c"): 257.9e3,
+               (16, 256, "k_final_exp_c"): 92.5e3}
 
 
 FE_LIMB_MAX = 6 * 152         # final exponentiations on blocks although warps are allowed
