@@ -390,7 +390,8 @@ FPG_NOINL GPt<fq> gec_g1_dbl_n(GEcs<fq>& sm, int lane, GPt<fq> acc, int n) {
 // doublings can run ahead: with B_w = 4^w P (G1, two bits of each GLV half per window) or
 // B_i = 2^i Q (G2, one bit of each GLS digit per position) and a table of the window's or
 // position's 16 combinations, k P is the sum of one table entry per window, and the additions of
-// that sum are independent of each other.
+// that sum are independent of each other.  The kernels use the G2 tables (the W proofs); the G1 tables and
+// gec_to_affine_quad are run by the host emulation's tests alone.
 // ---------------------------------------------------------------------------------------
 // -phi(P) = (omega X : -Y : Z) for a projective P on G1 (phi: (x, y) -> (omega x, y))
 FPG_DEV GPt<fq> gec_g1_mphi(const GPt<fq>& P) {

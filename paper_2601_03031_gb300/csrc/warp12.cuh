@@ -4,7 +4,9 @@
 // whatever their dependency structure, so a single lane cannot make one faster; what shortens a
 // chain of Fq12 operations is doing all of an operation's products at once.  (Where a launch is a few
 // blocks, a value with one limb per lane is faster still: limb12.cuh and limb_miller.cuh run the final
-// exponentiations and Miller loops that this file's blocks ran.)  Values
+// exponentiations and Miller loops that this file's blocks ran.  Kernels use the final exponentiation on a warp,
+// and on a block the Miller loop, products and squarings of the look-ahead schedule; the Miller loop on a warp
+// and the final exponentiation on a block are run by the host emulation's tests alone.)  Values
 // live in shared memory, flat as Fq2[w]/(w^6 - xi) (xi = 1 + u): Fq index 2k + e holds component
 // e (0 = real, 1 = u) of the coefficient of w^k, k = 0..5 (w^2 = v, so flat k = 0,2,4 are the tower's
 // c0.c0, c0.c1, c0.c2 and k = 1,3,5 are c1.c0, c1.c1, c1.c2).  Every operation is
