@@ -347,7 +347,9 @@ __global__ void __launch_bounds__(LEC2_THREADS) k_vb_muls(VBlk* st, uint32_t nb,
 
 // the G1 multiplications of k_vb_muls for many of them: the first `used` slots of every block (the others are
 // cleared by the caller), then g1^beta - z g1 of every block.  One block of 8219 terms (R = 2^13, b = R): 3.4 ms in
-// k_vb_muls, 0.24 + 2.0 with the groups; 1024 blocks of 22 terms: 6.0 ms here
+// k_vb_muls, 0.24 + 2.0 with the groups; of 4123 terms 1.76 and 0.24 + 1.03, of 2074 terms 1.02 and 0.24 + 0.83 (the G2 part
+// is a launch of its own then, so the line lies a little higher); 1024 blocks of 22 terms: 6.0 ms here
+constexpr uint64_t VB_BLOCKS_MAX = LEC_MULS_MAX + 256;
 __global__ void __launch_bounds__(128) k_vb_muls8(const VBlk* st, uint32_t nb, uint32_t tpb, uint32_t used, const g1a* tP,
                                                   const fr* tk, const g1a* g1beta, g1j* T, g1a* P) {
     __shared__ GEc<fq> sm[16];
@@ -677,7 +679,7 @@ void block_transcripts(const VSrc& S, const uint8_t* C_be, const fq12* Cd, Block
 template <class A>
 void block_muls(const VSrc& S, uint32_t tpb, uint32_t used, const g1a* g1beta, BlockBufs<A>& Bb, cudaStream_t s) {
     const uint64_t nt = (uint64_t)S.nb * tpb, muls = (uint64_t)S.nb * used + S.nb;
-    const bool groups = muls > LEC_MULS_MAX;
+    const bool groups = muls > VB_BLOCKS_MAX;
     FP_KERNEL("k_vb_muls", s, k_vb_muls<<<(unsigned)(S.nb + (groups ? 0 : (nt + S.nb + 1) / 2)), LEC2_THREADS, 0, s>>>(
                                   Bb.st, S.nb, Bb.tP, Bb.tk, nt, g1beta, Bb.T, Bb.P, Bb.Q));
     if (groups) {

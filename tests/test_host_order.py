@@ -250,12 +250,12 @@ def test_many_evaluation_proof_terms_take_the_groups(lib, log_c):
     lib.fp_pp_free(p)
 
 
-@pytest.mark.parametrize("log_r,log_c,b,groups", [(5, 6, 32, set()), (9, 1, 3, {"k_vb_muls8"}), (8, 1, 2, {"k_vb_muls8"}),
+@pytest.mark.parametrize("log_r,log_c,b,groups", [(5, 6, 32, set()), (11, 1, 2048, set()), (9, 1, 3, {"k_vb_muls8"}), (8, 1, 2, {"k_vb_muls8"}),
                                                   (12, 1, 1024, {"k_vb_muls8", "k_va_rows8"}), (1, 12, 2, {"k_va_colE8"}),
                                                   (1, 13, 2, {"k_va_colE8"}), (1, 14, 2, {"k_va_colE8", "k_vp_prod"})])
 def test_many_multiplications_of_the_verifier_take_the_groups(lib, log_r, log_c, b, groups):
-    """Block terms, rows and columns: half a block each up to 2048 per launch, above that 8 lanes each; a column's
-    product of pairings on a block up to 8192 of them, above that on a thread."""
+    """Rows and columns: half a block each up to 2048 per launch, block terms up to 2304, above that 8 lanes each; a
+    column's product of pairings on a block up to 8192 of them, above that on a thread."""
     p, h, pf = vp(), vp(), vp()
     N = 1 << (log_r + log_c)
     assert lib.vc_setup_split(u32(log_r), u32(log_c), u32(b), u64(1), None, ctypes.byref(p)) == 0
